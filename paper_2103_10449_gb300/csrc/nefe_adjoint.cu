@@ -669,14 +669,15 @@ int nefe_sw_dual(const double* x, const double* w, int n, const double box[3], d
     double* part = nullptr;
     unsigned* err = nullptr;
     const int nb = ad_blocks(n);
-    NEFE_CU(cudaMallocAsync(&part, sizeof(double) * kRed * (size_t)(nb > 0 ? nb : 1), s));
-    NEFE_CU(cudaMallocAsync(&err, sizeof(unsigned), s));
+    Scratch1 S;
+    S.s = s;
+    S.want(&part, sizeof(double) * kRed * (size_t)(nb > 0 ? nb : 1));
+    S.want(&err, sizeof(unsigned));
+    NEFE_CU(S.commit());
     NEFE_CU(cudaMemsetAsync(err, 0, sizeof(unsigned), s));
     launch_sw_ad(x, w, n, box, nbr, cnt, cap, *prm, dtheta, true, f, fd, part, out16, err, s);
     unsigned e = 0;
     NEFE_CU(cudaMemcpyAsync(&e, err, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(part, s);
-    cudaFreeAsync(err, s);
     NEFE_CU(cudaStreamSynchronize(s));
     NEFE_CU(cudaGetLastError());
     if (e & NEFE_ERR_SHELL_OVERFLOW) return fail(NEFE_EOVERFLOW, "nefe_sw_dual: shell above 32 neighbours");
@@ -713,7 +714,8 @@ int nefe_adjoint_create(nefe_adj** out, int device, void* stream, const nefe_adj
     const int n = A->n;
     const size_t b3 = sizeof(double) * 3 * (size_t)n;
     auto bail = [&](int code) { cudaStreamSynchronize(A->s); delete A; return code; };
-    if ((rc = prepare1(A->L, n, d->box, rcs, (int)total, NEFE_FP32, true))) return bail(rc);
+    want1(A->L, n, n3, NEFE_FP32, true);
+    if ((rc = commit1(A->L, n, d->box, rcs, n3, NEFE_FP32))) return bail(rc);
     A->lb = bufs_of(A->L, nullptr, n);
     double** arrs[] = {&A->x0, &A->v0, &A->x, &A->v, &A->F, &A->vh, &A->fsw, &A->fswd, &A->X, &A->V, &A->Fd,
                        &A->VH, &A->xb, &A->vb, &A->fb, &A->w, &A->xi};

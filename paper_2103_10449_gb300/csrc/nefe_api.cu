@@ -1,7 +1,9 @@
 // Stateless C-ABI entry points of libnefe (caller-owned device buffers) and error reporting.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "nefe.h"
@@ -48,12 +50,101 @@ int check_box(const double box[3], double rcs) {
     return NEFE_OK;
 }
 
-int prepare1(Scratch1& S, int n, const double box[3], double rcs, int ncell_cap, int prec,
-                    bool cells, const nefe_uf_params* uf, double skin) {
+// The library's scratch pool of a device.  The default pool hands its memory back to the driver
+// at every synchronisation, so each call mapped its scratch anew (457 -> 207 us for a waited-for
+// list and force call of 1723 atoms); this one keeps up to kScratchKeep bytes mapped between calls
+// (anything above goes back at the next synchronisation).  Allocation and release are stream
+// ordered, so calls on several streams and threads share it safely.
+constexpr uint64_t kScratchKeep = 256ull << 20;
+constexpr int kPoolDevices = 64;
+
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pool[kPoolDevices] = {};
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+    *p = nullptr;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= kPoolDevices) return cudaMallocAsync(p, bytes < 16 ? 16 : bytes, s);
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (!g_pool[dev]) {
+            cudaMemPoolProps props;
+            std::memset(&props, 0, sizeof(props));
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            if ((e = cudaMemPoolCreate(&g_pool[dev], &props)) != cudaSuccess) {
+                g_pool[dev] = nullptr;
+                return e;
+            }
+            uint64_t keep = kScratchKeep;
+            e = cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) return e;
+        }
+        pool = g_pool[dev];
+    }
+    return cudaMallocFromPoolAsync(p, bytes < 16 ? 16 : bytes, pool, s);
+}
+
+namespace {
+struct SwcBytes {
+    alignas(16) unsigned char b[sizeof(SWc<double>)];
+};
+
+__device__ __forceinline__ void copy_words(void* dst, const void* src, int bytes, int t) {
+    if (4 * t < bytes) static_cast<unsigned*>(dst)[t] = static_cast<const unsigned*>(src)[t];
+}
+
+__global__ void __launch_bounds__(256) k_scratch_init(const __grid_constant__ DevSys hs, const __grid_constant__ DevState st,
+                                                      const __grid_constant__ SwcBytes swc, DevSys* dsys, DevState* dst,
+                                                      void* dswc, int* tile_sys, int ntiles, long long* acc, int nacc,
+                                                      int* counts, int ncells) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    static_assert(sizeof(DevSys) <= 1024 && sizeof(DevState) <= 1024, "one word per thread of the first block");
+    copy_words(dsys, &hs, (int)sizeof(hs), t);
+    copy_words(dst, &st, (int)sizeof(st), t);
+    copy_words(dswc, &swc, (int)sizeof(swc), t);
+    for (int i = t; i < ntiles; i += stride) tile_sys[i] = 0;
+    for (int i = t; i < nacc; i += stride) acc[i] = 0;
+    for (int i = t; i < ncells; i += stride) counts[i] = 0;
+}
+}  // namespace
+
+void want1(Scratch1& S, int n, const int n3[3], int prec, bool cells) {
+    const size_t ntiles = (size_t)(n + kTile - 1) / kTile, N = (size_t)n;
+    S.ncells = cells ? n3[0] * n3[1] * n3[2] : 0;
+    S.want(&S.sys, sizeof(DevSys));
+    S.want(&S.st, sizeof(DevState));
+    S.want(&S.tile_sys, sizeof(int) * (ntiles > 0 ? ntiles : 1));
+    S.want(&S.acc, sizeof(long long) * ACC_N * kSlots);
+    S.want(&S.swc, sizeof(SwcBytes));
+    const size_t v4 = prec == NEFE_FP64 ? sizeof(double4) : sizeof(float4);
+    S.want(&S.xs, v4 * N);
+    if (cells) {
+        const size_t C = (size_t)S.ncells;
+        S.want(&S.xa, v4 * N);
+        S.want(&S.xcs, v4 * N);
+        S.want(&S.q, sizeof(int4) * N);
+        S.want(&S.cell_of, sizeof(int) * N);
+        S.want(&S.perm, sizeof(int) * N);
+        S.want(&S.cell_start, sizeof(int) * (C + 1));
+        S.want(&S.cell_count, sizeof(int) * C);
+        S.want(&S.cell_cursor, sizeof(int) * C);
+        S.want(&S.scan_sums, sizeof(int) * 1024);
+    }
+}
+
+int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3], int prec,
+            const nefe_sw_params* prm, const nefe_uf_params* uf, double skin) {
     const int ntiles = (n + kTile - 1) / kTile;
     DevSys hs;
     std::memset(&hs, 0, sizeof(hs));
-    hs.off = 0; hs.n = n; hs.tile0 = 0; hs.ntile = ntiles; hs.cell0 = 0; hs.ncell_cap = ncell_cap;
+    hs.off = 0; hs.n = n; hs.tile0 = 0; hs.ntile = ntiles; hs.cell0 = 0;
+    hs.ncell_cap = n3[0] * n3[1] * n3[2];
     hs.rcs = rcs; hs.pair = -1; hs.prm = 0; hs.mass_e = 1.0;
     hs.rcs2_lo_f = (float)(rcs * rcs) * (1.0f - 1e-4f);
     hs.rcs2_hi_f = (float)(rcs * rcs) * (1.0f + 1e-4f);
@@ -63,30 +154,24 @@ int prepare1(Scratch1& S, int n, const double box[3], double rcs, int ncell_cap,
     }
     DevState st;
     std::memset(&st, 0, sizeof(st));
-    for (int k = 0; k < 3; ++k) st.box[k] = box[k];
+    set_grid(st, box, n3);
     st.rebuild = 1;
     st.scale_int = 1.0;
-    NEFE_CU(S.alloc(&S.sys, sizeof(DevSys)));
-    NEFE_CU(S.alloc(&S.st, sizeof(DevState)));
-    NEFE_CU(S.alloc(&S.tile_sys, sizeof(int) * (size_t)(ntiles > 0 ? ntiles : 1)));
-    NEFE_CU(S.alloc(&S.acc, sizeof(long long) * ACC_N * kSlots));
-    NEFE_CU(cudaMemcpyAsync(S.sys, &hs, sizeof(hs), cudaMemcpyHostToDevice, S.s));
-    NEFE_CU(cudaMemcpyAsync(S.st, &st, sizeof(st), cudaMemcpyHostToDevice, S.s));
-    NEFE_CU(cudaMemsetAsync(S.tile_sys, 0, sizeof(int) * (size_t)(ntiles > 0 ? ntiles : 1), S.s));
-    NEFE_CU(cudaMemsetAsync(S.acc, 0, sizeof(long long) * ACC_N * kSlots, S.s));
-    const size_t v4 = prec == NEFE_FP64 ? sizeof(double4) : sizeof(float4);
-    NEFE_CU(S.alloc(&S.xs, v4 * (size_t)n));
-    if (cells) {
-        NEFE_CU(S.alloc(&S.xa, v4 * (size_t)n));
-        NEFE_CU(S.alloc(&S.xcs, v4 * (size_t)n));
-        NEFE_CU(S.alloc(&S.q, sizeof(int4) * (size_t)n));
-        NEFE_CU(S.alloc(&S.cell_of, sizeof(int) * (size_t)n));
-        NEFE_CU(S.alloc(&S.perm, sizeof(int) * (size_t)n));
-        NEFE_CU(S.alloc(&S.cell_start, sizeof(int) * (size_t)(ncell_cap + 1)));
-        NEFE_CU(S.alloc(&S.cell_count, sizeof(int) * (size_t)ncell_cap));
-        NEFE_CU(S.alloc(&S.cell_cursor, sizeof(int) * (size_t)ncell_cap));
-        NEFE_CU(cudaMemsetAsync(S.cell_count, 0, sizeof(int) * (size_t)ncell_cap, S.s));
+    SwcBytes sw;
+    std::memset(&sw, 0, sizeof(sw));
+    if (prm && prec == NEFE_FP64) {
+        const SWc<double> c = make_swc<double>(*prm);
+        std::memcpy(sw.b, &c, sizeof(c));
+    } else if (prm) {
+        const SWc<float> c = make_swc<float>(*prm);
+        std::memcpy(sw.b, &c, sizeof(c));
     }
+    NEFE_CU(S.commit());
+    const int nacc = ACC_N * kSlots;
+    const int work = std::max(std::max(ntiles, S.ncells), nacc);
+    k_scratch_init<<<std::min((work + 255) / 256, 608), 256, 0, S.s>>>(
+        hs, st, sw, S.sys, S.st, S.swc, S.tile_sys, ntiles, S.acc, nacc, S.cell_count, S.ncells);
+    NEFE_CU(cudaGetLastError());
     return NEFE_OK;
 }
 
@@ -99,12 +184,29 @@ Bufs bufs_of(const Scratch1& S, const double* x, int n) {
     b.shd = S.shd; b.shj = S.shj; b.shn = S.shn; b.P = S.P;
     b.cell_start = S.cell_start; b.cell_count = S.cell_count; b.cell_cursor = S.cell_cursor;
     b.ntot = n; b.swc = S.swc;
+    b.scan_sums = S.scan_sums; b.ncells_host = S.ncells;
     return b;
 }
 
 }  // namespace nefe
 
 using namespace nefe;
+
+// The call's error word, after its work on the stream.
+static int read_error(const Scratch1& S, unsigned* err) {
+    NEFE_CU(cudaMemcpyAsync(err, &S.st->err, sizeof(*err), cudaMemcpyDeviceToHost, S.s));
+    NEFE_CU(cudaStreamSynchronize(S.s));
+    return NEFE_OK;
+}
+
+// The shells, leg forces and partial forces of the two force passes.
+static void want_shells(Scratch1& S, int n, int precision) {
+    const size_t v4 = precision == NEFE_FP64 ? sizeof(double4) : sizeof(float4), N = (size_t)n;
+    S.want(&S.shd, v4 * N * kShell);
+    S.want(&S.shj, sizeof(int) * N * kShell);
+    S.want(&S.shn, sizeof(int) * N);
+    S.want(&S.P, 3 * v4 * N);
+}
 
 extern "C" {
 
@@ -133,15 +235,17 @@ int nefe_cell_bin(const double* x, int n, const double box[3], double rcs, int n
     for (int k = 0; k < 3; ++k) ncell3[k] = n3[k];
     Scratch1 S;
     S.s = (cudaStream_t)stream;
-    rc = prepare1(S, n, box, rcs, (int)total, NEFE_FP32, true);
-    if (rc) return rc;
     if (n == 0) {
         NEFE_CU(cudaMemsetAsync(cell_start, 0, sizeof(int) * (size_t)(total + 1), S.s));
         return NEFE_OK;
     }
+    want1(S, n, n3, NEFE_FP32, true);
+    rc = commit1(S, n, box, rcs, n3, NEFE_FP32);
+    if (rc) return rc;
     Bufs b = bufs_of(S, x, n);
     b.cell_of = cell_of; b.perm = perm; b.cell_start = cell_start;
     launch_cells(b, NEFE_FP32, (n + kTile - 1) / kTile, 1, 1, S.s, nullptr);
+    launch_cells_sort(b, (int)total, S.s);
     NEFE_CU(cudaGetLastError());
     return NEFE_OK;
 }
@@ -162,16 +266,16 @@ int nefe_neighbor_build(const double* x, int n, const double box[3], double rcs,
     if (total > (1LL << 30)) return fail(NEFE_EINVAL, "nefe_neighbor_build: cell grid too large");
     Scratch1 S;
     S.s = (cudaStream_t)stream;
-    rc = prepare1(S, n, box, rcs, (int)total, NEFE_FP32, true);
+    want1(S, n, n3, NEFE_FP32, true);
+    rc = commit1(S, n, box, rcs, n3, NEFE_FP32);
     if (rc) return rc;
     Bufs b = bufs_of(S, x, n);
     b.nbr = nbr; b.cnt = cnt; b.cap = cap;
     launch_cells_and_list(b, NEFE_FP32, (n + kTile - 1) / kTile, 1, 1, S.s, nullptr);
     NEFE_CU(cudaGetLastError());
-    DevState st;
-    NEFE_CU(cudaMemcpyAsync(&st, S.st, sizeof(st), cudaMemcpyDeviceToHost, S.s));
-    NEFE_CU(cudaStreamSynchronize(S.s));
-    const int ovf = (st.err & NEFE_ERR_NBR_OVERFLOW) ? 1 : 0;
+    unsigned err = 0;
+    if ((rc = read_error(S, &err))) return rc;
+    const int ovf = (err & NEFE_ERR_NBR_OVERFLOW) ? 1 : 0;
     if (overflow) *overflow = ovf;
     if (ovf) return fail(NEFE_EOVERFLOW, "nefe_neighbor_build: a row exceeded cap %d", cap);
     return NEFE_OK;
@@ -190,26 +294,13 @@ int nefe_sw_forces(const double* x, int n, const double box[3], double rcs, cons
     if (shell_overflow) *shell_overflow = 0;
     int n3[3];
     if (!host_grid(box, rcs, n3)) return fail(NEFE_EINVAL, "nefe_sw_forces: fewer than 2 cells on an axis");
-    const long long total = (long long)n3[0] * n3[1] * n3[2];
+    cap_grid(n3, 1LL << 30);
     Scratch1 S;
     S.s = (cudaStream_t)stream;
-    rc = prepare1(S, n, box, rcs, (int)(total > (1LL << 30) ? (1LL << 30) : total), precision, false);
-    if (rc) return rc;
-    if (precision == NEFE_FP64) {
-        SWc<double> c = make_swc<double>(*prm);
-        NEFE_CU(S.alloc(&S.swc, sizeof(c)));
-        NEFE_CU(cudaMemcpyAsync(S.swc, &c, sizeof(c), cudaMemcpyHostToDevice, S.s));
-    } else {
-        SWc<float> c = make_swc<float>(*prm);
-        NEFE_CU(S.alloc(&S.swc, sizeof(c)));
-        NEFE_CU(cudaMemcpyAsync(S.swc, &c, sizeof(c), cudaMemcpyHostToDevice, S.s));
-    }
+    want1(S, n, n3, precision, false);
+    want_shells(S, n, precision);
+    if ((rc = commit1(S, n, box, rcs, n3, precision, prm))) return rc;
     if (n > 0) {
-        const size_t v4 = precision == NEFE_FP64 ? sizeof(double4) : sizeof(float4);
-        NEFE_CU(S.alloc(&S.shd, v4 * (size_t)n * kShell));
-        NEFE_CU(S.alloc(&S.shj, sizeof(int) * (size_t)n * kShell));
-        NEFE_CU(S.alloc(&S.shn, sizeof(int) * (size_t)n));
-        NEFE_CU(S.alloc(&S.P, 3 * v4 * (size_t)n));
         Bufs b = bufs_of(S, x, n);
         b.nbr = const_cast<int*>(nbr); b.cnt = const_cast<int*>(cnt); b.cap = cap;
         b.f_out = f; b.e_atom = e_atom;
@@ -222,10 +313,9 @@ int nefe_sw_forces(const double* x, int n, const double box[3], double rcs, cons
     if (energy_virial) launch_decode_ev(S.acc, energy_virial, S.s);
     NEFE_CU(cudaGetLastError());
     if (shell_overflow) {
-        DevState st;
-        NEFE_CU(cudaMemcpyAsync(&st, S.st, sizeof(st), cudaMemcpyDeviceToHost, S.s));
-        NEFE_CU(cudaStreamSynchronize(S.s));
-        *shell_overflow = (st.err & NEFE_ERR_SHELL_OVERFLOW) ? 1 : 0;
+        unsigned err = 0;
+        if ((rc = read_error(S, &err))) return rc;
+        *shell_overflow = (err & NEFE_ERR_SHELL_OVERFLOW) ? 1 : 0;
         if (*shell_overflow) return fail(NEFE_EOVERFLOW, "nefe_sw_forces: shell above 32 neighbours");
     }
     return NEFE_OK;
@@ -243,28 +333,15 @@ int nefe_sw_energy_grad(const double* x, int n, const double box[3], double rcs,
     if (rc) return rc;
     int n3[3];
     if (!host_grid(box, rcs, n3)) return fail(NEFE_EINVAL, "nefe_sw_energy_grad: fewer than 2 cells on an axis");
-    const long long total = (long long)n3[0] * n3[1] * n3[2];
+    cap_grid(n3, 1LL << 30);
     Scratch1 S;
     S.s = (cudaStream_t)stream;
-    rc = prepare1(S, n, box, rcs, (int)(total > (1LL << 30) ? (1LL << 30) : total), precision, false);
-    if (rc) return rc;
-    if (precision == NEFE_FP64) {
-        SWc<double> c = make_swc<double>(*prm);
-        NEFE_CU(S.alloc(&S.swc, sizeof(c)));
-        NEFE_CU(cudaMemcpyAsync(S.swc, &c, sizeof(c), cudaMemcpyHostToDevice, S.s));
-    } else {
-        SWc<float> c = make_swc<float>(*prm);
-        NEFE_CU(S.alloc(&S.swc, sizeof(c)));
-        NEFE_CU(cudaMemcpyAsync(S.swc, &c, sizeof(c), cudaMemcpyHostToDevice, S.s));
-    }
+    want1(S, n, n3, precision, false);
+    double* fo = f;
+    if (!fo) S.want(&fo, sizeof(double) * 3 * (size_t)n);
+    want_shells(S, n, precision);
+    if ((rc = commit1(S, n, box, rcs, n3, precision, prm))) return rc;
     if (n > 0) {
-        const size_t v4 = precision == NEFE_FP64 ? sizeof(double4) : sizeof(float4);
-        double* fo = f;
-        if (!fo) NEFE_CU(S.alloc(&fo, sizeof(double) * 3 * (size_t)n));
-        NEFE_CU(S.alloc(&S.shd, v4 * (size_t)n * kShell));
-        NEFE_CU(S.alloc(&S.shj, sizeof(int) * (size_t)n * kShell));
-        NEFE_CU(S.alloc(&S.shn, sizeof(int) * (size_t)n));
-        NEFE_CU(S.alloc(&S.P, 3 * v4 * (size_t)n));
         Bufs b = bufs_of(S, x, n);
         b.nbr = const_cast<int*>(nbr); b.cnt = const_cast<int*>(cnt); b.cap = cap;
         b.f_out = fo; b.e_atom = nullptr; b.want_grad = 1;
@@ -276,12 +353,11 @@ int nefe_sw_energy_grad(const double* x, int n, const double box[3], double rcs,
     }
     launch_decode_grad(S.acc, energy_grad, S.s);
     NEFE_CU(cudaGetLastError());
-    DevState st;
-    NEFE_CU(cudaMemcpyAsync(&st, S.st, sizeof(st), cudaMemcpyDeviceToHost, S.s));
-    NEFE_CU(cudaStreamSynchronize(S.s));
-    if (st.err & NEFE_ERR_SHELL_OVERFLOW)
+    unsigned err = 0;
+    if ((rc = read_error(S, &err))) return rc;
+    if (err & NEFE_ERR_SHELL_OVERFLOW)
         return fail(NEFE_EOVERFLOW, "nefe_sw_energy_grad: shell above 32 neighbours");
-    if (st.err & NEFE_ERR_NAN) return fail(NEFE_ENAN, "nefe_sw_energy_grad: non-finite sum");
+    if (err & NEFE_ERR_NAN) return fail(NEFE_ENAN, "nefe_sw_energy_grad: non-finite sum");
     return NEFE_OK;
 }
 
@@ -307,13 +383,13 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
     if (total > (1LL << 30)) return fail(NEFE_EINVAL, "nefe_uf_forces: cell grid too large");
     Scratch1 S;
     S.s = (cudaStream_t)stream;
-    rc = prepare1(S, n, box, rcs, (int)total, precision, true, uf, skin);
-    if (rc) return rc;
+    want1(S, n, n3, precision, true);
+    int* uf_nbr = nullptr;
+    int* uf_cnt = nullptr;
+    S.want(&uf_nbr, sizeof(int) * (size_t)n * kUfCap);
+    S.want(&uf_cnt, sizeof(int) * (size_t)n);
+    if ((rc = commit1(S, n, box, rcs, n3, precision, nullptr, uf, skin))) return rc;
     if (n > 0) {
-        int* uf_nbr = nullptr;
-        int* uf_cnt = nullptr;
-        NEFE_CU(S.alloc(&uf_nbr, sizeof(int) * (size_t)n * kUfCap));
-        NEFE_CU(S.alloc(&uf_cnt, sizeof(int) * (size_t)n));
         Bufs b = bufs_of(S, x, n);
         b.uf_nbr = uf_nbr; b.uf_cnt = uf_cnt; b.uf_tiles = nullptr;
         b.f_out = f; b.e_atom = e_atom;
@@ -325,11 +401,10 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
     }
     if (energy_virial) launch_decode_ev(S.acc, energy_virial, S.s);
     NEFE_CU(cudaGetLastError());
-    DevState st;
-    NEFE_CU(cudaMemcpyAsync(&st, S.st, sizeof(st), cudaMemcpyDeviceToHost, S.s));
-    NEFE_CU(cudaStreamSynchronize(S.s));
-    if (st.err & NEFE_ERR_NBR_OVERFLOW) return fail(NEFE_EOVERFLOW, "nefe_uf_forces: a row exceeded %d", kUfCap);
-    if (st.err & (NEFE_ERR_BOX | NEFE_ERR_CELL)) return fail(NEFE_EINVAL, "nefe_uf_forces: cell grid error");
+    unsigned err = 0;
+    if ((rc = read_error(S, &err))) return rc;
+    if (err & NEFE_ERR_NBR_OVERFLOW) return fail(NEFE_EOVERFLOW, "nefe_uf_forces: a row exceeded %d", kUfCap);
+    if (err & (NEFE_ERR_BOX | NEFE_ERR_CELL)) return fail(NEFE_EINVAL, "nefe_uf_forces: cell grid error");
     return NEFE_OK;
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cmath>
+#include <utility>
 #include <vector>
 
 #include "nefe.h"
@@ -35,6 +36,31 @@ inline bool host_grid(const double box[3], double rcs, int n3[3]) {
         n3[k] = m < 2 ? 2 : m;
     }
     return ok;
+}
+
+// The device side's reduction of a grid above the cell capacity: the longest axis loses cells
+// (wider cells stay valid).
+inline void cap_grid(int n3[3], long long cap) {
+    while ((long long)n3[0] * n3[1] * n3[2] > cap) {
+        const int k = (n3[0] >= n3[1] && n3[0] >= n3[2]) ? 0 : (n3[1] >= n3[2] ? 1 : 2);
+        if (n3[k] <= 2) break;
+        --n3[k];
+    }
+}
+
+// Box and cell grid of a one-system state (the stateless calls; the engine sets them on the
+// device when a list is built).
+inline void set_grid(DevState& st, const double box[3], const int n3[3]) {
+    for (int k = 0; k < 3; ++k) {
+        st.box[k] = box[k];
+        st.ncell[k] = n3[k];
+        st.h[k] = st.hb[k] = box[k] / (double)n3[k];
+        st.ibox[k] = 1.0 / box[k];
+        st.h_f[k] = st.hb_f[k] = (float)st.h[k];
+        st.rho_f[k] = 1.0f;
+    }
+    st.hmoved = 0;
+    st.nbuild = 1;
 }
 
 template <typename T>
@@ -89,8 +115,12 @@ inline bool valid_uf(const nefe_uf_params* u) {
            std::isfinite(u->sigma) && std::isfinite(u->T) && std::isfinite(u->rc);
 }
 
-// Single-system descriptors and scratch for the stateless calls and the adjoint context
-// (stream-ordered allocations, released on the same stream).
+// Stream-ordered device scratch from the library's own memory pool of the current device.
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+
+// Single-system descriptors and scratch for the stateless calls and the adjoint context: the
+// arrays are collected with want() and carved out of one stream-ordered allocation by commit(),
+// which is released on the same stream.
 struct Scratch1 {
     DevSys* sys = nullptr;
     DevState* st = nullptr;
@@ -110,28 +140,38 @@ struct Scratch1 {
     int* cell_start = nullptr;
     int* cell_count = nullptr;
     int* cell_cursor = nullptr;
+    int* scan_sums = nullptr;
+    int ncells = 0;
     cudaStream_t s = nullptr;
-    std::vector<void*> owned;
+    void* base = nullptr;
+    std::vector<std::pair<void**, size_t>> wanted;   // pointer to set, offset
+    size_t total = 0;
 
     template <typename P>
-    cudaError_t alloc(P** p, size_t bytes) {
-        void* q = nullptr;
-        cudaError_t e = cudaMallocAsync(&q, bytes < 16 ? 16 : bytes, s);
-        if (e == cudaSuccess) owned.push_back(q);
-        *p = static_cast<P*>(q);
+    void want(P** p, size_t bytes) {
+        wanted.emplace_back(reinterpret_cast<void**>(p), total);
+        total += (bytes + 255) / 256 * 256;
+    }
+    cudaError_t commit() {
+        const cudaError_t e = scratch_alloc(&base, total, s);
+        for (auto& w : wanted) *w.first = e == cudaSuccess ? static_cast<char*>(base) + w.second : nullptr;
         return e;
     }
     ~Scratch1() {
-        for (void* p : owned) cudaFreeAsync(p, s);
+        if (base) cudaFreeAsync(base, s);
     }
 };
 
 // NEFE_OK when every box length is positive, finite and at least 2 rcs.
 int check_box(const double box[3], double rcs);
-// Sets up the one-system descriptors, the tile table and (cells) the cell arrays.
-// With uf, the system carries a Uhlenbeck-Ford term as U_int (list radius uf->rc + skin).
-int prepare1(Scratch1& S, int n, const double box[3], double rcs, int ncell_cap, int prec, bool cells,
-             const nefe_uf_params* uf = nullptr, double skin = 0.0);
+// Collects the one-system descriptors, the tile table, the sums and (cells) the cell arrays in S.
+void want1(Scratch1& S, int n, const int n3[3], int prec, bool cells);
+// Allocates what was collected and writes the descriptors, the tile table and zeroed sums and cell
+// counts with one kernel (arguments by value: no copy from host memory).  With prm, the potential
+// constants of precision prec go to S.swc; with uf, the system carries a Uhlenbeck-Ford term as
+// U_int (list radius uf->rc + skin).
+int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3], int prec,
+            const nefe_sw_params* prm = nullptr, const nefe_uf_params* uf = nullptr, double skin = 0.0);
 // Launch arguments over S for n atoms at FP64 positions x.
 Bufs bufs_of(const Scratch1& S, const double* x, int n);
 

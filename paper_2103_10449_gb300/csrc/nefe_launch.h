@@ -62,6 +62,8 @@ struct Bufs {
     int* uf_cnt;             // [ntot] their lengths
     void* uf_F;              // [ntot] UF force and atom energy of the step (T4)
     const int* uf_tiles;     // tiles of the UF systems (per-step UF kernel), or NULL: every tile
+    int* scan_sums;          // stateless: span sums of a multi-block cell scan (NULL: one block)
+    int ncells_host;         // stateless: number of cells of the grid
     int* lacc;               // [ntot][4] int32 force accumulators of the scatter form (2^-21 eV/A)
     int* any_rebuild;        // engine: [0] some system's rebuild flag is set this step, [1] some
                              // rebuild_next is set (fused epilogue); NULL in the stateless calls
@@ -71,9 +73,13 @@ struct Bufs {
 
 enum ForceMode { FM_FORCES = 0, FM_SETUP = 1, FM_STEP = 2 };
 
-// Cell count / scan / fill / sort only (the stateless cell sort).
+// Cell count / scan / fill only.
 void launch_cells(const Bufs& b, int precision, int ntiles, int nsys, int force_all,
                   cudaStream_t s, long* launches);
+// Orders the atoms of each cell by index (the stateless cell sort, after launch_cells).
+void launch_cells_sort(const Bufs& b, int ncells, cudaStream_t s);
+// Cells per block of the multi-block scan (its scratch: one int per block, at most 1024).
+int cells_scan_span(int ncells);
 // Decodes one system's fixed-point sums into [U_int, virial xx yy zz xy xz yz] (FP64, device).
 void launch_decode_ev(const long long* acc, double* out7, cudaStream_t s);
 // Decodes [U_int, dE/dA, dE/dB, dE/dp, dE/dq, dE/da, dE/dlambda3, dE/dgamma] (FP64, device).

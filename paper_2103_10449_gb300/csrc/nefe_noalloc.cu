@@ -110,7 +110,7 @@ extern "C" int nefe_cell_bin_noalloc(const double* x, int n, const double box[3]
     hs.rcs = rcs; hs.pair = -1; hs.mass_e = 1.0;
     DevState st;
     std::memset(&st, 0, sizeof(st));
-    for (int k = 0; k < 3; ++k) st.box[k] = box[k];
+    set_grid(st, box, n3);
     st.rebuild = 1;
     // descriptors, tile table and zeroed occupancy counts, all written by one kernel
     {
@@ -139,6 +139,7 @@ extern "C" int nefe_cell_bin_noalloc(const double* x, int n, const double box[3]
     b.cell_start = cell_start;
     b.ntot = n;
     launch_cells(b, NEFE_FP32, ntiles, 1, 1, s, nullptr);
+    launch_cells_sort(b, (int)total, s);
     NEFE_CU(cudaGetLastError());
     return NEFE_OK;
 }
