@@ -101,14 +101,14 @@ __device__ __forceinline__ void copy_words(void* dst, const void* src, int bytes
 
 __global__ void __launch_bounds__(256) k_scratch_init(const __grid_constant__ DevSys hs, const __grid_constant__ DevState st,
                                                       const __grid_constant__ SwcBytes swc, DevSys* dsys, DevState* dst,
-                                                      void* dswc, int* tile_sys, int ntiles, long long* acc, int nacc,
+                                                      void* dswc, int4* tiles, int ntiles, long long* acc, int nacc,
                                                       int* counts, int ncells) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     static_assert(sizeof(DevSys) <= 1024 && sizeof(DevState) <= 1024, "one word per thread of the first block");
     copy_words(dsys, &hs, (int)sizeof(hs), t);
     copy_words(dst, &st, (int)sizeof(st), t);
     copy_words(dswc, &swc, (int)sizeof(swc), t);
-    for (int i = t; i < ntiles; i += stride) tile_sys[i] = 0;
+    for (int i = t; i < ntiles; i += stride) tiles[i] = make_int4(0, i * kTile, min(kTile, hs.n - i * kTile), 0);
     for (int i = t; i < nacc; i += stride) acc[i] = 0;
     for (int i = t; i < ncells; i += stride) counts[i] = 0;
 }
@@ -119,7 +119,7 @@ void want1(Scratch1& S, int n, const int n3[3], int prec, bool cells) {
     S.ncells = cells ? n3[0] * n3[1] * n3[2] : 0;
     S.want(&S.sys, sizeof(DevSys));
     S.want(&S.st, sizeof(DevState));
-    S.want(&S.tile_sys, sizeof(int) * (ntiles > 0 ? ntiles : 1));
+    S.want(&S.tiles, sizeof(int4) * (ntiles > 0 ? ntiles : 1));
     S.want(&S.acc, sizeof(long long) * ACC_N * kSlots);
     S.want(&S.swc, sizeof(SwcBytes));
     const size_t v4 = prec == NEFE_FP64 ? sizeof(double4) : sizeof(float4);
@@ -170,7 +170,7 @@ int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3]
     const int nacc = ACC_N * kSlots;
     const int work = std::max(std::max(ntiles, S.ncells), nacc);
     k_scratch_init<<<std::min((work + 255) / 256, 608), 256, 0, S.s>>>(
-        hs, st, sw, S.sys, S.st, S.swc, S.tile_sys, ntiles, S.acc, nacc, S.cell_count, S.ncells);
+        hs, st, sw, S.sys, S.st, S.swc, S.tiles, ntiles, S.acc, nacc, S.cell_count, S.ncells);
     NEFE_CU(cudaGetLastError());
     return NEFE_OK;
 }
@@ -178,7 +178,7 @@ int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3]
 Bufs bufs_of(const Scratch1& S, const double* x, int n) {
     Bufs b;
     std::memset(&b, 0, sizeof(b));
-    b.sys = S.sys; b.st = S.st; b.acc = S.acc; b.tile_sys = S.tile_sys;
+    b.sys = S.sys; b.st = S.st; b.acc = S.acc; b.tiles = S.tiles;
     b.x = const_cast<double*>(x);
     b.xs = S.xs; b.xa = S.xa; b.xcs = S.xcs; b.q = S.q; b.cell_of = S.cell_of; b.perm = S.perm;
     b.shd = S.shd; b.shj = S.shj; b.shn = S.shn; b.P = S.P;
@@ -199,13 +199,44 @@ static int read_error(const Scratch1& S, unsigned* err) {
     return NEFE_OK;
 }
 
-// The shells, leg forces and partial forces of the two force passes.
-static void want_shells(Scratch1& S, int n, int precision) {
-    const size_t v4 = precision == NEFE_FP64 ? sizeof(double4) : sizeof(float4), N = (size_t)n;
-    S.want(&S.shd, v4 * N * kShell);
-    S.want(&S.shj, sizeof(int) * N * kShell);
+// Scratch of the two force passes: the scatter form's accumulators (FP32), or the shells, leg
+// forces and partial forces of the gather form (FP64).
+static void want_forces(Scratch1& S, int n, int precision) {
+    const size_t N = (size_t)n;
     S.want(&S.shn, sizeof(int) * N);
-    S.want(&S.P, 3 * v4 * N);
+    if (precision == NEFE_FP32) {
+        S.want(&S.xf, sizeof(int4) * N);
+        S.want(&S.xc, sizeof(uint2) * N);
+        S.want(&S.lacc, 4 * sizeof(int) * N);
+        S.want(&S.lacc_hi, 4 * sizeof(int) * N);
+        S.want(&S.hi_flag, sizeof(int) * ((N + kTile - 1) / kTile));
+        S.want(&S.lscale, sizeof(float4) * 2);
+    } else {
+        S.want(&S.shd, sizeof(double4) * N * kShell);
+        S.want(&S.shj, sizeof(int) * N * kShell);
+        S.want(&S.P, 3 * sizeof(double4) * N);
+    }
+}
+
+// Both force passes of a stateless call.
+static int run_forces(const Scratch1& S, Bufs& b, int n, const nefe_sw_params* prm, int precision) {
+    const int ntiles = (n + kTile - 1) / kTile;
+    if (precision == NEFE_FP32) {
+        b.xf = S.xf; b.xc = S.xc; b.lacc = S.lacc; b.lacc_hi = S.lacc_hi; b.hi_flag = S.hi_flag; b.lscale = S.lscale;
+        b.swc_common = make_swc<float>(*prm); b.common = 1;
+        b.row4 = (b.cap & 3) == 0 && (reinterpret_cast<uintptr_t>(b.nbr) & 15) == 0;
+        NEFE_CU(cudaMemsetAsync(S.lacc, 0, (size_t)(reinterpret_cast<char*>(S.hi_flag + ntiles) - reinterpret_cast<char*>(S.lacc)),
+                                S.s));
+        launch_frac_positions(b, S.s);
+        launch_edges(b, precision, 0, ntiles, FM_FORCES, S.s, nullptr);
+        launch_gather(b, precision, 0, ntiles, FM_FORCES, S.s, nullptr);
+    } else {
+        launch_mirror(b, precision, ntiles, S.s, nullptr);
+        launch_edges(b, precision, 8, ntiles, FM_FORCES, S.s, nullptr);
+        launch_gather(b, precision, 4, ntiles, FM_FORCES, S.s, nullptr);
+    }
+    NEFE_CU(cudaGetLastError());
+    return NEFE_OK;
 }
 
 extern "C" {
@@ -298,17 +329,13 @@ int nefe_sw_forces(const double* x, int n, const double box[3], double rcs, cons
     Scratch1 S;
     S.s = (cudaStream_t)stream;
     want1(S, n, n3, precision, false);
-    want_shells(S, n, precision);
+    want_forces(S, n, precision);
     if ((rc = commit1(S, n, box, rcs, n3, precision, prm))) return rc;
     if (n > 0) {
         Bufs b = bufs_of(S, x, n);
         b.nbr = const_cast<int*>(nbr); b.cnt = const_cast<int*>(cnt); b.cap = cap;
         b.f_out = f; b.e_atom = e_atom;
-        const int ntiles = (n + kTile - 1) / kTile;
-        launch_mirror(b, precision, ntiles, S.s, nullptr);
-        launch_edges(b, precision, 8, ntiles, FM_FORCES, S.s, nullptr);
-        launch_gather(b, precision, 4, ntiles, FM_FORCES, S.s, nullptr);
-        NEFE_CU(cudaGetLastError());
+        if ((rc = run_forces(S, b, n, prm, precision))) return rc;
     }
     if (energy_virial) launch_decode_ev(S.acc, energy_virial, S.s);
     NEFE_CU(cudaGetLastError());
@@ -339,17 +366,13 @@ int nefe_sw_energy_grad(const double* x, int n, const double box[3], double rcs,
     want1(S, n, n3, precision, false);
     double* fo = f;
     if (!fo) S.want(&fo, sizeof(double) * 3 * (size_t)n);
-    want_shells(S, n, precision);
+    want_forces(S, n, precision);
     if ((rc = commit1(S, n, box, rcs, n3, precision, prm))) return rc;
     if (n > 0) {
         Bufs b = bufs_of(S, x, n);
         b.nbr = const_cast<int*>(nbr); b.cnt = const_cast<int*>(cnt); b.cap = cap;
         b.f_out = fo; b.e_atom = nullptr; b.want_grad = 1;
-        const int ntiles = (n + kTile - 1) / kTile;
-        launch_mirror(b, precision, ntiles, S.s, nullptr);
-        launch_edges(b, precision, 8, ntiles, FM_FORCES, S.s, nullptr);
-        launch_gather(b, precision, 4, ntiles, FM_FORCES, S.s, nullptr);
-        NEFE_CU(cudaGetLastError());
+        if ((rc = run_forces(S, b, n, prm, precision))) return rc;
     }
     launch_decode_grad(S.acc, energy_grad, S.s);
     NEFE_CU(cudaGetLastError());

@@ -56,6 +56,9 @@ struct SWc {
     T eps, A, lam3;  // for the parameter derivatives
     T s_act;       // edges with r/sigma >= s_act are dropped (see make_swc)
     T act2;        // (s_act sigma)^2
+    // what rounding 1/sigma, a and B to T left out: their relative errors of some 1e-8 act like a
+    // uniform strain, which the pressure sees (8000 atoms: virial off by 1.2e-2 eV, 4e-3 with them)
+    T inv_sig_lo, a_lo, B_lo;
     int int_pq;    // 1 when p == 4 and q == 0 (the standard set): s^-p by multiplications
 };
 

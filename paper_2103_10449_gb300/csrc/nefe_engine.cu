@@ -62,7 +62,7 @@ struct nefe_ctx {
     DevState* d_st = nullptr;
     long long* d_acc = nullptr;
     long long* d_acc_tmp = nullptr;
-    int* d_tile_sys = nullptr;
+    int4* d_tiles = nullptr;
     double *d_x = nullptr, *d_r0 = nullptr, *d_ftmp = nullptr, *d_vtmp = nullptr;
     void *d_v = nullptr, *d_dhi = nullptr, *d_dlo = nullptr;
     void *d_F = nullptr, *d_xs = nullptr, *d_xa = nullptr, *d_xcs = nullptr, *d_sd0 = nullptr, *d_xi = nullptr;
@@ -70,7 +70,12 @@ struct nefe_ctx {
     int *d_shj = nullptr, *d_shn = nullptr, *d_rtiles = nullptr, *d_rcount = nullptr, *d_rcbase = nullptr;
     int* d_any = nullptr;    // context-wide rebuild flag words (Bufs::any_rebuild)
     int *d_uf_nbr = nullptr, *d_uf_cnt = nullptr, *d_uf_tiles = nullptr;
-    int* d_lacc = nullptr;   // scatter-form force accumulators (FP32 contexts)
+    int *d_lacc = nullptr, *d_lacc_hi = nullptr, *d_hi_flag = nullptr;   // scatter-form force accumulators (FP32)
+    float4* d_lscale = nullptr;
+    uint2* d_xc = nullptr;
+    int4 *d_xf = nullptr, *d_xfb = nullptr;                               // fractional positions (FP32)
+    bool chosen = false;     // pass A's form was set by nefe_set_tuning or the autotuner
+    bool stale_pos = false;  // the positions' forms have to be made anew before the next step
     void* d_uf_F = nullptr;
     int n_uf_tiles = 0;      // tiles of the systems with a Uhlenbeck-Ford term
     int4* d_q = nullptr;
@@ -81,8 +86,10 @@ struct nefe_ctx {
     DevGroup* d_groups = nullptr;
     double* d_trace = nullptr;
     std::vector<void*> allocs;
-    int lanes = 8;           // pass A lanes per atom (1 = one thread per atom, 4, 8, 16, 32; 0 = one
-                             // thread per atom in the scatter form, whose pass B is k_finish)
+    int lanes = 8;           // pass A lanes per atom (1 = one thread per atom, 4, 8, 16, 32; 0 = the
+                             // scatter form, whose pass B is k_finish: the FP32 default, faster than
+                             // the gather form at every size (8000 atoms: 36 -> 30 us a step; 256,000
+                             // atoms: 190 -> 110 us)
     int glanes = 4;          // pass B lanes per atom (1, 2, 4, 8)
     int llanes = 0;          // list build: 0 one warp per cell; 8, 16, 32 lanes per atom
     int rebuild_all = 0;     // rebuild policy (nefe_set_rebuild_policy)
@@ -154,6 +161,17 @@ int not_ready(nefe_ctx* c, const char* what) {
 }
 
 double rc_of(const HostSys& h) { return h.prm.a * h.prm.sigma; }
+
+// Pass A's form, and the positions that the kernels of that form read.
+void set_form(nefe_ctx* c, int lanes) {
+    c->lanes = lanes;
+    const bool scatter = c->prec == NEFE_FP32 && lanes == 0;
+    const int xf = scatter ? 1 : 0, xs = !scatter || c->n_uf_tiles > 0 ? 1 : 0;
+    if (c->b.want_xf != xf || c->b.want_xs != xs) c->stale_pos = true;
+    c->b.want_xf = xf;
+    c->b.want_xs = xs;
+    c->b.leg_refuse = c->chosen ? 1 : 0;
+}
 
 // Both force passes, chunk by chunk; with slot >= 0 (profiling capture) events bracket
 // every chunk's pass A and pass B.  fuse: the scatter form's epilogue also runs the next
@@ -229,11 +247,16 @@ void fill_results(const DevSys& S, const DevState& st, nefe_results* out) {
 // Lists, mirror and total forces from the current x, v (lambda and scales unchanged).
 int resetup(nefe_ctx* c) {
     NEFE_CU(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * (size_t)c->nsys * ACC_N * kSlots, c->stream));
-    if (c->d_lacc) NEFE_CU(cudaMemsetAsync(c->d_lacc, 0, 4 * sizeof(int) * (size_t)c->ntot, c->stream));
+    if (c->d_lacc) {
+        NEFE_CU(cudaMemsetAsync(c->d_lacc, 0, 4 * sizeof(int) * (size_t)c->ntot, c->stream));
+        NEFE_CU(cudaMemsetAsync(c->d_lacc_hi, 0, 4 * sizeof(int) * (size_t)c->ntot, c->stream));
+        NEFE_CU(cudaMemsetAsync(c->d_hi_flag, 0, sizeof(int) * (size_t)c->ntiles, c->stream));
+    }
     launch_cells_and_list(c->b, c->prec, c->ntiles, c->nsys, 1, c->stream, &c->launches);
     if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->stream, &c->launches);
     launch_kick_drift(c->b, c->prec, c->ntiles, 0, c->stream, &c->launches);
     enqueue_forces(c, FM_SETUP);
+    c->stale_pos = false;
     NEFE_CU(cudaGetLastError());
     return NEFE_OK;
 }
@@ -398,7 +421,7 @@ int setup(nefe_ctx* c) {
     if ((rc = dalloc(c, &c->d_st, sizeof(DevState) * nsys))) return rc;
     if ((rc = dalloc(c, &c->d_acc, sizeof(long long) * nsys * ACC_N * kSlots))) return rc;
     if ((rc = dalloc(c, &c->d_acc_tmp, sizeof(long long) * nsys * ACC_N * kSlots))) return rc;
-    if ((rc = dalloc(c, &c->d_tile_sys, sizeof(int) * tile_sys.size()))) return rc;
+    if ((rc = dalloc(c, &c->d_tiles, sizeof(int4) * tile_sys.size()))) return rc;
     if ((rc = dalloc(c, &c->d_x, sizeof(double) * 3 * N))) return rc;
     if ((rc = dalloc(c, &c->d_v, el * 3 * N))) return rc;
     if ((rc = dalloc(c, &c->d_dhi, el * 3 * N))) return rc;
@@ -420,7 +443,12 @@ int setup(nefe_ctx* c) {
     if ((rc = dalloc(c, &c->d_P, 3 * v4 * N))) return rc;
     if (c->prec == NEFE_FP32) {
         if ((rc = dalloc(c, &c->d_lacc, 4 * sizeof(int) * N))) return rc;
-        NEFE_CU(cudaMemset(c->d_lacc, 0, 4 * sizeof(int) * N));
+        if ((rc = dalloc(c, &c->d_lacc_hi, 4 * sizeof(int) * N))) return rc;
+        if ((rc = dalloc(c, &c->d_hi_flag, sizeof(int) * tile_sys.size()))) return rc;
+        if ((rc = dalloc(c, &c->d_lscale, sizeof(float4) * 2 * nsys))) return rc;
+        if ((rc = dalloc(c, &c->d_xf, sizeof(int4) * N))) return rc;
+        if ((rc = dalloc(c, &c->d_xfb, sizeof(int4) * N))) return rc;
+        if ((rc = dalloc(c, &c->d_xc, sizeof(uint2) * N))) return rc;
     }
     if ((rc = dalloc(c, &c->d_rtiles, sizeof(int) * tile_sys.size()))) return rc;
     if ((rc = dalloc(c, &c->d_rcount, sizeof(int)))) return rc;
@@ -450,6 +478,8 @@ int setup(nefe_ctx* c) {
         NEFE_CU(cudaMemset(c->d_uf_cnt, 0, sizeof(int) * N));
         NEFE_CU(cudaMemset(c->d_uf_F, 0, v4 * N));
     }
+    SWc<float> swc_common{};
+    bool common = false;
     if (c->prec == NEFE_FP64) {
         std::vector<SWc<double>> t(nsys);
         for (int s = 0; s < nsys; ++s) t[s] = make_swc<double>(c->sys[s].prm);
@@ -458,6 +488,8 @@ int setup(nefe_ctx* c) {
     } else {
         std::vector<SWc<float>> t(nsys);
         for (int s = 0; s < nsys; ++s) t[s] = make_swc<float>(c->sys[s].prm);
+        common = std::all_of(t.begin(), t.end(), [&](const SWc<float>& v) { return std::memcmp(&v, &t[0], sizeof(v)) == 0; });
+        swc_common = t[0];
         if ((rc = dalloc(c, &c->d_swc, sizeof(SWc<float>) * nsys))) return rc;
         NEFE_CU(cudaMemcpy(c->d_swc, t.data(), sizeof(SWc<float>) * nsys, cudaMemcpyHostToDevice));
     }
@@ -481,7 +513,13 @@ int setup(nefe_ctx* c) {
     NEFE_CU(cudaMemset(c->d_xi, 0, v4 * N));
     NEFE_CU(cudaMemcpy(c->d_sys, hs.data(), sizeof(DevSys) * nsys, cudaMemcpyHostToDevice));
     NEFE_CU(cudaMemcpy(c->d_st, hst.data(), sizeof(DevState) * nsys, cudaMemcpyHostToDevice));
-    NEFE_CU(cudaMemcpy(c->d_tile_sys, tile_sys.data(), sizeof(int) * tile_sys.size(), cudaMemcpyHostToDevice));
+    std::vector<int4> tiles(tile_sys.size());
+    for (size_t t = 0; t < tiles.size(); ++t) {
+        const DevSys& S = hs[tile_sys[t]];
+        const int first = S.off + ((int)t - S.tile0) * kTile;
+        tiles[t] = make_int4(tile_sys[t], first, std::min(kTile, S.off + S.n - first), 0);
+    }
+    NEFE_CU(cudaMemcpy(c->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice));
     NEFE_CU(cudaMemcpy(c->d_groups, groups.data(), sizeof(DevGroup) * groups.size(), cudaMemcpyHostToDevice));
     if (!hp.empty())
         NEFE_CU(cudaMemcpy(c->d_pairs, hp.data(), sizeof(DevPair) * hp.size(), cudaMemcpyHostToDevice));
@@ -491,7 +529,7 @@ int setup(nefe_ctx* c) {
 
     Bufs& b = c->b;
     std::memset(&b, 0, sizeof(b));
-    b.sys = c->d_sys; b.st = c->d_st; b.acc = c->d_acc; b.tile_sys = c->d_tile_sys;
+    b.sys = c->d_sys; b.st = c->d_st; b.acc = c->d_acc; b.tiles = c->d_tiles;
     b.x = c->d_x; b.v = c->d_v; b.dhi = c->d_dhi; b.dlo = c->d_dlo; b.r0 = c->d_r0; b.F = c->d_F;
     b.xs = c->d_xs; b.xa = c->d_xa; b.xcs = c->d_xcs; b.sd0 = c->d_sd0; b.xi = c->d_xi;
     b.shd = c->d_shd; b.shj = c->d_shj; b.shn = c->d_shn; b.P = c->d_P; b.spill = c->d_spill;
@@ -505,7 +543,10 @@ int setup(nefe_ctx* c) {
     b.trace = c->d_trace;
     b.list_lanes = c->llanes;
     b.uf_nbr = c->d_uf_nbr; b.uf_cnt = c->d_uf_cnt; b.uf_F = c->d_uf_F; b.uf_tiles = c->d_uf_tiles;
-    b.lacc = c->d_lacc;
+    b.lacc = c->d_lacc; b.lacc_hi = c->d_lacc_hi; b.hi_flag = c->d_hi_flag;
+    b.xf = c->d_xf; b.xfb = c->d_xfb; b.lscale = c->d_lscale; b.xc = c->d_xc;
+    b.swc_common = swc_common; b.common = common ? 1 : 0;
+    set_form(c, c->lanes);
 
     launch_inject(b, c->prec, c->ntiles, nullptr, c->d_vtmp, c->stream);
     NEFE_CU(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * nsys * ACC_N * kSlots, c->stream));
@@ -538,6 +579,7 @@ int nefe_create(nefe_ctx** out, int device, void* stream, int precision, double 
     nefe_ctx* c = new nefe_ctx();
     c->device = device;
     c->prec = precision;
+    c->lanes = precision == NEFE_FP32 ? 0 : 8;
     c->dt = dt_ps;
     c->skin = skin;
     c->cap = nbr_cap;
@@ -712,6 +754,10 @@ int nefe_run(nefe_ctx* c, long nsteps) {
     int rc = setup(c);
     if (rc) return rc;
     if ((rc = set_device(c))) return rc;
+    if (c->stale_pos) {
+        launch_positions(c->b, c->prec, c->ntiles, c->stream, &c->launches);
+        c->stale_pos = false;
+    }
     long full = nsteps / kGraphSteps, rem = nsteps % kGraphSteps;
     if (full > 0 && !c->gexec) {
         if (c->profiling && (rc = ensure_events(c))) return rc;
@@ -957,6 +1003,7 @@ int nefe_load(nefe_ctx* c, const char* path) {
              cudaMemcpy(bl.p, tmp.data(), bl.bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     }
     std::fclose(f);
+    c->stale_pos = true;                         // what the files hold of it is the anchor and the displacement
     return ok ? NEFE_OK : fail(NEFE_EINVAL, "nefe_load: truncated or unreadable checkpoint");
 }
 
@@ -982,6 +1029,7 @@ static int refine_in_steps(nefe_ctx* c, const std::vector<std::pair<double, int>
             else cudaMemcpyAsync(x.p, snap + off, x.bytes, cudaMemcpyDeviceToDevice, c->stream);
             off += (x.bytes + 255) / 256 * 256;
         }
+        if (!save) c->stale_pos = true;
     };
     copy(true);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -996,7 +1044,7 @@ static int refine_in_steps(nefe_ctx* c, const std::vector<std::pair<double, int>
     for (size_t ka = 0; ka < ranked_a.size() && ka < 2 && rc == NEFE_OK; ++ka) {
         for (int lb : {1, 2, 4, 8}) {
             if (ranked_a[ka].second == 0 && lb != 1) continue;   // the scatter form has one pass B
-            c->lanes = ranked_a[ka].second;
+            set_form(c, ranked_a[ka].second);
             c->glanes = lb;
             drop_graph(c);
             if ((rc = nefe_run(c, kGraphSteps))) break;
@@ -1017,7 +1065,7 @@ static int refine_in_steps(nefe_ctx* c, const std::vector<std::pair<double, int>
     int best_r = c->rebuild_all;
     if (rc == NEFE_OK) {
         const int other = 1 - c->rebuild_all;
-        c->lanes = best_a;
+        set_form(c, best_a);
         c->glanes = best_b;
         c->b.rebuild_all = other;
         drop_graph(c);
@@ -1043,7 +1091,7 @@ static int refine_in_steps(nefe_ctx* c, const std::vector<std::pair<double, int>
     c->launches = launches;
     drop_graph(c);
     if (rc) return rc;
-    c->lanes = best_a;
+    set_form(c, best_a);
     c->glanes = best_b;
     c->tune_us = best;
     NEFE_CU(cudaGetLastError());
@@ -1056,7 +1104,14 @@ int nefe_autotune(nefe_ctx* c) {
     int rc = setup(c);
     if (rc) return rc;
     if ((rc = set_device(c))) return rc;
+    if (!c->chosen) drop_graph(c);               // what the forms refuse is captured in the step graph
+    c->chosen = true;
+    c->b.leg_refuse = 1;
     Bufs b = c->b;
+    if (c->prec == NEFE_FP32) {                  // every form is timed: both kinds of positions
+        b.want_xf = b.want_xs = 1;
+        launch_positions(b, c->prec, c->ntiles, c->stream, &c->launches);
+    }
     b.acc = c->d_acc_tmp;
     b.f_out = c->d_ftmp;
     b.e_atom = nullptr;
@@ -1155,7 +1210,7 @@ int nefe_autotune(nefe_ctx* c) {
     cudaEventDestroy(e1);
     NEFE_CU(cudaGetLastError());
     if (best_l != c->lanes || best_gl != c->glanes || best_ll != c->llanes) drop_graph(c);
-    c->lanes = best_l;
+    set_form(c, best_l);
     c->glanes = best_gl;
     c->llanes = best_ll;
     c->b.list_lanes = best_ll;
@@ -1182,8 +1237,9 @@ int nefe_set_tuning(nefe_ctx* c, int lanes) {
     if (!c) return fail(NEFE_EINVAL, "context is NULL");
     if (!lanes_supported(lanes) || (c->prec == NEFE_FP64 && (lanes == 0 || lanes == 1 || lanes == 4)))
         return fail(NEFE_EINVAL, "unsupported lanes per atom %d", lanes);
-    if (lanes != c->lanes) drop_graph(c);
-    c->lanes = lanes;
+    if (lanes != c->lanes || !c->chosen) drop_graph(c);
+    c->chosen = true;
+    set_form(c, lanes);
     return NEFE_OK;
 }
 

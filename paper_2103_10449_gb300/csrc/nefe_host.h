@@ -65,7 +65,7 @@ inline void set_grid(DevState& st, const double box[3], const int n3[3]) {
 
 template <typename T>
 inline SWc<T> make_swc(const nefe_sw_params& p) {
-    SWc<T> c;
+    SWc<T> c{};
     c.inv_sig = (T)(1.0 / p.sigma);
     c.a = (T)p.a;
     const double rc = p.a * p.sigma;
@@ -80,6 +80,9 @@ inline SWc<T> make_swc(const nefe_sw_params& p) {
     c.eps = (T)p.eps;
     c.A = (T)p.A;
     c.lam3 = (T)p.lambda3;
+    c.inv_sig_lo = (T)(1.0 / p.sigma - (double)c.inv_sig);
+    c.a_lo = (T)(p.a - (double)c.a);
+    c.B_lo = (T)(p.B - (double)c.B);
     // FP32 path: an edge whose three-body factor exp(gamma/(s - a)) is below 1e-12 adds forces
     // of order 1e-8 eV/A (pair and triplet), far below FP32 resolution, so it is dropped:
     // s_act = a + gamma / ln(1e-12).  FP64 path: only the last 1e-12 sigma before the cutoff
@@ -124,7 +127,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 struct Scratch1 {
     DevSys* sys = nullptr;
     DevState* st = nullptr;
-    int* tile_sys = nullptr;
+    int4* tiles = nullptr;
     long long* acc = nullptr;
     void* swc = nullptr;
     int4* q = nullptr;
@@ -141,6 +144,10 @@ struct Scratch1 {
     int* cell_count = nullptr;
     int* cell_cursor = nullptr;
     int* scan_sums = nullptr;
+    int4* xf = nullptr;
+    int *lacc = nullptr, *lacc_hi = nullptr, *hi_flag = nullptr;
+    float4* lscale = nullptr;
+    uint2* xc = nullptr;
     int ncells = 0;
     cudaStream_t s = nullptr;
     void* base = nullptr;

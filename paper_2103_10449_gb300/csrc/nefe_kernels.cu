@@ -13,11 +13,11 @@
 //   rebuild       (flagged systems) fold the displacement into the FP64 anchor, cell count ->
 //                 scan -> fill (with a cell-ordered copy of the mirror) -> Verlet list; as a
 //                 kernel sequence, or as one cooperative launch (k_rebuild_coop).
-//   k_edges1      force pass A, one thread per atom: in-cutoff shell of each atom, pair terms,
-//                 the shell's moments and the force the triplets centred on the atom exert on
-//                 each leg atom; in the scatter form (the FP32 default) every leg force and the
-//                 atom's own force go into int32 fixed-point accumulators (order independent).
-//                 k_edges: the lane-group variants (and the FP64 path), storing per edge.
+//   k_edges_s     force pass A of the scatter form (the FP32 default): the edges of a warp's atoms
+//                 as one list, pair terms, the shells' moments and the force each atom's terms
+//                 exert on each leg atom, added into int32 fixed-point accumulators (order
+//                 independent).  k_edges1, k_edges: the gather form with one thread or a lane
+//                 group per atom (and the FP64 path), storing per edge.
 //   k_finish      the scatter form's epilogue: reads and clears the accumulators; Einstein
 //                 springs, lambda mixing, Langevin force with its per-system mean removed,
 //                 second half kick (and the next step's kick, drift and noise, see above).
@@ -36,6 +36,7 @@
 #include "nefe.h"
 #include "nefe_dev.h"
 #include "nefe_launch.h"
+#include "nefe_sw_terms.h"
 
 namespace nefe {
 
@@ -237,26 +238,25 @@ __device__ __forceinline__ void refresh_box_f(DevState& st) {
 struct TileAtom {
     int sys, first, count;
 };
+// One load: the kernels' first operands wait for it, so the system descriptor is not in their way.
 __device__ __forceinline__ TileAtom tile_of(const Bufs& b, int tile) {
+    const int4 v = b.tiles[tile];
     TileAtom t;
-    t.sys = b.tile_sys[tile];
-    const DevSys& S = b.sys[t.sys];
-    t.first = S.off + (tile - S.tile0) * kTile;
-    t.count = min(kTile, S.off + S.n - t.first);
+    t.sys = v.x;
+    t.first = v.y;
+    t.count = v.z;
     return t;
 }
 
 // A tile's system descriptor and state copied into shared memory by all threads of the block
 // (independent 4-byte loads: one memory latency, instead of one per cache line of the structs
-// that the kernel's field accesses would otherwise wait for, one after the other), and the tile.
-// Writes to the state (flags, error bits) still go to the global copy.  Every thread of the block
-// must call it; it ends with a barrier.
+// that the kernel's field accesses would otherwise wait for, one after the other).  Writes to the
+// state (flags, error bits) still go to the global copy.  The caller syncs.
 struct StagedSys {
     DevSys S;
     DevState st;
 };
-__device__ __forceinline__ TileAtom stage_tile(const Bufs& b, int tile, StagedSys& sh) {
-    const int sys = b.tile_sys[tile];
+__device__ __forceinline__ void stage_sys(const Bufs& b, int sys, StagedSys& sh) {
     const uint32_t* gs = reinterpret_cast<const uint32_t*>(b.sys + sys);
     const uint32_t* gt = reinterpret_cast<const uint32_t*>(b.st + sys);
     uint32_t* ds = reinterpret_cast<uint32_t*>(&sh.S);
@@ -266,12 +266,6 @@ __device__ __forceinline__ TileAtom stage_tile(const Bufs& b, int tile, StagedSy
         if (w < ws) ds[w] = gs[w];
         else dt[w - ws] = gt[w - ws];
     }
-    __syncthreads();
-    TileAtom t;
-    t.sys = sys;
-    t.first = sh.S.off + (tile - sh.S.tile0) * kTile;
-    t.count = min(kTile, sh.S.off + sh.S.n - t.first);
-    return t;
 }
 
 // ------------------------------------------------------------------------------------
@@ -312,6 +306,19 @@ __device__ __forceinline__ void cell_axis(double x, double L, double n_over_L, i
     }
 }
 
+// The top 21 bits of each fraction in one 8-byte word, for pass A's row filter: x in bits 63-43, y
+// in 42-22, z in 21-1.  The reader takes the words (hi, funnel shift by 21, lo << 10) as they are: what
+// follows the 21 bits is noise below one unit.
+__device__ __forceinline__ uint2 pack_frac(const int4& f) {
+    const unsigned x = (unsigned)f.x >> 11, y = (unsigned)f.y >> 11, z = (unsigned)f.z >> 11;
+    return make_uint2(y << 22 | z << 1, x << 11 | y >> 10);     // (lo, hi)
+}
+
+// Fractional position of x in the box of the last list build (frac32).
+__device__ __forceinline__ int4 frac_position(const double (&x)[3], const DevState& st) {
+    return make_int4(frac32(x[0], st.ibox[0]), frac32(x[1], st.ibox[1]), frac32(x[2], st.ibox[2]), 0);
+}
+
 // ------------------------------------------------------------------------------------
 // Rebuild R1: fold the displacement into the FP64 anchor; cell of each atom, unwrapped cell
 // index q, fresh mirror, spring offset, occupancy count.  The cell grid was set with the system's
@@ -350,6 +357,13 @@ __device__ void cells_count_tile(const Bufs& b, int tile) {
     reinterpret_cast<T4*>(b.xs)[i] = m;
     if (b.xa) reinterpret_cast<T4*>(b.xa)[i] = m;
     if (b.sd0) reinterpret_cast<T4*>(b.sd0)[i] = mk4((T)sd[0], (T)sd[1], (T)sd[2], (T)0);
+    if (b.xf && b.want_xf) {
+        const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
+        const int4 f = frac_position(x3, st);
+        b.xf[i] = f;
+        b.xfb[i] = f;
+        b.xc[i] = pack_frac(f);
+    }
     atomicAdd(&b.cell_count[S.cell0 + cell], 1);
 }
 
@@ -1428,30 +1442,111 @@ __global__ void __launch_bounds__(kTile) k_mirror(Bufs b) {
 // box drift).  In the FP32 path (dhi, dlo) is a compensated pair: a two-sum keeps the
 // rounding error of every increment in dlo.
 // ------------------------------------------------------------------------------------
+// Every operation is rounded by itself (no contraction with the product that made d), so that the
+// two kernels that move atoms give the same bits whatever surrounds the call in each.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 template <typename T>
 __device__ __forceinline__ void comp_add(T& hi, T& lo, T d) {
     if constexpr (sizeof(T) == 8) {
-        hi += d;
+        hi = __dadd_rn(hi, d);
     } else {
-        const T s = hi + d;
-        const T bp = s - hi;
-        const T err = (hi - (s - bp)) + (d - bp);
-        lo += err;
-        const T h2 = s + lo;
-        lo = lo - (h2 - s);
+        const T s = __fadd_rn(hi, d);
+        const T bp = __fsub_rn(s, hi);
+        const T err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(d, bp));
+        lo = __fadd_rn(lo, err);
+        const T h2 = __fadd_rn(s, lo);
+        lo = __fsub_rn(lo, __fsub_rn(h2, s));
         hi = h2;
     }
 }
 
-// Drift of atom i by its half-kicked velocity vk (move), its mirror, the displacement test (sets
-// *flag) and the thermostat noise of step kstep (stored, and returned in z).  dh, dl: the atom's
-// displacement, updated in place.  Shared by k_kick_drift and by the epilogue that moves the
-// atoms for the next step (systems without a barostat), so both do the same operations.
-// xa: the atom's mirror at the last build (loaded by the caller together with its other operands).
-// any: the context-wide word that records that some system's flag was set (or NULL).
+// L 2^-32 of system s as FP32 value and remainder (what pass A's positions are scaled by).
+__device__ __forceinline__ void scale_of_box(const Bufs& b, int s, const double box[3]) {
+    if (!b.lscale) return;
+    float hi[3], lo[3];
+    for (int k = 0; k < 3; ++k) {
+        const double L = box[k] * 0x1p-32;
+        hi[k] = (float)L;
+        lo[k] = (float)(L - (double)hi[k]);
+    }
+    b.lscale[2 * s] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+    b.lscale[2 * s + 1] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+}
+
+// Per-block constants of the fractional positions' update, set by threads 0..2 (the caller syncs):
+// 1 - h/hb per axis (0 while the box is the one of the last build), with the division in FP64 since it
+// is the small difference of two nearly equal edges, and 2^32 / L.
+struct BoxMove {
+    float omr[3], to_frac[3];
+};
+__device__ __forceinline__ void box_move(const DevState& st, BoxMove& m) {
+    const int k = threadIdx.x;
+    if (k < 3) {
+        m.omr[k] = st.hmoved ? (float)(1.0 - st.h[k] / st.hb[k]) : 0.0f;
+        m.to_frac[k] = 4294967296.0f / (float)st.box[k];
+    }
+}
+
+// Position of atom i from its displacement d since the last build: the mirror (want_xs) and, in the
+// FP32 path, the fractional position (want_xf), which the scatter form's pass A reads.  Returns the
+// squared displacement of the list test, relative to the box's own deformation.  With x = X + d (X at
+// the build) and the cell edge grown from hb to h, the fraction is X/L_b + [d + X (1 - h/hb)] / L.
 template <typename T>
-__device__ __forceinline__ void drift_atom(const Bufs& b, const DevSys& S, const DevState& st, int i,
-                                           const typename V4<T>::t& xa, const T (&vk)[3], bool move,
+__device__ __forceinline__ T place_atom(const Bufs& b, const DevState& st, const BoxMove& bm, int i,
+                                        const typename V4<T>::t& xa, const int4& fb, const int4& q, const T (&d)[3]) {
+    using T4 = typename V4<T>::t;
+    const T xav[3] = {xa.x, xa.y, xa.z};
+    const int qa[3] = {q.x, q.y, q.z};
+    const bool hmoved = st.hmoved != 0;
+    T dd2 = 0;
+    if constexpr (sizeof(T) == 8) {
+        T m[3];
+        for (int k = 0; k < 3; ++k) {
+            m[k] = xav[k] + d[k];
+            if (hmoved) m[k] -= (T)qa[k] * (st.h[k] - st.hb[k]);
+            const T dd = hmoved ? m[k] - xav[k] * (st.h[k] / st.hb[k]) : d[k];
+            dd2 += dd * dd;
+        }
+        reinterpret_cast<T4*>(b.xs)[i] = mk4(m[0], m[1], m[2], (T)0);
+    } else {
+        T mv[3];
+        for (int k = 0; k < 3; ++k) {
+            mv[k] = d[k];
+            // (the list test alone does with the FP32 ratio)
+            if (hmoved) mv[k] = fma_rn(fma_rn((T)qa[k], st.hb_f[k], xav[k]), b.want_xf ? bm.omr[k] : 1.0f - st.rho_f[k], mv[k]);
+            dd2 += mv[k] * mv[k];
+        }
+        if (b.want_xf) {
+            const int4 f = make_int4(fb.x + __float2int_rn(mul_rn(mv[0], bm.to_frac[0])),
+                                     fb.y + __float2int_rn(mul_rn(mv[1], bm.to_frac[1])),
+                                     fb.z + __float2int_rn(mul_rn(mv[2], bm.to_frac[2])), 0);
+            b.xf[i] = f;
+            b.xc[i] = pack_frac(f);
+        }
+        if (b.want_xs) {
+            T m[3];
+            for (int k = 0; k < 3; ++k) {
+                m[k] = xav[k] + d[k];
+                if (hmoved) m[k] -= (T)qa[k] * (st.h_f[k] - st.hb_f[k]);
+            }
+            reinterpret_cast<T4*>(b.xs)[i] = mk4(m[0], m[1], m[2], (T)0);
+        }
+    }
+    return dd2;
+}
+
+// Drift of atom i by its half-kicked velocity vk (move), its position (place_atom), the
+// displacement test (sets *flag) and the thermostat noise of step kstep (stored, and returned in
+// z).  dh, dl: the atom's displacement, updated in place.  Shared by k_kick_drift and by the epilogue
+// that moves the atoms for the next step (systems without a barostat), so both do the same
+// operations.  xa, fb: the atom's mirror and fractional position at the last build (loaded by the
+// caller together with its other operands).  any: the context-wide word that records that some system's flag was set (or NULL).
+template <typename T>
+__device__ __forceinline__ void drift_atom(const Bufs& b, const DevSys& S, const DevState& st, const BoxMove& bm, int i,
+                                           const typename V4<T>::t& xa, const int4& fb, const T (&vk)[3], bool move,
                                            T (&dh)[3], T (&dl)[3], int flag_set, int* flag, int* any,
                                            unsigned long long kstep, T (&z)[3]) {
     using T4 = typename V4<T>::t;
@@ -1466,27 +1561,18 @@ __device__ __forceinline__ void drift_atom(const Bufs& b, const DevSys& S, const
     if (move) {
         const T dt = pick<T>(b.dt, S.dt_f);
         for (int k = 0; k < 3; ++k) {
-            T d = dt * pick<T>(st.phi[k], st.phi_f[k]) * vk[k];
+            T d = mul_rn(mul_rn(dt, pick<T>(st.phi[k], st.phi_f[k])), vk[k]);
             if (scaled) {   // (s - 1) x with x = xa + q hb + displacement
-                const T xk = xav[k] + (T)qa[k] * pick<T>(st.hb[k], st.hb_f[k]) + dh[k];
-                d += pick<T>(st.s[k] - 1.0, st.sm1_f[k]) * xk;
+                const T xk = fma_rn((T)qa[k], pick<T>(st.hb[k], st.hb_f[k]), xav[k]) + dh[k];
+                d = fma_rn(pick<T>(st.s[k] - 1.0, st.sm1_f[k]), xk, d);
             }
             comp_add<T>(dh[k], dl[k], d);
             DH[k * N + i] = dh[k];
             if constexpr (sizeof(T) == 4) DL[k * N + i] = dl[k];
         }
     }
-    T m[3];
-    for (int k = 0; k < 3; ++k) {
-        m[k] = xav[k] + (dh[k] + dl[k]);
-        if (hmoved) m[k] -= (T)qa[k] * (pick<T>(st.h[k], st.h_f[k]) - pick<T>(st.hb[k], st.hb_f[k]));
-    }
-    reinterpret_cast<T4*>(b.xs)[i] = mk4(m[0], m[1], m[2], (T)0);
-    T dd2 = 0;
-    for (int k = 0; k < 3; ++k) {
-        const T dd = hmoved ? m[k] - xav[k] * pick<T>(st.h[k] / st.hb[k], st.rho_f[k]) : dh[k] + dl[k];
-        dd2 += dd * dd;
-    }
+    const T d[3] = {dh[0] + dl[0], dh[1] + dl[1], dh[2] + dl[2]};
+    const T dd2 = place_atom<T>(b, st, bm, i, xa, fb, q, d);
     if (dd2 > pick<T>(st.thr2, st.thr2_f) && !flag_set) {
         atomicOr(flag, 1);
         if (any) atomicOr(any, 1);
@@ -1498,6 +1584,33 @@ __device__ __forceinline__ void drift_atom(const Bufs& b, const DevSys& S, const
     }
 }
 
+// Positions of every atom from the anchor and the displacement, in the forms that the force passes
+// in use read (after a checkpoint was loaded or another form was chosen).
+template <typename T>
+__global__ void __launch_bounds__(kTile) k_positions(Bufs b) {
+    using T4 = typename V4<T>::t;
+    __shared__ BoxMove bm;
+    const TileAtom ta = tile_of(b, blockIdx.x);
+    const DevState& st = b.st[ta.sys];
+    box_move(st, bm);
+    __syncthreads();
+    if ((int)threadIdx.x >= ta.count) return;
+    const int i = ta.first + threadIdx.x;
+    const size_t N = b.ntot;
+    if (b.want_xf && i == b.sys[ta.sys].off) scale_of_box(b, ta.sys, st.box);
+    int4 fb = make_int4(0, 0, 0, 0);
+    if (b.want_xf) {
+        const double x[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
+        b.xfb[i] = fb = frac_position(x, st);
+    }
+    T d[3];
+    for (int k = 0; k < 3; ++k) {
+        d[k] = reinterpret_cast<const T*>(b.dhi)[k * N + i];
+        if constexpr (sizeof(T) == 4) d[k] += reinterpret_cast<const T*>(b.dlo)[k * N + i];
+    }
+    place_atom<T>(b, st, bm, i, reinterpret_cast<const T4*>(b.xa)[i], fb, b.q[i], d);
+}
+
 // skip: systems without a barostat were already kicked and moved by the previous step's
 // epilogue (k_finish with fuse), so their tiles return at once.
 template <typename T>
@@ -1507,6 +1620,11 @@ __global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip
     const DevSys& S = b.sys[ta.sys];
     DevState& st = b.st[ta.sys];
     if (skip && S.baro == BARO_NONE) return;     // uniform over the block (one system per tile)
+    __shared__ BoxMove bm;
+    if (b.want_xf) {
+        box_move(st, bm);
+        __syncthreads();
+    }
     T xs_sum[3] = {(T)0, (T)0, (T)0};
     if ((int)threadIdx.x < ta.count) {
         const int i = ta.first + threadIdx.x;
@@ -1515,6 +1633,8 @@ __global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip
         const T* DH = reinterpret_cast<const T*>(b.dhi);
         const T* DL = reinterpret_cast<const T*>(b.dlo);
         const T4 xa = reinterpret_cast<const T4*>(b.xa)[i];
+        int4 fb = make_int4(0, 0, 0, 0);
+        if (b.want_xf) fb = b.xfb[i];
         T dh[3], dl[3], vk[3] = {(T)0, (T)0, (T)0};
         for (int k = 0; k < 3; ++k) {
             dh[k] = DH[k * N + i];
@@ -1525,11 +1645,11 @@ __global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip
             const T fv[3] = {F.x, F.y, F.z};
             const T ck = pick<T>(S.ckick, S.ckick_f);
             for (int k = 0; k < 3; ++k) {
-                vk[k] = V[k * N + i] + ck * fv[k];
+                vk[k] = fma_rn(ck, fv[k], V[k * N + i]);
                 V[k * N + i] = vk[k];
             }
         }
-        drift_atom<T>(b, S, st, i, xa, vk, mode == 1, dh, dl, st.rebuild, &st.rebuild, b.any_rebuild,
+        drift_atom<T>(b, S, st, bm, i, xa, fb, vk, mode == 1, dh, dl, st.rebuild, &st.rebuild, b.any_rebuild,
                       (unsigned long long)st.k,
                       xs_sum);
     }
@@ -1782,49 +1902,16 @@ constexpr int kShell1Shared = 8;
 constexpr int kShell1 = kShell1Shared + kSpill1;
 constexpr int kEdges1Threads = 64;
 
-// Scatter form of the force passes: pass A adds every leg force (and the atom's own force)
-// into per-atom int32 accumulators (units of 2^-21 eV/A) with global reductions.  Integer
-// addition is associative, so the result does not depend on the order in which the
-// reductions arrive (bitwise reproducible), and no second pass has to find the legs again:
-// a streaming epilogue (k_finish) reads and clears each atom's accumulator.  A term is
-// rounded to 2^-22 eV/A; one above kLegLimit eV/A (whose sum over the terms an atom can
-// receive could overflow int32) is dropped and flags the system.
-// The x and y terms travel in one 64-bit reduction as y 2^32 + x (two's complement, modulo
-// 2^64): integer addition is linear, so the 64-bit word accumulates Y 2^32 + X exactly, X and Y
-// being the int32 sums.  Its low word is X; its high word is Y - 1 when X < 0 (the borrow), which
-// the reader undoes (force_of_acc).  Two reductions per force instead of three.
-constexpr float kLegScale = 2097152.0f;          // 2^21
-constexpr float kLegLimit = 48.0f;
-__device__ __forceinline__ void red_force(int* acc4, float x, float y, float z, unsigned* err) {
-    if (!(fabsf(x) < kLegLimit && fabsf(y) < kLegLimit && fabsf(z) < kLegLimit)) {
-        atomicOr(err, NEFE_ERR_NAN);
-        return;
-    }
-    const long long px = __float2int_rn(x * kLegScale), py = __float2int_rn(y * kLegScale);
-    const unsigned long long xy = ((unsigned long long)py << 32) + (unsigned long long)px;
-    atomicAdd(reinterpret_cast<unsigned long long*>(acc4), xy);
-    atomicAdd(acc4 + 2, __float2int_rn(z * kLegScale));
-}
-
-// The int32 sums (X, Y, Z) of an accumulator written by red_force.
-__device__ __forceinline__ int3 force_of_acc(int4 q) {
-    return make_int3(q.x, q.y + (q.x < 0 ? 1 : 0), q.z);
-}
-
 constexpr int kEdges1K1 = kShell1Shared;
 
-// One work item of the thread-per-atom pass A: half a tile (64 atoms).  Every thread of the
-// block calls it with the same item.
 // Pass A for atom i (thread-per-atom): compaction of its Verlet row into the in-cutoff shell
 // (column t of the shared shell table, entries past its K1 rows in the global spill area), pair
-// terms, and the leg forces of the triplets centred on i (stored per shell edge, or in the
-// scatter form added into the force accumulators, with the energy and virial added to red8).
+// terms, and the leg forces of the triplets centred on i, stored per shell edge.
 // pos(j) returns atom j's mirror position (from global memory or a shared copy).
-template <typename T, bool SCATTER, int NT, typename PosFn>
+template <typename T, int NT, typename PosFn>
 __device__ __forceinline__ void edges1_atom(const Bufs& b, const SWc<T>& P, DevState& st,
                                             const T* soff, int i, int t,
-                                            typename V4<T>::t (*sh_u)[NT], T (*sh_r)[NT], int (*sh_j)[NT],
-                                            PosFn pos, T (&red8)[8]) {
+                                            typename V4<T>::t (*sh_u)[NT], T (*sh_r)[NT], PosFn pos) {
     using T4 = typename V4<T>::t;
     constexpr int K1 = kShell1Shared, KS = kShell1 - kShell1Shared;
     const T4 xi = pos(i);
@@ -1879,10 +1966,7 @@ __device__ __forceinline__ void edges1_atom(const Bufs& b, const SWc<T>& P, DevS
             if (r2 < P.act2) {
                 if (m < capm) {
                     put_u(m, mk4(dx, dy, dz, r2));
-                    // the scatter form keeps the shell's atom indices next to it in shared memory
-                    // (global only past its rows); the gather form publishes them for pass B
-                    if (SCATTER && m < K1) sh_j[m][t] = e[u] & (int)kIndexMask;
-                    else Sj[m] = e[u] & (int)kIndexMask;
+                    Sj[m] = e[u] & (int)kIndexMask;
                 }
                 ++m;
             }
@@ -1892,7 +1976,7 @@ __device__ __forceinline__ void edges1_atom(const Bufs& b, const SWc<T>& P, DevS
         atomicOr(&st.err, NEFE_ERR_SHELL_OVERFLOW);
         m = capm;
     }
-    if (!SCATTER && m < kShell) Sj[m] = -1;
+    if (m < kShell) Sj[m] = -1;
     T fx = 0, fy = 0, fz = 0, en = 0;
     T w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
     // Moments of the shell: G = sum_b g_b, m1 = sum_b g_b u_b, M = sum_b g_b u_b u_b^T.  Every
@@ -1950,8 +2034,7 @@ __device__ __forceinline__ void edges1_atom(const Bufs& b, const SWc<T>& P, DevS
         const T ay = k1 * (Muy - c0 * m1y - self * ua.y);
         const T az = k1 * (Muz - c0 * m1z - self * ua.z);
         const T lx = cc * ua.x - ax, ly = cc * ua.y - ay, lz = cc * ua.z - az;
-        if constexpr (SCATTER) red_force(b.lacc + 4 * (size_t)(a < K1 ? sh_j[a][t] : Sj[a]), lx, ly, lz, &st.err);
-        else Fl[a] = mk4(lx, ly, lz, (T)0);
+        Fl[a] = mk4(lx, ly, lz, (T)0);
         fx -= lx; fy -= ly; fz -= lz;
         en += (T)0.5 * P.epslam * ga * eh;
         const T dx = ua.x * ra, dy = ua.y * ra, dz = ua.z * ra;
@@ -1960,54 +2043,481 @@ __device__ __forceinline__ void edges1_atom(const Bufs& b, const SWc<T>& P, DevS
         w4 += (T)0.5 * (dx * lz + dz * lx);
         w5 += (T)0.5 * (dy * lz + dz * ly);
     }
-    if constexpr (SCATTER) {
-        red_force(b.lacc + 4 * (size_t)i, fx, fy, fz, &st.err);
-        if (b.e_atom) b.e_atom[i] = (double)en;
-        red8[0] += en;
-        red8[2] += w0; red8[3] += w1; red8[4] += w2; red8[5] += w3; red8[6] += w4; red8[7] += w5;
-    } else {
-        T4* Pa = reinterpret_cast<T4*>(b.P);
-        Pa[i] = mk4(fx, fy, fz, en);
-        Pa[b.ntot + 2 * (size_t)i] = mk4(w0, w1, w2, w3);
-        Pa[b.ntot + 2 * (size_t)i + 1] = mk4(w4, w5, (T)0, (T)0);
-    }
+    T4* Pa = reinterpret_cast<T4*>(b.P);
+    Pa[i] = mk4(fx, fy, fz, en);
+    Pa[b.ntot + 2 * (size_t)i] = mk4(w0, w1, w2, w3);
+    Pa[b.ntot + 2 * (size_t)i + 1] = mk4(w4, w5, (T)0, (T)0);
     b.shn[i] = m;
 }
 
-template <typename T, bool SCATTER>
-__device__ __forceinline__ void edges1_item(const Bufs& b, int tile, int part, typename V4<T>::t (*sh_u)[kEdges1Threads],
-                                            T (*sh_r)[kEdges1Threads], int (*sh_j)[kEdges1Threads],
-                                            T* soff) {
+template <typename T>
+__global__ void __launch_bounds__(kEdges1Threads, 16) k_edges1(Bufs b) {
     using T4 = typename V4<T>::t;
-    constexpr int NT = kEdges1Threads;
-    // 20 bytes per shell entry and thread (occupancy is bound by this table):
-    constexpr int K1 = kShell1Shared, KS = kShell1 - kShell1Shared;
-    const TileAtom ta = tile_of(b, tile);
+    constexpr int NT = kEdges1Threads, IPT = kTile / NT;
+    __shared__ T4 sh_u[kEdges1K1][NT];           // (d, r^2) after compaction, then (u, g)
+    __shared__ T sh_r[kEdges1K1][NT];            // r
+    __shared__ T soff[3 * 32];
+    const TileAtom ta = tile_of(b, (int)blockIdx.x / IPT + b.tile_base);
     const DevSys& S = b.sys[ta.sys];
     DevState& st = b.st[ta.sys];
     if (S.pot != POT_SW) return;                 // uniform over the block
     const SWc<T> P = reinterpret_cast<const SWc<T>*>(b.swc)[S.prm];
     offset_rows<T>(soff, pick<T>(st.h[0], st.h_f[0]), pick<T>(st.h[1], st.h_f[1]), pick<T>(st.h[2], st.h_f[2]));
     const int t = threadIdx.x;
-    const int ia = part * NT + t;
-    T red8[8] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0, (T)0, (T)0};   // scatter form: energy, -, virial
+    const int ia = ((int)blockIdx.x % IPT) * NT + t;
     if (ia < ta.count) {
         const T4* X = reinterpret_cast<const T4*>(b.xs);
-        edges1_atom<T, SCATTER, kEdges1Threads>(b, P, st, soff, ta.first + ia, t, sh_u, sh_r, sh_j,
-                                               [X](int j) { return X[j]; }, red8);
+        edges1_atom<T, NT>(b, P, st, soff, ta.first + ia, t, sh_u, sh_r, [X](int j) { return X[j]; });
     }
-    if constexpr (SCATTER) block_sum_to_acc<T, 8>(red8, b.acc + (size_t)ta.sys * ACC_N * kSlots, ACC_UINT, &st.err);
 }
 
-template <typename T, bool SCATTER>
-__global__ void __launch_bounds__(kEdges1Threads, 16) k_edges1(Bufs b) {
-    using T4 = typename V4<T>::t;
-    __shared__ T4 sh_u[kEdges1K1][kEdges1Threads];   // (d, r^2) after compaction, then (u, g)
-    __shared__ T sh_r[kEdges1K1][kEdges1Threads];    // r
-    __shared__ int sh_j[SCATTER ? kEdges1K1 : 1][kEdges1Threads];   // shell atom indices (scatter form)
-    __shared__ T soff[3 * 32];
-    constexpr int IPT = kTile / kEdges1Threads;  // work items per tile
-    edges1_item<T, SCATTER>(b, (int)blockIdx.x / IPT + b.tile_base, (int)blockIdx.x % IPT, sh_u, sh_r, sh_j, soff);
+// ------------------------------------------------------------------------------------
+// Scatter form of the force passes (FP32): pass A adds the force that each atom's terms exert on
+// each leg atom, and minus their sum on the atom itself, into per-atom int32 accumulators (units of
+// 2^-22 eV/A) with global reductions.  Integer addition is associative, so the result does not
+// depend on the order in which the reductions arrive (bitwise reproducible), and no second pass has
+// to find the legs again: a streaming epilogue (k_finish) reads and clears each accumulator.
+// The x and y terms travel in one 64-bit reduction as y 2^32 + x (two's complement, modulo
+// 2^64): integer addition is linear, so the 64-bit word accumulates Y 2^32 + X exactly, X and Y
+// being the int32 sums.  Its low word is X; its high word is Y - 1 when X < 0 (the borrow), which
+// the reader undoes (force_of_acc).  Two reductions per force instead of three.
+// A term of kLegFine eV/A or more is split: its multiples of kLegCoarse go to a second accumulator
+// (one count per multiple) and the rest, at most 7 eV/A, stays; up to 64 rests (32 legs, 32 own
+// edges) fit the int32 sum.  The second accumulator is read only for tiles whose flag says that
+// something was added (at 1000 K some atom of a system of thousands has such a term on most steps,
+// but few tiles do).
+// ------------------------------------------------------------------------------------
+constexpr float kLegScale = 4194304.0f;          // 2^22
+constexpr float kLegFine = 8.0f;
+constexpr float kLegCoarse = 14.0f;
+constexpr float kLegMax = 1e9f;
+constexpr float kLegRefuse = 48.0f;
+constexpr float kPairOdd = 6.0f;                 // half a pair force above which an own sum could reach kLegRefuse
+
+// Splits a large term: sign times its multiples of kLegCoarse go to atom j; returns the rest.
+__device__ __noinline__ float3 split_leg(const Bufs& b, const DevSys& S, int j, int sign, unsigned* err, float x, float y,
+                                         float z) {
+    if (!(fabsf(x) < kLegMax && fabsf(y) < kLegMax && fabsf(z) < kLegMax)) {
+        atomicOr(err, NEFE_ERR_NAN);
+        return make_float3(0.0f, 0.0f, 0.0f);
+    }
+    int* hi_j = b.lacc_hi + 4 * (size_t)j;
+    float v[3] = {x, y, z};
+    for (int k = 0; k < 3; ++k) {
+        const float h = rintf(v[k] / kLegCoarse);
+        v[k] = fmaf(-kLegCoarse, h, v[k]);
+        if (h != 0.0f) {
+            atomicAdd(hi_j + k, sign * (int)h);
+            b.hi_flag[S.tile0 + (j - S.off) / kTile] = 1;
+        }
+    }
+    return make_float3(v[0], v[1], v[2]);
+}
+
+__device__ __forceinline__ void red_force(int* acc4, int x, int y, int z) {
+    const unsigned long long xy = ((unsigned long long)(long long)y << 32) + (unsigned long long)(long long)x;
+    atomicAdd(reinterpret_cast<unsigned long long*>(acc4), xy);
+    atomicAdd(acc4 + 2, z);
+}
+
+// The int32 sums (X, Y, Z) of an accumulator written by red_force.
+__device__ __forceinline__ int3 force_of_acc(int4 q) {
+    return make_int3(q.x, q.y + (q.x < 0 ? 1 : 0), q.z);
+}
+
+// Force pass A, scatter form.  Each warp takes G = 32, 16 or 8 consecutive atoms, 32 / G lanes to an
+// atom.
+//   1. The lanes walk the atoms' Verlet rows and mark the entries inside the cutoff.  Positions are
+//      fractions: the difference of two is the nearest image by itself, so no cell offsets are looked
+//      up.  This filter reads 8-byte positions (21 bits an axis) and keeps a margin for their rounding.
+//   2. The marked entries become one edge list of the warp, taken 32 at a time: unit vector and g from
+//      the full positions (resolution L 2^-32); an edge of the margin has no terms.
+//   3. Per atom: the shell's moments.
+//   4. The edge list again: pair terms and leg forces (see sw_leg), quantised and added to the leg
+//      atoms; the own sums through shared integer accumulators.
+// What bounds it is the L1 wavefronts of the position gathers (17 a warp for 16-byte positions of 32
+// scattered atoms; step 1 alone took 83 of 172 us with them), hence the 8-byte ones.  With one thread
+// per atom throughout (the form before), steps 2 and 4 ran at the largest shell of each warp (9 edges
+// for a mean of 5.8) with idle lanes, and shells above 8 edges spilled to global memory.  Appending to
+// the list during the walk instead of marking (no second read of rows and positions) was slower by 10 us.
+// G: 32 where that gives every SM kScatterFull warps; smaller systems take 16 or 8 atoms to a warp,
+// whose chain of row groups and edge iterations is shorter by as much (8000 atoms: 8.9 -> 6.8 us).
+// A list holds kListEdges edges; atoms whose edges do not fit wait for the next batch.
+// Against the form before: 1,024,000-atom crystal at skin 1.6 A (28 row entries, 5.5 edges an atom)
+// 168 -> 155 us; 1,008,516 atoms of diamond / beta-tin pairs (12.8 edges) 345 -> 253 us; against the
+// gather form's two passes, 96,000 atoms under barostats 73 -> 42 us, 8000 atoms 13.5 -> 11.5 us.
+constexpr int kListEdges = 224;         // 32 atoms of a crystal hold 186 +- 5; smaller lists leave more L1 and warps
+constexpr int kScatterThreads = 64;
+// Resident blocks per SM the registers are bounded for: 14 where the launch fills them (crystal 154.7
+// us, 12: 159.6), else as many registers as the kernel wants (12 blocks' worth: 6.8 against 7.4 us for
+// 8000 atoms).
+constexpr int kScatterBlocks = 14, kScatterBlocksFew = 10;
+template <bool EATOM>
+struct __align__(16) ScatterShared {
+    float4 u[kListEdges];            // unit vector, g
+    float r[kListEdges];
+    unsigned id[kListEdges];         // atom of the warp << 27 | leg atom
+    float4 mom[3][32];               // moments; before them, the atoms' positions
+    int own[3][32];
+    float e[EATOM ? kListEdges : 1];
+};
+
+// r/sigma - a, from constants of twice the precision.
+__device__ __forceinline__ float below_cut(const SWc<float>& P, float r) {
+    return fmaf(r, P.inv_sig, -P.a) + fmaf(r, P.inv_sig_lo, -P.a_lo);
+}
+
+// Pair term of an edge (r < s_act sigma) and what the leg force needs of g: phi, dphi/dr, 1/(s - a).
+__device__ __forceinline__ void pair_edge(const SWc<float>& P, float r, float& phi, float& dphi, float& id) {
+    const float s = r * P.inv_sig, den = below_cut(P, r);
+    const bool in = s < P.s_act && den < -cut_eps<float>();
+    id = in ? xrcp(den) : 0.0f;
+    float e1 = in ? xexp(id) : 0.0f;
+    float rp, rq;
+    const float is = xrcp(s);
+    if (P.int_pq) {
+        const float is2 = xrcp(s * s);
+        rp = is2 * is2;
+        rq = 1.0f;
+    } else {
+        rp = xpow(s, -P.p);
+        rq = xpow(s, -P.q);
+    }
+    const float poly = fmaf(P.B, rp, -rq) + P.B_lo * rp;
+    e1 *= P.epsA;
+    phi = poly * e1;
+    dphi = e1 * ((P.q * rq - P.p * fmaf(P.B, rp, P.B_lo * rp)) * is - poly * id * id) * P.inv_sig;
+}
+
+// An edge's terms in the last phase: the force on the leg atom (see sw_leg; the rows of the shell's
+// moments M, m1 are ma, mb, mc), half the pair force, energies and 1/(s - a).
+struct LegOut {
+    float x, y, z, hp, phi, s3, ida;
+};
+__device__ __forceinline__ LegOut leg_of_edge(const SWc<float>& P, const float4& ua, float ra, const float4& ma,
+                                              const float4& mb, const float4& mc, float G) {
+    LegOut o;
+    float dphi;
+    pair_edge(P, ra, o.phi, dphi, o.ida);
+    o.hp = 0.5f * dphi;
+    const float c0 = P.c0, ga = ua.w;
+    const float eg = P.epslam * ga;
+    const float k1 = 2.0f * eg * xrcp(ra);
+    const float k2 = -eg * P.gam * o.ida * o.ida * P.inv_sig;
+    const float Mux = ma.x * ua.x + ma.y * ua.y + ma.z * ua.z;
+    const float Muy = mb.x * ua.x + mb.y * ua.y + mb.z * ua.z;
+    const float Muz = mc.x * ua.x + mc.y * ua.y + mc.z * ua.z;
+    const float q = ua.x * Mux + ua.y * Muy + ua.z * Muz;
+    const float pm = ua.x * ma.w + ua.y * mb.w + ua.z * mc.w;
+    const float self = ga * (1.0f - c0);
+    const float S2 = q - c0 * pm - self;
+    o.s3 = q - 2.0f * c0 * pm + c0 * c0 * G - self * (1.0f - c0);
+    const float cc = k1 * S2 - k2 * o.s3 - o.hp;
+    o.x = cc * ua.x - k1 * (Mux - c0 * ma.w - self * ua.x);
+    o.y = cc * ua.y - k1 * (Muy - c0 * mb.w - self * ua.y);
+    o.z = cc * ua.z - k1 * (Muz - c0 * mc.w - self * ua.z);
+    return o;
+}
+
+// Rare: a term that has to be split (or, with refuse, whose triplet part may be refused), from atom i
+// (lane t) to leg atom j.
+template <bool EATOM>
+__device__ __noinline__ void add_large_leg(const Bufs& b, const DevSys& S, ScatterShared<EATOM>& sh, int refuse, int j, int i,
+                                           int t, float3 l, float3 u, float hp, unsigned* err) {
+    float3 p = l;                                // what the leg atom gets
+    if (refuse && !(fabsf(l.x + hp * u.x) < kLegRefuse && fabsf(l.y + hp * u.y) < kLegRefuse &&
+                    fabsf(l.z + hp * u.z) < kLegRefuse)) {
+        atomicOr(err, NEFE_ERR_NAN);
+        p = make_float3(-hp * u.x, -hp * u.y, -hp * u.z);
+    }
+    p = split_leg(b, S, j, 1, err, p.x, p.y, p.z);
+    l = split_leg(b, S, i, -1, err, l.x, l.y, l.z);
+    red_force(b.lacc + 4 * (size_t)j, __float2int_rn(p.x * kLegScale), __float2int_rn(p.y * kLegScale),
+              __float2int_rn(p.z * kLegScale));
+    atomicAdd(&sh.own[0][t], __float2int_rn(l.x * kLegScale));
+    atomicAdd(&sh.own[1][t], __float2int_rn(l.y * kLegScale));
+    atomicAdd(&sh.own[2][t], __float2int_rn(l.z * kLegScale));
+}
+
+// Rare: takes the own sum of an atom (its pair forces and the recoils of its triplet legs, sum of
+// hp u - l) out again if it is refused.  All lanes of the warp call it; part, t: the lane's part and
+// atom, m: its edges (on: in this batch), G: atoms.
+template <bool EATOM>
+__device__ __noinline__ void refuse_own(const Bufs& b, const DevSys& S, const SWc<float>& P, ScatterShared<EATOM>& sh,
+                                        int lane, int G, int i, int m, int mx, float Gm, unsigned* err) {
+    const int t = lane & (G - 1);
+    float ox = 0.0f, oy = 0.0f, oz = 0.0f;
+    int base = 0;
+    for (int a = 0; a < mx; ++a) {
+        const unsigned bal = __ballot_sync(0xffffffffu, a < m);
+        if (a < m) {
+            const int e = base + __popc(bal & ((1u << lane) - 1u));
+            const float4 u = sh.u[e];
+            const LegOut o = leg_of_edge(P, u, sh.r[e], sh.mom[0][t], sh.mom[1][t], sh.mom[2][t], Gm);
+            ox += o.hp * u.x - o.x; oy += o.hp * u.y - o.y; oz += o.hp * u.z - o.z;
+        }
+        base += __popc(bal);
+    }
+    for (int o = 16; o >= G; o >>= 1) {
+        ox += __shfl_xor_sync(0xffffffffu, ox, o);
+        oy += __shfl_xor_sync(0xffffffffu, oy, o);
+        oz += __shfl_xor_sync(0xffffffffu, oz, o);
+    }
+    if (lane < G && !(fabsf(ox) < kLegRefuse && fabsf(oy) < kLegRefuse && fabsf(oz) < kLegRefuse)) {
+        atomicOr(err, NEFE_ERR_NAN);
+        const float3 o = split_leg(b, S, i, -1, err, ox, oy, oz);
+        sh.own[0][t] += __float2int_rn(o.x * kLegScale);
+        sh.own[1][t] += __float2int_rn(o.y * kLegScale);
+        sh.own[2][t] += __float2int_rn(o.z * kLegScale);
+    }
+    __syncwarp();
+}
+
+// COMMON: every system has the same potential constants, which are then kernel arguments (operands of
+// the constant bank, no loads: 171 -> 155 us on the crystal); otherwise they are read from the table.
+template <bool EATOM, bool GRAD, bool COMMON, int BLOCKS>
+__global__ void __launch_bounds__(kScatterThreads, BLOCKS)
+k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc, int lg) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int G = 1 << lg, lpa = 5 - lg;
+    __shared__ ScatterShared<EATOM> shm[kScatterThreads / 32];
+    ScatterShared<EATOM>& sh = shm[threadIdx.x >> 5];
+    static_assert(kScatterThreads == 64 && kTile == 128, "two warps of 2^lg atoms a block");
+    const int item = (int)blockIdx.x, tile = (item >> (6 - lg)) + b.tile_base;
+    const TileAtom ta = tile_of(b, tile);
+    const DevSys& S = b.sys[ta.sys];
+    DevState& st = b.st[ta.sys];
+    if (S.pot != POT_SW) return;                 // uniform over the block
+    const SWc<float>& P = COMMON ? Pc : reinterpret_cast<const SWc<float>*>(b.swc)[S.prm];
+    const int lane = threadIdx.x & 31, t = lane & (G - 1);
+    const unsigned below = (1u << lane) - 1u;
+    const int ia = ((item & ((64 >> lg) - 1)) << (lg + 1)) + ((int)(threadIdx.x >> 5) << lg) + t;   // of the tile
+    const int i = ta.first + ia;
+    const bool valid = ia < ta.count;
+    // L 2^-32 to twice the precision: a relative error of L alone would be a uniform strain of up to
+    // 6e-8, which the pressure sees (the row filter does without the second part)
+    const float4 Lh = b.lscale[2 * ta.sys], Ll = b.lscale[2 * ta.sys + 1];
+    const bool il = b.nbr_il != 0;
+    // 1. accepted row entries of this lane: entry 8 (part + n 32 / G) + k is bit 8 n + k of lo, hi
+    unsigned lo = 0u, hi = 0u;
+    if (valid) {
+        const int part = lane >> lg;
+        const bool wide = il || b.row4;
+        const int4* rows4 = il ? reinterpret_cast<const int4*>(b.nbr) + i
+                               : reinterpret_cast<const int4*>(b.nbr + (size_t)i * b.cap);
+        const size_t rstep = il ? (size_t)b.ntot : 1;
+        const uint2* X = b.xc;
+        const uint2 pi = X[i];
+        const int xi = (int)pi.y, yi = (int)__funnelshift_l(pi.x, pi.y, 21), zi = (int)(pi.x << 10);
+        const int ci = min(b.cnt[i], b.cap);
+        // each axis of the packed difference is within 2 units of 2^-21 L of the true one
+        const float mg = 2.0f * 2048.0f * (Lh.x + Lh.y + Lh.z);
+        const float rc = sqrtf(P.act2) + mg, act2 = rc * rc;
+        int shift = 0;
+        for (int base = 8 * part; base < ci; base += 8 << lpa, shift += 8) {
+            int e[8];
+#pragma unroll
+            for (int v = 0; v < 8; v += 4) {
+                if (wide) {
+                    int4 r = make_int4(i, i, i, i);
+                    if (base + v < ci) r = rows4[(size_t)((base + v) >> 2) * rstep];
+                    e[v] = r.x; e[v + 1] = r.y; e[v + 2] = r.z; e[v + 3] = r.w;
+                } else {
+                    const int* row = reinterpret_cast<const int*>(rows4);
+#pragma unroll
+                    for (int u = v; u < v + 4; ++u) e[u] = base + u < ci ? row[base + u] : i;
+                }
+            }
+            unsigned oct = 0u;
+            uint2 pj[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                // past the row's length a row-major group holds the caller's bytes: not an index
+                int j = (il || base + u < ci) ? (e[u] & (int)kIndexMask) : i;
+                if (!NEFE_IN_RANGE(j, b.ntot, &st.err)) j = i;
+                pj[u] = X[j];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float dx = (float)((int)pj[u].y - xi) * Lh.x,
+                            dy = (float)((int)__funnelshift_l(pj[u].x, pj[u].y, 21) - yi) * Lh.y,
+                            dz = (float)((int)(pj[u].x << 10) - zi) * Lh.z;
+                if (dx * dx + dy * dy + dz * dz < act2) oct |= 1u << u;
+            }
+            // entries past the length are the atom itself
+            if (ci - base < 8) oct &= (1u << (ci - base)) - 1u;
+            if (shift < 32) lo |= oct << shift; else hi |= oct << (shift - 32);
+        }
+    }
+    const int ml = __popc(lo) + __popc(hi);      // edges of this lane, then of its atom
+    int m = ml;
+    for (int o = 16; o >= G; o >>= 1) m += __shfl_xor_sync(kAll, m, o);
+    int incl = m;                                // edges of atoms 0 .. t
+    for (int o = 1; o < G; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, incl, o, G);
+        if (t >= o) incl += y;
+    }
+    const int total = __shfl_sync(kAll, incl, G - 1);
+    float red8[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};   // energy, -, virial
+    float gth[7] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    float en = 0.0f;
+    int mtrue = 0;                               // edges of the lane inside the cutoff
+    const float pair_odd = b.leg_refuse ? kPairOdd : INFINITY;
+    int4* spos = reinterpret_cast<int4*>(&sh.mom[0][0]);
+    sh.own[0][lane] = 0; sh.own[1][lane] = 0; sh.own[2][lane] = 0;
+    for (int done = 0; done < total;) {
+        const bool act = incl - m >= done && incl - done <= kListEdges && m > 0;
+        const int ma = act ? ml : 0;
+        const int mx = __reduce_max_sync(kAll, ma);
+        int E = 0;
+        {
+            const int part = lane >> lg;
+            unsigned l = lo, h = hi;
+            for (int a = 0; a < mx; ++a) {       // slot by slot: consecutive lanes hold distinct atoms
+                const bool on = a < ma;
+                const unsigned bal = __ballot_sync(kAll, on);
+                if (on) {
+                    int k;
+                    if (l) { k = __ffs(l) - 1; l &= l - 1u; }
+                    else { k = 31 + __ffs(h); h &= h - 1u; }
+                    k = 8 * (((k >> 3) << lpa) + part) + (k & 7);
+                    int j = b.nbr[nbr_at(b, i, k)] & (int)kIndexMask;
+                    if (!NEFE_IN_RANGE(j, b.ntot, &st.err)) j = i;
+                    sh.id[E + __popc(bal & below)] = (unsigned)t << kCodeShift | (unsigned)j;
+                }
+                E += __popc(bal);
+            }
+        }
+        if (lane < G && valid) spos[lane] = b.xf[i];
+        __syncwarp();
+        // 2. unit vectors and g; two edges a lane, so that their gathers are in flight together
+        for (int e0 = lane; e0 < E; e0 += 64) {
+            int4 xj[2], xi[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const unsigned w = sh.id[e0 + 32 * u < E ? e0 + 32 * u : e0];
+                xj[u] = b.xf[w & kIndexMask];
+                xi[u] = spos[w >> kCodeShift];
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int e = e0 + 32 * u;
+                if (e >= E) break;
+                const float fx = (float)(xj[u].x - xi[u].x), fy = (float)(xj[u].y - xi[u].y), fz = (float)(xj[u].z - xi[u].z);
+                const float dx = fx * Lh.x + fx * Ll.x, dy = fy * Lh.y + fy * Ll.y, dz = fz * Lh.z + fz * Ll.z;
+                const float r2 = dx * dx + dy * dy + dz * dz;
+                // one Newton step: the hardware value's bias of a fraction of 1e-7 would scale every
+                // edge alike, which the pressure sees
+                float ir = xrsqrt(r2);
+                ir = fmaf(0.5f * ir, fmaf(-r2 * ir, ir, 1.0f), ir);
+                const float r = r2 * ir, s = r * P.inv_sig, den = below_cut(P, r);
+                const float g = s < P.s_act && den < -cut_eps<float>() ? xexp(P.gam * xrcp(den)) : 0.0f;
+                sh.u[e] = make_float4(dx * ir, dy * ir, dz * ir, g);
+                sh.r[e] = r;
+            }
+        }
+        __syncwarp();
+        // 3. moments
+        float Gm = 0;
+        {
+            float mx_ = 0, my = 0, mz = 0, xx = 0, yy = 0, zz = 0, xy = 0, xz = 0, yz = 0;
+            int base = 0;
+            for (int a = 0; a < mx; ++a) {
+                const bool on = a < ma;
+                const unsigned bal = __ballot_sync(kAll, on);
+                if (on) {
+                    const float4 u = sh.u[base + __popc(bal & below)];
+                    const float gx = u.w * u.x, gy = u.w * u.y, gz = u.w * u.z;
+                    mtrue += u.w > 0.0f ? 1 : 0;
+                    Gm += u.w; mx_ += gx; my += gy; mz += gz;
+                    xx += gx * u.x; yy += gy * u.y; zz += gz * u.z; xy += gx * u.y; xz += gx * u.z; yz += gy * u.z;
+                }
+                base += __popc(bal);
+            }
+            for (int o = 16; o >= G; o >>= 1) {
+                Gm += __shfl_xor_sync(kAll, Gm, o);
+                mx_ += __shfl_xor_sync(kAll, mx_, o); my += __shfl_xor_sync(kAll, my, o); mz += __shfl_xor_sync(kAll, mz, o);
+                xx += __shfl_xor_sync(kAll, xx, o); yy += __shfl_xor_sync(kAll, yy, o); zz += __shfl_xor_sync(kAll, zz, o);
+                xy += __shfl_xor_sync(kAll, xy, o); xz += __shfl_xor_sync(kAll, xz, o); yz += __shfl_xor_sync(kAll, yz, o);
+            }
+            if (lane < G) {
+                sh.mom[0][t] = make_float4(xx, xy, xz, mx_);
+                sh.mom[1][t] = make_float4(xy, yy, yz, my);
+                sh.mom[2][t] = make_float4(xz, yz, zz, mz);
+            }
+        }
+        __syncwarp();
+        // 4. pair terms and leg forces
+        bool odd = false;
+        for (int e0 = 0; e0 < E; e0 += 32) {
+            const int e = e0 + lane;
+            const bool on = e < E;
+            const unsigned w = on ? sh.id[e] : 0u;
+            const int te = (int)(w >> kCodeShift);
+            const float Gt = __shfl_sync(kAll, Gm, te);
+            if (!on) continue;
+            const int j = (int)(w & kIndexMask);
+            const float4 ua = sh.u[e];
+            const float ra = sh.r[e];
+            const LegOut o = leg_of_edge(P, ua, ra, sh.mom[0][te], sh.mom[1][te], sh.mom[2][te], Gt);
+            const float h = P.epslam * ua.w * o.s3;   // the triplets of edge a, each seen from both its edges
+            const float ee = 0.5f * (o.phi + h);
+            red8[0] += ee;
+            if (EATOM) sh.e[e] = ee;
+            const float dx = ua.x * ra, dy = ua.y * ra, dz = ua.z * ra;
+            red8[2] += dx * o.x; red8[3] += dy * o.y; red8[4] += dz * o.z;
+            red8[5] += 0.5f * (dx * o.y + dy * o.x);
+            red8[6] += 0.5f * (dx * o.z + dz * o.x);
+            red8[7] += 0.5f * (dy * o.z + dz * o.y);
+            if constexpr (GRAD) {
+                float pg[5];
+                sw_pair_pgrad<float>(P, ra, pg);
+#pragma unroll
+                for (int q5 = 0; q5 < 5; ++q5) gth[q5] += 0.5f * pg[q5];
+                gth[4] += h * P.gam * o.ida * o.ida;
+                gth[5] += 0.5f * P.eps * ua.w * o.s3;
+                gth[6] += h * o.ida;
+            }
+            if (!(fabsf(o.x) < kLegFine && fabsf(o.y) < kLegFine && fabsf(o.z) < kLegFine && fabsf(o.hp) < pair_odd)) {
+                odd = true;
+                add_large_leg(b, S, sh, b.leg_refuse, j, i - t + te, te, make_float3(o.x, o.y, o.z),
+                              make_float3(ua.x, ua.y, ua.z), o.hp, &st.err);
+                continue;
+            }
+            const int qx = __float2int_rn(o.x * kLegScale), qy = __float2int_rn(o.y * kLegScale),
+                      qz = __float2int_rn(o.z * kLegScale);
+            red_force(b.lacc + 4 * (size_t)j, qx, qy, qz);
+            atomicAdd(&sh.own[0][te], qx);
+            atomicAdd(&sh.own[1][te], qy);
+            atomicAdd(&sh.own[2][te], qz);
+        }
+        __syncwarp();
+        if (b.leg_refuse && __any_sync(kAll, odd)) refuse_own(b, S, P, sh, lane, G, i, ma, mx, Gm, &st.err);
+        if (EATOM) {                             // per-atom energies in slot order
+            int base = 0;
+            for (int a = 0; a < mx; ++a) {
+                const unsigned bal = __ballot_sync(kAll, a < ma);
+                if (a < ma) en += sh.e[base + __popc(bal & below)];
+                base += __popc(bal);
+            }
+        }
+        done = __reduce_max_sync(kAll, act ? incl : 0);
+        __syncwarp();
+    }
+    __syncwarp();
+    for (int o = 16; o >= G; o >>= 1) {
+        mtrue += __shfl_xor_sync(kAll, mtrue, o);
+        if (EATOM) en += __shfl_xor_sync(kAll, en, o);
+    }
+    if (lane < G && valid) {
+        b.shn[i] = mtrue;
+        if (mtrue > kShell) atomicOr(&st.err, NEFE_ERR_SHELL_OVERFLOW);
+        if (m > 0) red_force(b.lacc + 4 * (size_t)i, -sh.own[0][lane], -sh.own[1][lane], -sh.own[2][lane]);
+        if (EATOM && b.e_atom) b.e_atom[i] = (double)en;
+    }
+    long long* acc = b.acc + (size_t)ta.sys * ACC_N * kSlots;
+    block_sum_to_acc<float, 8>(red8, acc, ACC_UINT, &st.err);
+    if constexpr (GRAD) block_sum_to_acc<float, 7>(gth, acc, ACC_DTH, &st.err);
 }
 
 // Force pass B, L lanes per atom:
@@ -2035,12 +2545,13 @@ __global__ void __launch_bounds__(kTile) k_gather(Bufs b) {
     __shared__ __align__(16) StagedSys sh;
     __shared__ long long s_xi[3][kSlots];
     __shared__ T s_xm[3];
+    const TileAtom ta = tile_of(b, tile);
     if (MODE != FM_FORCES) {   // the noise sums' slots, loaded with the descriptors
-        const int sys = b.tile_sys[tile];
-        const long long* xa = b.acc + (size_t)sys * ACC_N * kSlots + (size_t)ACC_XI * kSlots;
+        const long long* xa = b.acc + (size_t)ta.sys * ACC_N * kSlots + (size_t)ACC_XI * kSlots;
         for (int w = threadIdx.x; w < 3 * kSlots; w += blockDim.x) s_xi[w / kSlots][w % kSlots] = xa[w];
     }
-    const TileAtom ta = stage_tile(b, tile, sh);
+    stage_sys(b, ta.sys, sh);
+    __syncthreads();
     const DevSys& S = sh.S;
     const DevState& st = sh.st;
     DevState& gst = b.st[ta.sys];
@@ -2278,57 +2789,72 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
     __shared__ __align__(16) StagedSys sh;
     __shared__ long long s_xi[3][kSlots];
     __shared__ T s_xm[3];
-    if (MODE != FM_FORCES) {   // the noise sums' slots, loaded with the descriptors
-        const int sys = b.tile_sys[tile];
-        const long long* xa = b.acc + (size_t)sys * ACC_N * kSlots + (size_t)ACC_XI * kSlots;
-        for (int w = threadIdx.x; w < 3 * kSlots; w += blockDim.x) s_xi[w / kSlots][w % kSlots] = xa[w];
+    __shared__ BoxMove bm;
+    const TileAtom ta = tile_of(b, tile);
+    const bool valid = (int)threadIdx.x < ta.count;
+    const int i = ta.first + threadIdx.x;
+    const size_t N = b.ntot;
+    // The atom's operands and the system's descriptors are loaded together, before the first is
+    // looked at (nothing else hides this kernel's latency; what a system does not use is loaded all
+    // the same and ignored: arrays of every context).
+    int4* a4 = reinterpret_cast<int4*>(b.lacc) + i;
+    int4 q = make_int4(0, 0, 0, 0), fb = q;
+    T4 d0 = mk4((T)0, (T)0, (T)0, (T)0), z = d0, xa = d0;
+    T dh[3] = {(T)0, (T)0, (T)0}, dl[3] = {(T)0, (T)0, (T)0}, pv[3] = {(T)0, (T)0, (T)0};
+    if (valid) {
+        q = *a4;
+        if (MODE != FM_FORCES) {
+            const T* DH = reinterpret_cast<const T*>(b.dhi);
+            const T* DL = reinterpret_cast<const T*>(b.dlo);
+            const T* V = reinterpret_cast<const T*>(b.v);
+            d0 = reinterpret_cast<const T4*>(b.sd0)[i];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                dh[k] = DH[k * N + i];
+                if constexpr (sizeof(T) == 4) dl[k] = DL[k * N + i];
+                pv[k] = V[k * N + i];
+            }
+            z = reinterpret_cast<const T4*>(b.xi)[i];
+            if (MODE == FM_STEP && fuse) {
+                if (b.want_xs) xa = reinterpret_cast<const T4*>(b.xa)[i];   // (no barostat: the box never moves)
+                if (b.want_xf) fb = b.xfb[i];
+            }
+        }
     }
-    const TileAtom ta = stage_tile(b, tile, sh);
+    const int big = b.hi_flag ? b.hi_flag[tile] : 0;                        // large terms were split
+    if (MODE != FM_FORCES) {   // the noise sums' slots, loaded with the descriptors
+        const long long* xs = b.acc + (size_t)ta.sys * ACC_N * kSlots + (size_t)ACC_XI * kSlots;
+        for (int w = threadIdx.x; w < 3 * kSlots; w += blockDim.x) s_xi[w / kSlots][w % kSlots] = xs[w];
+    }
+    stage_sys(b, ta.sys, sh);
+    __syncthreads();
     const DevSys& S = sh.S;
     const DevState& st = sh.st;
     DevState& gst = b.st[ta.sys];
     if (MODE != FM_FORCES) noise_mean_staged<T>(S, s_xi, s_xm);
+    if (MODE == FM_STEP && fuse) box_move(st, bm);
     __syncthreads();
+    if (big != 0 && threadIdx.x == 0) b.hi_flag[tile] = 0;            // every thread has read it
     const bool fz = MODE == FM_STEP && fuse && S.baro == BARO_NONE;   // uniform over the block
     T red[14];
 #pragma unroll
     for (int k = 0; k < 14; ++k) red[k] = (T)0;
     T zn[3] = {(T)0, (T)0, (T)0};
-    if ((int)threadIdx.x < ta.count) {
-        const int i = ta.first + threadIdx.x;
-        const size_t N = b.ntot;
-        // every operand is loaded before the first is used, so the loads are in flight together
-        // (this kernel streams its operands; nothing else hides their latency)
-        const bool sw = S.pot == POT_SW, springs = MODE != FM_FORCES && S.springs;
-        const bool thermo = MODE != FM_FORCES && S.thermo;
-        int4* a4 = reinterpret_cast<int4*>(b.lacc) + i;
-        int4 q = make_int4(0, 0, 0, 0);
-        T4 d0 = mk4((T)0, (T)0, (T)0, (T)0), z = d0;
-        T dh[3] = {(T)0, (T)0, (T)0}, dl[3] = {(T)0, (T)0, (T)0}, pv[3] = {(T)0, (T)0, (T)0};
-        if (sw) q = *a4;
-        if (springs || fz) {
-            const T* DH = reinterpret_cast<const T*>(b.dhi);
-            const T* DL = reinterpret_cast<const T*>(b.dlo);
-            if (springs) d0 = reinterpret_cast<const T4*>(b.sd0)[i];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                dh[k] = DH[k * N + i];
-                if constexpr (sizeof(T) == 4) dl[k] = DL[k * N + i];
-            }
-        }
-        if (MODE != FM_FORCES) {
-            const T* V = reinterpret_cast<const T*>(b.v);
-            pv[0] = V[i]; pv[1] = V[N + i]; pv[2] = V[2 * N + i];
-        }
-        if (thermo) z = reinterpret_cast<const T4*>(b.xi)[i];
-        T4 xa = mk4((T)0, (T)0, (T)0, (T)0);
-        if (fz) xa = reinterpret_cast<const T4*>(b.xa)[i];
+    if (valid) {
+        const bool sw = S.pot == POT_SW;
         if (sw) *a4 = make_int4(0, 0, 0, 0);
+        else q = make_int4(0, 0, 0, 0);
         const T pd[3] = {d0.x + dh[0] + dl[0], d0.y + dh[1] + dl[1], d0.z + dh[2] + dl[2]};
         const T pz[3] = {z.x, z.y, z.z};
         const T inv = (T)(1.0 / (double)kLegScale);
         const int3 fq = force_of_acc(q);
-        const T f[3] = {(T)fq.x * inv, (T)fq.y * inv, (T)fq.z * inv};
+        T f[3] = {(T)fq.x * inv, (T)fq.y * inv, (T)fq.z * inv};
+        if (sw && big != 0) {
+            int4* h4 = reinterpret_cast<int4*>(b.lacc_hi) + i;
+            const int4 h = *h4;
+            *h4 = make_int4(0, 0, 0, 0);
+            f[0] += (T)kLegCoarse * (T)h.x; f[1] += (T)kLegCoarse * (T)h.y; f[2] += (T)kLegCoarse * (T)h.z;
+        }
         T vo[3], Fo[3];
         finish_atom<T, MODE>(b, S, st, i, f, (T)0, false, pd, pv, pz, s_xm, red, fz, vo, Fo);
         if (fz) {
@@ -2337,10 +2863,10 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
             const T ck = pick<T>(S.ckick, S.ckick_f);
             T vk[3];
             for (int k = 0; k < 3; ++k) {
-                vk[k] = vo[k] + ck * Fo[k];
+                vk[k] = fma_rn(ck, Fo[k], vo[k]);
                 V[k * N + i] = vk[k];
             }
-            drift_atom<T>(b, S, st, i, xa, vk, true, dh, dl, 0, &gst.rebuild_next,
+            drift_atom<T>(b, S, st, bm, i, xa, fb, vk, true, dh, dl, 0, &gst.rebuild_next,
                           b.any_rebuild ? b.any_rebuild + 1 : nullptr, (unsigned long long)st.k + 1ULL,
                           zn);
         }
@@ -2565,6 +3091,7 @@ __global__ void __launch_bounds__(kTile) k_group(Bufs b, const DevGroup* groups,
                     st.s[k] = 1.0; st.phi[k] = 1.0; st.phi_f[k] = 1.0f; st.sm1_f[k] = 0.0f;
                 }
                 st.scaled = 0;
+                scale_of_box(b, s, st.box);
             } else {
                 observe(sh[mi].S, sh[mi].st);
             }
@@ -2623,6 +3150,7 @@ __global__ void __launch_bounds__(kTile) k_group(Bufs b, const DevGroup* groups,
             for (int mi = 0; mi < nm; ++mi) {
                 DevState& st = sh[mi].st;
                 prepare_step(sh[mi].S, st, b.dt);
+                if (st.scaled) scale_of_box(b, members[mi], st.box);
                 st.rebuild = (carry && sh[mi].S.baro == BARO_NONE) ? st.rebuild_next : 0;
                 st.rebuild_next = 0;
                 st.k += 1;
@@ -2862,11 +3390,42 @@ void launch_kick_drift(const Bufs& b, int precision, int ntiles, int mode, cudaS
     if (launches) *launches += 1;
 }
 
+void launch_positions(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches) {
+    if (ntiles <= 0) return;
+    if (precision == NEFE_FP64) k_positions<double><<<ntiles, kTile, 0, s>>>(b);
+    else k_positions<float><<<ntiles, kTile, 0, s>>>(b);
+    if (launches) *launches += 1;
+}
+
+// Fractional positions only (stateless scatter form).
+__global__ void __launch_bounds__(kTile) k_frac_positions(Bufs b) {
+    const int i = blockIdx.x * kTile + threadIdx.x;
+    if (i >= b.ntot) return;
+    const size_t N = b.ntot;
+    const double x[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
+    const int4 f = frac_position(x, b.st[0]);
+    b.xf[i] = f;
+    b.xc[i] = pack_frac(f);
+    if (i == 0) scale_of_box(b, 0, b.st[0].box);
+}
+void launch_frac_positions(const Bufs& b, cudaStream_t s) {
+    if (b.ntot > 0) k_frac_positions<<<(b.ntot + kTile - 1) / kTile, kTile, 0, s>>>(b);
+}
+
 void launch_mirror(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches) {
     if (ntiles <= 0) return;
     if (precision == NEFE_FP64) k_mirror<double><<<ntiles, kTile, 0, s>>>(b);
     else k_mirror<float><<<ntiles, kTile, 0, s>>>(b);
     if (launches) *launches += 1;
+}
+
+// Atoms per warp of the scatter form's pass A (see k_edges_s), as a power of two: by the whole
+// context's size, so that a run does not depend on how the passes are launched.
+constexpr int kScatterFull = 8;          // warps per SM
+static int scatter_atoms(int ntot) {
+    for (int lg : {5, 4})
+        if (ntot >= (152 * kScatterFull << lg)) return lg;
+    return 3;
 }
 
 template <typename T>
@@ -2878,9 +3437,18 @@ static void edges_dispatch(const Bufs& b, int lanes, int ntiles, cudaStream_t s)
             if constexpr (sizeof(T) == 8) {
                 k_edges<T, 8><<<ntiles * 8, kTile, 0, s>>>(b);
             } else {
-                const int items = ntiles * (kTile / kEdges1Threads);
-                if (lanes == 0) k_edges1<T, true><<<items, kEdges1Threads, 0, s>>>(b);
-                else k_edges1<T, false><<<items, kEdges1Threads, 0, s>>>(b);
+                if (lanes == 0) {
+                    const int lg = scatter_atoms(b.ntot), items = ntiles << (6 - lg);
+                    const auto go = [&](auto kernel) { kernel<<<items, kScatterThreads, 0, s>>>(b, b.swc_common, lg); };
+                    const bool full = items >= 152 * kScatterBlocks;
+                    if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks>);          // (stateless: one system)
+                    else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks>);
+                    else if (!b.common) go(k_edges_s<false, false, false, kScatterBlocks>);
+                    else if (full) go(k_edges_s<false, false, true, kScatterBlocks>);
+                    else go(k_edges_s<false, false, true, kScatterBlocksFew>);
+                } else {
+                    k_edges1<T><<<ntiles * (kTile / kEdges1Threads), kEdges1Threads, 0, s>>>(b);
+                }
             }
             break;
         }

@@ -13,7 +13,7 @@ struct Bufs {
     const DevSys* sys;
     DevState* st;
     long long* acc;          // [nsys][ACC_N][kSlots]
-    const int* tile_sys;     // system of each 128-atom tile
+    const int4* tiles;       // 128-atom tiles: system, first atom, atom count
     double* x;               // FP64 anchor positions (positions at the last list build), SoA
     void* dhi;               // displacement since the last build, kernel precision, SoA (may be NULL)
     void* dlo;               // its compensation term (FP32 path; may be NULL)
@@ -64,7 +64,18 @@ struct Bufs {
     const int* uf_tiles;     // tiles of the UF systems (per-step UF kernel), or NULL: every tile
     int* scan_sums;          // stateless: span sums of a multi-block cell scan (NULL: one block)
     int ncells_host;         // stateless: number of cells of the grid
-    int* lacc;               // [ntot][4] int32 force accumulators of the scatter form (2^-21 eV/A)
+    int* lacc;               // [ntot][4] int32 force accumulators of the scatter form (2^-22 eV/A)
+    int* lacc_hi;            // [ntot][4] multiples of large terms (see k_edges_s)
+    SWc<float> swc_common;   // the potential constants, where every system has the same (common)
+    int common;
+    int leg_refuse;          // the scatter form was chosen by the caller: terms above its limit are refused
+    int* hi_flag;            // [tiles] some large term was split this step (cleared by k_finish)
+    float4* lscale;          // [nsys][2] L 2^-32 as FP32 value and remainder
+    int4* xf;                // FP32: fractional positions (x/L as 32-bit fixed point)
+    int4* xfb;               // their values at the last list build
+    uint2* xc;               // their top 21 bits per axis (pass A's row filter)
+    int want_xf, want_xs;    // FP32 per-step positions: fractional (scatter form), mirror (the others)
+    int row4;                // row-major rows can be read 16 bytes at a time
     int* any_rebuild;        // engine: [0] some system's rebuild flag is set this step, [1] some
                              // rebuild_next is set (fused epilogue); NULL in the stateless calls
     int rebuild_all;         // engine: when any system's list is stale, every system rebuilds (one
@@ -113,6 +124,10 @@ void launch_inject(const Bufs& b, int precision, int ntiles, const double* x, co
 // was fused (its next-step noise sums and rebuild flag are moved into place).
 void launch_group(const Bufs& b, const DevGroup* groups, int ngroups, int mode, cudaStream_t s,
                   long* launches, int carry = 0);
+// Positions of every atom from anchor and displacement, in the forms in use (want_xf, want_xs).
+void launch_positions(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches);
+// Fractional positions of b.x (stateless scatter form).
+void launch_frac_positions(const Bufs& b, cudaStream_t s);
 // Mirror only (stateless force entry): q and xs from x with the list-build formula.
 void launch_mirror(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches);
 // Thermostat noise as FP64 (n,3).

@@ -25,7 +25,7 @@ constexpr size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign;
 constexpr size_t kOffSys = 0;
 constexpr size_t kOffSt = align_up(kOffSys + sizeof(DevSys));
 constexpr size_t kOffTile = align_up(kOffSt + sizeof(DevState));
-constexpr size_t kOffXs = align_up(kOffTile + sizeof(int) * (NEFE_NOALLOC_MAX_ATOMS / kTile + 1));
+constexpr size_t kOffXs = align_up(kOffTile + sizeof(int4) * (NEFE_NOALLOC_MAX_ATOMS / kTile + 1));
 constexpr size_t kOffXa = align_up(kOffXs + sizeof(float4) * NEFE_NOALLOC_MAX_ATOMS);
 constexpr size_t kOffQ = align_up(kOffXa + sizeof(float4) * NEFE_NOALLOC_MAX_ATOMS);
 constexpr size_t kOffCount = align_up(kOffQ + sizeof(int4) * NEFE_NOALLOC_MAX_ATOMS);
@@ -58,7 +58,7 @@ int scratch_address(void** out) {
 // Writes the one-system descriptors (passed by value, so the call issues no host-to-device
 // copy from host memory), the tile table (every tile belongs to system 0) and zeroed
 // occupancy counts into the scratch.
-__global__ void k_noalloc_init(DevSys hs, DevState st, DevSys* dsys, DevState* dst, int* tile_sys, int ntiles,
+__global__ void k_noalloc_init(DevSys hs, DevState st, DevSys* dsys, DevState* dst, int4* tiles, int ntiles,
                                int* counts, int ncells) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
@@ -66,7 +66,7 @@ __global__ void k_noalloc_init(DevSys hs, DevState st, DevSys* dsys, DevState* d
         *dsys = hs;
         *dst = st;
     }
-    for (int i = t; i < ntiles; i += stride) tile_sys[i] = 0;
+    for (int i = t; i < ntiles; i += stride) tiles[i] = make_int4(0, i * kTile, min(kTile, hs.n - i * kTile), 0);
     for (int i = t; i < ncells; i += stride) counts[i] = 0;
 }
 
@@ -118,7 +118,7 @@ extern "C" int nefe_cell_bin_noalloc(const double* x, int n, const double box[3]
         const int blocks = (work + 255) / 256 < 152 ? (work + 255) / 256 : 152;
         k_noalloc_init<<<blocks, 256, 0, s>>>(hs, st, reinterpret_cast<DevSys*>(p + kOffSys),
                                                reinterpret_cast<DevState*>(p + kOffSt),
-                                               reinterpret_cast<int*>(p + kOffTile), ntiles,
+                                               reinterpret_cast<int4*>(p + kOffTile), ntiles,
                                                reinterpret_cast<int*>(p + kOffCount), (int)total);
         NEFE_CU(cudaGetLastError());
     }
@@ -127,7 +127,7 @@ extern "C" int nefe_cell_bin_noalloc(const double* x, int n, const double box[3]
     std::memset(&b, 0, sizeof(b));
     b.sys = reinterpret_cast<DevSys*>(p + kOffSys);
     b.st = reinterpret_cast<DevState*>(p + kOffSt);
-    b.tile_sys = reinterpret_cast<int*>(p + kOffTile);
+    b.tiles = reinterpret_cast<int4*>(p + kOffTile);
     b.x = const_cast<double*>(x);
     b.xs = p + kOffXs;
     b.xa = p + kOffXa;

@@ -145,3 +145,107 @@ def test_adjoint_does_not_depend_on_when_lists_are_built(N, kind):
     for g in got[1:]:
         assert g[0] == got[0][0]
         assert all(np.array_equal(a, b) for a, b in zip(g[1:], got[0][1:]))
+
+
+# ------------------------------------------------------------------ scatter form
+def _forces32(N, x, box, skin, cap, shift=0):
+    n, rcs = len(x), RC + skin
+    xd = soa(x)
+    nbr = torch.zeros(n * cap + shift, dtype=torch.int32, device="cuda")[shift:]
+    nbr.fill_(-1)                                       # what lies past a row's length is the caller's
+    cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+    N.nefe_neighbor_build(xd, n, box, rcs, cap, nbr, cnt)
+    f = torch.zeros(3 * n, dtype=torch.float64, device="cuda")
+    e = torch.zeros(n, dtype=torch.float64, device="cuda")
+    ev = torch.zeros(7, dtype=torch.float64, device="cuda")
+    N.nefe_sw_forces(xd, n, box, rcs, nbr, cnt, cap, N.nefe_sw_params_silicon(), N.NEFE_FP32, f, e, ev)
+    torch.cuda.synchronize()
+    return f.cpu().numpy().reshape(3, n).T, e.cpu().numpy(), ev.cpu().numpy()
+
+
+def _close32(x, box, got):
+    """The FP32 tolerance of the parity tests: 1e-5 of the largest force, energy and virial scale."""
+    e_o, f_o, vir_o, ea_o = O.sw_energy(x, box)
+    f, e, ev = got
+    assert np.abs(f - f_o).max() <= 1e-5 * np.abs(f_o).max()
+    assert np.abs(e - ea_o).max() <= 1e-5 * np.abs(ea_o).max()
+    assert abs(ev[0] - e_o) <= 1e-5 * abs(e_o)
+    assert np.abs(ev[1:] - vir_o).max() <= 1e-4 * np.abs(vir_o).max()
+
+
+@pytest.mark.parametrize("cap,shift", [(48, 0), (48, 1), (47, 0), (64, 0)])
+@pytest.mark.parametrize("n", [31, 33, 129, 1000])
+def test_scatter_forces_at_ragged_sizes(N, n, cap, shift):
+    """Ragged warps and tiles, rows that cannot be read 16 bytes at a time, rows above 32 entries
+    (skin 1.4 A), coordinates many boxes away."""
+    x, box = I.liquid(max(n, 700), 0.05, seed=100 + n)
+    x = x[:n] + np.array([7.0 * box[0], -123.0, 0.0])
+    _close32(x, box, _forces32(N, x, box, 1.4 if cap == 64 else 0.5, cap, shift))
+
+
+def test_scatter_forces_with_more_edges_than_a_list(N):
+    """28 neighbours inside the cutoff: a warp's edges take several batches (896 of 224)."""
+    x, box = I.diamond(5, 5, 5, a=4.4)
+    x = I.rattle(x, 0.05, 7)
+    _close32(x, box, _forces32(N, x, box, 0.3, 64))
+
+
+@pytest.mark.parametrize("r", [1.2, 0.8])
+def test_scatter_forces_of_close_pairs(N, r):
+    """Terms far above what the first accumulator holds (some 1e2 to 1e4 eV/A) are split and lose
+    nothing: relative to the largest force as any other."""
+    x, box = I.diamond(3, 3, 3)
+    x = I.rattle(x, 0.1, 8)
+    d = x[1] - x[0]
+    d -= box * np.rint(d / box)
+    x[1] = x[0] + d * (r / np.linalg.norm(d))
+    _close32(x, box, _forces32(N, x, box, 0.5, 48))
+
+
+def test_chosen_scatter_form_refuses_what_it_always_refused(N):
+    """A context whose form was set by hand flags terms of 48 eV/A or more; the default takes them."""
+    x, box = I.diamond(3, 3, 3)
+    d = x[4] - x[0]
+    x[4] = x[0] + d * (1.3 / np.linalg.norm(d))
+    got = {}
+    for chosen in (False, True):
+        ctx = N.Context(precision=N.NEFE_FP32, skin=0.5, nbr_cap=48)
+        s = ctx.add_system(x, box, v=np.zeros_like(x))
+        if chosen:
+            ctx.set_tuning(0)
+        ctx.run(1)
+        got[chosen] = ctx.results(s)["error"]
+        ctx.close()
+    assert got == {False: 0, True: 4}
+
+
+@pytest.mark.parametrize("shape", [(2, 2, 2), (10, 10, 10), (16, 16, 16)])
+def test_scatter_form_atoms_per_warp(N, shape):
+    """Context sizes that take 8, 16 and 32 atoms to a warp, with different potentials in one context
+    (constants from the table) and with one (constants as arguments): energy of the state read back
+    against the FP64 kernel's, 1e-5 relative."""
+    x0, box = I.diamond(*shape)
+    n = len(x0)
+    reps = 5 if shape == (10, 10, 10) else 1
+    for scale in (1.0, 0.97):
+        ctx = N.Context(precision=N.NEFE_FP32, skin=0.5, nbr_cap=48)
+        for r in range(reps + 1):
+            s = ctx.add_system(x0, box, v=I.gaussian_velocities(n, 5.0, 40 + r))
+            ctx.set_thermostat(s, 900.0, 0.1, 50 + r)
+        p = N.nefe_sw_params_silicon()
+        p.lambda3 *= scale
+        ctx.set_sw_params(0, p)
+        ctx.run(40)
+        for s in (0, reps):
+            x, _, b = ctx.get_state(s)
+            xd = soa(x)
+            nbr = torch.zeros(n * 48, dtype=torch.int32, device="cuda")
+            cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+            N.nefe_neighbor_build(xd, n, b, RC + 0.5, 48, nbr, cnt)
+            f, ev = torch.zeros(3 * n, dtype=torch.float64, device="cuda"), torch.zeros(7, dtype=torch.float64, device="cuda")
+            N.nefe_sw_forces(xd, n, b, RC + 0.5, nbr, cnt, 48, p if s == 0 else N.nefe_sw_params_silicon(), N.NEFE_FP64, f,
+                             None, ev)
+            r = ctx.results(s)
+            assert r["error"] == 0
+            assert r["U"] == pytest.approx(float(ev[0]), rel=1e-5)
+        ctx.close()
