@@ -80,6 +80,7 @@ struct DevSys {
     double amp;                 // Langevin noise amplitude sqrt(2 m kB T / (tdamp dt)) (eV/A)
     double gam;                 // Langevin friction m / tdamp (eV ps / A^2)
     double ckick;               // dt / (2 m) (A^2 / (eV ps))
+    double baro_c;              // dt / Q_b of the barostat, Q_b = (N + 1) kB T tau_P^2 (1 / (eV ps))
     // FP32 copies and flags read by the FP32 kernels (no FP64 instruction per atom)
     float amp_f, gam_f, ckick_f, mass_f, kE_f, kint_f, dt_f, inv_n_f;
     float rcs2_lo_f, rcs2_hi_f; // list radius^2 times (1 -/+ 1e-4): FP32 filter band

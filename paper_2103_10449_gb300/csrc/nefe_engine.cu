@@ -355,6 +355,7 @@ int setup(nefe_ctx* c) {
         d.amp = h.tdamp > 0.0 ? std::sqrt(2.0 * d.mass_e * kB * h.T / (h.tdamp * c->dt)) : 0.0;
         d.gam = h.tdamp > 0.0 ? d.mass_e / h.tdamp : 0.0;
         d.ckick = 0.5 * c->dt / d.mass_e;
+        d.baro_c = h.baro != NEFE_BARO_NONE ? c->dt / ((h.n + 1) * kB * h.T * h.pdamp * h.pdamp) : 0.0;
         d.amp_f = (float)d.amp; d.gam_f = (float)d.gam; d.ckick_f = (float)d.ckick;
         d.mass_f = (float)d.mass_e; d.kE_f = (float)d.k_E; d.kint_f = (float)d.k_int;
         d.dt_f = (float)c->dt;
