@@ -92,7 +92,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
 
 namespace {
 struct SwcBytes {
-    alignas(16) unsigned char b[sizeof(SWc<double>)];
+    alignas(16) unsigned char b[sizeof(SWc<float>)];
 };
 
 __device__ __forceinline__ void copy_words(void* dst, const void* src, int bytes, int t) {
@@ -159,10 +159,7 @@ int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3]
     st.scale_int = 1.0;
     SwcBytes sw;
     std::memset(&sw, 0, sizeof(sw));
-    if (prm && prec == NEFE_FP64) {
-        const SWc<double> c = make_swc<double>(*prm);
-        std::memcpy(sw.b, &c, sizeof(c));
-    } else if (prm) {
+    if (prm && prec == NEFE_FP32) {
         const SWc<float> c = make_swc<float>(*prm);
         std::memcpy(sw.b, &c, sizeof(c));
     }
@@ -204,13 +201,13 @@ static int read_error(const Scratch1& S, unsigned* err) {
 static void want_forces(Scratch1& S, int n, int precision) {
     const size_t N = (size_t)n;
     S.want(&S.shn, sizeof(int) * N);
+    S.want(&S.xc, sizeof(uint2) * N);
+    S.want(&S.lscale, sizeof(float4) * 2);
     if (precision == NEFE_FP32) {
         S.want(&S.xf, sizeof(int4) * N);
-        S.want(&S.xc, sizeof(uint2) * N);
         S.want(&S.lacc, 4 * sizeof(int) * N);
         S.want(&S.lacc_hi, 4 * sizeof(int) * N);
         S.want(&S.hi_flag, sizeof(int) * ((N + kTile - 1) / kTile));
-        S.want(&S.lscale, sizeof(float4) * 2);
     } else {
         S.want(&S.shd, sizeof(double4) * N * kShell);
         S.want(&S.shj, sizeof(int) * N * kShell);
@@ -218,22 +215,28 @@ static void want_forces(Scratch1& S, int n, int precision) {
     }
 }
 
-// Both force passes of a stateless call.
+// Both force passes of a stateless call.  FP64 pass B: one lane per atom from kGatherOne atoms on (its
+// epilogue runs on one lane per atom, so more lanes cost FP64 issue; fewer atoms want shorter chains).
+constexpr int kGatherOne = 20000;
 static int run_forces(const Scratch1& S, Bufs& b, int n, const nefe_sw_params* prm, int precision) {
     const int ntiles = (n + kTile - 1) / kTile;
+    b.xc = S.xc; b.lscale = S.lscale;
+    b.row4 = (b.cap & 3) == 0 && (reinterpret_cast<uintptr_t>(b.nbr) & 15) == 0;
+    b.lg = atoms_per_warp_log2(precision, n);
+    b.common = 1;
     if (precision == NEFE_FP32) {
-        b.xf = S.xf; b.xc = S.xc; b.lacc = S.lacc; b.lacc_hi = S.lacc_hi; b.hi_flag = S.hi_flag; b.lscale = S.lscale;
-        b.swc_common = make_swc<float>(*prm); b.common = 1;
-        b.row4 = (b.cap & 3) == 0 && (reinterpret_cast<uintptr_t>(b.nbr) & 15) == 0;
+        b.xf = S.xf; b.lacc = S.lacc; b.lacc_hi = S.lacc_hi; b.hi_flag = S.hi_flag;
+        b.swc_common = make_swc<float>(*prm);
         NEFE_CU(cudaMemsetAsync(S.lacc, 0, (size_t)(reinterpret_cast<char*>(S.hi_flag + ntiles) - reinterpret_cast<char*>(S.lacc)),
                                 S.s));
         launch_frac_positions(b, S.s);
         launch_edges(b, precision, 0, ntiles, FM_FORCES, S.s, nullptr);
         launch_gather(b, precision, 0, ntiles, FM_FORCES, S.s, nullptr);
     } else {
+        b.swp_common = sw_params_real(*prm);
         launch_mirror(b, precision, ntiles, S.s, nullptr);
         launch_edges(b, precision, 8, ntiles, FM_FORCES, S.s, nullptr);
-        launch_gather(b, precision, 4, ntiles, FM_FORCES, S.s, nullptr);
+        launch_gather(b, precision, n >= kGatherOne ? 1 : 4, ntiles, FM_FORCES, S.s, nullptr);
     }
     NEFE_CU(cudaGetLastError());
     return NEFE_OK;

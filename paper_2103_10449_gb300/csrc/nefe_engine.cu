@@ -75,6 +75,7 @@ struct nefe_ctx {
     uint2* d_xc = nullptr;
     int4 *d_xf = nullptr, *d_xfb = nullptr;                               // fractional positions (FP32)
     bool chosen = false;     // pass A's form was set by nefe_set_tuning or the autotuner
+    bool gchosen = false;    // pass B's lanes likewise
     bool stale_pos = false;  // the positions' forms have to be made anew before the next step
     void* d_uf_F = nullptr;
     int n_uf_tiles = 0;      // tiles of the systems with a Uhlenbeck-Ford term
@@ -166,7 +167,9 @@ double rc_of(const HostSys& h) { return h.prm.a * h.prm.sigma; }
 void set_form(nefe_ctx* c, int lanes) {
     c->lanes = lanes;
     const bool scatter = c->prec == NEFE_FP32 && lanes == 0;
-    const int xf = scatter ? 1 : 0, xs = !scatter || c->n_uf_tiles > 0 ? 1 : 0;
+    const int xf = scatter || c->prec == NEFE_FP64 ? 1 : 0, xs = !scatter || c->n_uf_tiles > 0 ? 1 : 0;
+    // FP64: 8, 16, 32 lanes per atom set by hand stand for 16, 8, 4 atoms per warp
+    c->b.lg = c->prec == NEFE_FP64 && c->chosen ? (lanes <= 8 ? 4 : lanes == 16 ? 3 : 2) : atoms_per_warp_log2(c->prec, c->ntot);
     if (c->b.want_xf != xf || c->b.want_xs != xs) c->stale_pos = true;
     c->b.want_xf = xf;
     c->b.want_xs = xs;
@@ -446,11 +449,11 @@ int setup(nefe_ctx* c) {
         if ((rc = dalloc(c, &c->d_lacc, 4 * sizeof(int) * N))) return rc;
         if ((rc = dalloc(c, &c->d_lacc_hi, 4 * sizeof(int) * N))) return rc;
         if ((rc = dalloc(c, &c->d_hi_flag, sizeof(int) * tile_sys.size()))) return rc;
-        if ((rc = dalloc(c, &c->d_lscale, sizeof(float4) * 2 * nsys))) return rc;
         if ((rc = dalloc(c, &c->d_xf, sizeof(int4) * N))) return rc;
-        if ((rc = dalloc(c, &c->d_xfb, sizeof(int4) * N))) return rc;
-        if ((rc = dalloc(c, &c->d_xc, sizeof(uint2) * N))) return rc;
     }
+    if ((rc = dalloc(c, &c->d_lscale, sizeof(float4) * 2 * nsys))) return rc;
+    if ((rc = dalloc(c, &c->d_xfb, sizeof(int4) * N))) return rc;
+    if ((rc = dalloc(c, &c->d_xc, sizeof(uint2) * N))) return rc;
     if ((rc = dalloc(c, &c->d_rtiles, sizeof(int) * tile_sys.size()))) return rc;
     if ((rc = dalloc(c, &c->d_rcount, sizeof(int)))) return rc;
     if ((rc = dalloc(c, &c->d_rcbase, sizeof(int) * (size_t)(nsys + 1)))) return rc;
@@ -480,12 +483,15 @@ int setup(nefe_ctx* c) {
         NEFE_CU(cudaMemset(c->d_uf_F, 0, v4 * N));
     }
     SWc<float> swc_common{};
+    SWp<double> swp_common{};
     bool common = false;
     if (c->prec == NEFE_FP64) {
-        std::vector<SWc<double>> t(nsys);
-        for (int s = 0; s < nsys; ++s) t[s] = make_swc<double>(c->sys[s].prm);
-        if ((rc = dalloc(c, &c->d_swc, sizeof(SWc<double>) * nsys))) return rc;
-        NEFE_CU(cudaMemcpy(c->d_swc, t.data(), sizeof(SWc<double>) * nsys, cudaMemcpyHostToDevice));
+        std::vector<SWp<double>> t(nsys);
+        for (int s = 0; s < nsys; ++s) t[s] = sw_params_real(c->sys[s].prm);
+        common = std::all_of(t.begin(), t.end(), [&](const SWp<double>& v) { return std::memcmp(&v, &t[0], sizeof(v)) == 0; });
+        swp_common = t[0];
+        if ((rc = dalloc(c, &c->d_swc, sizeof(SWp<double>) * nsys))) return rc;
+        NEFE_CU(cudaMemcpy(c->d_swc, t.data(), sizeof(SWp<double>) * nsys, cudaMemcpyHostToDevice));
     } else {
         std::vector<SWc<float>> t(nsys);
         for (int s = 0; s < nsys; ++s) t[s] = make_swc<float>(c->sys[s].prm);
@@ -545,8 +551,11 @@ int setup(nefe_ctx* c) {
     b.list_lanes = c->llanes;
     b.uf_nbr = c->d_uf_nbr; b.uf_cnt = c->d_uf_cnt; b.uf_F = c->d_uf_F; b.uf_tiles = c->d_uf_tiles;
     b.lacc = c->d_lacc; b.lacc_hi = c->d_lacc_hi; b.hi_flag = c->d_hi_flag;
+    // FP64 pass B: its epilogue runs on one lane per atom, so more lanes cost FP64 issue (16 x 8000 atoms:
+    // 149 us with 4, 56 us with 1); below 20,000 atoms the shorter chain of 4 lanes wins
+    if (c->prec == NEFE_FP64 && !c->gchosen) c->glanes = c->ntot >= 20000 ? 1 : 4;
     b.xf = c->d_xf; b.xfb = c->d_xfb; b.lscale = c->d_lscale; b.xc = c->d_xc;
-    b.swc_common = swc_common; b.common = common ? 1 : 0;
+    b.swc_common = swc_common; b.swp_common = swp_common; b.common = common ? 1 : 0;
     set_form(c, c->lanes);
 
     launch_inject(b, c->prec, c->ntiles, nullptr, c->d_vtmp, c->stream);
@@ -1106,7 +1115,7 @@ int nefe_autotune(nefe_ctx* c) {
     if (rc) return rc;
     if ((rc = set_device(c))) return rc;
     if (!c->chosen) drop_graph(c);               // what the forms refuse is captured in the step graph
-    c->chosen = true;
+    c->chosen = c->gchosen = true;
     c->b.leg_refuse = 1;
     Bufs b = c->b;
     if (c->prec == NEFE_FP32) {                  // every form is timed: both kinds of positions
@@ -1120,6 +1129,7 @@ int nefe_autotune(nefe_ctx* c) {
     NEFE_CU(cudaEventCreate(&e0));
     NEFE_CU(cudaEventCreate(&e1));
     // best of three trials of five launches each, after two warm-up launches
+    auto lg_of = [&](int l) { return c->prec == NEFE_FP64 ? (l == 8 ? 4 : l == 16 ? 3 : 2) : c->b.lg; };
     auto time_us = [&](auto&& launch) {
         for (int w = 0; w < 2; ++w) launch();
         double best_trial = 1e30;
@@ -1159,6 +1169,7 @@ int nefe_autotune(nefe_ctx* c) {
             });
             scatter_us = us;
         } else {
+            b.lg = lg_of(l);
             us = time_us([&] { launch_edges(b, c->prec, l, c->ntiles, FM_FORCES, c->stream, &c->launches); });
         }
         ranked_a.push_back({us, l});
@@ -1168,6 +1179,7 @@ int nefe_autotune(nefe_ctx* c) {
     cudaFree(tv0);
     cudaFree(tf0);
     std::sort(ranked_a.begin(), ranked_a.end());
+    b.lg = lg_of(best_l);
     launch_edges(b, c->prec, best_l == 0 ? 1 : best_l, c->ntiles, FM_FORCES, c->stream, &c->launches);
     double best_g = 1e30;
     int best_gl = c->glanes;
@@ -1413,6 +1425,7 @@ int nefe_set_gather_tuning(nefe_ctx* c, int lanes) {
     if (lanes != 1 && lanes != 2 && lanes != 4 && lanes != 8)
         return fail(NEFE_EINVAL, "pass B supports 1, 2, 4 or 8 lanes per atom");
     if (lanes != c->glanes) drop_graph(c);
+    c->gchosen = true;
     c->glanes = lanes;
     return NEFE_OK;
 }

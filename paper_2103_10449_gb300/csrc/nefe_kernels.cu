@@ -126,10 +126,40 @@ template <> struct Noise<float> {
 // moving it to the 2^-32 scale, so a block's contribution carries at most 2^-17 of rounding
 // on top of its FP32 summation error.  Integer addition makes the per-system total independent
 // of the order in which blocks arrive.  Every thread of the block must call it.
+// In FP64 the threads' values are converted first (2^-40 units) and summed as integers: FP64 adds
+// run at 2 lanes a cycle, and five of them per value and warp were a third of the epilogue.  Values
+// of 2^22 or more (or not finite) take the FP64 sums.
 // ------------------------------------------------------------------------------------
 template <typename T, int K>
 __device__ __forceinline__ void block_sum_to_acc(T (&v)[K], long long* acc_sys, int first,
                                                  unsigned* err) {
+    if constexpr (sizeof(T) == 8) {
+        __shared__ long long ired[kTile / 32][K];
+        bool big = false;
+#pragma unroll
+        for (int k = 0; k < K; ++k) big = big || !(fabs(v[k]) < 4194304.0);
+        if (!__syncthreads_or(big)) {
+            const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                long long q = __double2ll_rn(v[k] * 0x1p40);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+                if (lane == 0) ired[w][k] = q;
+            }
+            __syncthreads();
+            if (threadIdx.x < K) {
+                long long s = 0;
+                for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += ired[i][threadIdx.x];
+                s = (s + 128) >> 8;
+                if (s != 0)
+                    atomicAdd(reinterpret_cast<unsigned long long*>(
+                                  &acc_sys[(size_t)(first + threadIdx.x) * kSlots + (blockIdx.x % kSlots)]),
+                              (unsigned long long)s);
+            }
+            return;
+        }
+    }
     __shared__ T red[kTile / 32][K];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
@@ -319,6 +349,19 @@ __device__ __forceinline__ int4 frac_position(const double (&x)[3], const DevSta
     return make_int4(frac32(x[0], st.ibox[0]), frac32(x[1], st.ibox[1]), frac32(x[2], st.ibox[2]), 0);
 }
 
+// L 2^-32 of system s as FP32 value and remainder (what pass A's positions are scaled by).
+__device__ __forceinline__ void scale_of_box(const Bufs& b, int s, const double box[3]) {
+    if (!b.lscale) return;
+    float hi[3], lo[3];
+    for (int k = 0; k < 3; ++k) {
+        const double L = box[k] * 0x1p-32;
+        hi[k] = (float)L;
+        lo[k] = (float)(L - (double)hi[k]);
+    }
+    b.lscale[2 * s] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+    b.lscale[2 * s + 1] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+}
+
 // ------------------------------------------------------------------------------------
 // Rebuild R1: fold the displacement into the FP64 anchor; cell of each atom, unwrapped cell
 // index q, fresh mirror, spring offset, occupancy count.  The cell grid was set with the system's
@@ -357,10 +400,10 @@ __device__ void cells_count_tile(const Bufs& b, int tile) {
     reinterpret_cast<T4*>(b.xs)[i] = m;
     if (b.xa) reinterpret_cast<T4*>(b.xa)[i] = m;
     if (b.sd0) reinterpret_cast<T4*>(b.sd0)[i] = mk4((T)sd[0], (T)sd[1], (T)sd[2], (T)0);
-    if (b.xf && b.want_xf) {
+    if (b.xfb && b.want_xf) {
         const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
         const int4 f = frac_position(x3, st);
-        b.xf[i] = f;
+        if (b.xf) b.xf[i] = f;
         b.xfb[i] = f;
         b.xc[i] = pack_frac(f);
     }
@@ -1434,6 +1477,12 @@ __global__ void __launch_bounds__(kTile) k_mirror(Bufs b) {
         xs[k] = xk - (double)q * st.h[k];
     }
     reinterpret_cast<T4*>(b.xs)[i] = mk4((T)xs[0], (T)xs[1], (T)xs[2], (T)0);
+    if (b.xc) {
+        const size_t N = b.ntot;
+        const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
+        b.xc[i] = pack_frac(frac_position(x3, st));
+        if (i == 0) scale_of_box(b, 0, st.box);
+    }
 }
 
 // ------------------------------------------------------------------------------------
@@ -1461,19 +1510,6 @@ __device__ __forceinline__ void comp_add(T& hi, T& lo, T d) {
         lo = __fsub_rn(lo, __fsub_rn(h2, s));
         hi = h2;
     }
-}
-
-// L 2^-32 of system s as FP32 value and remainder (what pass A's positions are scaled by).
-__device__ __forceinline__ void scale_of_box(const Bufs& b, int s, const double box[3]) {
-    if (!b.lscale) return;
-    float hi[3], lo[3];
-    for (int k = 0; k < 3; ++k) {
-        const double L = box[k] * 0x1p-32;
-        hi[k] = (float)L;
-        lo[k] = (float)(L - (double)hi[k]);
-    }
-    b.lscale[2 * s] = make_float4(hi[0], hi[1], hi[2], 0.0f);
-    b.lscale[2 * s + 1] = make_float4(lo[0], lo[1], lo[2], 0.0f);
 }
 
 // Per-block constants of the fractional positions' update, set by threads 0..2 (the caller syncs):
@@ -1511,6 +1547,15 @@ __device__ __forceinline__ T place_atom(const Bufs& b, const DevState& st, const
             dd2 += dd * dd;
         }
         reinterpret_cast<T4*>(b.xs)[i] = mk4(m[0], m[1], m[2], (T)0);
+        if (b.want_xf) {                         // the row filter's position (FP32 does for it)
+            float mv[3];
+            for (int k = 0; k < 3; ++k) {
+                mv[k] = (float)d[k];
+                if (hmoved) mv[k] = fmaf(fmaf((float)qa[k], st.hb_f[k], (float)xav[k]), bm.omr[k], mv[k]);
+            }
+            b.xc[i] = pack_frac(make_int4(fb.x + __float2int_rn(mv[0] * bm.to_frac[0]), fb.y + __float2int_rn(mv[1] * bm.to_frac[1]),
+                                          fb.z + __float2int_rn(mv[2] * bm.to_frac[2]), 0));
+        }
     } else {
         T mv[3];
         for (int k = 0; k < 3; ++k) {
@@ -1724,8 +1769,7 @@ __device__ __forceinline__ void sw_pair_pgrad(const SWc<T>& P, T r, T out[5]) {
 //     and stores the leg force L_a = sum_b F_a(b) in shd[i][a] for pass B.  Atom i gets -L_a
 //     (the three forces of a triplet sum to zero) and half of h(i; a, b) per ordered pair.
 // Each ordered pair costs ~14 flops and every triplet force is computed exactly once.
-// P[i] = (pair + own triplet force, atom energy); block sums of energy and virial (and, with
-// want_grad, of dE/d(A, B, p, q, a, lambda3, gamma)).
+// P[i] = (pair + own triplet force, atom energy), then the atom's virial.
 template <typename T, int L>
 __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
     using T4 = typename V4<T>::t;
@@ -1734,7 +1778,6 @@ __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
     __shared__ T4 sh_u[G][kShell + 1];     // (d, r^2) after compaction, then (u, r)
     __shared__ T sh_g[G][kShell + 1];
     __shared__ T sh_dg[G][kShell + 1];
-    __shared__ T sh_id[G][kShell + 1];     // 1/(s - a), parameter gradients only
     __shared__ T4 soff[27];
 
     const int tile = blockIdx.x / L + b.tile_base, part = blockIdx.x % L;
@@ -1753,8 +1796,6 @@ __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
 
     T fx = 0, fy = 0, fz = 0, en = 0;
     T w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
-    T gth[7] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0, (T)0};   // dE/d(A, B, p, q, a, lambda3, gamma)
-    const bool grad = b.want_grad != 0;
     if (valid) {
         const T4 xi = reinterpret_cast<const T4*>(b.xs)[i];
         const int ci = min(b.cnt[i], b.cap);
@@ -1821,13 +1862,6 @@ __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
             sh_u[grp][a] = mk4(d.x * ir, d.y * ir, d.z * ir, r);
             sh_g[grp][a] = g;
             sh_dg[grp][a] = dg;
-            if (grad) {   // each pair is seen from both ends: half of each derivative
-                T pg[5];
-                sw_pair_pgrad<T>(P, r, pg);
-                for (int k = 0; k < 5; ++k) gth[k] += (T)0.5 * pg[k];
-                const T den = r * P.inv_sig - P.a;
-                sh_id[grp][a] = den < -cut_eps<T>() ? xrcp(den) : (T)0;
-            }
         }
         __syncwarp(gmask);
         // 3. leg forces
@@ -1836,7 +1870,7 @@ __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
             const T ga = sh_g[grp][a];
             const T k1 = (T)2 * P.epslam * ga * xrcp(ua.w);
             const T k2 = P.epslam * sh_dg[grp][a];
-            T ax = 0, ay = 0, az = 0, cc = 0, eh = 0, e1 = 0, e2 = 0;
+            T ax = 0, ay = 0, az = 0, cc = 0, eh = 0;
             for (int bb = 0; bb < m; ++bb) {
                 if (bb == a) continue;
                 const T4 ub = sh_u[grp][bb];
@@ -1849,11 +1883,6 @@ __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
                 cc += t1 * c - k2 * dc * s1;
                 const T hb = dc * s1;                    // (c - c0)^2 g_b
                 eh += hb;
-                if (grad) {
-                    const T idb = sh_id[grp][bb];
-                    e1 += hb * idb;
-                    e2 += hb * idb * idb;
-                }
             }
             const T lx = cc * ua.x - ax, ly = cc * ua.y - ay, lz = cc * ua.z - az;
             Fl[a] = mk4(lx, ly, lz, (T)0);
@@ -1865,13 +1894,6 @@ __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
             w3 += (T)0.5 * (dx * ly + dy * lx);
             w4 += (T)0.5 * (dx * lz + dz * lx);
             w5 += (T)0.5 * (dy * lz + dz * ly);
-            if (grad) {
-                const T ida = sh_id[grp][a];
-                const T hh = (T)0.5 * P.epslam * ga;
-                gth[4] += hh * P.gam * (ida * ida * eh + e2);
-                gth[5] += (T)0.5 * P.eps * ga * eh;
-                gth[6] += hh * (ida * eh + e1);
-            }
         }
         // the atom's force, energy and virial (summed over its lanes); pass B adds the energy
         // and virial to its block sums, so this pass has no block reduction
@@ -1888,7 +1910,6 @@ __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
             b.shn[i] = m;
         }
     }
-    if (grad) block_sum_to_acc<T, 7>(gth, b.acc + (size_t)ta.sys * ACC_N * kSlots, ACC_DTH, &st.err);
 }
 
 // Force pass A, one thread per atom (64-thread blocks, half a tile each), FP32: the same
@@ -2273,6 +2294,58 @@ __device__ __noinline__ void refuse_own(const Bufs& b, const DevSys& S, const SW
     __syncwarp();
 }
 
+// Step 1 of the edge-list kernels for atom i: the lane takes the row's octets part, part + 2^lpa, ...
+// and marks their entries closer than sqrt(rc2) (with the margin of the packed positions): entry
+// 8 (part + n 2^lpa) + k is bit 8 n + k of (lo, hi).
+__device__ __forceinline__ void mark_row(const Bufs& b, int i, int part, int lpa, const float4& L, float rc2, unsigned* err,
+                                         unsigned& lo, unsigned& hi) {
+    const bool il = b.nbr_il != 0, wide = il || b.row4;
+    const int4* rows4 = il ? reinterpret_cast<const int4*>(b.nbr) + i : reinterpret_cast<const int4*>(b.nbr + (size_t)i * b.cap);
+    const size_t rstep = il ? (size_t)b.ntot : 1;
+    const uint2* X = b.xc;
+    const uint2 pi = X[i];
+    const int xi = (int)pi.y, yi = (int)__funnelshift_l(pi.x, pi.y, 21), zi = (int)(pi.x << 10);
+    const int ci = min(b.cnt[i], b.cap);
+    // each axis of the packed difference is within 2 units of 2^-21 L of the true one
+    const float mg = 2.0f * 2048.0f * (L.x + L.y + L.z);
+    const float rc = sqrtf(rc2) + mg, act2 = rc * rc;
+    int shift = 0;
+    for (int base = 8 * part; base < ci; base += 8 << lpa, shift += 8) {
+        int e[8];
+#pragma unroll
+        for (int v = 0; v < 8; v += 4) {
+            if (wide) {
+                int4 r = make_int4(i, i, i, i);
+                if (base + v < ci) r = rows4[(size_t)((base + v) >> 2) * rstep];
+                e[v] = r.x; e[v + 1] = r.y; e[v + 2] = r.z; e[v + 3] = r.w;
+            } else {
+                const int* row = reinterpret_cast<const int*>(rows4);
+#pragma unroll
+                for (int u = v; u < v + 4; ++u) e[u] = base + u < ci ? row[base + u] : i;
+            }
+        }
+        unsigned oct = 0u;
+        uint2 pj[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            // past the row's length a row-major group holds the caller's bytes: not an index
+            int j = (il || base + u < ci) ? (e[u] & (int)kIndexMask) : i;
+            if (!NEFE_IN_RANGE(j, b.ntot, err)) j = i;
+            pj[u] = X[j];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float dx = (float)((int)pj[u].y - xi) * L.x,
+                        dy = (float)((int)__funnelshift_l(pj[u].x, pj[u].y, 21) - yi) * L.y,
+                        dz = (float)((int)(pj[u].x << 10) - zi) * L.z;
+            if (dx * dx + dy * dy + dz * dz < act2) oct |= 1u << u;
+        }
+        // entries past the length are the atom itself
+        if (ci - base < 8) oct &= (1u << (ci - base)) - 1u;
+        if (shift < 32) lo |= oct << shift; else hi |= oct << (shift - 32);
+    }
+}
+
 // COMMON: every system has the same potential constants, which are then kernel arguments (operands of
 // the constant bank, no loads: 171 -> 155 us on the crystal); otherwise they are read from the table.
 template <bool EATOM, bool GRAD, bool COMMON, int BLOCKS>
@@ -2297,58 +2370,9 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc,
     // L 2^-32 to twice the precision: a relative error of L alone would be a uniform strain of up to
     // 6e-8, which the pressure sees (the row filter does without the second part)
     const float4 Lh = b.lscale[2 * ta.sys], Ll = b.lscale[2 * ta.sys + 1];
-    const bool il = b.nbr_il != 0;
-    // 1. accepted row entries of this lane: entry 8 (part + n 32 / G) + k is bit 8 n + k of lo, hi
+    // 1. accepted row entries
     unsigned lo = 0u, hi = 0u;
-    if (valid) {
-        const int part = lane >> lg;
-        const bool wide = il || b.row4;
-        const int4* rows4 = il ? reinterpret_cast<const int4*>(b.nbr) + i
-                               : reinterpret_cast<const int4*>(b.nbr + (size_t)i * b.cap);
-        const size_t rstep = il ? (size_t)b.ntot : 1;
-        const uint2* X = b.xc;
-        const uint2 pi = X[i];
-        const int xi = (int)pi.y, yi = (int)__funnelshift_l(pi.x, pi.y, 21), zi = (int)(pi.x << 10);
-        const int ci = min(b.cnt[i], b.cap);
-        // each axis of the packed difference is within 2 units of 2^-21 L of the true one
-        const float mg = 2.0f * 2048.0f * (Lh.x + Lh.y + Lh.z);
-        const float rc = sqrtf(P.act2) + mg, act2 = rc * rc;
-        int shift = 0;
-        for (int base = 8 * part; base < ci; base += 8 << lpa, shift += 8) {
-            int e[8];
-#pragma unroll
-            for (int v = 0; v < 8; v += 4) {
-                if (wide) {
-                    int4 r = make_int4(i, i, i, i);
-                    if (base + v < ci) r = rows4[(size_t)((base + v) >> 2) * rstep];
-                    e[v] = r.x; e[v + 1] = r.y; e[v + 2] = r.z; e[v + 3] = r.w;
-                } else {
-                    const int* row = reinterpret_cast<const int*>(rows4);
-#pragma unroll
-                    for (int u = v; u < v + 4; ++u) e[u] = base + u < ci ? row[base + u] : i;
-                }
-            }
-            unsigned oct = 0u;
-            uint2 pj[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                // past the row's length a row-major group holds the caller's bytes: not an index
-                int j = (il || base + u < ci) ? (e[u] & (int)kIndexMask) : i;
-                if (!NEFE_IN_RANGE(j, b.ntot, &st.err)) j = i;
-                pj[u] = X[j];
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float dx = (float)((int)pj[u].y - xi) * Lh.x,
-                            dy = (float)((int)__funnelshift_l(pj[u].x, pj[u].y, 21) - yi) * Lh.y,
-                            dz = (float)((int)(pj[u].x << 10) - zi) * Lh.z;
-                if (dx * dx + dy * dy + dz * dz < act2) oct |= 1u << u;
-            }
-            // entries past the length are the atom itself
-            if (ci - base < 8) oct &= (1u << (ci - base)) - 1u;
-            if (shift < 32) lo |= oct << shift; else hi |= oct << (shift - 32);
-        }
-    }
+    if (valid) mark_row(b, i, lane >> lg, lpa, Lh, P.act2, &st.err, lo, hi);
     const int ml = __popc(lo) + __popc(hi);      // edges of this lane, then of its atom
     int m = ml;
     for (int o = 16; o >= G; o >>= 1) m += __shfl_xor_sync(kAll, m, o);
@@ -2520,6 +2544,197 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc,
     if constexpr (GRAD) block_sum_to_acc<float, 7>(gth, acc, ACC_DTH, &st.err);
 }
 
+// Force pass A in FP64: the same edge list, with the terms of nefe_sw_terms.h.  The row filter is FP32, so
+// FP64 (2 lanes a cycle and SM) sees only the edges; they are walked 32 at a time, and the triplets of
+// an atom cost O(m).  Leg forces (each with half of its pair force) are stored per shell slot for pass
+// B, the atom's own force is minus their sum; energy and virial go to the system's sums here.
+// What bounds it is FP64 issue: about 160 operations an edge.  The form before computed distances of
+// all row entries, divided and took the exponentials on partly idle lanes, and every triplet pair:
+// 16 x 8000 atoms 988 -> 384 us, with dE/dtheta 32,768 liquid atoms 736 -> 268 us.
+constexpr int kListEdgesD = 192;
+struct __align__(16) EdgesDShared {
+    double v[8][kListEdgesD];        // unit vector, 1/r, 1/(s - a), g, dphi, r; then the leg force
+    unsigned id[kListEdgesD];        // atom of the warp << 27 | leg atom
+    unsigned short slot[kListEdgesD];   // cell-offset code << 8 | shell slot
+    double mom[10][32];
+};
+template <bool GRAD, bool COMMON>
+__global__ void __launch_bounds__(64)
+k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc, int lg) {
+    constexpr unsigned kAll = 0xffffffffu;
+    __shared__ EdgesDShared shm[2];
+    EdgesDShared& sh = shm[threadIdx.x >> 5];
+    const int G = 1 << lg, lpa = 5 - lg;
+    const int item = (int)blockIdx.x, tile = (item >> (6 - lg)) + b.tile_base;
+    const TileAtom ta = tile_of(b, tile);
+    const DevSys& S = b.sys[ta.sys];
+    DevState& st = b.st[ta.sys];
+    if (S.pot != POT_SW) return;                 // uniform over the block
+    const SWp<double>& P = COMMON ? Pc : reinterpret_cast<const SWp<double>*>(b.swc)[S.prm];
+    const int lane = threadIdx.x & 31, t = lane & (G - 1);
+    const unsigned below = (1u << lane) - 1u;
+    const int ia = ((item & ((64 >> lg) - 1)) << (lg + 1)) + ((int)(threadIdx.x >> 5) << lg) + t;   // of the tile
+    const int i = ta.first + ia;
+    const bool valid = ia < ta.count;
+    const double hx = st.h[0], hy = st.h[1], hz = st.h[2];
+    const double4* X = reinterpret_cast<const double4*>(b.xs);
+    unsigned lo = 0u, hi = 0u;
+    if (valid) mark_row(b, i, lane >> lg, lpa, b.lscale[2 * ta.sys], (float)P.rc2, &st.err, lo, hi);
+    const int ml = __popc(lo) + __popc(hi);      // edges of this lane, then of its atom
+    int m = ml, before = 0;                      // before: of the atom's lanes before this one
+    for (int o = 16; o >= G; o >>= 1) m += __shfl_xor_sync(kAll, m, o);
+    {
+        int inc = ml;                            // inclusive scan over the atom's lanes (stride G)
+        for (int o = G; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kAll, inc, o);
+            if (lane >= o) inc += y;
+        }
+        before = inc - ml;
+    }
+    int incl = m;                                // edges of atoms 0 .. t
+    for (int o = 1; o < G; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, incl, o, G);
+        if (t >= o) incl += y;
+    }
+    const int total = __shfl_sync(kAll, incl, G - 1);
+    int mtrue = 0;
+    double red8[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // energy, -, virial
+    double gth[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    double fx = 0.0, fy = 0.0, fz = 0.0, en = 0.0;
+    for (int done = 0; done < total;) {
+        const bool act = incl - m >= done && incl - done <= kListEdgesD && m > 0;
+        const int ma = act ? ml : 0;
+        const int mx = __reduce_max_sync(kAll, ma);
+        int E = 0;
+        {
+            const int part = lane >> lg;
+            unsigned l = lo, h = hi;
+            for (int a = 0; a < mx; ++a) {       // slot by slot: consecutive lanes hold distinct atoms
+                const bool on = a < ma;
+                const unsigned bal = __ballot_sync(kAll, on);
+                if (on) {
+                    int k;
+                    if (l) { k = __ffs(l) - 1; l &= l - 1u; }
+                    else { k = 31 + __ffs(h); h &= h - 1u; }
+                    k = 8 * (((k >> 3) << lpa) + part) + (k & 7);
+                    const unsigned w = (unsigned)b.nbr[nbr_at(b, i, k)];
+                    int j = (int)(w & kIndexMask);
+                    if (!NEFE_IN_RANGE(j, b.ntot, &st.err)) j = i;
+                    const int e = E + __popc(bal & below), slot = before + a;
+                    sh.id[e] = (unsigned)t << kCodeShift | (unsigned)j;
+                    sh.slot[e] = (unsigned short)((w >> kCodeShift) << 8 | (unsigned)slot);
+                    if (slot < kShell) b.shj[(size_t)i * kShell + slot] = j;
+                }
+                E += __popc(bal);
+            }
+        }
+        __syncwarp();
+        for (int e = lane; e < E; e += 32) {     // edge terms
+            const unsigned w = sh.id[e];
+            const int code = sh.slot[e] >> 8, ai = i - t + (int)(w >> kCodeShift);
+            const double4 xj = X[w & kIndexMask], xi = X[ai];
+            const int ox = code % 3 - 1, oy = (code / 3) % 3 - 1, oz = code / 9 - 1;
+            const double d[3] = {(xj.x - xi.x) + (ox == 0 ? 0.0 : ox < 0 ? -hx : hx),
+                                 (xj.y - xi.y) + (oy == 0 ? 0.0 : oy < 0 ? -hy : hy),
+                                 (xj.z - xi.z) + (oz == 0 ? 0.0 : oz < 0 ? -hz : hz)};
+            const double none[3] = {0.0, 0.0, 0.0};
+            EdgeT<double> q;
+            sw_edge_terms<double, double, GRAD>(P, d, none, q);
+            if constexpr (GRAD)
+                for (int k = 0; k < 5; ++k) gth[k] += 0.5 * q.pg[k];
+            sh.v[0][e] = q.ux; sh.v[1][e] = q.uy; sh.v[2][e] = q.uz;
+            sh.v[3][e] = q.ir; sh.v[4][e] = q.id; sh.v[5][e] = q.g;
+            sh.v[6][e] = q.dphi; sh.v[7][e] = q.r;
+            red8[0] = fma(0.5, q.phi, red8[0]);
+            if (b.e_atom) reinterpret_cast<double4*>(b.shd)[(size_t)ai * kShell + min(sh.slot[e] & 255, kShell - 1)].w = 0.5 * q.phi;
+        }
+        __syncwarp();
+        MomT<double> M = {};
+        int base = 0;
+        for (int a = 0; a < mx; ++a) {           // moments
+            const bool on = a < ma;
+            const unsigned bal = __ballot_sync(kAll, on);
+            if (on) {
+                const int e = base + __popc(bal & below);
+                const double g = sh.v[5][e];
+                mtrue += g > 0.0 ? 1 : 0;
+                mom_add(M, sh.v[0][e], sh.v[1][e], sh.v[2][e], g);
+            }
+            base += __popc(bal);
+        }
+        double mv[10] = {M.G, M.x, M.y, M.z, M.xx, M.yy, M.zz, M.xy, M.xz, M.yz};
+        for (int o = 16; o >= G; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 10; ++k) mv[k] += __shfl_xor_sync(kAll, mv[k], o);
+        if (lane < G)
+#pragma unroll
+            for (int k = 0; k < 10; ++k) sh.mom[k][t] = mv[k];
+        __syncwarp();
+        for (int e = lane; e < E; e += 32) {     // leg forces
+            const int te = (int)(sh.id[e] >> kCodeShift), slot = sh.slot[e] & 255, ai = i - t + te;
+            MomT<double> Q;
+            Q.G = sh.mom[0][te];  Q.x = sh.mom[1][te];  Q.y = sh.mom[2][te];  Q.z = sh.mom[3][te];
+            Q.xx = sh.mom[4][te]; Q.yy = sh.mom[5][te]; Q.zz = sh.mom[6][te];
+            Q.xy = sh.mom[7][te]; Q.xz = sh.mom[8][te]; Q.yz = sh.mom[9][te];
+            const double ux = sh.v[0][e], uy = sh.v[1][e], uz = sh.v[2][e], ir = sh.v[3][e], id = sh.v[4][e], g = sh.v[5][e];
+            double lx, ly, lz, s3;
+            sw_leg(P, Q, ux, uy, uz, ir, id, g, sh.v[6][e], lx, ly, lz, s3);
+            const double gs = g * s3, h = P.eps * P.lam * gs;   // the triplets of edge a, each seen from both its edges
+            red8[0] = fma(0.5, h, red8[0]);
+            if constexpr (GRAD) {
+                const double hi_ = h * id;
+                gth[4] = fma(P.gam * hi_, id, gth[4]);
+                gth[5] = fma(0.5 * P.eps, gs, gth[5]);
+                gth[6] += hi_;
+            }
+            const double r = sh.v[7][e];
+            const double ax = r * lx, ay = r * ly, az = r * lz;
+            red8[2] = fma(ux, ax, red8[2]); red8[3] = fma(uy, ay, red8[3]); red8[4] = fma(uz, az, red8[4]);
+            red8[5] = fma(ux, ay, fma(uy, ax, red8[5]));
+            red8[6] = fma(ux, az, fma(uz, ax, red8[6]));
+            red8[7] = fma(uy, az, fma(uz, ay, red8[7]));
+            if (slot < kShell) {
+                double4* leg = reinterpret_cast<double4*>(b.shd) + (size_t)ai * kShell + slot;
+                if (b.e_atom) *leg = mk4(lx, ly, lz, leg->w + 0.5 * h);
+                else *leg = mk4(lx, ly, lz, 0.0);
+            }
+            sh.v[0][e] = lx; sh.v[1][e] = ly; sh.v[2][e] = lz;
+        }
+        __syncwarp();
+        base = 0;
+        for (int a = 0; a < mx; ++a) {           // the atoms' own forces
+            const bool on = a < ma;
+            const unsigned bal = __ballot_sync(kAll, on);
+            if (on) {
+                const int e = base + __popc(bal & below), slot = min(before + a, kShell - 1);
+                fx -= sh.v[0][e]; fy -= sh.v[1][e]; fz -= sh.v[2][e];
+                if (b.e_atom) en += reinterpret_cast<const double4*>(b.shd)[(size_t)i * kShell + slot].w;
+            }
+            base += __popc(bal);
+        }
+        done = __reduce_max_sync(kAll, act ? incl : 0);
+        __syncwarp();
+    }
+    red8[5] *= 0.5; red8[6] *= 0.5; red8[7] *= 0.5;
+    for (int o = 16; o >= G; o >>= 1) {
+        mtrue += __shfl_xor_sync(kAll, mtrue, o);
+        fx += __shfl_xor_sync(kAll, fx, o);
+        fy += __shfl_xor_sync(kAll, fy, o);
+        fz += __shfl_xor_sync(kAll, fz, o);
+        if (b.e_atom) en += __shfl_xor_sync(kAll, en, o);
+    }
+    if (lane < G && valid) {
+        if (m > kShell) atomicOr(&st.err, NEFE_ERR_SHELL_OVERFLOW);
+        const int ms = min(m, kShell);
+        b.shn[i] = ms;
+        if (ms < kShell) b.shj[(size_t)i * kShell + ms] = -1;
+        reinterpret_cast<double4*>(b.P)[i] = mk4(fx, fy, fz, en);
+    }
+    long long* acc = b.acc + (size_t)ta.sys * ACC_N * kSlots;
+    block_sum_to_acc<double, 8>(red8, acc, ACC_UINT, &st.err);
+    if constexpr (GRAD) block_sum_to_acc<double, 7>(gth, acc, ACC_DTH, &st.err);
+}
+
 // Force pass B, L lanes per atom:
 //   F_SW(i) = P(i) + sum_{j in shell(i)} L_j(i),
 // L_j(i) being the leg force that the triplets centred on neighbour j exert on i, stored by
@@ -2658,7 +2873,7 @@ __global__ void __launch_bounds__(kTile) k_gather(Bufs b) {
             const T4* Pa = reinterpret_cast<const T4*>(b.P);
             const T4 p = Pa[i];
             f[0] += p.x; f[1] += p.y; f[2] += p.z; e_i = p.w;
-            if (lane == 0) {
+            if (sizeof(T) == 4 && lane == 0) {   // (FP64: summed by pass A)
                 const T4 wa = Pa[b.ntot + 2 * (size_t)i], wb = Pa[b.ntot + 2 * (size_t)i + 1];
                 red[0] = e_i;
                 red[2] = wa.x; red[3] = wa.y; red[4] = wa.z; red[5] = wa.w; red[6] = wb.x; red[7] = wb.y;
@@ -3441,55 +3656,50 @@ void launch_mirror(const Bufs& b, int precision, int ntiles, cudaStream_t s, lon
     if (launches) *launches += 1;
 }
 
-// Atoms per warp of the scatter form's pass A (see k_edges_s), as a power of two: by the whole
-// context's size, so that a run does not depend on how the passes are launched.
-constexpr int kScatterFull = 8;          // warps per SM
-static int scatter_atoms(int ntot) {
-    for (int lg : {5, 4})
-        if (ntot >= (152 * kScatterFull << lg)) return lg;
-    return 3;
+// Atoms per warp of the edge-list kernels, as a power of two: by the whole context's size, so that a
+// run does not depend on how the passes are launched.  FP32 (see k_edges_s): 32 where that gives every
+// SM 8 warps, else 16 or 8.  FP64, where one warp a SM quarter fills the unit: 16 (32 atoms' edges do
+// not fit one list) where that gives 4 warps a SM, 8 down to 2 warps, else 4.
+int atoms_per_warp_log2(int precision, int ntot) {
+    if (precision == NEFE_FP64) return ntot >= 16 * 152 * 4 ? 4 : ntot >= 8 * 152 * 2 ? 3 : 2;
+    return ntot >= 32 * 152 * 8 ? 5 : ntot >= 16 * 152 * 8 ? 4 : 3;
 }
 
-template <typename T>
-static void edges_dispatch(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
-    // an FP64 shell of 32 atoms per block does not fit the 48 KB static shared limit: 4 -> 8
+static void edges_fp32(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
     switch (lanes) {
-        case 0:   // one thread per atom, scatter form: FP32 only
-        case 1: { // one thread per atom: FP32 only (the FP64 columns exceed the shared limit)
-            if constexpr (sizeof(T) == 8) {
-                k_edges<T, 8><<<ntiles * 8, kTile, 0, s>>>(b);
-            } else {
-                if (lanes == 0) {
-                    const int lg = scatter_atoms(b.ntot), items = ntiles << (6 - lg);
-                    const auto go = [&](auto kernel) { kernel<<<items, kScatterThreads, 0, s>>>(b, b.swc_common, lg); };
-                    const bool full = items >= 152 * kScatterBlocks;
-                    if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks>);          // (stateless: one system)
-                    else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks>);
-                    else if (!b.common) go(k_edges_s<false, false, false, kScatterBlocks>);
-                    else if (full) go(k_edges_s<false, false, true, kScatterBlocks>);
-                    else go(k_edges_s<false, false, true, kScatterBlocksFew>);
-                } else {
-                    k_edges1<T><<<ntiles * (kTile / kEdges1Threads), kEdges1Threads, 0, s>>>(b);
-                }
-            }
+        case 0: {
+            const int lg = b.lg, items = ntiles << (6 - lg);
+            const auto go = [&](auto kernel) { kernel<<<items, kScatterThreads, 0, s>>>(b, b.swc_common, lg); };
+            const bool full = items >= 152 * kScatterBlocks;
+            if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks>);          // (stateless: one system)
+            else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks>);
+            else if (!b.common) go(k_edges_s<false, false, false, kScatterBlocks>);
+            else if (full) go(k_edges_s<false, false, true, kScatterBlocks>);
+            else go(k_edges_s<false, false, true, kScatterBlocksFew>);
             break;
         }
-        case 4:
-            if constexpr (sizeof(T) == 8) k_edges<T, 8><<<ntiles * 8, kTile, 0, s>>>(b);
-            else k_edges<T, 4><<<ntiles * 4, kTile, 0, s>>>(b);
-            break;
-        case 8: k_edges<T, 8><<<ntiles * 8, kTile, 0, s>>>(b); break;
-        case 16: k_edges<T, 16><<<ntiles * 16, kTile, 0, s>>>(b); break;
-        default: k_edges<T, 32><<<ntiles * 32, kTile, 0, s>>>(b); break;
+        case 1: k_edges1<float><<<ntiles * (kTile / kEdges1Threads), kEdges1Threads, 0, s>>>(b); break;
+        case 4: k_edges<float, 4><<<ntiles * 4, kTile, 0, s>>>(b); break;
+        case 8: k_edges<float, 8><<<ntiles * 8, kTile, 0, s>>>(b); break;
+        case 16: k_edges<float, 16><<<ntiles * 16, kTile, 0, s>>>(b); break;
+        default: k_edges<float, 32><<<ntiles * 32, kTile, 0, s>>>(b); break;
     }
+}
+
+static void edges_fp64(const Bufs& b, int ntiles, cudaStream_t s) {
+    const int lg = b.lg, items = ntiles << (6 - lg);
+    const auto go = [&](auto kernel) { kernel<<<items, 64, 0, s>>>(b, b.swp_common, lg); };
+    if (b.want_grad) go(k_edges_d<true, true>);          // (stateless: one system)
+    else if (b.common) go(k_edges_d<false, true>);
+    else go(k_edges_d<false, false>);
 }
 
 void launch_edges(const Bufs& b, int precision, int lanes, int ntiles, int mode, cudaStream_t s,
                   long* launches) {
     (void)mode;
     if (ntiles <= 0) return;
-    if (precision == NEFE_FP64) edges_dispatch<double>(b, lanes, ntiles, s);
-    else edges_dispatch<float>(b, lanes, ntiles, s);
+    if (precision == NEFE_FP64) edges_fp64(b, ntiles, s);
+    else edges_fp32(b, lanes, ntiles, s);
     if (launches) *launches += 1;
 }
 

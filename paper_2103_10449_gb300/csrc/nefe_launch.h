@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include "nefe_dev.h"
+#include "nefe_sw_terms.h"
 
 namespace nefe {
 
@@ -51,7 +52,7 @@ struct Bufs {
     int* rcbase;             // [nsys + 1] first worklist cell of each system (cells of flagged
                              // systems, in system order; the last entry is their number) or NULL
     double dt;
-    const void* swc;         // SWc<float> or SWc<double> table
+    const void* swc;         // SWc<float> (FP32) or SWp<double> (FP64) table
     DevPair* pairs;
     double* trace;
     double* f_out;           // stateless: FP64 SoA forces
@@ -67,6 +68,8 @@ struct Bufs {
     int* lacc;               // [ntot][4] int32 force accumulators of the scatter form (2^-22 eV/A)
     int* lacc_hi;            // [ntot][4] multiples of large terms (see k_edges_s)
     SWc<float> swc_common;   // the potential constants, where every system has the same (common)
+    SWp<double> swp_common;
+    int lg;                  // atoms per warp of the edge-list kernels, as a power of two
     int common;
     int leg_refuse;          // the scatter form was chosen by the caller: terms above its limit are refused
     int* hi_flag;            // [tiles] some large term was split this step (cleared by k_finish)
@@ -74,7 +77,7 @@ struct Bufs {
     int4* xf;                // FP32: fractional positions (x/L as 32-bit fixed point)
     int4* xfb;               // their values at the last list build
     uint2* xc;               // their top 21 bits per axis (pass A's row filter)
-    int want_xf, want_xs;    // FP32 per-step positions: fractional (scatter form), mirror (the others)
+    int want_xf, want_xs;    // per-step positions: fractional (scatter form; FP64: xc only), FP32 mirror (the others)
     int row4;                // row-major rows can be read 16 bytes at a time
     int* any_rebuild;        // engine: [0] some system's rebuild flag is set this step, [1] some
                              // rebuild_next is set (fused epilogue); NULL in the stateless calls
@@ -108,6 +111,7 @@ void launch_uf_list(const Bufs& b, int precision, int ntiles, cudaStream_t s, lo
 // Uhlenbeck-Ford forces and energies over `ntiles` tiles (b.uf_tiles, or every tile when NULL);
 // mode FM_FORCES writes b.f_out / b.e_atom (stateless), otherwise b.uf_F for pass B.
 void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches);
+int atoms_per_warp_log2(int precision, int ntot);
 // Force pass A (edges: pair terms, triplets centred on each atom, leg forces per edge).
 void launch_edges(const Bufs& b, int precision, int lanes, int ntiles, int mode, cudaStream_t s,
                   long* launches);

@@ -79,6 +79,7 @@ struct EdgeT {
     T ux, uy, uz;       // unit vector
     T ir, id, g;        // 1/r, 1/(r/sigma - a), exp(gamma id)
     T phi, dphi;        // pair term, dphi/dr
+    double r;           // length (real part)
     T pg[5];            // d phi / d(A, B, p, q, a) (GRAD)
 };
 
@@ -89,6 +90,7 @@ __device__ __forceinline__ bool sw_edge_terms(const SWp<TP>& P, const double (&d
     const double r2 = __fma_rn(d[2], d[2], __fma_rn(d[1], d[1], __dmul_rn(d[0], d[0])));
     const double ir = rsqrt(r2);
     const double r = __dmul_rn(r2, ir);
+    e.r = r;
     const double den = __fma_rn(r, P.inv_sig, -val(P.a));
     const bool in = r2 < P.rc2 && !(den >= -1e-12);   // (coincident atoms give NaN and stay in)
     const double id = 1.0 / (in ? den : -1.0);

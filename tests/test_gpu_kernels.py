@@ -249,3 +249,72 @@ def test_scatter_form_atoms_per_warp(N, shape):
             assert r["error"] == 0
             assert r["U"] == pytest.approx(float(ev[0]), rel=1e-5)
         ctx.close()
+
+
+# ------------------------------------------------------------------ FP64 edge lists
+@pytest.mark.parametrize("cap,shift", [(48, 0), (48, 1), (47, 0)])
+@pytest.mark.parametrize("n", [31, 65, 130, 2433])
+def test_fp64_forces_at_ragged_sizes(N, n, cap, shift):
+    """Ragged warps and tiles of 4 and 8 atoms to a warp, rows that cannot be read 16 bytes at a time:
+    forces, energies per atom, virial and dE/dtheta's energy to the FP64 tolerance (1e-10)."""
+    x, box = I.liquid(max(n, 700), 0.05, seed=200 + n)
+    x = x[:n]
+    rcs = RC + 0.5
+    xd = soa(x)
+    nbr = torch.full((n * cap + shift,), -1, dtype=torch.int32, device="cuda")[shift:]
+    cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+    N.nefe_neighbor_build(xd, n, box, rcs, cap, nbr, cnt)
+    f, f2 = (torch.zeros(3 * n, dtype=torch.float64, device="cuda") for _ in range(2))
+    e = torch.zeros(n, dtype=torch.float64, device="cuda")
+    ev, eg = torch.zeros(7, dtype=torch.float64, device="cuda"), torch.zeros(8, dtype=torch.float64, device="cuda")
+    prm = N.nefe_sw_params_silicon()
+    N.nefe_sw_forces(xd, n, box, rcs, nbr, cnt, cap, prm, N.NEFE_FP64, f, e, ev)
+    N.nefe_sw_energy_grad(xd, n, box, rcs, nbr, cnt, cap, prm, N.NEFE_FP64, f2, eg)
+    torch.cuda.synchronize()
+    e_o, f_o, vir_o, ea_o = O.sw_energy(x, box)
+    scale = np.abs(f_o).max()
+    assert np.abs(f.cpu().numpy().reshape(3, n).T - f_o).max() <= 1e-10 * scale
+    assert np.array_equal(f.cpu().numpy(), f2.cpu().numpy())
+    assert np.abs(e.cpu().numpy() - ea_o).max() <= 1e-10 * np.abs(ea_o).max()
+    assert abs(float(ev[0]) - e_o) <= 1e-10 * abs(e_o) and abs(float(eg[0]) - e_o) <= 1e-10 * abs(e_o)
+    assert np.abs(ev.cpu().numpy()[1:] - vir_o).max() <= 1e-9 * np.abs(vir_o).max()
+
+
+@pytest.mark.parametrize("lanes", [8, 16, 32])
+def test_fp64_forces_with_more_edges_than_a_list(N, lanes):
+    """28 neighbours inside the cutoff, 16 atoms to a warp (448 edges of 192), through the engine:
+    its energy and one step's motion against the oracle."""
+    x, box = I.diamond(4, 4, 4, a=4.4)
+    x = I.rattle(x, 0.02, 9)
+    ctx = N.Context(precision=N.NEFE_FP64, skin=0.3, nbr_cap=64)
+    s = ctx.add_system(x, box, v=np.zeros_like(x))
+    ctx.set_tuning(lanes)
+    ctx.run(3)
+    got, v, _ = ctx.get_state(s)
+    r = ctx.results(s)
+    ctx.close()
+    orc = O.System(x=x.copy(), v=np.zeros_like(x), box=box.copy())
+    orc.run(3)
+    assert r["error"] == 0
+    assert r["U"] == pytest.approx(orc.results()["U"], rel=1e-10)
+    assert np.abs(got - orc.x).max() < 1e-10 and np.abs(v - orc.v).max() <= 1e-9 * np.abs(orc.v).max()
+
+
+def test_block_sums_of_large_values(N):
+    """Per-atom values beyond the integer sums' range (a pair at 0.05 A: some 1e7 eV) take the FP64
+    sums: energy and virial still match the oracle."""
+    x, box = I.diamond(3, 3, 3)
+    d = x[4] - x[0]
+    x[4] = x[0] + d * (0.05 / np.linalg.norm(d))
+    n = len(x)
+    xd = soa(x)
+    nbr = torch.zeros(n * 48, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+    N.nefe_neighbor_build(xd, n, box, RC + 0.5, 48, nbr, cnt)
+    f, ev = torch.zeros(3 * n, dtype=torch.float64, device="cuda"), torch.zeros(7, dtype=torch.float64, device="cuda")
+    N.nefe_sw_forces(xd, n, box, RC + 0.5, nbr, cnt, 48, N.nefe_sw_params_silicon(), N.NEFE_FP64, f, None, ev)
+    torch.cuda.synchronize()
+    e_o, f_o, vir_o, _ = O.sw_energy(x, box)
+    assert np.abs(vir_o).max() > 2 * 2 ** 22       # each end of the pair is above 2^22
+    assert abs(float(ev[0]) - e_o) <= 1e-10 * abs(e_o)
+    assert np.abs(ev.cpu().numpy()[1:] - vir_o).max() <= 1e-9 * np.abs(vir_o).max()
