@@ -414,14 +414,21 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
     int* uf_cnt = nullptr;
     S.want(&uf_nbr, sizeof(int) * (size_t)n * kUfCap);
     S.want(&uf_cnt, sizeof(int) * (size_t)n);
+    if (precision == NEFE_FP32) {
+        S.want(&S.xf, sizeof(int4) * (size_t)n);
+        S.want(&S.xc, sizeof(uint2) * (size_t)n);
+        S.want(&S.lscale, sizeof(float4) * 2);
+    }
     if ((rc = commit1(S, n, box, rcs, n3, precision, nullptr, uf, skin))) return rc;
     if (n > 0) {
         Bufs b = bufs_of(S, x, n);
         b.uf_nbr = uf_nbr; b.uf_cnt = uf_cnt; b.uf_tiles = nullptr;
+        b.xf = b.xfb = S.xf; b.xc = S.xc; b.lscale = S.lscale;
+        b.want_xf = precision == NEFE_FP32 ? 1 : 0;
         b.f_out = f; b.e_atom = e_atom;
         const int ntiles = (n + kTile - 1) / kTile;
         launch_cells(b, precision, ntiles, 1, 1, S.s, nullptr);
-        launch_uf_list(b, precision, ntiles, S.s, nullptr);
+        launch_uf_list(b, precision, ntiles, 1, S.s, nullptr);
         launch_uf(b, precision, ntiles, FM_FORCES, S.s, nullptr);
         NEFE_CU(cudaGetLastError());
     }

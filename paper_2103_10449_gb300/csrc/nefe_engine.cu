@@ -167,7 +167,8 @@ double rc_of(const HostSys& h) { return h.prm.a * h.prm.sigma; }
 void set_form(nefe_ctx* c, int lanes) {
     c->lanes = lanes;
     const bool scatter = c->prec == NEFE_FP32 && lanes == 0;
-    const int xf = scatter || c->prec == NEFE_FP64 ? 1 : 0, xs = !scatter || c->n_uf_tiles > 0 ? 1 : 0;
+    // (the Uhlenbeck-Ford kernel reads fractions in FP32)
+    const int xf = scatter || c->prec == NEFE_FP64 || c->n_uf_tiles > 0 ? 1 : 0, xs = !scatter ? 1 : 0;
     // FP64: 8, 16, 32 lanes per atom set by hand stand for 16, 8, 4 atoms per warp
     c->b.lg = c->prec == NEFE_FP64 && c->chosen ? (lanes <= 8 ? 4 : lanes == 16 ? 3 : 2) : atoms_per_warp_log2(c->prec, c->ntot);
     if (c->b.want_xf != xf || c->b.want_xs != xs) c->stale_pos = true;
@@ -214,7 +215,7 @@ void enqueue_step(nefe_ctx* c, int slot = -1, bool first = true, bool last = tru
         launch_rebuild_coop(c->b, c->prec, c->coop_blocks, c->nsys, c->stream, &c->launches);
     } else {
         launch_cells_and_list(c->b, c->prec, c->ntiles, c->nsys, 0, c->stream, &c->launches);
-        if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->stream, &c->launches);
+        if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->nsys, c->stream, &c->launches);
     }
     enqueue_forces(c, FM_STEP, slot, fused && !last);
 }
@@ -256,7 +257,7 @@ int resetup(nefe_ctx* c) {
         NEFE_CU(cudaMemsetAsync(c->d_hi_flag, 0, sizeof(int) * (size_t)c->ntiles, c->stream));
     }
     launch_cells_and_list(c->b, c->prec, c->ntiles, c->nsys, 1, c->stream, &c->launches);
-    if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->stream, &c->launches);
+    if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->nsys, c->stream, &c->launches);
     launch_kick_drift(c->b, c->prec, c->ntiles, 0, c->stream, &c->launches);
     enqueue_forces(c, FM_SETUP);
     c->stale_pos = false;

@@ -401,6 +401,7 @@ __device__ void cells_count_tile(const Bufs& b, int tile) {
     if (b.xa) reinterpret_cast<T4*>(b.xa)[i] = m;
     if (b.sd0) reinterpret_cast<T4*>(b.sd0)[i] = mk4((T)sd[0], (T)sd[1], (T)sd[2], (T)0);
     if (b.xfb && b.want_xf) {
+        if (i == S.off) scale_of_box(b, ta.sys, st.box);
         const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
         const int4 f = frac_position(x3, st);
         if (b.xf) b.xf[i] = f;
@@ -1176,10 +1177,8 @@ __device__ __forceinline__ void nlist_cell(const Bufs& b, int s, int c, CellList
 // Each warp takes a contiguous range of the worklist cells: with a worklist, the cells of the
 // flagged systems in system order (rcbase[s] = first worklist cell of system s, rcbase[nsys] =
 // their number); without one (stateless calls, one system), every cell of system 0.
-template <typename T>
-__device__ void nlist_cells_of_grid(const Bufs& b, int nsys, CellListShared<T>* shm) {
-    const int lane = threadIdx.x & 31;
-    CellListShared<T>& sh = shm[threadIdx.x >> 5];
+template <typename F>
+__device__ __forceinline__ void for_cells_of_grid(const Bufs& b, int nsys, F&& body) {
     const int nw = gridDim.x * (kTile / 32);
     const int wid = blockIdx.x * (kTile / 32) + (int)(threadIdx.x >> 5);
     int C;
@@ -1205,8 +1204,15 @@ __device__ void nlist_cells_of_grid(const Bufs& b, int nsys, CellListShared<T>* 
         if (b.rcbase) {
             while (s + 1 < nsys && b.rcbase[s + 1] <= g) ++s;
         }
-        nlist_cell<T>(b, s, g - (b.rcbase ? b.rcbase[s] : 0), sh, lane);
+        body(s, g - (b.rcbase ? b.rcbase[s] : 0));
     }
+}
+
+template <typename T>
+__device__ void nlist_cells_of_grid(const Bufs& b, int nsys, CellListShared<T>* shm) {
+    const int lane = threadIdx.x & 31;
+    CellListShared<T>& sh = shm[threadIdx.x >> 5];
+    for_cells_of_grid(b, nsys, [&](int s, int c) { nlist_cell<T>(b, s, c, sh, lane); });
 }
 
 template <typename T>
@@ -1300,73 +1306,145 @@ __global__ void __launch_bounds__(kTile) k_barrier_selftest(unsigned* word, int*
 // ------------------------------------------------------------------------------------
 // Uhlenbeck-Ford fluid (the liquid's reference system, Sec. 2.1):
 //   u(r) = -p kT ln(1 - exp(-r^2/sigma^2)) - u(rc),  r < rc.
-// R6 (rebuild): UF pair rows.  One thread per atom walks the 125 cells o in {-2..2}^3 around its
-// own (cells are at least rcs wide and rc + skin <= 2 rcs, so they cover the list radius; with
-// at least 5 cells per axis no cell is visited twice) and appends every j within the list
-// radius (rc + skin, FP32 mirror distance with a relative margin of 1e-5: the list only has
-// to contain every pair that can come within rc before the next rebuild).  Rows are in cell
-// order, not sorted: the force kernel sums in fixed point, so the order does not matter.
+// R6 (rebuild): UF pair rows, one warp per cell as in R5: the atoms of a cell share the 125 cells
+// o in {-2..2}^3 around it (cells are at least rcs wide and rc + skin <= 2 rcs, so they cover the list
+// radius; with at least 5 cells per axis no cell is visited twice).  Lane r < 25 looks up x-run r, one
+// piece or two where it wraps at the box edge; the warp then walks the runs' candidates as one
+// sequence, 32 at a time, and every candidate is tested against each atom of the cell (up to kUfHome
+// at a time): j is appended when it lies within the list radius (rc + skin, mirror distance with a
+// relative margin of 1e-5: the list only has to contain every pair that can come within rc before the
+// next rebuild).  Rows are in cell order, not sorted: the force kernel sums in fixed point, so the
+// order does not matter.  Bound by load latency: one thread per atom took its 490 candidates one after
+// the other, 4 x 8000 atoms 57 us averaged over the steps -> 10.5 us.
 // ------------------------------------------------------------------------------------
+constexpr int kUfHome = 16;              // cell atoms per walk
+constexpr int kUfPieces = 50;            // two per run (the second empty unless the run wraps)
 template <typename T>
-__device__ void uflist_tile(const Bufs& b, int tile) {
+struct UfListShared {
     using T4 = typename V4<T>::t;
-    const TileAtom ta = tile_of(b, tile);
-    const DevSys& S = b.sys[ta.sys];
-    if (S.uf_mode == UF_NONE) return;            // uniform over the block
-    DevState& st = b.st[ta.sys];
-    if ((int)threadIdx.x >= ta.count) return;
-    const int i = ta.first + threadIdx.x;
+    T4 home[kUfHome];
+    int4 edge[kUfPieces];                // first candidate of the piece's 2nd .. 5th cell
+    int4 info[kUfPieces];                // first candidate, first flat index, code and x offset of the first cell
+    int pw[kUfPieces];                   // first flat index again
+};
+
+template <typename T>
+__device__ __forceinline__ void uflist_cell(const Bufs& b, int s, int c, UfListShared<T>& sh, int lane) {
+    using T4 = typename V4<T>::t;
+    constexpr unsigned kAll = 0xffffffffu;
+    const DevSys& S = b.sys[s];
+    if (S.uf_mode == UF_NONE) return;
+    DevState& st = b.st[s];
+    const int* start = b.cell_start + S.cell0 + s;
+    const int n = S.n, off = S.off;
+    const int hs = max(0, min(start[c], n)), m = max(hs, min(start[c + 1], n)) - hs;
+    if (m == 0) return;
+    const T4* xc = reinterpret_cast<const T4*>(b.xcs) + off;
     const int nx = st.ncell[0], ny = st.ncell[1], nz = st.ncell[2];
     if (nx < 5 || ny < 5 || nz < 5) {
-        b.uf_cnt[i] = 0;
+        for (int q = lane; q < m; q += 32) {
+            const int i = unpack_index(xc[hs + q].w);
+            if ((unsigned)(i - off) < (unsigned)n) b.uf_cnt[i] = 0;
+        }
         atomicOr(&st.err, NEFE_ERR_BOX);
         return;
     }
-    const int cell = b.cell_of[i];
-    const int cx = cell % nx, cy = (cell / nx) % ny, cz = cell / (nx * ny);
-    const int* start = b.cell_start + S.cell0 + ta.sys;
-    const T4 xi = reinterpret_cast<const T4*>(b.xs)[i];
     const T hx = pick<T>(st.h[0], st.h_f[0]), hy = pick<T>(st.h[1], st.h_f[1]), hz = pick<T>(st.h[2], st.h_f[2]);
     const T R2 = pick<T>(S.uf_R2 * (1.0 + 1e-5), S.uf_R2_f * (1.0f + 1e-5f));
-    const T4* xc = reinterpret_cast<const T4*>(b.xcs) + S.off;
-    int* row = b.uf_nbr + (size_t)i * kUfCap;
-    int count = 0;
-    for (int oz = -2; oz <= 2; ++oz) {
-        int zz = cz + oz;
+    const int cx = c % nx, cy = (c / nx) % ny, cz = c / (nx * ny);
+    // run r = (oy, oz): cells cx - 2 .. cx + 2 as piece A = ox < brk and piece B = the rest, past the edge
+    const int brk = cx < 2 ? -cx : (cx + 2 >= nx ? nx - cx : 3);
+    const int na = brk + 2, nb = 3 - brk;
+    const int xa = cx < 2 ? cx - 2 + nx : cx - 2;
+    int pa[6], pb[6];                            // starts of the cells of each piece, then its end
+    int len = 0;
+    if (lane < 25) {
+        int yy = cy + lane % 5 - 2, zz = cz + lane / 5 - 2;
+        yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
         zz = zz < 0 ? zz + nz : (zz >= nz ? zz - nz : zz);
-        for (int oy = -2; oy <= 2; ++oy) {
-            int yy = cy + oy;
-            yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
-            for (int ox = -2; ox <= 2; ++ox) {
-                int xx = cx + ox;
-                xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-                const int c2 = xx + nx * (yy + ny * zz);
-                const int lo = max(0, min(start[c2], S.n)), hi = max(lo, min(start[c2 + 1], S.n));
-                const T offx = (T)ox * hx, offy = (T)oy * hy, offz = (T)oz * hz;
-                const unsigned code = (unsigned)((ox + 2) + 5 * (oy + 2) + 25 * (oz + 2));
-                for (int q = lo; q < hi; ++q) {
-                    const T4 xj = xc[q];
-                    const int j = unpack_index(xj.w);
-                    if (j < S.off || j >= S.off + S.n) {
-                        atomicOr(&st.err, NEFE_ERR_CELL);
-                        continue;
-                    }
-                    if (j == i) continue;
-                    const T dx = xj.x - xi.x + offx, dy = xj.y - xi.y + offy, dz = xj.z - xi.z + offz;
-                    if (dx * dx + dy * dy + dz * dz < R2) {
-                        if (count < kUfCap) row[count] = (int)((unsigned)j | (code << kUfShift));
-                        ++count;
-                    }
+        const int* row = start + nx * (yy + ny * zz);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            pa[k] = max(0, min(row[xa + min(k, na)], n));
+            pb[k] = max(0, min(row[min(k, nb)], n));
+        }
+        len = max(0, pa[5] - pa[0]) + max(0, pb[5] - pb[0]);
+    }
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(kAll, incl, 31);
+    if (lane < 25) {
+        const int f0 = incl - len, f1 = f0 + max(0, pa[5] - pa[0]);
+        const int code = 5 * (lane % 5) + 25 * (lane / 5);
+        sh.pw[2 * lane] = f0;
+        sh.pw[2 * lane + 1] = f1;
+        sh.edge[2 * lane] = make_int4(pa[1], pa[2], pa[3], pa[4]);
+        sh.edge[2 * lane + 1] = make_int4(pb[1], pb[2], pb[3], pb[4]);
+        sh.info[2 * lane] = make_int4(pa[0], f0, code, -2);
+        sh.info[2 * lane + 1] = make_int4(pb[0], f1, code, brk);
+    }
+    for (int h0 = 0; h0 < m; h0 += kUfHome) {
+        const int mh = min(kUfHome, m - h0);
+        __syncwarp();
+        if (lane < mh) sh.home[lane] = xc[hs + h0 + lane];
+        __syncwarp();
+        int cnt = 0;                             // lane a: entries of cell atom a
+        for (int t0 = 0; t0 < total; t0 += 32) {
+            const int t = t0 + lane;
+            int j = -1, o = 0;
+            // a candidate that is not one (past the sequence, or a bad index) sits far away
+            T cxj = (T)1e15, cyj = (T)1e15, czj = (T)1e15;
+            if (t < total) {
+                int e = 0;                       // piece of t: last one whose flat start is <= t
+#pragma unroll
+                for (int step = 32; step > 0; step >>= 1) {
+                    const int q = e + step;
+                    if (q < kUfPieces && sh.pw[q] <= t) e = q;
+                }
+                const int4 in = sh.info[e], ed = sh.edge[e];
+                const int p = in.x + (t - in.y);
+                const T4 xj = xc[p];
+                j = unpack_index(xj.w);
+                const int ox = in.w + (p >= ed.x) + (p >= ed.y) + (p >= ed.z) + (p >= ed.w);
+                o = in.z + ox + 2;
+                if ((unsigned)(j - off) < (unsigned)n) {
+                    cxj = xj.x + (T)ox * hx;
+                    cyj = xj.y + (T)((e >> 1) % 5 - 2) * hy;
+                    czj = xj.z + (T)((e >> 1) / 5 - 2) * hz;
+                } else {
+                    atomicOr(&st.err, NEFE_ERR_CELL);
                 }
             }
+            const unsigned ent = (unsigned)j | (unsigned)o << kUfShift;
+            for (int a = 0; a < mh; ++a) {
+                const T4 ha = sh.home[a];
+                const int ia = unpack_index(ha.w);
+                const T dx = cxj - ha.x, dy = cyj - ha.y, dz = czj - ha.z;
+                const bool in = dx * dx + dy * dy + dz * dz < R2 && j != ia;
+                const unsigned bal = __ballot_sync(kAll, in);
+                const int pos = __shfl_sync(kAll, cnt, a) + __popc(bal & ((1u << lane) - 1u));
+                if (in && pos < kUfCap && (unsigned)(ia - off) < (unsigned)n) b.uf_nbr[(size_t)ia * kUfCap + pos] = (int)ent;
+                if (lane == a) cnt += __popc(bal);
+            }
+        }
+        if (lane < mh) {
+            const int ia = unpack_index(sh.home[lane].w);
+            if ((unsigned)(ia - off) < (unsigned)n) b.uf_cnt[ia] = cnt;
+            if (cnt > kUfCap) atomicOr(&st.err, NEFE_ERR_NBR_OVERFLOW);
         }
     }
-    b.uf_cnt[i] = count;
-    if (count > kUfCap) atomicOr(&st.err, NEFE_ERR_NBR_OVERFLOW);
+    __syncwarp();                                // the tables are reused
 }
 template <typename T>
-__global__ void __launch_bounds__(kTile) k_uflist(Bufs b) {
-    NEFE_FOR_TILES(b, uflist_tile<T>(b, tile));
+__global__ void __launch_bounds__(kTile) k_uflist(Bufs b, int nsys) {
+    __shared__ UfListShared<T> shm[kTile / 32];
+    UfListShared<T>& sh = shm[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    for_cells_of_grid(b, nsys, [&](int s, int c) { uflist_cell<T>(b, s, c, sh, lane); });
 }
 
 // Fixed-point accumulation of the UF pair sums (order independent, so the unsorted rows give
@@ -1375,74 +1453,202 @@ template <typename T> struct UfFix;
 template <> struct UfFix<float> {
     __device__ static long long to(float v) { return __float2ll_rn(v * 4294967296.0f); }
     __device__ static float from(long long q) { return (float)((double)q * 0x1p-32); }
+    __device__ static long long sum_unit(long long q) { return q; }                // to the sums' 2^-32
 };
 template <> struct UfFix<double> {
     __device__ static long long to(double v) { return __double2ll_rn(v * 0x1p40); }
     __device__ static double from(long long q) { return (double)q * 0x1p-40; }
+    __device__ static long long sum_unit(long long q) { return (q + 128) >> 8; }
 };
-__device__ __forceinline__ float xexpm1(float v) { return expm1f(v); }
-__device__ __forceinline__ double xexpm1(double v) { return ::expm1(v); }
-__device__ __forceinline__ float xlogf_acc(float v) { return logf(v); }
-__device__ __forceinline__ double xlogf_acc(double v) { return ::log(v); }
 
-// Per step (or stateless): UF force and energy of each atom of a UF system from its row.
+// A lane's sums.  FP32: a conversion to int64 runs on the FP64 pipe (it was 68 % busy with them), so
+// round(v 2^32) is taken by two FP32 additions instead, for |v| < 64: v + 192 rounds v to 2^-16, the
+// exact remainder plus 1.5 2^-9 rounds to 2^-32, and the bits of both less those of their constants are the
+// integers, added as such.  The same integer as the conversion's, which larger values still take.
+template <typename T, int K>
+struct UfSum {
+    long long q[K];
+    __device__ __forceinline__ void clear(long long*) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) q[k] = 0;
+    }
+    template <int M>
+    __device__ __forceinline__ void add(const T (&v)[M], bool) {
+#pragma unroll
+        for (int k = 0; k < M; ++k) q[k] += UfFix<T>::to(v[k]);
+    }
+    __device__ __forceinline__ long long get(int k) const { return q[k]; }
+};
+template <int K>
+struct UfSum<float, K> {
+    int hi[K], lo[K];
+    long long* q;                        // the larger values' sums: memory of the thread, hardly ever used
+    bool any;
+    __device__ __forceinline__ void clear(long long* local) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) hi[k] = lo[k] = 0;
+        q = local;
+        any = false;
+    }
+    template <int M>
+    __device__ __forceinline__ void add(const float (&v)[M], bool small) {
+        if (__builtin_expect(small, 1)) {
+            const float C = 192.0f, C2 = 0x1.8p-9f;
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                const float t = __fadd_rn(v[k], C);
+                hi[k] += __float_as_int(t) - __float_as_int(C);
+                lo[k] += __float_as_int(__fadd_rn(__fsub_rn(v[k], __fsub_rn(t, C)), C2)) - __float_as_int(C2);
+            }
+        } else {
+            if (!any)
+                for (int k = 0; k < K; ++k) q[k] = 0;
+            any = true;
+#pragma unroll 1
+            for (int k = 0; k < M; ++k) q[k] += UfFix<float>::to(v[k]);
+        }
+    }
+    __device__ __forceinline__ long long get(int k) const {
+        return (any ? q[k] : 0LL) + (long long)hi[k] * 65536 + lo[k];
+    }
+};
+
+// Energy u (without the shift) and force coefficient c (force on j along d: c d; on i: -c d) of a pair
+// at xx = r^2/sigma^2: u = -pk ln(1 - e), c = (2 pk / sigma^2) e / (1 - e), e = exp(-xx).  FP32: from
+// xx = 0.7 on, where 1 - e is at least one half, it is taken as it stands, and -ln(1 - e) = e + e^2 q(e)
+// with q fitted (Chebyshev nodes, 8th degree) on [0, 1/2]: within 1.2e-7 of u, where ln of the rounded
+// 1 - e loses the small e.
+__device__ __forceinline__ void uf_pair(float xx, float pk, float c0, float& u, float& c) {
+    const float e = expf(-xx);
+    if (xx >= 0.7f) {
+        constexpr float a[9] = {0x1.0p-1f, 0x1.555394p-2f, 0x1.0059eep-2f, 0x1.8bdac4p-3f, 0x1.da2ab2p-3f,
+                                -0x1.9d06dcp-3f, 0x1.2944ccp+0f, -0x1.942780p+0f, 0x1.54cfd0p+0f};
+        float q = a[8];
+#pragma unroll
+        for (int k = 7; k >= 0; --k) q = fmaf(q, e, a[k]);
+        u = pk * fmaf(e * e, q, e);
+        c = c0 * __fdividef(e, 1.0f - e);
+    } else {
+        const float m = -expm1f(-xx);
+        u = -pk * logf(m);
+        c = c0 * (e / m);
+    }
+}
+__device__ __forceinline__ void uf_pair(double xx, double pk, double c0, double& u, double& c) {
+    u = -pk * ::log(-::expm1(-xx));
+    c = c0 / ::expm1(xx);
+}
+
+// Per step (or stateless): UF force and energy of each atom of a UF system from its row, kUfLanes
+// lanes to an atom (the row read 32 bytes at a time; the fixed-point sums of the lanes add exactly).
 // Each pair is seen from both ends: half its energy and virial per end, the full force.
 // The energy goes to U_int (pot = UF) or to the FL reference energy U_E (UF reference); the
-// virial enters the pressure only when the UF term is U_int.
+// virial enters the pressure only when the UF term is U_int.  FP32 distances come from fractional
+// positions, FP64 ones from the mirror and the entry's cell offset.
+// One thread per atom left most of the chip idle (142 entries one after the other, each lane in a row
+// of its own): 4 x 8000 atoms 155 -> 34 us.
+// (FP64 keeps a tile to a block: its block sums are rounded to 2^-32 once per 128 atoms.)
+template <typename T> constexpr int kUfLanes = sizeof(T) == 8 ? 4 : 8;
+template <typename T> constexpr int kUfThreads = sizeof(T) == 8 ? 4 * kTile : kTile;
+template <typename T> constexpr int kUfBlocks = kTile * kUfLanes<T> / kUfThreads<T>;   // per tile
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kTile) k_uf(Bufs b) {
+__global__ void __launch_bounds__(kUfThreads<T>, sizeof(T) == 4 ? 5 : 1) k_uf(Bufs b) {
     using T4 = typename V4<T>::t;
-    __shared__ T4 soff[125];
-    const int tile = b.uf_tiles ? b.uf_tiles[blockIdx.x] : (int)blockIdx.x;
-    const TileAtom ta = tile_of(b, tile);
+    constexpr bool kFrac = sizeof(T) == 4;
+    constexpr int L = kUfLanes<T>, PARTS = kUfBlocks<T>, G = kTile / PARTS;   // atoms per block
+    __shared__ T4 soff[kFrac ? 1 : 125];
+    const int item = (int)blockIdx.x / PARTS, part = (int)blockIdx.x % PARTS;
+    const TileAtom ta = tile_of(b, b.uf_tiles ? b.uf_tiles[item] : item);
     const DevSys& S = b.sys[ta.sys];
     DevState& st = b.st[ta.sys];
     if (S.uf_mode == UF_NONE) return;            // uniform over the block
-    if (threadIdx.x < 125) {
-        const int c = threadIdx.x;
-        const int ox = c % 5 - 2, oy = (c / 5) % 5 - 2, oz = c / 25 - 2;
-        soff[c] = mk4((T)ox * pick<T>(st.h[0], st.h_f[0]), (T)oy * pick<T>(st.h[1], st.h_f[1]),
-                      (T)oz * pick<T>(st.h[2], st.h_f[2]), (T)0);
+    const bool pressure = S.uf_mode == UF_INT;
+    if constexpr (!kFrac) {
+        if (threadIdx.x < 125) {
+            const int c = threadIdx.x;
+            soff[c] = mk4((T)(c % 5 - 2) * (T)st.h[0], (T)((c / 5) % 5 - 2) * (T)st.h[1], (T)(c / 25 - 2) * (T)st.h[2], (T)0);
+        }
+        __syncthreads();
     }
-    __syncthreads();
     const T pk = pick<T>(S.uf_pk, S.uf_pk_f), is2 = pick<T>(S.uf_is2, S.uf_is2_f);
     const T rc2 = pick<T>(S.uf_rc2, S.uf_rc2_f), shift = pick<T>(S.uf_shift, S.uf_shift_f);
-    long long q[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // f xyz, energy, virial xx yy zz xy xz yz
-    const bool valid = (int)threadIdx.x < ta.count;
-    const int i = ta.first + threadIdx.x;
+    const T c0 = (T)2 * pk * is2;
+    const T cmax = (T)64 / fmax(sqrt(rc2), (T)0.5 * rc2);   // below it no term reaches 64
+    UfSum<T, 10> sum;                            // f xyz, energy, virial xx yy zz xy xz yz
+    long long large[kFrac ? 10 : 1];
+    sum.clear(large);
+    const int lane = threadIdx.x % L, ia = part * G + (int)threadIdx.x / L;
+    const bool valid = ia < ta.count;
+    const int i = ta.first + ia;
     if (valid) {
-        const T4* X = reinterpret_cast<const T4*>(b.xs);
-        const T4 xi = X[i];
         const int cnt = min(b.uf_cnt[i], kUfCap);
         const int* row = b.uf_nbr + (size_t)i * kUfCap;
-        for (int a = 0; a < cnt; ++a) {
-            const unsigned e = (unsigned)row[a];
+        int4 fi = make_int4(0, 0, 0, 0);
+        T4 xi = mk4((T)0, (T)0, (T)0, (T)0);
+        float4 Lh = make_float4(0.f, 0.f, 0.f, 0.f), Ll = Lh;
+        if constexpr (kFrac) {
+            fi = b.xf[i];
+            Lh = b.lscale[2 * ta.sys];
+            Ll = b.lscale[2 * ta.sys + 1];
+        } else {
+            xi = reinterpret_cast<const T4*>(b.xs)[i];
+        }
+        // the entry two turns ahead and the position one turn ahead are loaded before a turn's arithmetic
+        const int last = cnt - 1;
+        auto entry = [&](int a) { return (unsigned)row[min(a, last)]; };
+        using P4 = std::conditional_t<kFrac, int4, T4>;
+        auto position = [&](unsigned e) {
+            const int j = (e & kUfMask) < (unsigned)b.ntot ? (int)(e & kUfMask) : i;
+            if constexpr (kFrac) return b.xf[j];
+            else return reinterpret_cast<const T4*>(b.xs)[j];
+        };
+        unsigned e1 = 0u, e2 = 0u;
+        P4 p1{};
+        if (lane < cnt) {
+            e1 = entry(lane);
+            e2 = entry(lane + L);
+            p1 = position(e1);
+        }
+        for (int a = lane; a < cnt; a += L) {
+            const unsigned e = e1;
+            const P4 xj = p1;
+            e1 = e2;
+            e2 = entry(a + 2 * L);
+            p1 = position(e1);
             if (!NEFE_IN_RANGE(e & kUfMask, b.ntot, &st.err)) continue;
-            const T4 xj = X[e & kUfMask];
-            const T4 oh = soff[e >> kUfShift];
-            const T dx = (xj.x - xi.x) + oh.x, dy = (xj.y - xi.y) + oh.y, dz = (xj.z - xi.z) + oh.z;
+            T dx, dy, dz;
+            if constexpr (kFrac) {
+                const float gx = (float)(xj.x - fi.x), gy = (float)(xj.y - fi.y), gz = (float)(xj.z - fi.z);
+                dx = gx * Lh.x + gx * Ll.x; dy = gy * Lh.y + gy * Ll.y; dz = gz * Lh.z + gz * Ll.z;
+            } else {
+                const T4 oh = soff[e >> kUfShift];
+                dx = (xj.x - xi.x) + oh.x; dy = (xj.y - xi.y) + oh.y; dz = (xj.z - xi.z) + oh.z;
+            }
             const T r2 = dx * dx + dy * dy + dz * dz;
             if (!(r2 < rc2)) continue;
-            const T xx = r2 * is2;
-            const T u = -pk * xlogf_acc(-xexpm1(-xx)) - shift;
-            const T c = (T)2 * pk * is2 / xexpm1(xx);      // force on j along d: c d; on i: -c d
-            const T hc = (T)0.5 * c;
-            q[0] += UfFix<T>::to(-c * dx);
-            q[1] += UfFix<T>::to(-c * dy);
-            q[2] += UfFix<T>::to(-c * dz);
-            q[3] += UfFix<T>::to((T)0.5 * u);
-            q[4] += UfFix<T>::to(hc * dx * dx);
-            q[5] += UfFix<T>::to(hc * dy * dy);
-            q[6] += UfFix<T>::to(hc * dz * dz);
-            q[7] += UfFix<T>::to(hc * dx * dy);
-            q[8] += UfFix<T>::to(hc * dx * dz);
-            q[9] += UfFix<T>::to(hc * dy * dz);
+            T u, c;
+            uf_pair(r2 * is2, pk, c0, u, c);
+            const bool small = c < cmax && u < (T)64;
+            const T hc = (T)0.5 * c, eh = (T)0.5 * (u - shift);
+            if (pressure) sum.add({-c * dx, -c * dy, -c * dz, eh, hc * dx * dx, hc * dy * dy, hc * dz * dz, hc * dx * dy, hc * dx * dz, hc * dy * dz}, small);
+            else sum.add({-c * dx, -c * dy, -c * dz, eh}, small);
         }
     }
-    T v[10];
+    long long q[10];
 #pragma unroll
-    for (int k = 0; k < 10; ++k) v[k] = UfFix<T>::from(q[k]);
-    if (valid) {
+    for (int k = 0; k < 10; ++k) q[k] = sum.get(k);
+    // the atom's sums, then (lanes of different atoms) the warp's.  An atom whose energy or virial left
+    // the range (a pair at zero distance saturates) is reported, and kept out of the block's sums.
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+        if (k > 3 && !pressure) break;           // (uniform)
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) q[k] += __shfl_xor_sync(0xffffffffu, q[k], o);
+    }
+    if (valid && lane == 0) {
+        T v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = UfFix<T>::from(q[k]);
         if (MODE == FM_FORCES) {
             const size_t N = b.ntot;
             b.f_out[i] = (double)v[0]; b.f_out[N + i] = (double)v[1]; b.f_out[2 * N + i] = (double)v[2];
@@ -1451,13 +1657,35 @@ __global__ void __launch_bounds__(kTile) k_uf(Bufs b) {
             reinterpret_cast<T4*>(b.uf_F)[i] = mk4(v[0], v[1], v[2], v[3]);
         }
     }
-    long long* acc = b.acc + (size_t)ta.sys * ACC_N * kSlots;
-    if (S.uf_mode == UF_INT) {
-        T red[8] = {v[3], (T)0, v[4], v[5], v[6], v[7], v[8], v[9]};   // U_int, (U_E), virial
-        block_sum_to_acc<T, 8>(red, acc, ACC_UINT, &st.err);
-    } else {
-        T red[1] = {v[3]};
-        block_sum_to_acc<T, 1>(red, acc, ACC_UREF, &st.err);
+    bool out = false;
+#pragma unroll
+    for (int k = 3; k < 10; ++k) {
+        const long long x = UfFix<T>::sum_unit(q[k]);
+        out = out || x >= (1LL << 47) || x <= -(1LL << 47);
+    }
+    if (out) atomicOr(&st.err, NEFE_ERR_NAN);
+    __shared__ long long red[kUfThreads<T> / 32][7];     // energy, virial
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        long long x = out ? 0 : q[3 + k];
+#pragma unroll
+        for (int o = 16; o >= L; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < (pressure ? 7 : 1)) {
+        const int k = threadIdx.x;
+        long long x = 0;
+        for (int w = 0; w < kUfThreads<T> / 32; ++w) x += red[w][k];
+        x = UfFix<T>::sum_unit(x);
+        if (x >= (1LL << 47) || x <= -(1LL << 47)) {
+            atomicOr(&st.err, NEFE_ERR_NAN);
+        } else if (x != 0) {
+            const int slot = !pressure ? ACC_UREF : k == 0 ? ACC_UINT : ACC_VIR + k - 1;
+            atomicAdd(reinterpret_cast<unsigned long long*>(
+                          &b.acc[((size_t)ta.sys * ACC_N + slot) * kSlots + (blockIdx.x % kSlots)]),
+                      (unsigned long long)x);
+        }
     }
 }
 
@@ -3599,22 +3827,22 @@ void launch_decode_ev(const long long* acc, double* out7, cudaStream_t s) {
     k_decode_ev<<<1, 32, 0, s>>>(acc, out7);
 }
 
-void launch_uf_list(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches) {
+void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, cudaStream_t s, long* launches) {
     if (ntiles <= 0 || !b.uf_nbr) return;
-    const int g = rebuild_grid(b, ntiles);
-    if (precision == NEFE_FP64) k_uflist<double><<<g, kTile, 0, s>>>(b);
-    else k_uflist<float><<<g, kTile, 0, s>>>(b);
+    const int g = b.rtiles ? kRebuildBlocks : max(1, min(kRebuildBlocks, ntiles * 8));
+    if (precision == NEFE_FP64) k_uflist<double><<<g, kTile, 0, s>>>(b, nsys);
+    else k_uflist<float><<<g, kTile, 0, s>>>(b, nsys);
     if (launches) *launches += 1;
 }
 
 void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches) {
     if (ntiles <= 0 || !b.uf_nbr) return;
     if (precision == NEFE_FP64) {
-        if (mode == FM_FORCES) k_uf<double, FM_FORCES><<<ntiles, kTile, 0, s>>>(b);
-        else k_uf<double, FM_STEP><<<ntiles, kTile, 0, s>>>(b);
+        if (mode == FM_FORCES) k_uf<double, FM_FORCES><<<ntiles * kUfBlocks<double>, kUfThreads<double>, 0, s>>>(b);
+        else k_uf<double, FM_STEP><<<ntiles * kUfBlocks<double>, kUfThreads<double>, 0, s>>>(b);
     } else {
-        if (mode == FM_FORCES) k_uf<float, FM_FORCES><<<ntiles, kTile, 0, s>>>(b);
-        else k_uf<float, FM_STEP><<<ntiles, kTile, 0, s>>>(b);
+        if (mode == FM_FORCES) k_uf<float, FM_FORCES><<<ntiles * kUfBlocks<float>, kUfThreads<float>, 0, s>>>(b);
+        else k_uf<float, FM_STEP><<<ntiles * kUfBlocks<float>, kUfThreads<float>, 0, s>>>(b);
     }
     if (launches) *launches += 1;
 }

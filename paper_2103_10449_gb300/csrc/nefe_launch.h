@@ -107,7 +107,7 @@ void launch_kick_drift(const Bufs& b, int precision, int ntiles, int mode, cudaS
                        long* launches, int skip = 0);
 // Uhlenbeck-Ford pair rows of the UF systems (after the cell fill; flagged systems only when a
 // rebuild worklist is set).
-void launch_uf_list(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches);
+void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, cudaStream_t s, long* launches);
 // Uhlenbeck-Ford forces and energies over `ntiles` tiles (b.uf_tiles, or every tile when NULL);
 // mode FM_FORCES writes b.f_out / b.e_atom (stateless), otherwise b.uf_F for pass B.
 void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches);

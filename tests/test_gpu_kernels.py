@@ -318,3 +318,40 @@ def test_block_sums_of_large_values(N):
     assert np.abs(vir_o).max() > 2 * 2 ** 22       # each end of the pair is above 2^22
     assert abs(float(ev[0]) - e_o) <= 1e-10 * abs(e_o)
     assert np.abs(ev.cpu().numpy()[1:] - vir_o).max() <= 1e-9 * np.abs(vir_o).max()
+
+
+# ------------------------------------------------------------------ Uhlenbeck-Ford rows and pair sums
+# Rows and sums by several lanes per atom: part-filled tiles, rows shorter than the lanes, runs of
+# cells that wrap at either edge of the smallest grid (5 cells, all of an axis in one run) and of a
+# wider one.  Energies and forces normwise within 1e-10 (FP64) and 1e-5 (FP32) of the oracle, as for
+# the other force kernels; pairs a bit closer than sigma to a few sigma apart.
+@pytest.mark.parametrize("precision,tol", [(1, 1e-10), (0, 1e-5)])
+@pytest.mark.parametrize("n,cells", [(2, (5, 5, 5)), (17, (5, 5, 5)), (129, (5, 6, 5)), (700, (5, 5, 9)), (1299, (7, 5, 6))])
+def test_uf_rows_and_sums_by_lanes(N, n, cells, precision, tol):
+    uf = (25.0, 2.0, 2200.0, 8.0)
+    skin = 0.5
+    rcs = O.SW_SI[6] * O.SW_SI[1] + skin
+    box = np.array(cells) * rcs * 1.001
+    rng = np.random.default_rng(100 + n)
+    x = rng.uniform(0.0, box, (n, 3))
+    for _ in range(40):                          # away from contacts: resample what is closer than 1 A
+        d = x[:, None] - x[None]
+        d -= box * np.round(d / box)
+        r2 = (d * d).sum(2) + 1e9 * np.eye(n)
+        bad = np.unique(np.argwhere(r2 < 1.0)[:, 0])
+        if not len(bad):
+            break
+        x[bad] = rng.uniform(0.0, box, (len(bad), 3))
+    if n == 2:
+        x = np.array([[0.2, 0.3, 0.1], box - 0.9])                       # a pair across three faces
+    x = x + box * rng.integers(-3, 4, (n, 3))
+    e_o, f_o, vir_o, ea_o = O.uf_energy(x, box, uf)
+    f = torch.zeros(3 * n, dtype=torch.float64, device="cuda")
+    ea = torch.zeros(n, dtype=torch.float64, device="cuda")
+    ev = torch.zeros(7, dtype=torch.float64, device="cuda")
+    N.nefe_uf_forces(soa(x), n, box, rcs, skin, N.uf_params(*uf), precision, f, ea, ev)
+    f = f.cpu().numpy().reshape(3, n).T
+    assert np.abs(f - f_o).max() <= tol * np.abs(f_o).max()
+    assert np.abs(ea.cpu().numpy() - ea_o).max() <= tol * np.abs(ea_o).max()
+    assert abs(float(ev[0]) - e_o) <= tol * np.abs(ea_o).sum()
+    assert np.abs(ev[1:].cpu().numpy() - vir_o).max() <= 10 * tol * np.abs(vir_o).max()
