@@ -202,7 +202,7 @@ static void want_forces(Scratch1& S, int n, int precision) {
     const size_t N = (size_t)n;
     S.want(&S.shn, sizeof(int) * N);
     S.want(&S.xc, sizeof(uint2) * N);
-    S.want(&S.lscale, sizeof(float4) * 2);
+    S.want(&S.lscale, sizeof(float4) * 4);
     if (precision == NEFE_FP32) {
         S.want(&S.xf, sizeof(int4) * N);
         S.want(&S.lacc, 4 * sizeof(int) * N);
@@ -417,7 +417,7 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
     if (precision == NEFE_FP32) {
         S.want(&S.xf, sizeof(int4) * (size_t)n);
         S.want(&S.xc, sizeof(uint2) * (size_t)n);
-        S.want(&S.lscale, sizeof(float4) * 2);
+        S.want(&S.lscale, sizeof(float4) * 4);
     }
     if ((rc = commit1(S, n, box, rcs, n3, precision, nullptr, uf, skin))) return rc;
     if (n > 0) {

@@ -452,7 +452,7 @@ int setup(nefe_ctx* c) {
         if ((rc = dalloc(c, &c->d_hi_flag, sizeof(int) * tile_sys.size()))) return rc;
         if ((rc = dalloc(c, &c->d_xf, sizeof(int4) * N))) return rc;
     }
-    if ((rc = dalloc(c, &c->d_lscale, sizeof(float4) * 2 * nsys))) return rc;
+    if ((rc = dalloc(c, &c->d_lscale, sizeof(float4) * 4 * nsys))) return rc;
     if ((rc = dalloc(c, &c->d_xfb, sizeof(int4) * N))) return rc;
     if ((rc = dalloc(c, &c->d_xc, sizeof(uint2) * N))) return rc;
     if ((rc = dalloc(c, &c->d_rtiles, sizeof(int) * tile_sys.size()))) return rc;

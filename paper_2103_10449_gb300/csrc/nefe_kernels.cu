@@ -349,17 +349,23 @@ __device__ __forceinline__ int4 frac_position(const double (&x)[3], const DevSta
     return make_int4(frac32(x[0], st.ibox[0]), frac32(x[1], st.ibox[1]), frac32(x[2], st.ibox[2]), 0);
 }
 
-// L 2^-32 of system s as FP32 value and remainder (what pass A's positions are scaled by).
-__device__ __forceinline__ void scale_of_box(const Bufs& b, int s, const double box[3]) {
+// The four rows of system s in lscale: L 2^-32 as FP32 value and remainder (what the fractional positions
+// are scaled by), 1 - h/hb (0 while the box is the one of the last build; the division in FP64, since it
+// is the small difference of two nearly equal edges) and 2^32 / L.  Kept per system and rewritten where
+// the box changes: a division per block of the kernels that move the atoms had the integration of
+// 128 x 4000 atoms under barostats at 45.4 us a launch, now 42.8 (an FP64 warp instruction issues in 16 cycles).
+__device__ __forceinline__ void scale_axis(const Bufs& b, int s, int k, double box, double omr) {
+    float* row = reinterpret_cast<float*>(b.lscale + 4 * s) + k;
+    const double L = box * 0x1p-32;
+    const float hi = (float)L;
+    row[0] = hi;
+    row[4] = (float)(L - (double)hi);
+    row[8] = (float)omr;
+    row[12] = 4294967296.0f / (float)box;
+}
+__device__ __forceinline__ void scale_of_box(const Bufs& b, int s, const DevState& st) {
     if (!b.lscale) return;
-    float hi[3], lo[3];
-    for (int k = 0; k < 3; ++k) {
-        const double L = box[k] * 0x1p-32;
-        hi[k] = (float)L;
-        lo[k] = (float)(L - (double)hi[k]);
-    }
-    b.lscale[2 * s] = make_float4(hi[0], hi[1], hi[2], 0.0f);
-    b.lscale[2 * s + 1] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+    for (int k = 0; k < 3; ++k) scale_axis(b, s, k, st.box[k], st.hmoved ? 1.0 - st.h[k] / st.hb[k] : 0.0);
 }
 
 // ------------------------------------------------------------------------------------
@@ -401,7 +407,7 @@ __device__ void cells_count_tile(const Bufs& b, int tile) {
     if (b.xa) reinterpret_cast<T4*>(b.xa)[i] = m;
     if (b.sd0) reinterpret_cast<T4*>(b.sd0)[i] = mk4((T)sd[0], (T)sd[1], (T)sd[2], (T)0);
     if (b.xfb && b.want_xf) {
-        if (i == S.off) scale_of_box(b, ta.sys, st.box);
+        if (i == S.off) scale_of_box(b, ta.sys, st);
         const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
         const int4 f = frac_position(x3, st);
         if (b.xf) b.xf[i] = f;
@@ -1587,8 +1593,8 @@ __global__ void __launch_bounds__(kUfThreads<T>, sizeof(T) == 4 ? 5 : 1) k_uf(Bu
         float4 Lh = make_float4(0.f, 0.f, 0.f, 0.f), Ll = Lh;
         if constexpr (kFrac) {
             fi = b.xf[i];
-            Lh = b.lscale[2 * ta.sys];
-            Ll = b.lscale[2 * ta.sys + 1];
+            Lh = b.lscale[4 * ta.sys];
+            Ll = b.lscale[4 * ta.sys + 1];
         } else {
             xi = reinterpret_cast<const T4*>(b.xs)[i];
         }
@@ -1708,7 +1714,7 @@ __global__ void __launch_bounds__(kTile) k_mirror(Bufs b) {
         const size_t N = b.ntot;
         const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
         b.xc[i] = pack_frac(frac_position(x3, st));
-        if (i == 0) scale_of_box(b, 0, st.box);
+        if (i == 0) scale_of_box(b, 0, st);
     }
 }
 
@@ -1739,18 +1745,13 @@ __device__ __forceinline__ void comp_add(T& hi, T& lo, T d) {
     }
 }
 
-// Per-block constants of the fractional positions' update, set by threads 0..2 (the caller syncs):
-// 1 - h/hb per axis (0 while the box is the one of the last build), with the division in FP64 since it
-// is the small difference of two nearly equal edges, and 2^32 / L.
+// Constants of the fractional positions' update (rows 2 and 3 of lscale).
 struct BoxMove {
     float omr[3], to_frac[3];
 };
-__device__ __forceinline__ void box_move(const DevState& st, BoxMove& m) {
-    const int k = threadIdx.x;
-    if (k < 3) {
-        m.omr[k] = st.hmoved ? (float)(1.0 - st.h[k] / st.hb[k]) : 0.0f;
-        m.to_frac[k] = 4294967296.0f / (float)st.box[k];
-    }
+__device__ __forceinline__ BoxMove box_move(const Bufs& b, int s) {
+    const float4 o = b.lscale[4 * s + 2], t = b.lscale[4 * s + 3];
+    return {{o.x, o.y, o.z}, {t.x, t.y, t.z}};
 }
 
 // Position of atom i from its displacement d since the last build: the mirror (want_xs) and, in the
@@ -1864,12 +1865,16 @@ __global__ void __launch_bounds__(kTile) k_positions(Bufs b) {
     __shared__ BoxMove bm;
     const TileAtom ta = tile_of(b, blockIdx.x);
     const DevState& st = b.st[ta.sys];
-    box_move(st, bm);
+    if (threadIdx.x < 3) {                       // (the rows of lscale are written below)
+        const int k = threadIdx.x;
+        bm.omr[k] = st.hmoved ? (float)(1.0 - st.h[k] / st.hb[k]) : 0.0f;
+        bm.to_frac[k] = 4294967296.0f / (float)st.box[k];
+    }
     __syncthreads();
     if ((int)threadIdx.x >= ta.count) return;
     const int i = ta.first + threadIdx.x;
     const size_t N = b.ntot;
-    if (b.want_xf && i == b.sys[ta.sys].off) scale_of_box(b, ta.sys, st.box);
+    if (b.want_xf && i == b.sys[ta.sys].off) scale_of_box(b, ta.sys, st);
     int4 fb = make_int4(0, 0, 0, 0);
     if (b.want_xf) {
         const double x[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
@@ -1892,11 +1897,7 @@ __global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip
     const DevSys& S = b.sys[ta.sys];
     DevState& st = b.st[ta.sys];
     if (skip && S.baro == BARO_NONE) return;     // uniform over the block (one system per tile)
-    __shared__ BoxMove bm;
-    if (b.want_xf) {
-        box_move(st, bm);
-        __syncthreads();
-    }
+    const BoxMove bm = b.want_xf ? box_move(b, ta.sys) : BoxMove{};
     T xs_sum[3] = {(T)0, (T)0, (T)0};
     if ((int)threadIdx.x < ta.count) {
         const int i = ta.first + threadIdx.x;
@@ -2596,7 +2597,7 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc,
     const bool valid = ia < ta.count;
     // L 2^-32 to twice the precision: a relative error of L alone would be a uniform strain of up to
     // 6e-8, which the pressure sees (the row filter does without the second part)
-    const float4 Lh = b.lscale[2 * ta.sys], Ll = b.lscale[2 * ta.sys + 1];
+    const float4 Lh = b.lscale[4 * ta.sys], Ll = b.lscale[4 * ta.sys + 1];
     // 1. accepted row entries
     unsigned lo = 0u, hi = 0u;
     if (valid) mark_row(b, i, lane >> lg, lpa, Lh, P.act2, &st.err, lo, hi);
@@ -2806,7 +2807,7 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
     const double hx = st.h[0], hy = st.h[1], hz = st.h[2];
     const double4* X = reinterpret_cast<const double4*>(b.xs);
     unsigned lo = 0u, hi = 0u;
-    if (valid) mark_row(b, i, lane >> lg, lpa, b.lscale[2 * ta.sys], (float)P.rc2, &st.err, lo, hi);
+    if (valid) mark_row(b, i, lane >> lg, lpa, b.lscale[4 * ta.sys], (float)P.rc2, &st.err, lo, hi);
     const int ml = __popc(lo) + __popc(hi);      // edges of this lane, then of its atom
     int m = ml, before = 0;                      // before: of the atom's lanes before this one
     for (int o = 16; o >= G; o >>= 1) m += __shfl_xor_sync(kAll, m, o);
@@ -3231,7 +3232,6 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
     __shared__ __align__(16) StagedSys sh;
     __shared__ long long s_xi[3][kSlots];
     __shared__ T s_xm[3];
-    __shared__ BoxMove bm;
     const TileAtom ta = tile_of(b, tile);
     const bool valid = (int)threadIdx.x < ta.count;
     const int i = ta.first + threadIdx.x;
@@ -3243,6 +3243,7 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
     int4 q = make_int4(0, 0, 0, 0), fb = q;
     T4 d0 = mk4((T)0, (T)0, (T)0, (T)0), z = d0, xa = d0;
     T dh[3] = {(T)0, (T)0, (T)0}, dl[3] = {(T)0, (T)0, (T)0}, pv[3] = {(T)0, (T)0, (T)0};
+    BoxMove bm{};
     if (valid) {
         q = *a4;
         if (MODE != FM_FORCES) {
@@ -3258,6 +3259,7 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
             }
             z = reinterpret_cast<const T4*>(b.xi)[i];
             if (MODE == FM_STEP && fuse) {
+                if (b.want_xf) bm = box_move(b, ta.sys);
                 if (b.want_xs) xa = reinterpret_cast<const T4*>(b.xa)[i];   // (no barostat: the box never moves)
                 if (b.want_xf) fb = b.xfb[i];
             }
@@ -3274,7 +3276,6 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
     const DevState& st = sh.st;
     DevState& gst = b.st[ta.sys];
     if (MODE != FM_FORCES) noise_mean_staged<T>(S, s_xi, s_xm);
-    if (MODE == FM_STEP && fuse) box_move(st, bm);
     __syncthreads();
     if (big != 0 && threadIdx.x == 0) b.hi_flag[tile] = 0;            // every thread has read it
     const bool fz = MODE == FM_STEP && fuse && S.baro == BARO_NONE;   // uniform over the block
@@ -3482,12 +3483,7 @@ __device__ __forceinline__ void prepare_step(const Bufs& b, int s, const DevSys&
             st.h_f[lane] = (float)h;
             st.hb_f[lane] = (float)st.hb[lane];
             st.rho_f[lane] = (float)ratio;
-            if (b.lscale) {                      // (scale_of_box, one axis per lane)
-                const double L = box * 0x1p-32;
-                const float hi = (float)L;
-                reinterpret_cast<float*>(b.lscale + 2 * s)[lane] = hi;
-                reinterpret_cast<float*>(b.lscale + 2 * s + 1)[lane] = (float)(L - (double)hi);
-            }
+            if (b.lscale) scale_axis(b, s, lane, box, hm ? 1.0 - ratio : 0.0);
         }
     }
     if (lane == 0) {
@@ -3569,7 +3565,7 @@ __global__ void __launch_bounds__(kTile) k_group(Bufs b, const DevGroup* groups,
                     st.s[k] = 1.0; st.phi[k] = 1.0; st.phi_f[k] = 1.0f; st.sm1_f[k] = 0.0f;
                 }
                 st.scaled = 0;
-                scale_of_box(b, mine, st.box);
+                scale_of_box(b, mine, st);
             }
         }
     } else if (mode == 1) {
@@ -3870,7 +3866,7 @@ __global__ void __launch_bounds__(kTile) k_frac_positions(Bufs b) {
     const int4 f = frac_position(x, b.st[0]);
     b.xf[i] = f;
     b.xc[i] = pack_frac(f);
-    if (i == 0) scale_of_box(b, 0, b.st[0].box);
+    if (i == 0) scale_of_box(b, 0, b.st[0]);
 }
 void launch_frac_positions(const Bufs& b, cudaStream_t s) {
     if (b.ntot > 0) k_frac_positions<<<(b.ntot + kTile - 1) / kTile, kTile, 0, s>>>(b);

@@ -73,7 +73,7 @@ struct Bufs {
     int common;
     int leg_refuse;          // the scatter form was chosen by the caller: terms above its limit are refused
     int* hi_flag;            // [tiles] some large term was split this step (cleared by k_finish)
-    float4* lscale;          // [nsys][2] L 2^-32 as FP32 value and remainder
+    float4* lscale;          // [nsys][4] L 2^-32 as FP32 value and remainder, 1 - h/hb, 2^32/L
     int4* xf;                // FP32: fractional positions (x/L as 32-bit fixed point)
     int4* xfb;               // their values at the last list build
     uint2* xc;               // their top 21 bits per axis (pass A's row filter)
