@@ -299,7 +299,7 @@ int setup(nefe_ctx* c) {
     std::vector<DevSys> hs(nsys);
     std::vector<DevState> hst(nsys);
     std::vector<int> tile_sys;
-    long long ntot = 0, ncell = 0, tr = 0;
+    long long ntot = 0, ncell = 0, ncell_now = 0, tr = 0;
     for (int s = 0; s < nsys; ++s) {
         HostSys& h = c->sys[s];
         const double rcs = rc_of(h) + c->skin;
@@ -309,6 +309,7 @@ int setup(nefe_ctx* c) {
         // room for the box to grow by 25 % per axis under a barostat
         long long cap = 1;
         for (int k = 0; k < 3; ++k) cap *= (long long)std::max(2, (int)std::floor(n3[k] * 1.25) + 1);
+        ncell_now += (long long)n3[0] * n3[1] * n3[2];
         DevSys& d = hs[s];
         std::memset(&d, 0, sizeof(d));
         d.off = (int)ntot;
@@ -547,6 +548,7 @@ int setup(nefe_ctx* c) {
     b.cap = c->cap; b.ntot = c->ntot; b.dt = c->dt; b.swc = c->d_swc; b.pairs = c->d_pairs;
     b.nbr_il = (c->cap & 3) == 0 ? 1 : 0;   // interleaved rows (the force passes read them 4 at a time)
     b.rebuild_all = c->rebuild_all;
+    b.ncells_host = (int)std::min<long long>(ncell_now, 1 << 30);
 
     b.trace = c->d_trace;
     b.list_lanes = c->llanes;

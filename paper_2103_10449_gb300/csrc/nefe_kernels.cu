@@ -40,6 +40,39 @@
 
 namespace nefe {
 
+// Every kernel here waits, before its first memory access, for the launch before it to have completed
+// (dep_wait; a kernel that does not use its result waits as well, so that completion stays transitive
+// along the stream), and is launched with programmatic stream serialization: its blocks are then
+// resident already when the last block before them ends.  A step is 8 to 10 dependent launches of a
+// few us each, and what this takes off is the start of each.  One 8000-atom FP32 system
+// 28.3 -> 26.0 us a step, 64 atoms in FP64 50.8 -> 48.0 us.  Not after a long launch that fills the chip: the blocks would
+// go to the SMs that finish first and leave the others idle (16 x 8000 atoms in FP64: gather 57 -> 90 us), so
+// the kernels that follow the pair passes use it up to kEarlyBlocks blocks only, and the group update
+// up to kEarlyGroups.  Launched without the attribute the two instructions do nothing.
+constexpr int kEarlyBlocks = 2 * 152, kEarlyGroups = 32;
+__device__ __forceinline__ void dep_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename T> struct Same { using t = T; };
+template <typename... P>
+static void launch_next_if(bool early, void (*kernel)(P...), int blocks, int threads, cudaStream_t s, typename Same<P>::t... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... P>
+static void launch_next(void (*kernel)(P...), int blocks, int threads, cudaStream_t s, typename Same<P>::t... args) {
+    launch_next_if(true, kernel, blocks, threads, s, args...);
+}
+
 template <typename T> struct V4;
 template <> struct V4<float> { using t = float4; };
 template <> struct V4<double> { using t = double4; };
@@ -435,6 +468,7 @@ __device__ void cells_count_tile(const Bufs& b, int tile) {
 
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_cells_count(Bufs b) {
+    dep_wait();
     NEFE_FOR_TILES(b, cells_count_tile<T>(b, tile));
 }
 
@@ -528,6 +562,7 @@ __device__ void build_worklist(const Bufs& b, int nsys, int force_all) {
 }
 
 __global__ void __launch_bounds__(256) k_rebuild_list(Bufs b, int nsys, int force_all) {
+    dep_wait();
     build_worklist(b, nsys, force_all);
 }
 
@@ -592,6 +627,7 @@ __device__ void scan_system_cells(const Bufs& b, int s) {
 // One 256-thread block per system; systems whose rebuild flag is clear return (all are scanned
 // with force_all).
 __global__ void __launch_bounds__(256) k_cells_scan(Bufs b, int force_all) {
+    dep_wait();
     const int s = blockIdx.x;
     if (!force_all && !b.st[s].rebuild) return;
     scan_system_cells(b, s);
@@ -605,6 +641,7 @@ __global__ void __launch_bounds__(256) k_cells_scan(Bufs b, int force_all) {
 constexpr int kScanBlocks = 1024;
 constexpr int kScanOneBlock = 4096;
 __global__ void __launch_bounds__(256) k_cells_span_sums(Bufs b, int span, int* sums) {
+    dep_wait();
     const DevState& st = b.st[0];
     const int ncells = st.ncell[0] * st.ncell[1] * st.ncell[2];
     const int lo = blockIdx.x * span, hi = min(ncells, lo + span);
@@ -620,6 +657,7 @@ __global__ void __launch_bounds__(256) k_cells_span_sums(Bufs b, int span, int* 
     }
 }
 __global__ void __launch_bounds__(256) k_cells_scan_spans(Bufs b, int span, const int* sums) {
+    dep_wait();
     const DevState& st = b.st[0];
     const int ncells = st.ncell[0] * st.ncell[1] * st.ncell[2];
     int v = 0;
@@ -663,6 +701,7 @@ __device__ void cells_fill_tile(const Bufs& b, int tile) {
 }
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_cells_fill(Bufs b) {
+    dep_wait();
     NEFE_FOR_TILES(b, cells_fill_tile<T>(b, tile));
 }
 
@@ -670,6 +709,7 @@ __global__ void __launch_bounds__(kTile) k_cells_fill(Bufs b) {
 // per thread over gridDim.x blocks.  Only the stateless cell sort runs it: the list builds rank
 // their rows themselves.
 __global__ void __launch_bounds__(256) k_cells_sort(Bufs b) {
+    dep_wait();
     constexpr int s = 0;
     const DevSys& S = b.sys[s];
     const DevState& st = b.st[s];
@@ -962,6 +1002,7 @@ __device__ void nlist_item(const Bufs& b, int tile, int part, unsigned (*keys)[k
 
 template <typename T, int L>
 __global__ void __launch_bounds__(kTile, 8) k_nlist(Bufs b) {
+    dep_wait();
     constexpr int G = kTile / L;
     __shared__ __align__(16) unsigned keys[G][kKeyRow];
     __shared__ NlistShared<T> tab[G];
@@ -1222,6 +1263,7 @@ __device__ void nlist_cells_of_grid(const Bufs& b, int nsys, CellListShared<T>* 
 
 template <typename T>
 __global__ void __launch_bounds__(kTile, 8) k_nlist_cell(Bufs b, int nsys) {
+    dep_wait();
     __shared__ CellListShared<T> shm[kTile / 32];
     nlist_cells_of_grid<T>(b, nsys, shm);
 }
@@ -1446,6 +1488,7 @@ __device__ __forceinline__ void uflist_cell(const Bufs& b, int s, int c, UfListS
 }
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_uflist(Bufs b, int nsys) {
+    dep_wait();
     __shared__ UfListShared<T> shm[kTile / 32];
     UfListShared<T>& sh = shm[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -1558,6 +1601,7 @@ template <typename T> constexpr int kUfThreads = sizeof(T) == 8 ? 4 * kTile : kT
 template <typename T> constexpr int kUfBlocks = kTile * kUfLanes<T> / kUfThreads<T>;   // per tile
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kUfThreads<T>, sizeof(T) == 4 ? 5 : 1) k_uf(Bufs b) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     constexpr bool kFrac = sizeof(T) == 4;
     constexpr int L = kUfLanes<T>, PARTS = kUfBlocks<T>, G = kTile / PARTS;   // atoms per block
@@ -1697,6 +1741,7 @@ __global__ void __launch_bounds__(kUfThreads<T>, sizeof(T) == 4 ? 5 : 1) k_uf(Bu
 // Mirror only (stateless forces): same q / xs formula as R1, without counting.
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_mirror(Bufs b) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     const TileAtom ta = tile_of(b, blockIdx.x);
     const DevState& st = b.st[ta.sys];
@@ -1861,6 +1906,7 @@ __device__ __forceinline__ void drift_atom(const Bufs& b, const DevSys& S, const
 // in use read (after a checkpoint was loaded or another form was chosen).
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_positions(Bufs b) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     __shared__ BoxMove bm;
     const TileAtom ta = tile_of(b, blockIdx.x);
@@ -1892,6 +1938,7 @@ __global__ void __launch_bounds__(kTile) k_positions(Bufs b) {
 // epilogue (k_finish with fuse), so their tiles return at once.
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     const TileAtom ta = tile_of(b, blockIdx.x);
     const DevSys& S = b.sys[ta.sys];
@@ -2000,6 +2047,7 @@ __device__ __forceinline__ void sw_pair_pgrad(const SWc<T>& P, T r, T out[5]) {
 // P[i] = (pair + own triplet force, atom energy), then the atom's virial.
 template <typename T, int L>
 __global__ void __launch_bounds__(kTile) k_edges(Bufs b) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     constexpr int G = kTile / L;
     // rows padded by one entry: the groups of a warp then start on different banks
@@ -2301,6 +2349,7 @@ __device__ __forceinline__ void edges1_atom(const Bufs& b, const SWc<T>& P, DevS
 
 template <typename T>
 __global__ void __launch_bounds__(kEdges1Threads, 16) k_edges1(Bufs b) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     constexpr int NT = kEdges1Threads, IPT = kTile / NT;
     __shared__ T4 sh_u[kEdges1K1][NT];           // (d, r^2) after compaction, then (u, g)
@@ -2579,6 +2628,7 @@ __device__ __forceinline__ void mark_row(const Bufs& b, int i, int part, int lpa
 template <bool EATOM, bool GRAD, bool COMMON, int BLOCKS>
 __global__ void __launch_bounds__(kScatterThreads, BLOCKS)
 k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc, int lg) {
+    dep_wait();
     constexpr unsigned kAll = 0xffffffffu;
     const int G = 1 << lg, lpa = 5 - lg;
     __shared__ ScatterShared<EATOM> shm[kScatterThreads / 32];
@@ -2789,6 +2839,7 @@ struct __align__(16) EdgesDShared {
 template <bool GRAD, bool COMMON>
 __global__ void __launch_bounds__(64)
 k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc, int lg) {
+    dep_wait();
     constexpr unsigned kAll = 0xffffffffu;
     __shared__ EdgesDShared shm[2];
     EdgesDShared& sh = shm[threadIdx.x >> 5];
@@ -2982,6 +3033,7 @@ __device__ __forceinline__ void noise_mean_staged(const DevSys& S, const long lo
 
 template <typename T, int MODE, int L>
 __global__ void __launch_bounds__(kTile) k_gather(Bufs b) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     constexpr int G = kTile / L;
     const int tile = blockIdx.x / L + b.tile_base, part = blockIdx.x % L;
@@ -3227,6 +3279,7 @@ __device__ __forceinline__ void noise_mean(const Bufs& b, const DevSys& S, int s
 // the usual one (positions and velocities at a full step).
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
+    dep_wait();
     using T4 = typename V4<T>::t;
     const int tile = blockIdx.x + b.tile_base;
     __shared__ __align__(16) StagedSys sh;
@@ -3321,6 +3374,7 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
 // FP64 positions and velocities for output, and replacement from FP64 input.
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_materialize(Bufs b, double* x, double* v) {
+    dep_wait();
     const TileAtom ta = tile_of(b, blockIdx.x);
     if ((int)threadIdx.x >= ta.count) return;
     const int i = ta.first + threadIdx.x;
@@ -3340,6 +3394,7 @@ __global__ void __launch_bounds__(kTile) k_materialize(Bufs b, double* x, double
 
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_inject(Bufs b, const double* x, const double* v) {
+    dep_wait();
     const TileAtom ta = tile_of(b, blockIdx.x);
     if ((int)threadIdx.x >= ta.count) return;
     const int i = ta.first + threadIdx.x;
@@ -3511,6 +3566,7 @@ struct GroupShared {
     double next[3];      // lambda (schedule); T or p at this step and the next (pair)
 };
 __global__ void __launch_bounds__(kTile) k_group(Bufs b, const DevGroup* groups, int mode, int carry) {
+    dep_wait();
     const DevGroup gr = groups[blockIdx.x];
     const int nm = gr.b >= 0 ? 2 : 1;
     __shared__ __align__(16) GroupShared sh;
@@ -3655,6 +3711,7 @@ __global__ void __launch_bounds__(kTile) k_group(Bufs b, const DevGroup* groups,
 
 __global__ void k_noise(unsigned long long seed, unsigned long long sys, unsigned long long step, int n,
                         int prec, double* xi) {
+    dep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (prec == NEFE_FP64) {
@@ -3670,12 +3727,14 @@ __global__ void k_noise(unsigned long long seed, unsigned long long sys, unsigne
 
 // (n,3) row-major <-> SoA with stride n.
 __global__ void k_aos_to_soa(const double* __restrict__ a, double* __restrict__ s, int n) {
+    dep_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 3 * n) return;
     const int i = t / 3, k = t % 3;
     s[(size_t)k * n + i] = a[t];
 }
 __global__ void k_soa_to_aos(const double* __restrict__ s, double* __restrict__ a, int n) {
+    dep_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 3 * n) return;
     const int i = t / 3, k = t % 3;
@@ -3683,6 +3742,7 @@ __global__ void k_soa_to_aos(const double* __restrict__ s, double* __restrict__ 
 }
 
 __global__ void k_decode_ev(const long long* acc, double* out7) {
+    dep_wait();
     const int t = threadIdx.x;
     if (t >= 7) return;
     const int a = t == 0 ? ACC_UINT : ACC_VIR + (t - 1);
@@ -3702,23 +3762,30 @@ static int rebuild_grid(const Bufs& b, int items) {
     return b.rtiles ? (items < kRebuildBlocks ? items : kRebuildBlocks) : items;
 }
 
+// Blocks of the list builds: a warp for every cell there can be (ncells_host), up to kRebuildBlocks; on a
+// step without a rebuild the launch costs what its blocks cost to start (1216 blocks 2.7 us).
+static int list_grid(const Bufs& b, int ntiles) {
+    const int most = b.ncells_host > 0 ? (b.ncells_host + kTile / 32 - 1) / (kTile / 32) : ntiles * 8;
+    return max(1, min(kRebuildBlocks, most));
+}
+
 void launch_cells(const Bufs& b, int precision, int ntiles, int nsys, int force_all,
                   cudaStream_t s, long* launches) {
     if (ntiles <= 0) return;
-    if (b.rtiles) k_rebuild_list<<<1, 256, 0, s>>>(b, nsys, force_all);
+    if (b.rtiles) launch_next(k_rebuild_list, 1, 256, s, b, nsys, force_all);
     const int g = rebuild_grid(b, ntiles);
-    if (precision == NEFE_FP64) k_cells_count<double><<<g, kTile, 0, s>>>(b);
-    else k_cells_count<float><<<g, kTile, 0, s>>>(b);
+    if (precision == NEFE_FP64) launch_next(k_cells_count<double>, g, kTile, s, b);
+    else launch_next(k_cells_count<float>, g, kTile, s, b);
     if (!b.rtiles && b.scan_sums && b.ncells_host > kScanOneBlock) {
         const int span = cells_scan_span(b.ncells_host);
         const int blocks = (b.ncells_host + span - 1) / span;
-        k_cells_span_sums<<<blocks, 256, 0, s>>>(b, span, b.scan_sums);
-        k_cells_scan_spans<<<blocks, 256, 0, s>>>(b, span, b.scan_sums);
+        launch_next(k_cells_span_sums, blocks, 256, s, b, span, b.scan_sums);
+        launch_next(k_cells_scan_spans, blocks, 256, s, b, span, b.scan_sums);
     } else {
-        k_cells_scan<<<nsys, 256, 0, s>>>(b, force_all || !b.rtiles);
+        launch_next(k_cells_scan, nsys, 256, s, b, force_all || !b.rtiles);
     }
-    if (precision == NEFE_FP64) k_cells_fill<double><<<g, kTile, 0, s>>>(b);
-    else k_cells_fill<float><<<g, kTile, 0, s>>>(b);
+    if (precision == NEFE_FP64) launch_next(k_cells_fill<double>, g, kTile, s, b);
+    else launch_next(k_cells_fill<float>, g, kTile, s, b);
     if (launches) *launches += 4;
 }
 
@@ -3729,7 +3796,7 @@ int cells_scan_span(int ncells) {
 
 void launch_cells_sort(const Bufs& b, int ncells, cudaStream_t s) {
     const int blocks = (ncells + 255) / 256;
-    k_cells_sort<<<blocks < 4096 ? blocks : 4096, 256, 0, s>>>(b);
+    launch_next(k_cells_sort, blocks < 4096 ? blocks : 4096, 256, s, b);
 }
 
 void launch_cells_and_list(const Bufs& b, int precision, int ntiles, int nsys, int force_all,
@@ -3738,21 +3805,21 @@ void launch_cells_and_list(const Bufs& b, int precision, int ntiles, int nsys, i
     launch_cells(b, precision, ntiles, nsys, force_all, s, launches);
     const int L = (b.list_lanes == 8 || b.list_lanes == 16 || b.list_lanes == 32) ? b.list_lanes : 0;
     if (L == 0) {
-        const int g = b.rtiles ? kRebuildBlocks : max(1, min(kRebuildBlocks, ntiles * 8));
-        if (precision == NEFE_FP64) k_nlist_cell<double><<<g, kTile, 0, s>>>(b, nsys);
-        else k_nlist_cell<float><<<g, kTile, 0, s>>>(b, nsys);
+        const int g = list_grid(b, ntiles);
+        if (precision == NEFE_FP64) launch_next(k_nlist_cell<double>, g, kTile, s, b, nsys);
+        else launch_next(k_nlist_cell<float>, g, kTile, s, b, nsys);
         if (launches) *launches += 1;
         return;
     }
     const int g = rebuild_grid(b, ntiles * L);
     if (precision == NEFE_FP64) {
-        if (L == 8) k_nlist<double, 8><<<g, kTile, 0, s>>>(b);
-        else if (L == 16) k_nlist<double, 16><<<g, kTile, 0, s>>>(b);
-        else k_nlist<double, 32><<<g, kTile, 0, s>>>(b);
+        if (L == 8) launch_next(k_nlist<double, 8>, g, kTile, s, b);
+        else if (L == 16) launch_next(k_nlist<double, 16>, g, kTile, s, b);
+        else launch_next(k_nlist<double, 32>, g, kTile, s, b);
     } else {
-        if (L == 8) k_nlist<float, 8><<<g, kTile, 0, s>>>(b);
-        else if (L == 16) k_nlist<float, 16><<<g, kTile, 0, s>>>(b);
-        else k_nlist<float, 32><<<g, kTile, 0, s>>>(b);
+        if (L == 8) launch_next(k_nlist<float, 8>, g, kTile, s, b);
+        else if (L == 16) launch_next(k_nlist<float, 16>, g, kTile, s, b);
+        else launch_next(k_nlist<float, 32>, g, kTile, s, b);
     }
     if (launches) *launches += 1;
 }
@@ -3803,11 +3870,12 @@ int check_barrier_timeout(double limit_ms) {
 void launch_aos_soa(const double* src, double* dst, int n, int to_soa, cudaStream_t s) {
     if (n <= 0) return;
     const int blocks = (3 * n + 255) / 256;
-    if (to_soa) k_aos_to_soa<<<blocks, 256, 0, s>>>(src, dst, n);
-    else k_soa_to_aos<<<blocks, 256, 0, s>>>(src, dst, n);
+    if (to_soa) launch_next(k_aos_to_soa, blocks, 256, s, src, dst, n);
+    else launch_next(k_soa_to_aos, blocks, 256, s, src, dst, n);
 }
 
 __global__ void k_decode_grad(const long long* acc, double* out8) {
+    dep_wait();
     const int t = threadIdx.x;
     if (t >= 8) return;
     const int a = t == 0 ? ACC_UINT : ACC_DTH + (t - 1);
@@ -3815,29 +3883,29 @@ __global__ void k_decode_grad(const long long* acc, double* out8) {
 }
 
 void launch_decode_grad(const long long* acc, double* out8, cudaStream_t s) {
-    k_decode_grad<<<1, 32, 0, s>>>(acc, out8);
+    launch_next(k_decode_grad, 1, 32, s, acc, out8);
 }
 
 void launch_decode_ev(const long long* acc, double* out7, cudaStream_t s) {
-    k_decode_ev<<<1, 32, 0, s>>>(acc, out7);
+    launch_next(k_decode_ev, 1, 32, s, acc, out7);
 }
 
 void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, cudaStream_t s, long* launches) {
     if (ntiles <= 0 || !b.uf_nbr) return;
-    const int g = b.rtiles ? kRebuildBlocks : max(1, min(kRebuildBlocks, ntiles * 8));
-    if (precision == NEFE_FP64) k_uflist<double><<<g, kTile, 0, s>>>(b, nsys);
-    else k_uflist<float><<<g, kTile, 0, s>>>(b, nsys);
+    const int g = list_grid(b, ntiles);
+    if (precision == NEFE_FP64) launch_next(k_uflist<double>, g, kTile, s, b, nsys);
+    else launch_next(k_uflist<float>, g, kTile, s, b, nsys);
     if (launches) *launches += 1;
 }
 
 void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches) {
     if (ntiles <= 0 || !b.uf_nbr) return;
     if (precision == NEFE_FP64) {
-        if (mode == FM_FORCES) k_uf<double, FM_FORCES><<<ntiles * kUfBlocks<double>, kUfThreads<double>, 0, s>>>(b);
-        else k_uf<double, FM_STEP><<<ntiles * kUfBlocks<double>, kUfThreads<double>, 0, s>>>(b);
+        if (mode == FM_FORCES) launch_next(k_uf<double, FM_FORCES>, ntiles * kUfBlocks<double>, kUfThreads<double>, s, b);
+        else launch_next(k_uf<double, FM_STEP>, ntiles * kUfBlocks<double>, kUfThreads<double>, s, b);
     } else {
-        if (mode == FM_FORCES) k_uf<float, FM_FORCES><<<ntiles * kUfBlocks<float>, kUfThreads<float>, 0, s>>>(b);
-        else k_uf<float, FM_STEP><<<ntiles * kUfBlocks<float>, kUfThreads<float>, 0, s>>>(b);
+        if (mode == FM_FORCES) launch_next(k_uf<float, FM_FORCES>, ntiles * kUfBlocks<float>, kUfThreads<float>, s, b);
+        else launch_next(k_uf<float, FM_STEP>, ntiles * kUfBlocks<float>, kUfThreads<float>, s, b);
     }
     if (launches) *launches += 1;
 }
@@ -3845,20 +3913,21 @@ void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t 
 void launch_kick_drift(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches,
                        int skip) {
     if (ntiles <= 0) return;
-    if (precision == NEFE_FP64) k_kick_drift<double><<<ntiles, kTile, 0, s>>>(b, mode, skip);
-    else k_kick_drift<float><<<ntiles, kTile, 0, s>>>(b, mode, skip);
+    if (precision == NEFE_FP64) launch_next(k_kick_drift<double>, ntiles, kTile, s, b, mode, skip);
+    else launch_next(k_kick_drift<float>, ntiles, kTile, s, b, mode, skip);
     if (launches) *launches += 1;
 }
 
 void launch_positions(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches) {
     if (ntiles <= 0) return;
-    if (precision == NEFE_FP64) k_positions<double><<<ntiles, kTile, 0, s>>>(b);
-    else k_positions<float><<<ntiles, kTile, 0, s>>>(b);
+    if (precision == NEFE_FP64) launch_next(k_positions<double>, ntiles, kTile, s, b);
+    else launch_next(k_positions<float>, ntiles, kTile, s, b);
     if (launches) *launches += 1;
 }
 
 // Fractional positions only (stateless scatter form).
 __global__ void __launch_bounds__(kTile) k_frac_positions(Bufs b) {
+    dep_wait();
     const int i = blockIdx.x * kTile + threadIdx.x;
     if (i >= b.ntot) return;
     const size_t N = b.ntot;
@@ -3869,13 +3938,13 @@ __global__ void __launch_bounds__(kTile) k_frac_positions(Bufs b) {
     if (i == 0) scale_of_box(b, 0, b.st[0]);
 }
 void launch_frac_positions(const Bufs& b, cudaStream_t s) {
-    if (b.ntot > 0) k_frac_positions<<<(b.ntot + kTile - 1) / kTile, kTile, 0, s>>>(b);
+    if (b.ntot > 0) launch_next(k_frac_positions, (b.ntot + kTile - 1) / kTile, kTile, s, b);
 }
 
 void launch_mirror(const Bufs& b, int precision, int ntiles, cudaStream_t s, long* launches) {
     if (ntiles <= 0) return;
-    if (precision == NEFE_FP64) k_mirror<double><<<ntiles, kTile, 0, s>>>(b);
-    else k_mirror<float><<<ntiles, kTile, 0, s>>>(b);
+    if (precision == NEFE_FP64) launch_next(k_mirror<double>, ntiles, kTile, s, b);
+    else launch_next(k_mirror<float>, ntiles, kTile, s, b);
     if (launches) *launches += 1;
 }
 
@@ -3892,7 +3961,7 @@ static void edges_fp32(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
     switch (lanes) {
         case 0: {
             const int lg = b.lg, items = ntiles << (6 - lg);
-            const auto go = [&](auto kernel) { kernel<<<items, kScatterThreads, 0, s>>>(b, b.swc_common, lg); };
+            const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, kScatterThreads, s, b, b.swc_common, lg); };
             const bool full = items >= 152 * kScatterBlocks;
             if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks>);          // (stateless: one system)
             else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks>);
@@ -3901,17 +3970,17 @@ static void edges_fp32(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
             else go(k_edges_s<false, false, true, kScatterBlocksFew>);
             break;
         }
-        case 1: k_edges1<float><<<ntiles * (kTile / kEdges1Threads), kEdges1Threads, 0, s>>>(b); break;
-        case 4: k_edges<float, 4><<<ntiles * 4, kTile, 0, s>>>(b); break;
-        case 8: k_edges<float, 8><<<ntiles * 8, kTile, 0, s>>>(b); break;
-        case 16: k_edges<float, 16><<<ntiles * 16, kTile, 0, s>>>(b); break;
-        default: k_edges<float, 32><<<ntiles * 32, kTile, 0, s>>>(b); break;
+        case 1: launch_next(k_edges1<float>, ntiles * (kTile / kEdges1Threads), kEdges1Threads, s, b); break;
+        case 4: launch_next(k_edges<float, 4>, ntiles * 4, kTile, s, b); break;
+        case 8: launch_next(k_edges<float, 8>, ntiles * 8, kTile, s, b); break;
+        case 16: launch_next(k_edges<float, 16>, ntiles * 16, kTile, s, b); break;
+        default: launch_next(k_edges<float, 32>, ntiles * 32, kTile, s, b); break;
     }
 }
 
 static void edges_fp64(const Bufs& b, int ntiles, cudaStream_t s) {
     const int lg = b.lg, items = ntiles << (6 - lg);
-    const auto go = [&](auto kernel) { kernel<<<items, 64, 0, s>>>(b, b.swp_common, lg); };
+    const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, 64, s, b, b.swp_common, lg); };
     if (b.want_grad) go(k_edges_d<true, true>);          // (stateless: one system)
     else if (b.common) go(k_edges_d<false, true>);
     else go(k_edges_d<false, false>);
@@ -3929,11 +3998,11 @@ void launch_edges(const Bufs& b, int precision, int lanes, int ntiles, int mode,
 template <typename T, int MODE>
 static void gather_dispatch(const Bufs& b, int lanes, int ntiles, cudaStream_t s, int fuse) {
     switch (lanes) {
-        case 0: k_finish<T, MODE><<<ntiles, kTile, 0, s>>>(b, fuse); break;
-        case 1: k_gather<T, MODE, 1><<<ntiles, kTile, 0, s>>>(b); break;
-        case 2: k_gather<T, MODE, 2><<<ntiles * 2, kTile, 0, s>>>(b); break;
-        case 8: k_gather<T, MODE, 8><<<ntiles * 8, kTile, 0, s>>>(b); break;
-        default: k_gather<T, MODE, 4><<<ntiles * 4, kTile, 0, s>>>(b); break;
+        case 0: launch_next_if(ntiles <= kEarlyBlocks, k_finish<T, MODE>, ntiles, kTile, s, b, fuse); break;
+        case 1: launch_next_if(ntiles <= kEarlyBlocks, k_gather<T, MODE, 1>, ntiles, kTile, s, b); break;
+        case 2: launch_next_if(ntiles * 2 <= kEarlyBlocks, k_gather<T, MODE, 2>, ntiles * 2, kTile, s, b); break;
+        case 8: launch_next_if(ntiles * 8 <= kEarlyBlocks, k_gather<T, MODE, 8>, ntiles * 8, kTile, s, b); break;
+        default: launch_next_if(ntiles * 4 <= kEarlyBlocks, k_gather<T, MODE, 4>, ntiles * 4, kTile, s, b); break;
     }
 }
 
@@ -3954,27 +4023,27 @@ void launch_gather(const Bufs& b, int precision, int lanes, int ntiles, int mode
 
 void launch_materialize(const Bufs& b, int precision, int ntiles, double* x, double* v, cudaStream_t s) {
     if (ntiles <= 0) return;
-    if (precision == NEFE_FP64) k_materialize<double><<<ntiles, kTile, 0, s>>>(b, x, v);
-    else k_materialize<float><<<ntiles, kTile, 0, s>>>(b, x, v);
+    if (precision == NEFE_FP64) launch_next(k_materialize<double>, ntiles, kTile, s, b, x, v);
+    else launch_next(k_materialize<float>, ntiles, kTile, s, b, x, v);
 }
 
 void launch_inject(const Bufs& b, int precision, int ntiles, const double* x, const double* v, cudaStream_t s) {
     if (ntiles <= 0) return;
-    if (precision == NEFE_FP64) k_inject<double><<<ntiles, kTile, 0, s>>>(b, x, v);
-    else k_inject<float><<<ntiles, kTile, 0, s>>>(b, x, v);
+    if (precision == NEFE_FP64) launch_next(k_inject<double>, ntiles, kTile, s, b, x, v);
+    else launch_next(k_inject<float>, ntiles, kTile, s, b, x, v);
 }
 
 void launch_group(const Bufs& b, const DevGroup* groups, int ngroups, int mode, cudaStream_t s,
                   long* launches, int carry) {
     if (ngroups <= 0) return;
-    k_group<<<ngroups, kTile, 0, s>>>(b, groups, mode, carry);
+    launch_next_if(ngroups <= kEarlyGroups, k_group, ngroups, kTile, s, b, groups, mode, carry);
     if (launches) *launches += 1;
 }
 
 void launch_noise(unsigned long long seed, unsigned long long sys_id, unsigned long long step, int n,
                   int precision, double* xi, cudaStream_t s) {
     if (n <= 0) return;
-    k_noise<<<(n + 127) / 128, 128, 0, s>>>(seed, sys_id, step, n, precision, xi);
+    launch_next(k_noise, (n + 127) / 128, 128, s, seed, sys_id, step, n, precision, xi);
 }
 
 }  // namespace nefe

@@ -64,7 +64,7 @@ struct Bufs {
     void* uf_F;              // [ntot] UF force and atom energy of the step (T4)
     const int* uf_tiles;     // tiles of the UF systems (per-step UF kernel), or NULL: every tile
     int* scan_sums;          // stateless: span sums of a multi-block cell scan (NULL: one block)
-    int ncells_host;         // stateless: number of cells of the grid
+    int ncells_host;         // number of cells of the grid (engine: of all systems at creation)
     int* lacc;               // [ntot][4] int32 force accumulators of the scatter form (2^-22 eV/A)
     int* lacc_hi;            // [ntot][4] multiples of large terms (see k_edges_s)
     SWc<float> swc_common;   // the potential constants, where every system has the same (common)
