@@ -222,7 +222,7 @@ static int run_forces(const Scratch1& S, Bufs& b, int n, const nefe_sw_params* p
     const int ntiles = (n + kTile - 1) / kTile;
     b.xc = S.xc; b.lscale = S.lscale;
     b.row4 = (b.cap & 3) == 0 && (reinterpret_cast<uintptr_t>(b.nbr) & 15) == 0;
-    b.lg = atoms_per_warp_log2(precision, n);
+    set_edge_items(b, precision, atoms_per_warp_log2(precision, n), ntiles);
     b.common = 1;
     if (precision == NEFE_FP32) {
         b.xf = S.xf; b.lacc = S.lacc; b.lacc_hi = S.lacc_hi; b.hi_flag = S.hi_flag;

@@ -170,7 +170,8 @@ void set_form(nefe_ctx* c, int lanes) {
     // (the Uhlenbeck-Ford kernel reads fractions in FP32)
     const int xf = scatter || c->prec == NEFE_FP64 || c->n_uf_tiles > 0 ? 1 : 0, xs = !scatter ? 1 : 0;
     // FP64: 8, 16, 32 lanes per atom set by hand stand for 16, 8, 4 atoms per warp
-    c->b.lg = c->prec == NEFE_FP64 && c->chosen ? (lanes <= 8 ? 4 : lanes == 16 ? 3 : 2) : atoms_per_warp_log2(c->prec, c->ntot);
+    set_edge_items(c->b, c->prec, c->prec == NEFE_FP64 && c->chosen ? (lanes <= 8 ? 4 : lanes == 16 ? 3 : 2) : atoms_per_warp_log2(c->prec, c->ntot),
+                   c->ntiles);
     if (c->b.want_xf != xf || c->b.want_xs != xs) c->stale_pos = true;
     c->b.want_xf = xf;
     c->b.want_xs = xs;
@@ -1172,7 +1173,7 @@ int nefe_autotune(nefe_ctx* c) {
             });
             scatter_us = us;
         } else {
-            b.lg = lg_of(l);
+            set_edge_items(b, c->prec, lg_of(l), c->ntiles);
             us = time_us([&] { launch_edges(b, c->prec, l, c->ntiles, FM_FORCES, c->stream, &c->launches); });
         }
         ranked_a.push_back({us, l});
@@ -1182,7 +1183,7 @@ int nefe_autotune(nefe_ctx* c) {
     cudaFree(tv0);
     cudaFree(tf0);
     std::sort(ranked_a.begin(), ranked_a.end());
-    b.lg = lg_of(best_l);
+    set_edge_items(b, c->prec, lg_of(best_l), c->ntiles);
     launch_edges(b, c->prec, best_l == 0 ? 1 : best_l, c->ntiles, FM_FORCES, c->stream, &c->launches);
     double best_g = 1e30;
     int best_gl = c->glanes;

@@ -2445,6 +2445,18 @@ __device__ __forceinline__ int3 force_of_acc(int4 q) {
 // 168 -> 155 us; 1,008,516 atoms of diamond / beta-tin pairs (12.8 edges) 345 -> 253 us; against the
 // gather form's two passes, 96,000 atoms under barostats 73 -> 42 us, 8000 atoms 13.5 -> 11.5 us.
 constexpr int kListEdges = 224;         // 32 atoms of a crystal hold 186 +- 5; smaller lists leave more L1 and warps
+constexpr int kEdgesDBlocks = 7;         // blocks of k_edges_d an SM holds (shared memory)
+// The atoms of a block of the edge-list kernels: of tile `tile`, from atom `first` on, 2^lg to a warp.
+// Tiles from b.tail_tile on are cut finer (2^lg_tail): see set_edge_items.
+struct EdgeItem {
+    int lg, tile, first;
+};
+__device__ __forceinline__ EdgeItem edge_item(const Bufs& b) {
+    const int big = max(0, b.tail_tile - b.tile_base), nbig = big << (6 - b.lg);
+    const bool tail = (int)blockIdx.x >= nbig;
+    const int lg = tail ? b.lg_tail : b.lg, item = (int)blockIdx.x - (tail ? nbig : 0);
+    return {lg, b.tile_base + (tail ? big : 0) + (item >> (6 - lg)), (item & ((64 >> lg) - 1)) << (lg + 1)};
+}
 constexpr int kScatterThreads = 64;
 // Resident blocks per SM the registers are bounded for: 14 where the launch fills them (crystal 154.7
 // us, 12: 159.6), else as many registers as the kernel wants (12 blocks' worth: 6.8 against 7.4 us for
@@ -2627,22 +2639,22 @@ __device__ __forceinline__ void mark_row(const Bufs& b, int i, int part, int lpa
 // the constant bank, no loads: 171 -> 155 us on the crystal); otherwise they are read from the table.
 template <bool EATOM, bool GRAD, bool COMMON, int BLOCKS>
 __global__ void __launch_bounds__(kScatterThreads, BLOCKS)
-k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc, int lg) {
+k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc) {
     dep_wait();
     constexpr unsigned kAll = 0xffffffffu;
-    const int G = 1 << lg, lpa = 5 - lg;
+    const EdgeItem it = edge_item(b);
+    const int lg = it.lg, G = 1 << lg, lpa = 5 - lg;
     __shared__ ScatterShared<EATOM> shm[kScatterThreads / 32];
     ScatterShared<EATOM>& sh = shm[threadIdx.x >> 5];
     static_assert(kScatterThreads == 64 && kTile == 128, "two warps of 2^lg atoms a block");
-    const int item = (int)blockIdx.x, tile = (item >> (6 - lg)) + b.tile_base;
-    const TileAtom ta = tile_of(b, tile);
+    const TileAtom ta = tile_of(b, it.tile);
     const DevSys& S = b.sys[ta.sys];
     DevState& st = b.st[ta.sys];
     if (S.pot != POT_SW) return;                 // uniform over the block
     const SWc<float>& P = COMMON ? Pc : reinterpret_cast<const SWc<float>*>(b.swc)[S.prm];
     const int lane = threadIdx.x & 31, t = lane & (G - 1);
     const unsigned below = (1u << lane) - 1u;
-    const int ia = ((item & ((64 >> lg) - 1)) << (lg + 1)) + ((int)(threadIdx.x >> 5) << lg) + t;   // of the tile
+    const int ia = it.first + ((int)(threadIdx.x >> 5) << lg) + t;   // of the tile
     const int i = ta.first + ia;
     const bool valid = ia < ta.count;
     // L 2^-32 to twice the precision: a relative error of L alone would be a uniform strain of up to
@@ -2838,21 +2850,21 @@ struct __align__(16) EdgesDShared {
 };
 template <bool GRAD, bool COMMON>
 __global__ void __launch_bounds__(64)
-k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc, int lg) {
+k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc) {
     dep_wait();
     constexpr unsigned kAll = 0xffffffffu;
     __shared__ EdgesDShared shm[2];
     EdgesDShared& sh = shm[threadIdx.x >> 5];
-    const int G = 1 << lg, lpa = 5 - lg;
-    const int item = (int)blockIdx.x, tile = (item >> (6 - lg)) + b.tile_base;
-    const TileAtom ta = tile_of(b, tile);
+    const EdgeItem it = edge_item(b);
+    const int lg = it.lg, G = 1 << lg, lpa = 5 - lg;
+    const TileAtom ta = tile_of(b, it.tile);
     const DevSys& S = b.sys[ta.sys];
     DevState& st = b.st[ta.sys];
     if (S.pot != POT_SW) return;                 // uniform over the block
     const SWp<double>& P = COMMON ? Pc : reinterpret_cast<const SWp<double>*>(b.swc)[S.prm];
     const int lane = threadIdx.x & 31, t = lane & (G - 1);
     const unsigned below = (1u << lane) - 1u;
-    const int ia = ((item & ((64 >> lg) - 1)) << (lg + 1)) + ((int)(threadIdx.x >> 5) << lg) + t;   // of the tile
+    const int ia = it.first + ((int)(threadIdx.x >> 5) << lg) + t;   // of the tile
     const int i = ta.first + ia;
     const bool valid = ia < ta.count;
     const double hx = st.h[0], hy = st.h[1], hz = st.h[2];
@@ -3957,11 +3969,28 @@ int atoms_per_warp_log2(int precision, int ntot) {
     return ntot >= 32 * 152 * 8 ? 5 : ntot >= 16 * 152 * 8 ? 4 : 3;
 }
 
+// The last quarter of what the chip holds at once is cut into blocks of half the size, where there is
+// more than that to do: the launch ends on the SMs that drew the last blocks.  192,000 atoms 44.1 ->
+// 41.8 us, 512,000 304.8 -> 297.0, 1,024,000 192.6 -> 190.8, 128,000 in FP64 448 -> 440; a larger share or
+// quarter-size blocks give less, their lists being shorter, and just above one filling (136,000 atoms)
+// it costs 5 %.
+void set_edge_items(Bufs& b, int precision, int lg, int ntiles) {
+    const int resident = 152 * (precision == NEFE_FP64 ? kEdgesDBlocks : kScatterBlocks);
+    const bool cut = (long long)ntiles << (6 - lg) > resident + resident / 4;
+    b.lg = lg;
+    b.lg_tail = max(2, lg - 1);
+    b.tail_tile = cut ? ntiles - (resident / 4 >> (6 - lg)) : ntiles;
+}
+static int edge_items(const Bufs& b, int ntiles) {
+    const int big = max(0, min(b.tail_tile - b.tile_base, ntiles));
+    return (big << (6 - b.lg)) + ((ntiles - big) << (6 - b.lg_tail));
+}
+
 static void edges_fp32(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
     switch (lanes) {
         case 0: {
-            const int lg = b.lg, items = ntiles << (6 - lg);
-            const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, kScatterThreads, s, b, b.swc_common, lg); };
+            const int items = edge_items(b, ntiles);
+            const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, kScatterThreads, s, b, b.swc_common); };
             const bool full = items >= 152 * kScatterBlocks;
             if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks>);          // (stateless: one system)
             else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks>);
@@ -3979,8 +4008,8 @@ static void edges_fp32(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
 }
 
 static void edges_fp64(const Bufs& b, int ntiles, cudaStream_t s) {
-    const int lg = b.lg, items = ntiles << (6 - lg);
-    const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, 64, s, b, b.swp_common, lg); };
+    const int items = edge_items(b, ntiles);
+    const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, 64, s, b, b.swp_common); };
     if (b.want_grad) go(k_edges_d<true, true>);          // (stateless: one system)
     else if (b.common) go(k_edges_d<false, true>);
     else go(k_edges_d<false, false>);

@@ -70,6 +70,7 @@ struct Bufs {
     SWc<float> swc_common;   // the potential constants, where every system has the same (common)
     SWp<double> swp_common;
     int lg;                  // atoms per warp of the edge-list kernels, as a power of two
+    int lg_tail, tail_tile;  // the same from tile tail_tile on (set_edge_items)
     int common;
     int leg_refuse;          // the scatter form was chosen by the caller: terms above its limit are refused
     int* hi_flag;            // [tiles] some large term was split this step (cleared by k_finish)
@@ -112,6 +113,7 @@ void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, cudaStre
 // mode FM_FORCES writes b.f_out / b.e_atom (stateless), otherwise b.uf_F for pass B.
 void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches);
 int atoms_per_warp_log2(int precision, int ntot);
+void set_edge_items(Bufs& b, int precision, int lg, int ntiles);
 // Force pass A (edges: pair terms, triplets centred on each atom, leg forces per edge).
 void launch_edges(const Bufs& b, int precision, int lanes, int ntiles, int mode, cudaStream_t s,
                   long* launches);

@@ -355,3 +355,30 @@ def test_uf_rows_and_sums_by_lanes(N, n, cells, precision, tol):
     assert np.abs(ea.cpu().numpy() - ea_o).max() <= tol * np.abs(ea_o).max()
     assert abs(float(ev[0]) - e_o) <= tol * np.abs(ea_o).sum()
     assert np.abs(ev[1:].cpu().numpy() - vir_o).max() <= 10 * tol * np.abs(vir_o).max()
+
+
+# ------------------------------------------------------------------ finer blocks at the end
+@pytest.mark.parametrize("precision,tol,copies", [(1, 1e-10, (2, 1, 1)), (1, 1e-10, (3, 2, 2)), (0, 1e-5, (5, 2, 4)),
+                                                  (0, 1e-5, (4, 4, 3))])
+def test_forces_where_the_last_blocks_are_cut_finer(N, precision, tol, copies):
+    """Sizes below and above the ones from which the last tiles are cut finer: a rattled crystal repeated
+    in space has the forces, energies and virial of one copy (the FP64 ones of 4096 atoms), normwise."""
+    x1, box1 = I.diamond(8, 8, 8)
+    x1 = I.rattle(x1, 0.1, 4)
+    _, f1, v1, e1 = O.sw_energy(x1, box1)
+    m = int(np.prod(copies))
+    shift = np.stack(np.meshgrid(*[np.arange(c) for c in copies], indexing="ij"), -1).reshape(-1, 1, 3) * box1
+    x, box, n = (x1[None] + shift).reshape(-1, 3), box1 * np.array(copies), m * len(x1)
+    xd = soa(x)
+    nbr = torch.zeros(n * 48, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+    N.nefe_neighbor_build(xd, n, box, RC + 0.5, 48, nbr, cnt)
+    f, e = torch.zeros(3 * n, dtype=torch.float64, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda")
+    ev = torch.zeros(7, dtype=torch.float64, device="cuda")
+    N.nefe_sw_forces(xd, n, box, RC + 0.5, nbr, cnt, 48, N.nefe_sw_params_silicon(), precision, f, e, ev)
+    torch.cuda.synchronize()
+    f, e, ev = f.cpu().numpy().reshape(3, n).T.reshape(m, -1, 3), e.cpu().numpy().reshape(m, -1), ev.cpu().numpy()
+    assert np.abs(f - f1).max() <= tol * np.abs(f1).max()
+    assert np.abs(e - e1).max() <= tol * np.abs(e1).max()
+    assert abs(ev[0] / m - e1.sum()) <= tol * np.abs(e1).sum()
+    assert np.abs(ev[1:] / m - v1).max() <= 10 * tol * np.abs(v1).max()
