@@ -65,7 +65,7 @@ struct nefe_ctx {
     int4* d_tiles = nullptr;
     double *d_x = nullptr, *d_r0 = nullptr, *d_ftmp = nullptr, *d_vtmp = nullptr;
     void *d_v = nullptr, *d_dhi = nullptr, *d_dlo = nullptr;
-    void *d_F = nullptr, *d_xs = nullptr, *d_xa = nullptr, *d_xcs = nullptr, *d_sd0 = nullptr, *d_xi = nullptr;
+    void *d_F = nullptr, *d_xs = nullptr, *d_xa = nullptr, *d_xcs = nullptr, *d_sd0 = nullptr, *d_xi = nullptr, *d_xi_next = nullptr;
     void *d_shd = nullptr, *d_P = nullptr, *d_spill = nullptr;
     int *d_shj = nullptr, *d_shn = nullptr, *d_rtiles = nullptr, *d_rcount = nullptr, *d_rcbase = nullptr;
     int* d_any = nullptr;    // context-wide rebuild flag words (Bufs::any_rebuild)
@@ -181,12 +181,14 @@ void set_form(nefe_ctx* c, int lanes) {
 // Both force passes, chunk by chunk; with slot >= 0 (profiling capture) events bracket
 // every chunk's pass A and pass B.  fuse: the scatter form's epilogue also runs the next
 // step's kick and drift for the systems without a barostat.
-void enqueue_forces(nefe_ctx* c, int mode, int slot = -1, int fuse = 0) {
+// ahead: FP64 pass A also draws the next step's noise.
+void enqueue_forces(nefe_ctx* c, int mode, int slot = -1, int fuse = 0, bool ahead = false) {
     if (c->n_uf_tiles > 0) launch_uf(c->b, c->prec, c->n_uf_tiles, mode, c->stream, &c->launches);
     const int nch = (int)c->chunk_tile0.size();
     for (int k = 0; k < nch; ++k) {
         Bufs b = c->b;
         b.tile_base = c->chunk_tile0[k];
+        b.noise_ahead = ahead ? 1 : 0;
         const int e = slot >= 0 ? slot * nch + k : -1;
         const bool prof = e >= 0 && e < (int)c->ev0.size();
         if (prof) cudaEventRecordWithFlags(c->ev0[e], c->stream, cudaEventRecordExternal);
@@ -206,10 +208,11 @@ void enqueue_forces(nefe_ctx* c, int mode, int slot = -1, int fuse = 0) {
 void enqueue_step(nefe_ctx* c, int slot = -1, bool first = true, bool last = true) {
     NvtxRange nvtx_("nefe step");
     const bool fused = c->lanes == 0;            // k_finish is the epilogue
+    const bool draws = c->d_xi_next && c->chunk_tile0.size() == 1;
     launch_group(c->b, c->d_groups, c->ngroups, 1, c->stream, &c->launches, fused && !first);
     // with every system moved by the previous epilogue there is nothing left for k_kick_drift
     if (!(fused && !first && !c->any_baro))
-        launch_kick_drift(c->b, c->prec, c->ntiles, 1, c->stream, &c->launches, fused && !first);
+        launch_kick_drift(c->b, c->prec, c->ntiles, 1, c->stream, &c->launches, fused && !first, draws && !first);
     // the rebuild: one cooperative launch (worklist, cells, lists between grid barriers), or the
     // kernel sequence where the list build has lanes per atom or UF rows are built too
     if (c->coop && c->coop_blocks > 0 && c->llanes == 0 && c->n_uf_tiles == 0) {
@@ -218,7 +221,7 @@ void enqueue_step(nefe_ctx* c, int slot = -1, bool first = true, bool last = tru
         launch_cells_and_list(c->b, c->prec, c->ntiles, c->nsys, 0, c->stream, &c->launches);
         if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->nsys, c->stream, &c->launches);
     }
-    enqueue_forces(c, FM_STEP, slot, fused && !last);
+    enqueue_forces(c, FM_STEP, slot, fused && !last, draws && !last);
 }
 
 void fill_results(const DevSys& S, const DevState& st, nefe_results* out) {
@@ -442,6 +445,7 @@ int setup(nefe_ctx* c) {
     if ((rc = dalloc(c, &c->d_xcs, v4 * N))) return rc;
     if ((rc = dalloc(c, &c->d_sd0, v4 * N))) return rc;
     if ((rc = dalloc(c, &c->d_xi, v4 * N))) return rc;
+    if (c->prec == NEFE_FP64 && c->ntiles < 152 && (rc = dalloc(c, &c->d_xi_next, v4 * N))) return rc;   // (draw_ahead)
     if ((rc = dalloc(c, &c->d_shd, v4 * N * (size_t)kShell))) return rc;
     // spill area of the thread-per-atom pass A (FP32 only): the last kSpill1 entries of a shell
     if (c->prec == NEFE_FP32 && (rc = dalloc(c, &c->d_spill, (v4 + sizeof(float)) * N * kSpill1))) return rc;
@@ -541,7 +545,7 @@ int setup(nefe_ctx* c) {
     std::memset(&b, 0, sizeof(b));
     b.sys = c->d_sys; b.st = c->d_st; b.acc = c->d_acc; b.tiles = c->d_tiles;
     b.x = c->d_x; b.v = c->d_v; b.dhi = c->d_dhi; b.dlo = c->d_dlo; b.r0 = c->d_r0; b.F = c->d_F;
-    b.xs = c->d_xs; b.xa = c->d_xa; b.xcs = c->d_xcs; b.sd0 = c->d_sd0; b.xi = c->d_xi;
+    b.xs = c->d_xs; b.xa = c->d_xa; b.xcs = c->d_xcs; b.sd0 = c->d_sd0; b.xi = c->d_xi; b.xi_next = c->d_xi_next;
     b.shd = c->d_shd; b.shj = c->d_shj; b.shn = c->d_shn; b.P = c->d_P; b.spill = c->d_spill;
     b.rtiles = c->d_rtiles; b.rcount = c->d_rcount; b.rcbase = c->d_rcbase; b.any_rebuild = c->d_any;
     b.q = c->d_q; b.cell_of = c->d_cell_of; b.perm = c->d_perm; b.cell_start = c->d_cell_start;

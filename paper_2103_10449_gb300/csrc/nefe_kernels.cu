@@ -123,16 +123,18 @@ template <> struct Noise<double> {
     __device__ static void xi3(uint64_t seed, uint64_t sys, uint64_t step, uint64_t id, double out[3]) {
         uint64_t c[4] = {step, id, sys, 0ULL};
         philox4x64_10(c, seed, 0ULL);
-        const double u0 = ((double)(c[0] >> 11) + 0.5) * 0x1p-53;
-        const double u1 = ((double)(c[1] >> 11) + 0.5) * 0x1p-53;
-        const double u2 = ((double)(c[2] >> 11) + 0.5) * 0x1p-53;
-        const double u3 = ((double)(c[3] >> 11) + 0.5) * 0x1p-53;
-        const double two_pi = 6.283185307179586476925286766559;
-        const double r0 = ::sqrt(-2.0 * ::log(u0)), r1 = ::sqrt(-2.0 * ::log(u2));
-        double s0, c0, s1, c1;
-        ::sincos(two_pi * u1, &s0, &c0);
-        ::sincos(two_pi * u3, &s1, &c1);
-        out[0] = r0 * c0; out[1] = r0 * s0; out[2] = r1 * c1;
+        double unused;
+        pair(c[0], c[1], out[0], out[1]);
+        pair(c[2], c[3], out[2], unused);
+    }
+    // Box-Muller pair of two words
+    __device__ __forceinline__ static void pair(uint64_t c0, uint64_t c1, double& a, double& b) {
+        const double u0 = ((double)(c0 >> 11) + 0.5) * 0x1p-53, u1 = ((double)(c1 >> 11) + 0.5) * 0x1p-53;
+        const double r = ::sqrt(__dmul_rn(-2.0, ::log(u0)));
+        double sn, cs;
+        ::sincospi(2.0 * u1, &sn, &cs);
+        a = __dmul_rn(r, cs);
+        b = __dmul_rn(r, sn);
     }
 };
 template <> struct Noise<float> {
@@ -1866,7 +1868,8 @@ template <typename T>
 __device__ __forceinline__ void drift_atom(const Bufs& b, const DevSys& S, const DevState& st, const BoxMove& bm, int i,
                                            const typename V4<T>::t& xa, const int4& fb, const T (&vk)[3], bool move,
                                            T (&dh)[3], T (&dl)[3], int flag_set, int* flag, int* any,
-                                           unsigned long long kstep, T (&z)[3]) {
+                                           unsigned long long kstep, T (&z)[3],
+                                           const typename V4<T>::t* drawn = nullptr) {
     using T4 = typename V4<T>::t;
     const size_t N = b.ntot;
     T* DH = reinterpret_cast<T*>(b.dhi);
@@ -1897,7 +1900,11 @@ __device__ __forceinline__ void drift_atom(const Bufs& b, const DevSys& S, const
     }
     z[0] = z[1] = z[2] = (T)0;
     if (S.thermo) {
-        Noise<T>::xi3(S.seed, (uint64_t)S.rng_id, (uint64_t)kstep, (uint64_t)(i - S.off), z);
+        if (drawn) {
+            z[0] = drawn->x; z[1] = drawn->y; z[2] = drawn->z;
+        } else {
+            Noise<T>::xi3(S.seed, (uint64_t)S.rng_id, (uint64_t)kstep, (uint64_t)(i - S.off), z);
+        }
         reinterpret_cast<T4*>(b.xi)[i] = mk4(z[0], z[1], z[2], (T)0);
     }
 }
@@ -1934,10 +1941,11 @@ __global__ void __launch_bounds__(kTile) k_positions(Bufs b) {
     place_atom<T>(b, st, bm, i, reinterpret_cast<const T4*>(b.xa)[i], fb, b.q[i], d);
 }
 
+// drawn: the step's noise is in xi_next (draw_ahead).
 // skip: systems without a barostat were already kicked and moved by the previous step's
 // epilogue (k_finish with fuse), so their tiles return at once.
 template <typename T>
-__global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip) {
+__global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip, int drawn) {
     dep_wait();
     using T4 = typename V4<T>::t;
     const TileAtom ta = tile_of(b, blockIdx.x);
@@ -1971,7 +1979,7 @@ __global__ void __launch_bounds__(kTile) k_kick_drift(Bufs b, int mode, int skip
         }
         drift_atom<T>(b, S, st, bm, i, xa, fb, vk, mode == 1, dh, dl, st.rebuild, &st.rebuild, b.any_rebuild,
                       (unsigned long long)st.k,
-                      xs_sum);
+                      xs_sum, drawn ? reinterpret_cast<const T4*>(b.xi_next) + i : nullptr);
     }
     block_sum_to_acc<T, 3>(xs_sum, b.acc + (size_t)ta.sys * ACC_N * kSlots, ACC_XI, &st.err);
 }
@@ -2848,6 +2856,24 @@ struct __align__(16) EdgesDShared {
     unsigned short slot[kListEdgesD];   // cell-offset code << 8 | shell slot
     double mom[10][32];
 };
+// The next step's thermostat noise of 32 atoms (a quarter of a tile, one warp per Box-Muller pair) into
+// xi_next, by blocks of pass A beyond the edges' own.  It depends on the step and the atom only, and in
+// a small context it is the longest part of k_kick_drift (a chain of FP64 logarithm, root and sine, on as
+// many SMs as there are tiles) while most SMs have no block of pass A: 64 atoms, k_kick_drift 10.0 us a
+// step, the step 48.0 -> 43.1 us.  From 152 tiles on k_kick_drift fills the chip by itself.
+__device__ __forceinline__ void draw_ahead(const Bufs& b, int item) {
+    const TileAtom ta = tile_of(b, item >> 2);
+    const DevSys& S = b.sys[ta.sys];
+    const int ia = (item & 3) * 32 + (int)(threadIdx.x & 31), half = (int)(threadIdx.x >> 5);
+    if (!S.thermo || ia >= ta.count) return;
+    const int i = ta.first + ia;
+    uint64_t c[4] = {(uint64_t)b.st[ta.sys].k + 1, (uint64_t)(i - S.off), (uint64_t)S.rng_id, 0ULL};
+    philox4x64_10(c, S.seed, 0ULL);
+    double z0, z1;
+    Noise<double>::pair(half ? c[2] : c[0], half ? c[3] : c[1], z0, z1);
+    reinterpret_cast<double2*>(b.xi_next)[2 * (size_t)i + half] = make_double2(z0, half ? 0.0 : z1);
+}
+
 template <bool GRAD, bool COMMON>
 __global__ void __launch_bounds__(64)
 k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc) {
@@ -2855,6 +2881,10 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
     constexpr unsigned kAll = 0xffffffffu;
     __shared__ EdgesDShared shm[2];
     EdgesDShared& sh = shm[threadIdx.x >> 5];
+    if (b.noise_first >= 0 && (int)blockIdx.x >= b.noise_first) {
+        draw_ahead(b, (int)blockIdx.x - b.noise_first);
+        return;
+    }
     const EdgeItem it = edge_item(b);
     const int lg = it.lg, G = 1 << lg, lpa = 5 - lg;
     const TileAtom ta = tile_of(b, it.tile);
@@ -3923,10 +3953,10 @@ void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t 
 }
 
 void launch_kick_drift(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches,
-                       int skip) {
+                       int skip, int drawn) {
     if (ntiles <= 0) return;
-    if (precision == NEFE_FP64) launch_next(k_kick_drift<double>, ntiles, kTile, s, b, mode, skip);
-    else launch_next(k_kick_drift<float>, ntiles, kTile, s, b, mode, skip);
+    if (precision == NEFE_FP64) launch_next(k_kick_drift<double>, ntiles, kTile, s, b, mode, skip, drawn);
+    else launch_next(k_kick_drift<float>, ntiles, kTile, s, b, mode, skip, 0);
     if (launches) *launches += 1;
 }
 
@@ -4009,7 +4039,10 @@ static void edges_fp32(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
 
 static void edges_fp64(const Bufs& b, int ntiles, cudaStream_t s) {
     const int items = edge_items(b, ntiles);
-    const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, 64, s, b, b.swp_common); };
+    Bufs bn = b;
+    bn.noise_first = b.noise_ahead ? items : -1;
+    const int blocks = items + (b.noise_ahead ? 4 * ntiles : 0);
+    const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || blocks <= kEarlyBlocks, kernel, blocks, 64, s, bn, b.swp_common); };
     if (b.want_grad) go(k_edges_d<true, true>);          // (stateless: one system)
     else if (b.common) go(k_edges_d<false, true>);
     else go(k_edges_d<false, false>);

@@ -70,6 +70,8 @@ struct Bufs {
     SWc<float> swc_common;   // the potential constants, where every system has the same (common)
     SWp<double> swp_common;
     int lg;                  // atoms per warp of the edge-list kernels, as a power of two
+    void* xi_next;           // FP64: noise drawn ahead by pass A (noise_ahead), 4 doubles per atom, or NULL
+    int noise_ahead, noise_first;   // draw it in this launch; first block that does (-1: none)
     int lg_tail, tail_tile;  // the same from tile tail_tile on (set_edge_items)
     int common;
     int leg_refuse;          // the scatter form was chosen by the caller: terms above its limit are refused
@@ -105,7 +107,7 @@ void launch_cells_and_list(const Bufs& b, int precision, int ntiles, int nsys, i
 // Half kick + drift + mirror + displacement check + noise sums (mode 0: no kick/drift).  skip:
 // the systems without a barostat were moved by the previous step's fused epilogue.
 void launch_kick_drift(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s,
-                       long* launches, int skip = 0);
+                       long* launches, int skip = 0, int drawn = 0);
 // Uhlenbeck-Ford pair rows of the UF systems (after the cell fill; flagged systems only when a
 // rebuild worklist is set).
 void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, cudaStream_t s, long* launches);

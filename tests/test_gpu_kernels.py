@@ -357,7 +357,34 @@ def test_uf_rows_and_sums_by_lanes(N, n, cells, precision, tol):
     assert np.abs(ev[1:].cpu().numpy() - vir_o).max() <= 10 * tol * np.abs(vir_o).max()
 
 
-# ------------------------------------------------------------------ finer blocks at the end
+# ------------------------------------------------------------------ noise drawn ahead, finer blocks at the end
+@pytest.mark.parametrize("baro", [False, True])
+@pytest.mark.parametrize("shapes", [((2, 2, 2), (3, 3, 3)), ((2, 2, 2), (12, 12, 11)), ((14, 14, 13),)])
+def test_noise_drawn_by_the_previous_step(N, shapes, baro):
+    """FP64 contexts below and above the size where pass A draws the next step's noise (152 tiles), of
+    part-filled tiles, with a system without a thermostat and with a box that moves: 23 steps in one
+    call, in calls of 1 to 7 steps (whose first step draws its own) and captured, bit for bit."""
+    got = []
+    for parts in ((23,), (1, 1, 5, 7, 2, 7), (16, 7)):
+        ctx = N.Context(precision=N.NEFE_FP64, skin=0.6, nbr_cap=48)
+        for r, shape in enumerate(shapes):
+            x, box = I.diamond(*shape)
+            s = ctx.add_system(x, box, v=I.gaussian_velocities(len(x), 4.0, 70 + r))
+            ctx.set_thermostat(s, 800.0, 0.1, 80 + r)
+            if baro:
+                ctx.set_barostat(s, N.NEFE_BARO_ISO, 0.0, 0.5)
+        x, box = I.diamond(2, 2, 2)
+        ctx.add_system(x, box, v=I.gaussian_velocities(len(x), 4.0, 79))
+        for k in parts:
+            ctx.run(k)
+        got.append([ctx.get_state(s) for s in range(len(shapes) + 1)])
+        assert all(ctx.results(s)["error"] == 0 for s in range(len(shapes) + 1))
+        ctx.close()
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert all(np.array_equal(u, v) for u, v in zip(a, b))
+
+
 @pytest.mark.parametrize("precision,tol,copies", [(1, 1e-10, (2, 1, 1)), (1, 1e-10, (3, 2, 2)), (0, 1e-5, (5, 2, 4)),
                                                   (0, 1e-5, (4, 4, 3))])
 def test_forces_where_the_last_blocks_are_cut_finer(N, precision, tol, copies):
