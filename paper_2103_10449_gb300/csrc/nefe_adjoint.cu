@@ -864,7 +864,6 @@ int nefe_adjoint_create(nefe_adj** out, int device, void* stream, const nefe_adj
     if (rc) return rc;
     int n3[3];
     if (!host_grid(d->box, rcs, n3)) return fail(NEFE_EINVAL, "nefe_adjoint_create: fewer than 2 cells on an axis");
-    const long long total = (long long)n3[0] * n3[1] * n3[2];
     nefe_adj* A = new nefe_adj();
     A->device = device;
     A->s = (cudaStream_t)stream;

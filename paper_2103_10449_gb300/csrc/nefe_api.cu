@@ -428,7 +428,7 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
         b.f_out = f; b.e_atom = e_atom;
         const int ntiles = (n + kTile - 1) / kTile;
         launch_cells(b, precision, ntiles, 1, 1, S.s, nullptr);
-        launch_uf_list(b, precision, ntiles, 1, S.s, nullptr);
+        launch_uf_list(b, precision, ntiles, 1, 1, S.s, nullptr);
         launch_uf(b, precision, ntiles, FM_FORCES, S.s, nullptr);
         NEFE_CU(cudaGetLastError());
     }

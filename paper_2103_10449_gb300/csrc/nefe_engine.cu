@@ -219,7 +219,7 @@ void enqueue_step(nefe_ctx* c, int slot = -1, bool first = true, bool last = tru
         launch_rebuild_coop(c->b, c->prec, c->coop_blocks, c->nsys, c->stream, &c->launches);
     } else {
         launch_cells_and_list(c->b, c->prec, c->ntiles, c->nsys, 0, c->stream, &c->launches);
-        if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->nsys, c->stream, &c->launches);
+        if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->nsys, 0, c->stream, &c->launches);
     }
     enqueue_forces(c, FM_STEP, slot, fused && !last, draws && !last);
 }
@@ -261,7 +261,7 @@ int resetup(nefe_ctx* c) {
         NEFE_CU(cudaMemsetAsync(c->d_hi_flag, 0, sizeof(int) * (size_t)c->ntiles, c->stream));
     }
     launch_cells_and_list(c->b, c->prec, c->ntiles, c->nsys, 1, c->stream, &c->launches);
-    if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->nsys, c->stream, &c->launches);
+    if (c->n_uf_tiles > 0) launch_uf_list(c->b, c->prec, c->ntiles, c->nsys, 1, c->stream, &c->launches);
     launch_kick_drift(c->b, c->prec, c->ntiles, 0, c->stream, &c->launches);
     enqueue_forces(c, FM_SETUP);
     c->stale_pos = false;
@@ -553,6 +553,7 @@ int setup(nefe_ctx* c) {
     b.cap = c->cap; b.ntot = c->ntot; b.dt = c->dt; b.swc = c->d_swc; b.pairs = c->d_pairs;
     b.nbr_il = (c->cap & 3) == 0 ? 1 : 0;   // interleaved rows (the force passes read them 4 at a time)
     b.rebuild_all = c->rebuild_all;
+    b.by_flag = cells_by_flag(nsys, c->ntiles);
     b.ncells_host = (int)std::min<long long>(ncell_now, 1 << 30);
 
     b.trace = c->d_trace;

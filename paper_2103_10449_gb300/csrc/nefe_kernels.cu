@@ -6,18 +6,23 @@
 //                 left point), applies the dCCI update (Eqs. Ps_coex_discreted /
 //                 l_coex_discreted), sets this step's drift factors and zeroes the sums.
 //   k_kick_drift  v += dt/2 F/m; displacement since the last list build += dt phi v (+ the
-//                 affine box drift), kept as a compensated pair in the FP32 path; mirror
-//                 xs = x - q h; displacement test -> rebuild flag; thermostat noise + its sum.
+//                 affine box drift), kept as a compensated pair in the FP32 path; position as
+//                 the force pass in use reads it (fractions of the box, packed fractions for the
+//                 row filter, mirror xs = x - q h); displacement test -> rebuild flag;
+//                 thermostat noise + its sum.
 //                 In the scatter form this work is done by the previous step's epilogue for the
 //                 systems without a barostat (k_finish with fuse), and the kernel skips them.
 //   rebuild       (flagged systems) fold the displacement into the FP64 anchor, cell count ->
-//                 scan -> fill (with a cell-ordered copy of the mirror) -> Verlet list; as a
-//                 kernel sequence, or as one cooperative launch (k_rebuild_coop).
+//                 scan -> fill (with a cell-ordered copy of the mirror) -> Verlet list: a cluster
+//                 of blocks per system up to the fill (k_cells_clusters, few small systems), or a
+//                 kernel sequence over a worklist, or one cooperative launch (k_rebuild_coop).
+//                 Uhlenbeck-Ford rows (k_uflist) by the same cells.
 //   k_edges_s     force pass A of the scatter form (the FP32 default): the edges of a warp's atoms
 //                 as one list, pair terms, the shells' moments and the force each atom's terms
 //                 exert on each leg atom, added into int32 fixed-point accumulators (order
-//                 independent).  k_edges1, k_edges: the gather form with one thread or a lane
-//                 group per atom (and the FP64 path), storing per edge.
+//                 independent).  k_edges1, k_edges: the FP32 gather form with one thread or a
+//                 lane group per atom, storing per edge.  k_edges_d: FP64, edge lists of a warp's
+//                 atoms, storing per edge.  k_uf: Uhlenbeck-Ford forces, several lanes per atom.
 //   k_finish      the scatter form's epilogue: reads and clears the accumulators; Einstein
 //                 springs, lambda mixing, Langevin force with its per-system mean removed,
 //                 second half kick (and the next step's kick, drift and noise, see above).
@@ -409,13 +414,13 @@ __device__ __forceinline__ void scale_of_box(const Bufs& b, int s, const DevStat
 // state (on the host for the stateless calls, by k_rebuild_list in the engine).
 // ------------------------------------------------------------------------------------
 template <typename T>
-__device__ void cells_count_tile(const Bufs& b, int tile) {
+__device__ void cells_count_tile(const Bufs& b, int tile, int th) {
     using T4 = typename V4<T>::t;
     const TileAtom ta = tile_of(b, tile);
     const DevSys& S = b.sys[ta.sys];
     const DevState& st = b.st[ta.sys];
-    if ((int)threadIdx.x >= ta.count) return;
-    const int i = ta.first + threadIdx.x;
+    if (th >= ta.count) return;
+    const int i = ta.first + th;
     const size_t N = b.ntot;
     int c3[3], qv[3];
     double xm[3], sd[3] = {0.0, 0.0, 0.0};
@@ -431,7 +436,7 @@ __device__ void cells_count_tile(const Bufs& b, int tile) {
             if (b.dlo) dl[k * N + i] = (T)0;
         }
         cell_axis(xk, st.box[k], st.ibox[k] * (double)st.ncell[k], st.ncell[k], qv[k], c3[k]);
-        xm[k] = xk - (double)qv[k] * st.h[k];
+        xm[k] = __fma_rn(-(double)qv[k], st.h[k], xk);   // (written out: the same in every kernel that builds)
         if (b.r0) sd[k] = xk - b.r0[k * N + i];
     }
     const int cell = c3[0] + st.ncell[0] * (c3[1] + st.ncell[1] * c3[2]);
@@ -471,7 +476,28 @@ __device__ void cells_count_tile(const Bufs& b, int tile) {
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_cells_count(Bufs b) {
     dep_wait();
-    NEFE_FOR_TILES(b, cells_count_tile<T>(b, tile));
+    NEFE_FOR_TILES(b, cells_count_tile<T>(b, tile, threadIdx.x));
+}
+
+// The cell grid of a system about to be rebuilt, at its current box.
+__device__ __forceinline__ void set_cell_grid(const DevSys& S, DevState& st) {
+    const double bx[3] = {st.box[0], st.box[1], st.box[2]};
+    const bool same = st.grcs == S.rcs && st.gbox[0] == bx[0] && st.gbox[1] == bx[1] &&
+                      st.gbox[2] == bx[2];
+    if (!same) {
+        int g3[3];
+        const bool ok = grid_for(bx, S.rcs, S.ncell_cap, g3);
+        for (int k = 0; k < 3; ++k) {
+            st.ncell[k] = g3[k];
+            st.h[k] = __ddiv_rn(bx[k], (double)g3[k]);
+            st.hb[k] = st.h[k];
+            st.ibox[k] = __ddiv_rn(1.0, bx[k]);
+            st.gbox[k] = bx[k];
+        }
+        st.grcs = S.rcs;
+        refresh_box_f(st);
+        if (!ok) atomicOr(&st.err, NEFE_ERR_BOX);
+    }
 }
 
 // Worklist of the tiles of every system whose rebuild flag is set (all with force_all), and the
@@ -509,23 +535,7 @@ __device__ void build_worklist(const Bufs& b, int nsys, int force_all) {
             const DevSys& S = b.sys[s];
             const int base = atomicAdd(&cnt, S.ntile);
             for (int t = 0; t < S.ntile; ++t) b.rtiles[base + t] = S.tile0 + t;
-            const double bx[3] = {st.box[0], st.box[1], st.box[2]};
-            const bool same = st.grcs == S.rcs && st.gbox[0] == bx[0] && st.gbox[1] == bx[1] &&
-                              st.gbox[2] == bx[2];
-            if (!same) {
-                int g3[3];
-                const bool ok = grid_for(bx, S.rcs, S.ncell_cap, g3);
-                for (int k = 0; k < 3; ++k) {
-                    st.ncell[k] = g3[k];
-                    st.h[k] = __ddiv_rn(bx[k], (double)g3[k]);
-                    st.hb[k] = st.h[k];
-                    st.ibox[k] = __ddiv_rn(1.0, bx[k]);
-                    st.gbox[k] = bx[k];
-                }
-                st.grcs = S.rcs;
-                refresh_box_f(st);
-                if (!ok) atomicOr(&st.err, NEFE_ERR_BOX);
-            }
+            set_cell_grid(S, st);
             st.nbuild += 1;
         }
     }
@@ -568,8 +578,10 @@ __global__ void __launch_bounds__(256) k_rebuild_list(Bufs b, int nsys, int forc
     build_worklist(b, nsys, force_all);
 }
 
+constexpr int kCellsCluster = 8, kCellsThreads = 512;   // k_cells_clusters: blocks per system, threads
+
 // R2: exclusive scan of cells [lo, hi) of system s's occupancy by one block (blockDim a multiple
-// of 32, at most 256; 8 consecutive cells per thread per pass), starting from `carry`; resets the
+// of 32, at most 512; 8 consecutive cells per thread per pass), starting from `carry`; resets the
 // counts.  The block that holds the last cell writes the total.
 __device__ void scan_cells_range(const Bufs& b, int s, int lo, int hi, int ncells, int carry) {
     constexpr int PT = 8;
@@ -577,7 +589,7 @@ __device__ void scan_cells_range(const Bufs& b, int s, int lo, int hi, int ncell
     int* start = b.cell_start + S.cell0 + s;
     int* count = b.cell_count + S.cell0;
     int* cursor = b.cell_cursor + S.cell0;
-    __shared__ int warp_tot[8];
+    __shared__ int warp_tot[kCellsThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
     const int span = (int)blockDim.x * PT;
     for (int base = lo; base < hi; base += span) {
@@ -684,12 +696,12 @@ __device__ __forceinline__ int unpack_index(double w) { return (int)w; }
 // R3: scatter atoms into their cell segment (order inside a cell fixed by R4), with a copy
 // of their mirror positions in the same order for the list build.
 template <typename T>
-__device__ void cells_fill_tile(const Bufs& b, int tile) {
+__device__ void cells_fill_tile(const Bufs& b, int tile, int th) {
     using T4 = typename V4<T>::t;
     const TileAtom ta = tile_of(b, tile);
     const DevSys& S = b.sys[ta.sys];
-    if ((int)threadIdx.x >= ta.count) return;
-    const int i = ta.first + threadIdx.x;
+    if (th >= ta.count) return;
+    const int i = ta.first + th;
     const int pos = atomicAdd(&b.cell_cursor[S.cell0 + b.cell_of[i]], 1);
     if (pos < 0 || pos >= S.n) {                 // inconsistent occupancy: record, never write out of range
         atomicOr(&b.st[ta.sys].err, NEFE_ERR_CELL);
@@ -704,7 +716,44 @@ __device__ void cells_fill_tile(const Bufs& b, int tile) {
 template <typename T>
 __global__ void __launch_bounds__(kTile) k_cells_fill(Bufs b) {
     dep_wait();
-    NEFE_FOR_TILES(b, cells_fill_tile<T>(b, tile));
+    NEFE_FOR_TILES(b, cells_fill_tile<T>(b, tile, threadIdx.x));
+}
+
+// Worklist, R1, R2 and R3 of a small context (at most 32 systems and kClusterTiles tiles) in one launch: a
+// cluster of 8 blocks per system, with cluster barriers between the passes.  There is no worklist:
+// the list builds go by the systems' own flags (for_cells_of_grid).  On most steps no flag is set
+// and the launch returns at once, where the four launches cost 1.1 us each: 64 atoms in FP64 43.1 -> 40.8 us
+// a step, one 8000-atom system (63 tiles) 26.0 -> 24.9.  Larger contexts keep the separate kernels, which
+// spread a rebuild over the whole chip: 4 x 8000 atoms (252 tiles) 96 us a step against 100 in clusters,
+// 12 x 8000 76.6 against 77.7.
+constexpr int kClusterSystems = 32, kClusterTiles = 128;
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <typename T>
+__global__ void __cluster_dims__(kCellsCluster) __launch_bounds__(kCellsThreads) k_cells_clusters(Bufs b, int nsys) {
+    dep_wait();
+    if (*(volatile int*)b.any_rebuild == 0) return;
+    const int s = (int)blockIdx.x / kCellsCluster, rank = (int)blockIdx.x % kCellsCluster;
+    const DevSys& S = b.sys[s];
+    DevState& st = b.st[s];
+    // with rebuild_all any system's flag flags all; a flag set meanwhile by another cluster implies it
+    const int mine = (int)threadIdx.x < nsys && (b.rebuild_all || (int)threadIdx.x == s)
+                         ? *(volatile int*)&b.st[threadIdx.x].rebuild : 0;
+    if (!__syncthreads_or(mine)) return;         // uniform over the cluster
+    if (rank == 0 && threadIdx.x == 0) {
+        *(volatile int*)&st.rebuild = 1;
+        set_cell_grid(S, st);
+        st.nbuild += 1;
+    }
+    cluster_sync();
+    const int sub = (int)threadIdx.x / kTile, th = (int)threadIdx.x % kTile;
+    const int t0 = rank * (kCellsThreads / kTile) + sub, step = kCellsCluster * (kCellsThreads / kTile);
+    for (int t = t0; t < S.ntile; t += step) cells_count_tile<T>(b, S.tile0 + t, th);
+    cluster_sync();
+    if (rank == 0) scan_system_cells(b, s);
+    cluster_sync();
+    for (int t = t0; t < S.ntile; t += step) cells_fill_tile<T>(b, S.tile0 + t, th);
 }
 
 // R4: insertion sort of each cell segment by atom index (stable order by (cell, atom)), one cell
@@ -1229,6 +1278,28 @@ template <typename F>
 __device__ __forceinline__ void for_cells_of_grid(const Bufs& b, int nsys, F&& body) {
     const int nw = gridDim.x * (kTile / 32);
     const int wid = blockIdx.x * (kTile / 32) + (int)(threadIdx.x >> 5);
+    if (b.by_flag) {                             // few systems: lane s holds the cells up to those of system s
+        if (*(volatile int*)b.any_rebuild == 0) return;
+        const int lane = threadIdx.x & 31;
+        int upto = 0;
+        if (lane < nsys) {
+            const DevState& st = b.st[lane];
+            if (st.rebuild) upto = st.ncell[0] * st.ncell[1] * st.ncell[2];
+        }
+        const int own = upto;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += y;
+        }
+        const int C = __shfl_sync(0xffffffffu, upto, 31), K = (C + nw - 1) / nw;
+        const int g1 = min(C, (wid + 1) * K);
+        for (int g = wid * K; g < g1; ++g) {
+            const int s = __popc(__ballot_sync(0xffffffffu, upto <= g));
+            body(s, g - __shfl_sync(0xffffffffu, upto - own, s));
+        }
+        return;
+    }
     int C;
     if (b.rcbase) {
         C = b.rcbase[nsys];
@@ -1336,12 +1407,12 @@ __global__ void __launch_bounds__(kTile, 8) k_rebuild_coop(Bufs b, int nsys) {
     const unsigned nb = gridDim.x;
     if (blockIdx.x == 0) build_worklist(b, nsys, 0);
     if (!grid_barrier(bar, tmo, kBarrierNs, nb)) { flag_timeout(b, nsys); return; }
-    NEFE_FOR_TILES(b, cells_count_tile<T>(b, tile));
+    NEFE_FOR_TILES(b, cells_count_tile<T>(b, tile, threadIdx.x));
     if (!grid_barrier(bar, tmo, kBarrierNs, nb)) { flag_timeout(b, nsys); return; }
     for (int sy = blockIdx.x; sy < nsys; sy += gridDim.x)
         if (b.st[sy].rebuild) scan_system_cells(b, sy);
     if (!grid_barrier(bar, tmo, kBarrierNs, nb)) { flag_timeout(b, nsys); return; }
-    NEFE_FOR_TILES(b, cells_fill_tile<T>(b, tile));
+    NEFE_FOR_TILES(b, cells_fill_tile<T>(b, tile, threadIdx.x));
     if (!grid_barrier(bar, tmo, kBarrierNs, nb)) { flag_timeout(b, nsys); return; }
     nlist_cells_of_grid<T>(b, nsys, shm);
 }
@@ -3841,10 +3912,20 @@ void launch_cells_sort(const Bufs& b, int ncells, cudaStream_t s) {
     launch_next(k_cells_sort, blocks < 4096 ? blocks : 4096, 256, s, b);
 }
 
-void launch_cells_and_list(const Bufs& b, int precision, int ntiles, int nsys, int force_all,
+int cells_by_flag(int nsys, int ntiles) { return nsys <= kClusterSystems && ntiles <= kClusterTiles ? 1 : 0; }
+
+void launch_cells_and_list(const Bufs& b0, int precision, int ntiles, int nsys, int force_all,
                            cudaStream_t s, long* launches) {
+    Bufs b = b0;
+    if (force_all || b.list_lanes != 0) b.by_flag = 0;   // (the worklist's own kernels)
     if (ntiles <= 0) return;
-    launch_cells(b, precision, ntiles, nsys, force_all, s, launches);
+    if (force_all || !b.by_flag) {
+        launch_cells(b, precision, ntiles, nsys, force_all, s, launches);
+    } else {
+        if (precision == NEFE_FP64) launch_next(k_cells_clusters<double>, nsys * kCellsCluster, kCellsThreads, s, b, nsys);
+        else launch_next(k_cells_clusters<float>, nsys * kCellsCluster, kCellsThreads, s, b, nsys);
+        if (launches) *launches += 1;
+    }
     const int L = (b.list_lanes == 8 || b.list_lanes == 16 || b.list_lanes == 32) ? b.list_lanes : 0;
     if (L == 0) {
         const int g = list_grid(b, ntiles);
@@ -3879,7 +3960,9 @@ int rebuild_coop_blocks(int precision) {
     return min(per_sm * sms, kRebuildBlocks);
 }
 
-void launch_rebuild_coop(const Bufs& b, int precision, int blocks, int nsys, cudaStream_t s, long* launches) {
+void launch_rebuild_coop(const Bufs& b0, int precision, int blocks, int nsys, cudaStream_t s, long* launches) {
+    Bufs b = b0;
+    b.by_flag = 0;                               // (its own worklist)
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(kTile);
@@ -3932,7 +4015,9 @@ void launch_decode_ev(const long long* acc, double* out7, cudaStream_t s) {
     launch_next(k_decode_ev, 1, 32, s, acc, out7);
 }
 
-void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, cudaStream_t s, long* launches) {
+void launch_uf_list(const Bufs& b0, int precision, int ntiles, int nsys, int force_all, cudaStream_t s, long* launches) {
+    Bufs b = b0;
+    if (force_all || b.list_lanes != 0) b.by_flag = 0;
     if (ntiles <= 0 || !b.uf_nbr) return;
     const int g = list_grid(b, ntiles);
     if (precision == NEFE_FP64) launch_next(k_uflist<double>, g, kTile, s, b, nsys);

@@ -64,6 +64,7 @@ struct Bufs {
     void* uf_F;              // [ntot] UF force and atom energy of the step (T4)
     const int* uf_tiles;     // tiles of the UF systems (per-step UF kernel), or NULL: every tile
     int* scan_sums;          // stateless: span sums of a multi-block cell scan (NULL: one block)
+    int by_flag;             // small context: cells by k_cells_clusters, list builds by the rebuild flags
     int ncells_host;         // number of cells of the grid (engine: of all systems at creation)
     int* lacc;               // [ntot][4] int32 force accumulators of the scatter form (2^-22 eV/A)
     int* lacc_hi;            // [ntot][4] multiples of large terms (see k_edges_s)
@@ -110,10 +111,11 @@ void launch_kick_drift(const Bufs& b, int precision, int ntiles, int mode, cudaS
                        long* launches, int skip = 0, int drawn = 0);
 // Uhlenbeck-Ford pair rows of the UF systems (after the cell fill; flagged systems only when a
 // rebuild worklist is set).
-void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, cudaStream_t s, long* launches);
+void launch_uf_list(const Bufs& b, int precision, int ntiles, int nsys, int force_all, cudaStream_t s, long* launches);
 // Uhlenbeck-Ford forces and energies over `ntiles` tiles (b.uf_tiles, or every tile when NULL);
 // mode FM_FORCES writes b.f_out / b.e_atom (stateless), otherwise b.uf_F for pass B.
 void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches);
+int cells_by_flag(int nsys, int ntiles);   // value of by_flag for a context
 int atoms_per_warp_log2(int precision, int ntot);
 void set_edge_items(Bufs& b, int precision, int lg, int ntiles);
 // Force pass A (edges: pair terms, triplets centred on each atom, leg forces per edge).

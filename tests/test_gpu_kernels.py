@@ -409,3 +409,32 @@ def test_forces_where_the_last_blocks_are_cut_finer(N, precision, tol, copies):
     assert np.abs(e - e1).max() <= tol * np.abs(e1).max()
     assert abs(ev[0] / m - e1.sum()) <= tol * np.abs(e1).sum()
     assert np.abs(ev[1:] / m - v1).max() <= 10 * tol * np.abs(v1).max()
+
+
+# ------------------------------------------------------------------ rebuild by clusters
+@pytest.mark.parametrize("policy", [0, 1])
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("shapes", [((2, 2, 2), (5, 5, 4)), ((16, 16, 7), (3, 3, 3)), ((16, 16, 10), (3, 3, 3))])
+def test_rebuild_by_clusters_and_by_worklist(N, shapes, precision, policy):
+    """The same systems in a context of at most 32 (cells by a cluster per system, up to 128 tiles in all) and of 35
+    (worklist): hot enough that lists are rebuilt every few steps, the same motion bit for bit.  (The FP64
+    passes' lanes are set: their sums' order, and so the last bits, go by the context's size otherwise.)"""
+    got = []
+    for extra in (0, 33):
+        ctx = N.Context(precision=precision, skin=0.3, nbr_cap=48)
+        for r, shape in enumerate(shapes):
+            x, box = I.diamond(*shape)
+            s = ctx.add_system(x, box, v=I.gaussian_velocities(len(x), 6.0, 90 + r))
+            ctx.set_thermostat(s, 1500.0, 0.1, 30 + r)
+        x, box = I.diamond(2, 2, 2)
+        for r in range(extra):
+            ctx.add_system(x, box, v=I.gaussian_velocities(len(x), 3.0, r))
+        if precision == 1:
+            ctx.set_tuning(8, 4)
+        ctx.set_rebuild_policy(policy)
+        ctx.run(60)
+        got.append([ctx.get_state(s) for s in range(len(shapes))])
+        assert all(ctx.results(s)["error"] == 0 for s in range(len(shapes)))
+        ctx.close()
+    for a, b in zip(*got):
+        assert all(np.array_equal(u, v) for u, v in zip(a, b))
