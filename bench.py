@@ -663,11 +663,12 @@ def main():
     bytes_a = PASS_A_FIXED + 4.0 * mean_cnt + 20.0 * m_shell
     bytes_b = PASS_B_FIXED + 20.0 * m_shell
     if lanes[0] == 0:
-        # scatter form: pass A reads own mirror, row length and row, and adds the leg forces into
+        # scatter form: pass A reads own position in two forms (fraction 16, packed for the row
+        # filter 8), row length and row, writes the shell size, and adds the edge and leg forces into
         # 16-byte accumulators (L2-resident reductions, not counted); pass B streams the
         # epilogue operands (accumulator 16, spring offset 16, displacement 24, noise 16, v 12 +
         # 12, force 16)
-        bytes_a = 16 + 4 + 4.0 * mean_cnt + 4
+        bytes_a = 16 + 8 + 4 + 4.0 * mean_cnt + 4
         bytes_b = 16 + 16 + 24 + 16 + 12 + 12 + 16
     if b_us > a_us:
         kkey, kname, kbytes, kus = "k_gather", "force pass B (gather or scatter-form epilogue: springs, Langevin, kick)", bytes_b, b_us

@@ -170,10 +170,10 @@ NEFE_API int nefe_neighbor_build(const double* x, int n, const double box[3], do
 
 /*
  * nefe_sw_forces - Stillinger-Weber energy, forces and virial on a list built by
- * nefe_neighbor_build from the same x and box.  Gather formulation: the force on i sums the
+ * nefe_neighbor_build from the same x and box.  FP64 is a gather: the force on i sums the
  * pair terms, the three-body terms centred on i, and the three-body terms centred on each
- * neighbour j in which i is a leg, so no atomics touch the forces and the result is
- * bitwise reproducible.
+ * neighbour j in which i is a leg.  FP32 adds the terms of each centre to its atoms in fixed
+ * point.  Both are bitwise reproducible.
  *   x, n, box, rcs, nbr, cnt, cap   as nefe_neighbor_build (same values).
  *   prm         host, potential parameters (prm->a * prm->sigma <= rcs).
  *   precision   NEFE_FP32 or NEFE_FP64 pair/triplet arithmetic.
@@ -404,7 +404,9 @@ NEFE_API int nefe_save(nefe_ctx* ctx, const char* path);
 NEFE_API int nefe_load(nefe_ctx* ctx, const char* path);
 
 /* Times the variants of both force passes on the current state and keeps the fastest:
- * pass A with 1 (one thread per atom), 4, 8, 16 or 32 lanes per atom (FP64: 8, 16, 32),
+ * pass A in the scatter form (0; the FP32 default: edge lists per warp, fixed-point force sums) or
+ * with 1 (one thread per atom), 4, 8, 16 or 32 lanes per atom (FP64: 8, 16, 32, which stand for edge
+ * lists of 16, 8 or 4 atoms to a warp; left alone, by the context's size),
  * pass B with 1, 2, 4 or 8 lanes per atom, and the rebuild policy (nefe_set_rebuild_policy); the
  * list build keeps its form (nefe_set_list_tuning).  Each force pass is first timed alone; then
  * the two fastest pass-A variants with every pass-B variant, and with the best pair each rebuild
@@ -532,7 +534,8 @@ typedef struct nefe_adjoint_desc {
 } nefe_adjoint_desc;
 
 /* Creates the context on `device` / `stream` (device memory ~ (17 + 3 K_c) n doubles plus
- * 9 n doubles per checkpoint).  NEFE_EINVAL on bad arguments, NEFE_ENOMEM. */
+ * 9 n doubles per checkpoint, and about 2.3 kB per atom and up to 140 MB for the list and its
+ * edges).  NEFE_EINVAL on bad arguments, NEFE_ENOMEM. */
 NEFE_API int nefe_adjoint_create(nefe_adj** out, int device, void* stream, const nefe_adjoint_desc* desc,
                                  const nefe_sw_params* prm);
 NEFE_API int nefe_adjoint_destroy(nefe_adj* adj);
@@ -540,7 +543,8 @@ NEFE_API int nefe_adjoint_destroy(nefe_adj* adj);
  * invalidates the checkpoints. */
 NEFE_API int nefe_adjoint_set_params(nefe_adj* adj, const nefe_sw_params* prm);
 /* Runs nsteps from the initial state, keeping the checkpoints; *W (host) = the work.  The neighbour
- * list is rebuilt at every force evaluation.  Blocking.  NEFE_EOVERFLOW / NEFE_ENAN on a bad run. */
+ * list holds every pair within the cutoff at each force evaluation: it is rebuilt where an atom has
+ * moved too far since it was built.  Blocking.  NEFE_EOVERFLOW / NEFE_ENAN on a bad run. */
 NEFE_API int nefe_adjoint_forward(nefe_adj* adj, long nsteps, double* W);
 /* Reverse sweep over the last forward run: dW/dtheta (host [7]) and, when not NULL, dW/dx0 and
  * dW/dv0 (host (n, 3)).  Each segment is recomputed from its checkpoint.  Blocking.
