@@ -120,7 +120,7 @@ void want1(Scratch1& S, int n, const int n3[3], int prec, bool cells) {
     S.want(&S.sys, sizeof(DevSys));
     S.want(&S.st, sizeof(DevState));
     S.want(&S.tiles, sizeof(int4) * (ntiles > 0 ? ntiles : 1));
-    S.want(&S.acc, sizeof(long long) * ACC_N * kSlots);
+    S.want(&S.acc, sizeof(long long) * 2 * ACC_N * kSlots);     // sums, then their remainders
     S.want(&S.swc, sizeof(SwcBytes));
     const size_t v4 = prec == NEFE_FP64 ? sizeof(double4) : sizeof(float4);
     S.want(&S.xs, v4 * N);
@@ -164,7 +164,7 @@ int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3]
         std::memcpy(sw.b, &c, sizeof(c));
     }
     NEFE_CU(S.commit());
-    const int nacc = ACC_N * kSlots;
+    const int nacc = 2 * ACC_N * kSlots;
     const int work = std::max(std::max(ntiles, S.ncells), nacc);
     k_scratch_init<<<std::min((work + 255) / 256, 608), 256, 0, S.s>>>(
         hs, st, sw, S.sys, S.st, S.swc, S.tiles, ntiles, S.acc, nacc, S.cell_count, S.ncells);
@@ -175,7 +175,7 @@ int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3]
 Bufs bufs_of(const Scratch1& S, const double* x, int n) {
     Bufs b;
     std::memset(&b, 0, sizeof(b));
-    b.sys = S.sys; b.st = S.st; b.acc = S.acc; b.tiles = S.tiles;
+    b.sys = S.sys; b.st = S.st; b.acc = S.acc; b.acc_lo = S.acc + ACC_N * kSlots; b.tiles = S.tiles;
     b.x = const_cast<double*>(x);
     b.xs = S.xs; b.xa = S.xa; b.xcs = S.xcs; b.q = S.q; b.cell_of = S.cell_of; b.perm = S.perm;
     b.shd = S.shd; b.shj = S.shj; b.shn = S.shn; b.P = S.P;

@@ -168,11 +168,13 @@ template <> struct Noise<float> {
 // of the order in which blocks arrive.  Every thread of the block must call it.
 // In FP64 the threads' values are converted first (2^-40 units) and summed as integers: FP64 adds
 // run at 2 lanes a cycle, and five of them per value and warp were a third of the epilogue.  Values
-// of 2^22 or more (or not finite) take the FP64 sums.
+// of 2^22 or more (or not finite) take the FP64 sums.  The remainders of the conversion to 2^-32 are
+// kept in their own slots where the caller has some (acc_lo: stateless calls, whose small blocks
+// would round several times as often as a 128-atom block does).
 // ------------------------------------------------------------------------------------
 template <typename T, int K>
 __device__ __forceinline__ void block_sum_to_acc(T (&v)[K], long long* acc_sys, int first,
-                                                 unsigned* err) {
+                                                 unsigned* err, long long* acc_lo = nullptr) {
     if constexpr (sizeof(T) == 8) {
         __shared__ long long ired[kTile / 32][K];
         bool big = false;
@@ -191,11 +193,12 @@ __device__ __forceinline__ void block_sum_to_acc(T (&v)[K], long long* acc_sys, 
             if (threadIdx.x < K) {
                 long long s = 0;
                 for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += ired[i][threadIdx.x];
+                const size_t slot = (size_t)(first + threadIdx.x) * kSlots + (blockIdx.x % kSlots);
+                const long long units = s;
                 s = (s + 128) >> 8;
-                if (s != 0)
-                    atomicAdd(reinterpret_cast<unsigned long long*>(
-                                  &acc_sys[(size_t)(first + threadIdx.x) * kSlots + (blockIdx.x % kSlots)]),
-                              (unsigned long long)s);
+                if (s != 0) atomicAdd(reinterpret_cast<unsigned long long*>(&acc_sys[slot]), (unsigned long long)s);
+                if (acc_lo && units != s * 256)
+                    atomicAdd(reinterpret_cast<unsigned long long*>(&acc_lo[slot]), (unsigned long long)(units - s * 256));
             }
             return;
         }
@@ -3123,8 +3126,8 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
         reinterpret_cast<double4*>(b.P)[i] = mk4(fx, fy, fz, en);
     }
     long long* acc = b.acc + (size_t)ta.sys * ACC_N * kSlots;
-    block_sum_to_acc<double, 8>(red8, acc, ACC_UINT, &st.err);
-    if constexpr (GRAD) block_sum_to_acc<double, 7>(gth, acc, ACC_DTH, &st.err);
+    block_sum_to_acc<double, 8>(red8, acc, ACC_UINT, &st.err, b.acc_lo);
+    if constexpr (GRAD) block_sum_to_acc<double, 7>(gth, acc, ACC_DTH, &st.err, b.acc_lo);
 }
 
 // Force pass B, L lanes per atom:
@@ -3854,12 +3857,17 @@ __global__ void k_soa_to_aos(const double* __restrict__ s, double* __restrict__ 
     a[t] = s[(size_t)k * n + i];
 }
 
+// Sum a of a stateless call: slots and remainders (stateless calls hold both, one after the other).
+__device__ __forceinline__ double decoded(const long long* acc, int a) {
+    const long long* lo = acc + (size_t)ACC_N * kSlots;
+    return (double)slot_sum(acc + (size_t)a * kSlots) / kFix + (double)slot_sum(lo + (size_t)a * kSlots) * 0x1p-40;
+}
 __global__ void k_decode_ev(const long long* acc, double* out7) {
     dep_wait();
     const int t = threadIdx.x;
     if (t >= 7) return;
     const int a = t == 0 ? ACC_UINT : ACC_VIR + (t - 1);
-    out7[t] = (double)slot_sum(acc + (size_t)a * kSlots) / kFix;
+    out7[t] = decoded(acc, a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -4004,7 +4012,7 @@ __global__ void k_decode_grad(const long long* acc, double* out8) {
     const int t = threadIdx.x;
     if (t >= 8) return;
     const int a = t == 0 ? ACC_UINT : ACC_DTH + (t - 1);
-    out8[t] = (double)slot_sum(acc + (size_t)a * kSlots) / kFix;
+    out8[t] = decoded(acc, a);
 }
 
 void launch_decode_grad(const long long* acc, double* out8, cudaStream_t s) {

@@ -14,6 +14,7 @@ struct Bufs {
     const DevSys* sys;
     DevState* st;
     long long* acc;          // [nsys][ACC_N][kSlots]
+    long long* acc_lo;       // stateless: remainders of the sums in 2^-40 units, the same layout, or NULL
     const int4* tiles;       // 128-atom tiles: system, first atom, atom count
     double* x;               // FP64 anchor positions (positions at the last list build), SoA
     void* dhi;               // displacement since the last build, kernel precision, SoA (may be NULL)

@@ -438,3 +438,26 @@ def test_rebuild_by_clusters_and_by_worklist(N, shapes, precision, policy):
         ctx.close()
     for a, b in zip(*got):
         assert all(np.array_equal(u, v) for u, v in zip(a, b))
+
+
+# ------------------------------------------------------------------ sums of a stateless FP64 call
+@pytest.mark.parametrize("seed", [1, 2, 3])
+def test_fp64_sums_keep_their_remainders(N, seed):
+    """Energy, virial and dE/d(A) of 64 atoms in blocks of 8: block sums in 2^-40 eV units, so some 500
+    conversions of at most 2^-41 eV each (1e-11 eV, 4e-14 of the energy), where one rounding to 2^-32 eV per
+    block is 1e-10 eV and more."""
+    x, box = I.diamond(2, 2, 2)
+    x = I.rattle(x, 0.1, seed)
+    n, cap = len(x), 48
+    xd = soa(x)
+    nbr, cnt = torch.zeros(n * cap, dtype=torch.int32, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    N.nefe_neighbor_build(xd, n, box, RC + 0.5, cap, nbr, cnt)
+    f = torch.zeros(3 * n, dtype=torch.float64, device="cuda")
+    ev, eg = torch.zeros(7, dtype=torch.float64, device="cuda"), torch.zeros(8, dtype=torch.float64, device="cuda")
+    N.nefe_sw_forces(xd, n, box, RC + 0.5, nbr, cnt, cap, N.nefe_sw_params_silicon(), N.NEFE_FP64, f, None, ev)
+    N.nefe_sw_energy_grad(xd, n, box, RC + 0.5, nbr, cnt, cap, N.nefe_sw_params_silicon(), N.NEFE_FP64, f, eg)
+    torch.cuda.synchronize()
+    e_o, _, vir_o, _ = O.sw_energy(x, box)
+    assert abs(float(ev[0]) - e_o) <= 1e-13 * abs(e_o)
+    assert abs(float(eg[0]) - e_o) <= 1e-13 * abs(e_o)
+    assert np.abs(ev.cpu().numpy()[1:] - vir_o).max() <= 1e-13 * abs(e_o)
