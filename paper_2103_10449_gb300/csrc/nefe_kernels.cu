@@ -167,8 +167,9 @@ template <> struct Noise<float> {
 // on top of its FP32 summation error.  Integer addition makes the per-system total independent
 // of the order in which blocks arrive.  Every thread of the block must call it.
 // In FP64 the threads' values are converted first (2^-40 units) and summed as integers: FP64 adds
-// run at 2 lanes a cycle, and five of them per value and warp were a third of the epilogue.  Values
-// of 2^22 or more (or not finite) take the FP64 sums.  The remainders of the conversion to 2^-32 are
+// run at 2 lanes a cycle, and five of them per value and warp were a third of the epilogue.  The
+// integer sum of a block (at most 128 threads) stays below 2^62 when every value is below 2^15; a
+// block that holds a larger value (or one that is not finite) takes the FP64 sums.  The remainders of the conversion to 2^-32 are
 // kept in their own slots where the caller has some (acc_lo: stateless calls, whose small blocks
 // would round several times as often as a 128-atom block does).
 // ------------------------------------------------------------------------------------
@@ -177,9 +178,10 @@ __device__ __forceinline__ void block_sum_to_acc(T (&v)[K], long long* acc_sys, 
                                                  unsigned* err, long long* acc_lo = nullptr) {
     if constexpr (sizeof(T) == 8) {
         __shared__ long long ired[kTile / 32][K];
+        constexpr double most = 4194304.0 / kTile;
         bool big = false;
 #pragma unroll
-        for (int k = 0; k < K; ++k) big = big || !(fabs(v[k]) < 4194304.0);
+        for (int k = 0; k < K; ++k) big = big || !(fabs(v[k]) < most);
         if (!__syncthreads_or(big)) {
             const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll

@@ -461,3 +461,59 @@ def test_fp64_sums_keep_their_remainders(N, seed):
     assert abs(float(ev[0]) - e_o) <= 1e-13 * abs(e_o)
     assert abs(float(eg[0]) - e_o) <= 1e-13 * abs(e_o)
     assert np.abs(ev.cpu().numpy()[1:] - vir_o).max() <= 1e-13 * abs(e_o)
+
+
+# ------------------------------------------------------------------ large sums
+def _sw(N, x, box, prm, precision, skin=0.5, cap=48, grad=False):
+    """Forces, energy and virial (or energy and dE/dtheta) of a stateless call, as numpy."""
+    n, rcs = len(x), RC + skin
+    xd = soa(x)
+    nbr, cnt = torch.zeros(n * cap, dtype=torch.int32, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    N.nefe_neighbor_build(xd, n, box, rcs, cap, nbr, cnt)
+    f = torch.zeros(3 * n, dtype=torch.float64, device="cuda")
+    out = torch.zeros(8 if grad else 7, dtype=torch.float64, device="cuda")
+    if grad:
+        N.nefe_sw_energy_grad(xd, n, box, rcs, nbr, cnt, cap, prm, precision, f, out)
+    else:
+        N.nefe_sw_forces(xd, n, box, rcs, nbr, cnt, cap, prm, precision, f, None, out)
+    torch.cuda.synchronize()
+    return f.cpu().numpy().reshape(3, n).T, out.cpu().numpy()
+
+
+def _silicon(N, **scale):
+    p = N.nefe_sw_params_silicon()
+    for k, v in scale.items():
+        setattr(p, k, getattr(p, k) * v)
+    return p
+
+
+@pytest.mark.parametrize("power", [12, 16, 17, 18, 19, 20, 21])
+def test_block_sums_whose_terms_are_in_range_but_not_their_total(N, power):
+    """eps times 2^power: the sums are those of silicon times the same number.  A block (8 atoms, some 35 eV)
+    crosses 2^22 eV at 2^17 and 2^23 at 2^18, a lane's term (some 2 eV) crosses 2^22 at 2^21 only.  Each of the
+    500 conversions is within 2^-33 eV of its term, and the reference's (2^-40 units) within 2^power 2^-41."""
+    x, box = I.diamond(2, 2, 2)
+    x = I.rattle(x, 0.1, 21)
+    k = 2.0 ** power
+    _, ev1 = _sw(N, x, box, _silicon(N), N.NEFE_FP64)
+    _, eg1 = _sw(N, x, box, _silicon(N), N.NEFE_FP64, grad=True)
+    _, ev = _sw(N, x, box, _silicon(N, eps=k), N.NEFE_FP64)
+    _, eg = _sw(N, x, box, _silicon(N, eps=k), N.NEFE_FP64, grad=True)
+    tol = 1e-12 * abs(ev1[0])
+    assert np.abs(ev / k - ev1).max() <= tol
+    assert np.abs(eg / k - eg1).max() <= 1e-12 * np.abs(eg1).max()
+
+
+def test_spring_energies_of_sites_in_other_images(N):
+    """Springs take no nearest image: sites 20 boxes away hold 3.5e5 eV an atom, 1.1e7 eV in the 32 atoms of a
+    block, in FP64 against the plain sum."""
+    x, box = I.diamond(2, 2, 2)
+    r0 = x + np.array([20.0, 20.0, 20.0]) * box
+    ctx = N.Context(precision=N.NEFE_FP64, skin=0.5, nbr_cap=48)
+    s = ctx.add_system(x, box, v=np.zeros_like(x), r0=r0)
+    ctx.set_schedule(s, N.NEFE_SCHED_FL, 1, 1000, k_E=5.0)
+    ctx.setup()
+    r = ctx.results(s)
+    ctx.close()
+    assert r["error"] == 0
+    assert r["U_E"] == pytest.approx(0.5 * 5.0 * float(((x - r0) ** 2).sum()), rel=1e-12)
