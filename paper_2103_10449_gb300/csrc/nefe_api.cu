@@ -206,7 +206,7 @@ static void want_forces(Scratch1& S, int n, int precision) {
     if (precision == NEFE_FP32) {
         S.want(&S.xf, sizeof(int4) * N);
         S.want(&S.lacc, 4 * sizeof(int) * N);
-        S.want(&S.lacc_hi, 4 * sizeof(int) * N);
+        S.want(&S.lacc_hi, 3 * sizeof(long long) * N);
         S.want(&S.hi_flag, sizeof(int) * ((N + kTile - 1) / kTile));
     } else {
         S.want(&S.shd, sizeof(double4) * N * kShell);
@@ -340,7 +340,7 @@ int nefe_sw_forces(const double* x, int n, const double box[3], double rcs, cons
         b.f_out = f; b.e_atom = e_atom;
         if ((rc = run_forces(S, b, n, prm, precision))) return rc;
     }
-    if (energy_virial) launch_decode_ev(S.acc, energy_virial, S.s);
+    if (energy_virial) launch_decode_ev(S.acc, energy_virial, &S.st->err, S.s);
     NEFE_CU(cudaGetLastError());
     if (shell_overflow) {
         unsigned err = 0;
@@ -432,7 +432,7 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
         launch_uf(b, precision, ntiles, FM_FORCES, S.s, nullptr);
         NEFE_CU(cudaGetLastError());
     }
-    if (energy_virial) launch_decode_ev(S.acc, energy_virial, S.s);
+    if (energy_virial) launch_decode_ev(S.acc, energy_virial, nullptr, S.s);
     NEFE_CU(cudaGetLastError());
     unsigned err = 0;
     if ((rc = read_error(S, &err))) return rc;

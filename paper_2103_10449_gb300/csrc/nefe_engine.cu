@@ -70,7 +70,8 @@ struct nefe_ctx {
     int *d_shj = nullptr, *d_shn = nullptr, *d_rtiles = nullptr, *d_rcount = nullptr, *d_rcbase = nullptr;
     int* d_any = nullptr;    // context-wide rebuild flag words (Bufs::any_rebuild)
     int *d_uf_nbr = nullptr, *d_uf_cnt = nullptr, *d_uf_tiles = nullptr;
-    int *d_lacc = nullptr, *d_lacc_hi = nullptr, *d_hi_flag = nullptr;   // scatter-form force accumulators (FP32)
+    int *d_lacc = nullptr, *d_hi_flag = nullptr;   // scatter-form force accumulators (FP32)
+    long long* d_lacc_hi = nullptr;
     float4* d_lscale = nullptr;
     uint2* d_xc = nullptr;
     int4 *d_xf = nullptr, *d_xfb = nullptr;                               // fractional positions (FP32)
@@ -257,7 +258,7 @@ int resetup(nefe_ctx* c) {
     NEFE_CU(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * (size_t)c->nsys * ACC_N * kSlots, c->stream));
     if (c->d_lacc) {
         NEFE_CU(cudaMemsetAsync(c->d_lacc, 0, 4 * sizeof(int) * (size_t)c->ntot, c->stream));
-        NEFE_CU(cudaMemsetAsync(c->d_lacc_hi, 0, 4 * sizeof(int) * (size_t)c->ntot, c->stream));
+        NEFE_CU(cudaMemsetAsync(c->d_lacc_hi, 0, 3 * sizeof(long long) * (size_t)c->ntot, c->stream));
         NEFE_CU(cudaMemsetAsync(c->d_hi_flag, 0, sizeof(int) * (size_t)c->ntiles, c->stream));
     }
     launch_cells_and_list(c->b, c->prec, c->ntiles, c->nsys, 1, c->stream, &c->launches);
@@ -454,7 +455,7 @@ int setup(nefe_ctx* c) {
     if ((rc = dalloc(c, &c->d_P, 3 * v4 * N))) return rc;
     if (c->prec == NEFE_FP32) {
         if ((rc = dalloc(c, &c->d_lacc, 4 * sizeof(int) * N))) return rc;
-        if ((rc = dalloc(c, &c->d_lacc_hi, 4 * sizeof(int) * N))) return rc;
+        if ((rc = dalloc(c, &c->d_lacc_hi, 3 * sizeof(long long) * N))) return rc;
         if ((rc = dalloc(c, &c->d_hi_flag, sizeof(int) * tile_sys.size()))) return rc;
         if ((rc = dalloc(c, &c->d_xf, sizeof(int4) * N))) return rc;
     }

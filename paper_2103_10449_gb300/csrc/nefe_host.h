@@ -145,7 +145,8 @@ struct Scratch1 {
     int* cell_cursor = nullptr;
     int* scan_sums = nullptr;
     int4* xf = nullptr;
-    int *lacc = nullptr, *lacc_hi = nullptr, *hi_flag = nullptr;
+    int *lacc = nullptr, *hi_flag = nullptr;
+    long long* lacc_hi = nullptr;
     float4* lscale = nullptr;
     uint2* xc = nullptr;
     int ncells = 0;

@@ -2464,34 +2464,40 @@ __global__ void __launch_bounds__(kEdges1Threads, 16) k_edges1(Bufs b) {
 // being the int32 sums.  Its low word is X; its high word is Y - 1 when X < 0 (the borrow), which
 // the reader undoes (force_of_acc).  Two reductions per force instead of three.
 // A term of kLegFine eV/A or more is split: its multiples of kLegCoarse go to a second accumulator
-// (one count per multiple) and the rest, at most 7 eV/A, stays; up to 64 rests (32 legs, 32 own
+// (int64, one count per multiple) and the rest, at most 7 eV/A, stays; up to 64 rests (32 legs, 32 own
 // edges) fit the int32 sum.  The second accumulator is read only for tiles whose flag says that
 // something was added (at 1000 K some atom of a system of thousands has such a term on most steps,
-// but few tiles do).
+// but few tiles do).  A term that is not finite, or of kLegMax (2.5e17 eV/A) and more, sets the atom's
+// count to kLegNan, from which no sum of counts (64 terms of up to 2^54) comes back below kLegLost:
+// the force is NaN, as a floating-point sum would have it.
 // ------------------------------------------------------------------------------------
 constexpr float kLegScale = 4194304.0f;          // 2^22
 constexpr float kLegFine = 8.0f;
 constexpr float kLegCoarse = 14.0f;
-constexpr float kLegMax = 1e9f;
+constexpr float kLegMax = 14.0f * 18014398509481984.0f;   // 14 2^54
+constexpr long long kLegNan = 1LL << 62, kLegLost = 1LL << 61;
 constexpr float kLegRefuse = 48.0f;
 constexpr float kPairOdd = 6.0f;                 // half a pair force above which an own sum could reach kLegRefuse
 
-// Splits a large term: sign times its multiples of kLegCoarse go to atom j; returns the rest.
+// Splits a large term: sign times its multiples of kLegCoarse go to atom j; returns the rest.  (FP64: the
+// multiples of a large FP32 value are not FP32 numbers; the rest is one.)
 __device__ __noinline__ float3 split_leg(const Bufs& b, const DevSys& S, int j, int sign, unsigned* err, float x, float y,
                                          float z) {
-    if (!(fabsf(x) < kLegMax && fabsf(y) < kLegMax && fabsf(z) < kLegMax)) {
-        atomicOr(err, NEFE_ERR_NAN);
-        return make_float3(0.0f, 0.0f, 0.0f);
-    }
-    int* hi_j = b.lacc_hi + 4 * (size_t)j;
+    unsigned long long* hi_j = reinterpret_cast<unsigned long long*>(b.lacc_hi + 3 * (size_t)j);
     float v[3] = {x, y, z};
     for (int k = 0; k < 3; ++k) {
-        const float h = rintf(v[k] / kLegCoarse);
-        v[k] = fmaf(-kLegCoarse, h, v[k]);
-        if (h != 0.0f) {
-            atomicAdd(hi_j + k, sign * (int)h);
-            b.hi_flag[S.tile0 + (j - S.off) / kTile] = 1;
+        if (!(fabsf(v[k]) < kLegMax)) {
+            atomicOr(err, NEFE_ERR_NAN);
+            v[k] = 0.0f;
+            if (b.leg_refuse) continue;          // (a refused term is left out)
+            atomicExch(hi_j + k, (unsigned long long)kLegNan);
+        } else {
+            const double h = rint((double)v[k] / (double)kLegCoarse);
+            if (h == 0.0) continue;
+            v[k] = (float)fma(-(double)kLegCoarse, h, (double)v[k]);
+            atomicAdd(hi_j + k, (unsigned long long)(sign * (long long)h));
         }
+        b.hi_flag[S.tile0 + (j - S.off) / kTile] = 1;
     }
     return make_float3(v[0], v[1], v[2]);
 }
@@ -3464,10 +3470,14 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
         const int3 fq = force_of_acc(q);
         T f[3] = {(T)fq.x * inv, (T)fq.y * inv, (T)fq.z * inv};
         if (sw && big != 0) {
-            int4* h4 = reinterpret_cast<int4*>(b.lacc_hi) + i;
-            const int4 h = *h4;
-            *h4 = make_int4(0, 0, 0, 0);
-            f[0] += (T)kLegCoarse * (T)h.x; f[1] += (T)kLegCoarse * (T)h.y; f[2] += (T)kLegCoarse * (T)h.z;
+            long long* h3 = b.lacc_hi + 3 * (size_t)i;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const long long h = h3[k];
+                h3[k] = 0;
+                if (h >= kLegLost || h <= -kLegLost) f[k] = (T)NAN;
+                else f[k] += (T)kLegCoarse * (T)h;
+            }
         }
         T vo[3], Fo[3];
         finish_atom<T, MODE>(b, S, st, i, f, (T)0, false, pd, pv, pz, s_xm, red, fz, vo, Fo);
@@ -3864,12 +3874,13 @@ __device__ __forceinline__ double decoded(const long long* acc, int a) {
     const long long* lo = acc + (size_t)ACC_N * kSlots;
     return (double)slot_sum(acc + (size_t)a * kSlots) / kFix + (double)slot_sum(lo + (size_t)a * kSlots) * 0x1p-40;
 }
-__global__ void k_decode_ev(const long long* acc, double* out7) {
+// (NaN where a block's sum was out of range or not finite and is missing: err, or NULL)
+__global__ void k_decode_ev(const long long* acc, double* out7, const unsigned* err) {
     dep_wait();
     const int t = threadIdx.x;
     if (t >= 7) return;
     const int a = t == 0 ? ACC_UINT : ACC_VIR + (t - 1);
-    out7[t] = decoded(acc, a);
+    out7[t] = err && (*err & NEFE_ERR_NAN) ? NAN : decoded(acc, a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -4021,8 +4032,8 @@ void launch_decode_grad(const long long* acc, double* out8, cudaStream_t s) {
     launch_next(k_decode_grad, 1, 32, s, acc, out8);
 }
 
-void launch_decode_ev(const long long* acc, double* out7, cudaStream_t s) {
-    launch_next(k_decode_ev, 1, 32, s, acc, out7);
+void launch_decode_ev(const long long* acc, double* out7, const unsigned* err, cudaStream_t s) {
+    launch_next(k_decode_ev, 1, 32, s, acc, out7, err);
 }
 
 void launch_uf_list(const Bufs& b0, int precision, int ntiles, int nsys, int force_all, cudaStream_t s, long* launches) {

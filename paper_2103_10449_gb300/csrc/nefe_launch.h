@@ -68,7 +68,7 @@ struct Bufs {
     int by_flag;             // small context: cells by k_cells_clusters, list builds by the rebuild flags
     int ncells_host;         // number of cells of the grid (engine: of all systems at creation)
     int* lacc;               // [ntot][4] int32 force accumulators of the scatter form (2^-22 eV/A)
-    int* lacc_hi;            // [ntot][4] multiples of large terms (see k_edges_s)
+    long long* lacc_hi;      // [ntot][3] multiples of large terms (see k_edges_s)
     SWc<float> swc_common;   // the potential constants, where every system has the same (common)
     SWp<double> swp_common;
     int lg;                  // atoms per warp of the edge-list kernels, as a power of two
@@ -99,8 +99,9 @@ void launch_cells(const Bufs& b, int precision, int ntiles, int nsys, int force_
 void launch_cells_sort(const Bufs& b, int ncells, cudaStream_t s);
 // Cells per block of the multi-block scan (its scratch: one int per block, at most 1024).
 int cells_scan_span(int ncells);
-// Decodes one system's fixed-point sums into [U_int, virial xx yy zz xy xz yz] (FP64, device).
-void launch_decode_ev(const long long* acc, double* out7, cudaStream_t s);
+// Decodes one system's fixed-point sums into [U_int, virial xx yy zz xy xz yz] (FP64, device); NaN
+// where the error word says that a block's sum is missing (err: device, or NULL).
+void launch_decode_ev(const long long* acc, double* out7, const unsigned* err, cudaStream_t s);
 // Decodes [U_int, dE/dA, dE/dB, dE/dp, dE/dq, dE/da, dE/dlambda3, dE/dgamma] (FP64, device).
 void launch_decode_grad(const long long* acc, double* out8, cudaStream_t s);
 // Rebuild sequence (only systems whose rebuild flag is set, or all when force_all).

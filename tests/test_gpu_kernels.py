@@ -517,3 +517,32 @@ def test_spring_energies_of_sites_in_other_images(N):
     ctx.close()
     assert r["error"] == 0
     assert r["U_E"] == pytest.approx(0.5 * 5.0 * float(((x - r0) ** 2).sum()), rel=1e-12)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_coincident_atoms_give_nan_and_only_there(N, precision):
+    """Two atoms at one place: NaN forces on them, energy and virial NaN (no finite sum stands for them),
+    every atom further away than two cutoffs as without them."""
+    x, box = I.diamond(4, 4, 4)
+    x = I.rattle(x, 0.05, 5)
+    x[9] = x[8]
+    f, ev = _sw(N, x, box, _silicon(N), precision)
+    assert np.isnan(f[8]).any() and np.isnan(f[9]).any()
+    assert np.isnan(ev).any()
+    d = x - x[8]
+    d -= box * np.rint(d / box)
+    far = np.flatnonzero((d * d).sum(1) > (2.0 * RC) ** 2)
+    f_o = O.sw_force_atoms(x, box, far)
+    assert len(far) > 100 and np.abs(f[far] - f_o).max() <= 1e-5 * np.abs(f_o).max()
+
+
+@pytest.mark.parametrize("r", [0.06, 0.03, 0.012])
+def test_scatter_forces_of_very_close_pairs(N, r):
+    """Forces of some 5e8 to 1e12 eV/A: finite, relative to the largest as any other."""
+    x, box = I.diamond(3, 3, 3)
+    d = x[4] - x[0]
+    x[4] = x[0] + d * (r / np.linalg.norm(d))
+    f, _ = _sw(N, x, box, _silicon(N), N.NEFE_FP32)
+    _, f_o, _, _ = O.sw_energy(x, box)
+    # the pair's distance carries 2 units of 16 A 2^-32 (7.6e-9 A) and 2^-23 of itself; the force goes as r^-5
+    assert np.abs(f - f_o).max() <= (1e-5 + 5 * 7.6e-9 / r) * np.abs(f_o).max()
