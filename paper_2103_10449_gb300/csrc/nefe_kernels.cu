@@ -164,8 +164,10 @@ template <> struct Noise<float> {
 // value into slot (blockIdx % kSlots).  The FP64 path converts the block sum at 2^-32; the
 // FP32 path rounds it to a multiple of 2^-16 (an int32 conversion, |block sum| < 32768) before
 // moving it to the 2^-32 scale, so a block's contribution carries at most 2^-17 of rounding
-// on top of its FP32 summation error.  Integer addition makes the per-system total independent
-// of the order in which blocks arrive.  Every thread of the block must call it.
+// on top of its FP32 summation error.  A larger block sum is converted warp by warp: what cannot be
+// summed (and is reported) are 32,768 eV in a warp (32 atoms at most; 65,536 for dE/dtheta), whatever
+// the block's size.  Integer addition makes the per-system total independent of the order in which
+// blocks arrive.  Every thread of the block must call it.
 // In FP64 the threads' values are converted first (2^-40 units) and summed as integers: FP64 adds
 // run at 2 lanes a cycle, and five of them per value and warp were a third of the epilogue.  The
 // integer sum of a block (at most 128 threads) stays below 2^62 when every value is below 2^15; a
@@ -226,6 +228,15 @@ __device__ __forceinline__ void block_sum_to_acc(T (&v)[K], long long* acc_sys, 
             const float t = s * 65536.0f;
             bad = !(fabsf(t) < 2147483520.0f);
             q = bad ? 0LL : (long long)__float2int_rn(t) * 65536LL;
+            if (bad) {                           // rare: the warps' sums one by one
+                constexpr float most = K == 7 ? 4294967040.0f : 2147483520.0f;   // (K = 7: dE/dtheta)
+                bad = false;
+                for (int i = 0; i < nw; ++i) {
+                    const float u = red[i][threadIdx.x] * 65536.0f;
+                    if (fabsf(u) < most) q += __float2ll_rn(u) * 65536LL;
+                    else bad = true;
+                }
+            }
         } else {
             bad = !isfinite(s);
             q = bad ? 0LL : __double2ll_rn(s * kFix);

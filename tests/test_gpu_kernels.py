@@ -546,3 +546,17 @@ def test_scatter_forces_of_very_close_pairs(N, r):
     _, f_o, _, _ = O.sw_energy(x, box)
     # the pair's distance carries 2 units of 16 A 2^-32 (7.6e-9 A) and 2^-23 of itself; the force goes as r^-5
     assert np.abs(f - f_o).max() <= (1e-5 + 5 * 7.6e-9 / r) * np.abs(f_o).max()
+
+
+def test_fp32_sums_out_of_range_for_a_block_but_not_for_its_warps(N):
+    """39,304 atoms of some 690 eV each (eps times 160): 64 atoms of a block exceed the 32,768 eV that an FP32 block
+    sum holds, the 32 of a warp do not (nor does dE/da, some 1500 eV an atom, the 65,536 of its own).  Energy against FP64,
+    1e-5."""
+    x, box = I.diamond(17, 17, 17)
+    x = I.rattle(x, 0.05, 3)
+    p = _silicon(N, eps=160.0)
+    _, ev = _sw(N, x, box, p, N.NEFE_FP32)
+    _, ev64 = _sw(N, x, box, p, N.NEFE_FP64)
+    assert abs(ev[0] - ev64[0]) <= 1e-5 * abs(ev64[0])
+    _, eg = _sw(N, x, box, p, N.NEFE_FP32, grad=True)
+    assert abs(eg[0] - ev64[0]) <= 1e-5 * abs(ev64[0])
