@@ -2490,9 +2490,9 @@ constexpr long long kLegNan = 1LL << 62, kLegLost = 1LL << 61;
 constexpr float kLegRefuse = 48.0f;
 constexpr float kPairOdd = 6.0f;                 // half a pair force above which an own sum could reach kLegRefuse
 
-// Splits a large term: sign times its multiples of kLegCoarse go to atom j; returns the rest.  (FP64: the
-// multiples of a large FP32 value are not FP32 numbers; the rest is one.)
-__device__ __noinline__ float3 split_leg(const Bufs& b, const DevSys& S, int j, int sign, unsigned* err, float x, float y,
+// Splits a large term: sign times its multiples of kLegCoarse go to atom j; returns the rest.  (A count
+// above 2^24 is rounded; what it leaves is split again.  Each remainder is an FP32 number.)
+__device__ __forceinline__ float3 split_leg(const Bufs& b, const DevSys& S, int j, int sign, unsigned* err, float x, float y,
                                          float z) {
     unsigned long long* hi_j = reinterpret_cast<unsigned long long*>(b.lacc_hi + 3 * (size_t)j);
     float v[3] = {x, y, z};
@@ -2503,10 +2503,13 @@ __device__ __noinline__ float3 split_leg(const Bufs& b, const DevSys& S, int j, 
             if (b.leg_refuse) continue;          // (a refused term is left out)
             atomicExch(hi_j + k, (unsigned long long)kLegNan);
         } else {
-            const double h = rint((double)v[k] / (double)kLegCoarse);
-            if (h == 0.0) continue;
-            v[k] = (float)fma(-(double)kLegCoarse, h, (double)v[k]);
-            atomicAdd(hi_j + k, (unsigned long long)(sign * (long long)h));
+            long long n = 0;
+            for (float h = rintf(v[k] / kLegCoarse); h != 0.0f; h = rintf(v[k] / kLegCoarse)) {
+                v[k] = fmaf(-kLegCoarse, h, v[k]);
+                n += (long long)h;
+            }
+            if (n == 0) continue;
+            atomicAdd(hi_j + k, (unsigned long long)(sign * n));
         }
         b.hi_flag[S.tile0 + (j - S.off) / kTile] = 1;
     }
@@ -2630,24 +2633,38 @@ __device__ __forceinline__ LegOut leg_of_edge(const SWc<float>& P, const float4&
     return o;
 }
 
-// Rare: a term that has to be split (or, with refuse, whose triplet part may be refused), from atom i
-// (lane t) to leg atom j.
+// Rare: the edges whose terms have to be split (or, with refuse, whose triplet part may be refused): bit k of
+// `odd` is edge 32 k + lane of the warp's list.  Their terms are computed again here, after the edge loop:
+// a call in the middle of it had the compiler spill (16 to 68 bytes by what was called; 64 pairs 64.9 ms a
+// pass with 16, 67.1 with 68, 63.7 with none).  All lanes of the warp come here; i0: the warp's first atom,
+// Gm: the lane's atom's moment.
 template <bool EATOM>
-__device__ __noinline__ void add_large_leg(const Bufs& b, const DevSys& S, ScatterShared<EATOM>& sh, int refuse, int j, int i,
-                                           int t, float3 l, float3 u, float hp, unsigned* err) {
-    float3 p = l;                                // what the leg atom gets
-    if (refuse && !(fabsf(l.x + hp * u.x) < kLegRefuse && fabsf(l.y + hp * u.y) < kLegRefuse &&
-                    fabsf(l.z + hp * u.z) < kLegRefuse)) {
-        atomicOr(err, NEFE_ERR_NAN);
-        p = make_float3(-hp * u.x, -hp * u.y, -hp * u.z);
+__device__ __forceinline__ void add_large_legs(const Bufs& b, const DevSys& S, const SWc<float>& P, ScatterShared<EATOM>& sh,
+                                            int lane, int i0, unsigned odd, float Gm, unsigned* err) {
+    for (unsigned any = __reduce_or_sync(0xffffffffu, odd); any; any &= any - 1u) {
+        const int k = __ffs(any) - 1, e = 32 * k + lane;
+        const bool on = (odd >> k & 1u) != 0u;
+        const unsigned w = on ? sh.id[e] : 0u;
+        const int t = (int)(w >> kCodeShift), j = (int)(w & kIndexMask), i = i0 + t;
+        const float Gt = __shfl_sync(0xffffffffu, Gm, t);
+        if (!on) continue;
+        const float4 u = sh.u[e];
+        const LegOut o = leg_of_edge(P, u, sh.r[e], sh.mom[0][t], sh.mom[1][t], sh.mom[2][t], Gt);
+        float3 l = make_float3(o.x, o.y, o.z), p = l;    // p: what the leg atom gets
+        if (b.leg_refuse && !(fabsf(l.x + o.hp * u.x) < kLegRefuse && fabsf(l.y + o.hp * u.y) < kLegRefuse &&
+                              fabsf(l.z + o.hp * u.z) < kLegRefuse)) {
+            atomicOr(err, NEFE_ERR_NAN);
+            p = make_float3(-o.hp * u.x, -o.hp * u.y, -o.hp * u.z);
+        }
+        p = split_leg(b, S, j, 1, err, p.x, p.y, p.z);
+        l = split_leg(b, S, i, -1, err, l.x, l.y, l.z);
+        red_force(b.lacc + 4 * (size_t)j, __float2int_rn(p.x * kLegScale), __float2int_rn(p.y * kLegScale),
+                  __float2int_rn(p.z * kLegScale));
+        atomicAdd(&sh.own[0][t], __float2int_rn(l.x * kLegScale));
+        atomicAdd(&sh.own[1][t], __float2int_rn(l.y * kLegScale));
+        atomicAdd(&sh.own[2][t], __float2int_rn(l.z * kLegScale));
     }
-    p = split_leg(b, S, j, 1, err, p.x, p.y, p.z);
-    l = split_leg(b, S, i, -1, err, l.x, l.y, l.z);
-    red_force(b.lacc + 4 * (size_t)j, __float2int_rn(p.x * kLegScale), __float2int_rn(p.y * kLegScale),
-              __float2int_rn(p.z * kLegScale));
-    atomicAdd(&sh.own[0][t], __float2int_rn(l.x * kLegScale));
-    atomicAdd(&sh.own[1][t], __float2int_rn(l.y * kLegScale));
-    atomicAdd(&sh.own[2][t], __float2int_rn(l.z * kLegScale));
+    __syncwarp();
 }
 
 // Rare: takes the own sum of an atom (its pair forces and the recoils of its triplet legs, sum of
@@ -2863,7 +2880,8 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
         }
         __syncwarp();
         // 4. pair terms and leg forces
-        bool odd = false;
+        unsigned odd = 0u;                       // edges whose terms are large (bit e / 32)
+        static_assert(kListEdges <= 32 * 32, "a bit for each turn");
         for (int e0 = 0; e0 < E; e0 += 32) {
             const int e = e0 + lane;
             const bool on = e < E;
@@ -2894,9 +2912,7 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
                 gth[6] += h * o.ida;
             }
             if (!(fabsf(o.x) < kLegFine && fabsf(o.y) < kLegFine && fabsf(o.z) < kLegFine && fabsf(o.hp) < pair_odd)) {
-                odd = true;
-                add_large_leg(b, S, sh, b.leg_refuse, j, i - t + te, te, make_float3(o.x, o.y, o.z),
-                              make_float3(ua.x, ua.y, ua.z), o.hp, &st.err);
+                odd |= 1u << (e0 >> 5);
                 continue;
             }
             const int qx = __float2int_rn(o.x * kLegScale), qy = __float2int_rn(o.y * kLegScale),
@@ -2907,7 +2923,10 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
             atomicAdd(&sh.own[2][te], qz);
         }
         __syncwarp();
-        if (b.leg_refuse && __any_sync(kAll, odd)) refuse_own(b, S, P, sh, lane, G, i, ma, mx, Gm, &st.err);
+        if (__any_sync(kAll, odd != 0u)) {
+            add_large_legs(b, S, P, sh, lane, i - t, odd, Gm, &st.err);
+            if (b.leg_refuse) refuse_own(b, S, P, sh, lane, G, i, ma, mx, Gm, &st.err);
+        }
         if (EATOM) {                             // per-atom energies in slot order
             int base = 0;
             for (int a = 0; a < mx; ++a) {
@@ -3486,7 +3505,8 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
             for (int k = 0; k < 3; ++k) {
                 const long long h = h3[k];
                 h3[k] = 0;
-                if (h >= kLegLost || h <= -kLegLost) f[k] = (T)NAN;
+                if (h == (long long)(int)h) f[k] += (T)kLegCoarse * (T)(int)h;
+                else if (h >= kLegLost || h <= -kLegLost) f[k] = (T)NAN;
                 else f[k] += (T)kLegCoarse * (T)h;
             }
         }
