@@ -173,9 +173,10 @@ NEFE_API int nefe_neighbor_build(const double* x, int n, const double box[3], do
  * nefe_neighbor_build from the same x and box.  FP64 is a gather: the force on i sums the
  * pair terms, the three-body terms centred on i, and the three-body terms centred on each
  * neighbour j in which i is a leg.  FP32 adds the terms of each centre to its atoms in fixed
- * point.  Both are bitwise reproducible.  Terms that are not finite (coincident atoms), or in FP32 of
- * 2.5e17 eV/A and more, give NaN forces; energy_virial is NaN where a sum is not finite, or in FP32
- * where that of a warp's atoms (at most 32) reaches 32768 eV.
+ * point (units of 2^-22 eV/A for silicon, finer or coarser by the power of two nearest to the ratio of
+ * eps/sigma).  Both are bitwise reproducible.  Terms that are not finite (coincident atoms), or in FP32
+ * of 2.5e17 eV/A and more at silicon's unit, give NaN forces; energy_virial is NaN where a sum is not
+ * finite, or in FP32 where that of a warp's atoms (at most 32) reaches 32768 eV.
  *   x, n, box, rcs, nbr, cnt, cap   as nefe_neighbor_build (same values).
  *   prm         host, potential parameters (prm->a * prm->sigma <= rcs).
  *   precision   NEFE_FP32 or NEFE_FP64 pair/triplet arithmetic.

@@ -162,6 +162,7 @@ int commit1(Scratch1& S, int n, const double box[3], double rcs, const int n3[3]
     if (prm && prec == NEFE_FP32) {
         const SWc<float> c = make_swc<float>(*prm);
         std::memcpy(sw.b, &c, sizeof(c));
+        hs.leg_unit_f = 1.0f / c.leg_scale;
     }
     NEFE_CU(S.commit());
     const int nacc = 2 * ACC_N * kSlots;

@@ -369,6 +369,7 @@ int setup(nefe_ctx* c) {
         d.amp_f = (float)d.amp; d.gam_f = (float)d.gam; d.ckick_f = (float)d.ckick;
         d.mass_f = (float)d.mass_e; d.kE_f = (float)d.k_E; d.kint_f = (float)d.k_int;
         d.dt_f = (float)c->dt;
+        d.leg_unit_f = 1.0f / make_swc<float>(h.prm).leg_scale;
         d.inv_n_f = (float)(1.0 / h.n);
         d.rcs2_lo_f = (float)(rcs * rcs) * (1.0f - 1e-4f);
         d.rcs2_hi_f = (float)(rcs * rcs) * (1.0f + 1e-4f);

@@ -63,6 +63,14 @@ inline void set_grid(DevState& st, const double box[3], const int n3[3]) {
     st.nbuild = 1;
 }
 
+// Power of two by which the scatter form's force unit is finer than silicon's (eps/sigma = 1.035, in
+// the middle of an octave, so that fitted parameters keep the unit).
+inline int leg_power(const nefe_sw_params& p) {
+    const double force = p.eps / p.sigma * (1.4142135623730951 / 1.035);
+    const int k = force > 0.0 && std::isfinite(force) ? -std::ilogb(force) : 0;
+    return k < -60 ? -60 : (k > 60 ? 60 : k);
+}
+
 template <typename T>
 inline SWc<T> make_swc(const nefe_sw_params& p) {
     SWc<T> c{};
@@ -92,6 +100,8 @@ inline SWc<T> make_swc(const nefe_sw_params& p) {
     const double ract = (double)c.s_act * p.sigma;
     c.act2 = (T)(ract * ract < rc * rc ? ract * ract : rc * rc);
     c.int_pq = (p.p == 4.0 && p.q == 0.0) ? 1 : 0;
+    c.leg_scale = (T)std::ldexp(kLegScale, leg_power(p));
+    c.leg_fine = (T)std::ldexp(kLegFine, -leg_power(p));
     return c;
 }
 

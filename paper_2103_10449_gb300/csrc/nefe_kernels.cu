@@ -2467,14 +2467,17 @@ __global__ void __launch_bounds__(kEdges1Threads, 16) k_edges1(Bufs b) {
 // ------------------------------------------------------------------------------------
 // Scatter form of the force passes (FP32): pass A adds the force that each atom's terms exert on
 // each leg atom, and minus their sum on the atom itself, into per-atom int32 accumulators (units of
-// 2^-22 eV/A) with global reductions.  Integer addition is associative, so the result does not
+// 2^-22 eV/A for silicon) with global reductions.  Integer addition is associative, so the result does not
 // depend on the order in which the reductions arrive (bitwise reproducible), and no second pass has
 // to find the legs again: a streaming epilogue (k_finish) reads and clears each accumulator.
 // The x and y terms travel in one 64-bit reduction as y 2^32 + x (two's complement, modulo
 // 2^64): integer addition is linear, so the 64-bit word accumulates Y 2^32 + X exactly, X and Y
 // being the int32 sums.  Its low word is X; its high word is Y - 1 when X < 0 (the borrow), which
 // the reader undoes (force_of_acc).  Two reductions per force instead of three.
-// A term of kLegFine eV/A or more is split: its multiples of kLegCoarse go to a second accumulator
+// The unit follows the potential: 2^-22 eV/A times a power of two near (eps/sigma) / (silicon's), see
+// leg_power, so that the rounding is relative to the potential's own forces (with eps a hundredth of
+// silicon's a fixed unit left 2e-5 of the largest force).  In these units:
+// a term of kLegFine eV/A or more is split: its multiples of kLegCoarse go to a second accumulator
 // (int64, one count per multiple) and the rest, at most 7 eV/A, stays; up to 64 rests (32 legs, 32 own
 // edges) fit the int32 sum.  The second accumulator is read only for tiles whose flag says that
 // something was added (at 1000 K some atom of a system of thousands has such a term on most steps,
@@ -2482,8 +2485,6 @@ __global__ void __launch_bounds__(kEdges1Threads, 16) k_edges1(Bufs b) {
 // count to kLegNan, from which no sum of counts (64 terms of up to 2^54) comes back below kLegLost:
 // the force is NaN, as a floating-point sum would have it.
 // ------------------------------------------------------------------------------------
-constexpr float kLegScale = 4194304.0f;          // 2^22
-constexpr float kLegFine = 8.0f;
 constexpr float kLegCoarse = 14.0f;
 constexpr float kLegMax = 14.0f * 18014398509481984.0f;   // 14 2^54
 constexpr long long kLegNan = 1LL << 62, kLegLost = 1LL << 61;
@@ -2656,8 +2657,9 @@ __device__ __forceinline__ void add_large_legs(const Bufs& b, const DevSys& S, c
             atomicOr(err, NEFE_ERR_NAN);
             p = make_float3(-o.hp * u.x, -o.hp * u.y, -o.hp * u.z);
         }
-        p = split_leg(b, S, j, 1, err, p.x, p.y, p.z);
-        l = split_leg(b, S, i, -1, err, l.x, l.y, l.z);
+        const float unit = P.leg_scale / kLegScale;
+        p = split_leg(b, S, j, 1, err, p.x * unit, p.y * unit, p.z * unit);
+        l = split_leg(b, S, i, -1, err, l.x * unit, l.y * unit, l.z * unit);
         red_force(b.lacc + 4 * (size_t)j, __float2int_rn(p.x * kLegScale), __float2int_rn(p.y * kLegScale),
                   __float2int_rn(p.z * kLegScale));
         atomicAdd(&sh.own[0][t], __float2int_rn(l.x * kLegScale));
@@ -2693,7 +2695,8 @@ __device__ __noinline__ void refuse_own(const Bufs& b, const DevSys& S, const SW
     }
     if (lane < G && !(fabsf(ox) < kLegRefuse && fabsf(oy) < kLegRefuse && fabsf(oz) < kLegRefuse)) {
         atomicOr(err, NEFE_ERR_NAN);
-        const float3 o = split_leg(b, S, i, -1, err, ox, oy, oz);
+        const float unit = P.leg_scale / kLegScale;
+        const float3 o = split_leg(b, S, i, -1, err, ox * unit, oy * unit, oz * unit);
         sh.own[0][t] += __float2int_rn(o.x * kLegScale);
         sh.own[1][t] += __float2int_rn(o.y * kLegScale);
         sh.own[2][t] += __float2int_rn(o.z * kLegScale);
@@ -2795,6 +2798,7 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
     float en = 0.0f;
     int mtrue = 0;                               // edges of the lane inside the cutoff
     const float pair_odd = b.leg_refuse ? kPairOdd : INFINITY;
+    const float fine = b.leg_refuse ? fminf(P.leg_fine, kLegFine) : P.leg_fine;   // (a refusal is in eV/A)
     int4* spos = reinterpret_cast<int4*>(&sh.mom[0][0]);
     sh.own[0][lane] = 0; sh.own[1][lane] = 0; sh.own[2][lane] = 0;
     for (int done = 0; done < total;) {
@@ -2911,12 +2915,12 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
                 gth[5] += 0.5f * P.eps * ua.w * o.s3;
                 gth[6] += h * o.ida;
             }
-            if (!(fabsf(o.x) < kLegFine && fabsf(o.y) < kLegFine && fabsf(o.z) < kLegFine && fabsf(o.hp) < pair_odd)) {
+            if (!(fabsf(o.x) < fine && fabsf(o.y) < fine && fabsf(o.z) < fine && fabsf(o.hp) < pair_odd)) {
                 odd |= 1u << (e0 >> 5);
                 continue;
             }
-            const int qx = __float2int_rn(o.x * kLegScale), qy = __float2int_rn(o.y * kLegScale),
-                      qz = __float2int_rn(o.z * kLegScale);
+            const int qx = __float2int_rn(o.x * P.leg_scale), qy = __float2int_rn(o.y * P.leg_scale),
+                      qz = __float2int_rn(o.z * P.leg_scale);
             red_force(b.lacc + 4 * (size_t)j, qx, qy, qz);
             atomicAdd(&sh.own[0][te], qx);
             atomicAdd(&sh.own[1][te], qy);
@@ -3496,18 +3500,19 @@ __global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
         else q = make_int4(0, 0, 0, 0);
         const T pd[3] = {d0.x + dh[0] + dl[0], d0.y + dh[1] + dl[1], d0.z + dh[2] + dl[2]};
         const T pz[3] = {z.x, z.y, z.z};
-        const T inv = (T)(1.0 / (double)kLegScale);
+        const T inv = (T)S.leg_unit_f;
         const int3 fq = force_of_acc(q);
         T f[3] = {(T)fq.x * inv, (T)fq.y * inv, (T)fq.z * inv};
         if (sw && big != 0) {
             long long* h3 = b.lacc_hi + 3 * (size_t)i;
+            const T coarse = (T)(kLegCoarse * kLegScale) * inv;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const long long h = h3[k];
                 h3[k] = 0;
-                if (h == (long long)(int)h) f[k] += (T)kLegCoarse * (T)(int)h;
+                if (h == (long long)(int)h) f[k] += coarse * (T)(int)h;
                 else if (h >= kLegLost || h <= -kLegLost) f[k] = (T)NAN;
-                else f[k] += (T)kLegCoarse * (T)h;
+                else f[k] += coarse * (T)h;
             }
         }
         T vo[3], Fo[3];

@@ -560,3 +560,26 @@ def test_fp32_sums_out_of_range_for_a_block_but_not_for_its_warps(N):
     assert abs(ev[0] - ev64[0]) <= 1e-5 * abs(ev64[0])
     _, eg = _sw(N, x, box, p, N.NEFE_FP32, grad=True)
     assert abs(eg[0] - ev64[0]) <= 1e-5 * abs(ev64[0])
+
+
+@pytest.mark.parametrize("scale", [1e-8, 1e-4, 1e-2, 0.5, 2.0, 100.0])
+def test_scatter_forces_of_weak_and_strong_potentials(N, scale):
+    """The FP32 tolerance is relative (1e-5 of the largest force) whatever the unit of energy, in a stateless call
+    and in a context (velocity after one step from rest, FP64 against FP32)."""
+    x, box = I.diamond(3, 3, 3)
+    x = I.rattle(x, 0.1, 8)
+    f, _ = _sw(N, x, box, _silicon(N, eps=scale), N.NEFE_FP32)
+    _, f_o, _, _ = O.sw_energy(x, box)
+    assert np.abs(f / scale - f_o).max() <= 1e-5 * np.abs(f_o).max()
+    v = []
+    for precision in (N.NEFE_FP32, N.NEFE_FP64):
+        ctx = N.Context(precision=precision, skin=0.5, nbr_cap=48)
+        for k in (scale, 1.0):                           # two potentials in one context
+            s = ctx.add_system(x, box, v=np.zeros_like(x), mass=28.0855 * k)
+            ctx.set_sw_params(s, _silicon(N, eps=k))
+        ctx.run(1)
+        assert all(ctx.results(s)["error"] == 0 for s in range(2))
+        v.append([ctx.get_state(s)[1] for s in range(2)])
+        ctx.close()
+    for a, b in zip(*v):
+        assert np.abs(a - b).max() <= 1e-5 * np.abs(b).max()
