@@ -2478,7 +2478,7 @@ __global__ void __launch_bounds__(kEdges1Threads, 16) k_edges1(Bufs b) {
 // leg_power, so that the rounding is relative to the potential's own forces (with eps a hundredth of
 // silicon's a fixed unit left 2e-5 of the largest force).  In these units:
 // a term of kLegFine eV/A or more is split: its multiples of kLegCoarse go to a second accumulator
-// (int64, one count per multiple) and the rest, at most 7 eV/A, stays; up to 64 rests (32 legs, 32 own
+// (int64, one count per multiple) and the rest, at most 7.5 eV/A, stays; up to 64 rests (32 legs, 32 own
 // edges) fit the int32 sum.  The second accumulator is read only for tiles whose flag says that
 // something was added (at 1000 K some atom of a system of thousands has such a term on most steps,
 // but few tiles do).  A term that is not finite, or of kLegMax (2.5e17 eV/A) and more, sets the atom's
@@ -2491,30 +2491,29 @@ constexpr long long kLegNan = 1LL << 62, kLegLost = 1LL << 61;
 constexpr float kLegRefuse = 48.0f;
 constexpr float kPairOdd = 6.0f;                 // half a pair force above which an own sum could reach kLegRefuse
 
-// Splits a large term: sign times its multiples of kLegCoarse go to atom j; returns the rest.  (A count
-// above 2^24 is rounded; what it leaves is split again.  Each remainder is an FP32 number.)
-__device__ __forceinline__ float3 split_leg(const Bufs& b, const DevSys& S, int j, int sign, unsigned* err, float x, float y,
-                                         float z) {
-    unsigned long long* hi_j = reinterpret_cast<unsigned long long*>(b.lacc_hi + 3 * (size_t)j);
-    float v[3] = {x, y, z};
-    for (int k = 0; k < 3; ++k) {
-        if (!(fabsf(v[k]) < kLegMax)) {
-            atomicOr(err, NEFE_ERR_NAN);
-            v[k] = 0.0f;
-            if (b.leg_refuse) continue;          // (a refused term is left out)
-            atomicExch(hi_j + k, (unsigned long long)kLegNan);
-        } else {
-            long long n = 0;
-            for (float h = rintf(v[k] / kLegCoarse); h != 0.0f; h = rintf(v[k] / kLegCoarse)) {
-                v[k] = fmaf(-kLegCoarse, h, v[k]);
-                n += (long long)h;
-            }
-            if (n == 0) continue;
-            atomicAdd(hi_j + k, (unsigned long long)(sign * n));
-        }
-        b.hi_flag[S.tile0 + (j - S.off) / kTile] = 1;
+// Splits a large term into n multiples of kLegCoarse and the rest (n = kLegNan: out of range or not
+// finite).  A count above 2^24 is rounded; what it leaves is split again.  Each remainder is an FP32
+// number, and the last is at most 7.5.
+__device__ __forceinline__ float split_term(float v, long long& n) {
+    n = 0;
+    if (!(fabsf(v) < kLegMax)) {
+        n = kLegNan;
+        return 0.0f;
     }
-    return make_float3(v[0], v[1], v[2]);
+    while (fabsf(v) > 7.5f) {
+        const float h = rintf(v * (1.0f / kLegCoarse));
+        v = fmaf(-kLegCoarse, h, v);
+        n += fabsf(h) < 1e9f ? (long long)(int)h : (long long)h;
+    }
+    return v;
+}
+
+// n multiples of kLegCoarse for component k of atom j.
+__device__ __forceinline__ void add_count(const Bufs& b, const DevSys& S, int j, int k, long long n) {
+    unsigned long long* hi = reinterpret_cast<unsigned long long*>(b.lacc_hi + 3 * (size_t)j) + k;
+    if (n == kLegNan || n == -kLegNan) atomicExch(hi, (unsigned long long)kLegNan);
+    else atomicAdd(hi, (unsigned long long)n);
+    b.hi_flag[S.tile0 + (j - S.off) / kTile] = 1;
 }
 
 __device__ __forceinline__ void red_force(int* acc4, int x, int y, int z) {
@@ -2634,37 +2633,52 @@ __device__ __forceinline__ LegOut leg_of_edge(const SWc<float>& P, const float4&
     return o;
 }
 
-// Rare: the edges whose terms have to be split (or, with refuse, whose triplet part may be refused): bit k of
-// `odd` is edge 32 k + lane of the warp's list.  Their terms are computed again here, after the edge loop:
-// a call in the middle of it had the compiler spill (16 to 68 bytes by what was called; 64 pairs 64.9 ms a
-// pass with 16, 67.1 with 68, 63.7 with none).  All lanes of the warp come here; i0: the warp's first atom,
-// Gm: the lane's atom's moment.
+// Rare: the edges whose terms have to be split (or, with leg_refuse, whose triplet part may be refused): bit k
+// of `odd` is edge 32 k + lane of the warp's list.  This comes after the edge loop, which leaves the force in
+// sh.u (leg_refuse: it is computed again): a call in the middle of the loop had the compiler spill (16 to 68
+// bytes by what was called; 64 pairs 64.9 ms a pass with 16, 67.1 with 68, 63.7 with none).  All lanes
+// of the warp come here; i0: the warp's first atom, Gm: the lane's atom's moment.
 template <bool EATOM>
 __device__ __forceinline__ void add_large_legs(const Bufs& b, const DevSys& S, const SWc<float>& P, ScatterShared<EATOM>& sh,
                                             int lane, int i0, unsigned odd, float Gm, unsigned* err) {
+    const float unit = P.leg_scale / kLegScale;
     for (unsigned any = __reduce_or_sync(0xffffffffu, odd); any; any &= any - 1u) {
-        const int k = __ffs(any) - 1, e = 32 * k + lane;
-        const bool on = (odd >> k & 1u) != 0u;
+        const int q = __ffs(any) - 1, e = 32 * q + lane;
+        const bool on = (odd >> q & 1u) != 0u;
         const unsigned w = on ? sh.id[e] : 0u;
         const int t = (int)(w >> kCodeShift), j = (int)(w & kIndexMask), i = i0 + t;
         const float Gt = __shfl_sync(0xffffffffu, Gm, t);
         if (!on) continue;
         const float4 u = sh.u[e];
-        const LegOut o = leg_of_edge(P, u, sh.r[e], sh.mom[0][t], sh.mom[1][t], sh.mom[2][t], Gt);
-        float3 l = make_float3(o.x, o.y, o.z), p = l;    // p: what the leg atom gets
-        if (b.leg_refuse && !(fabsf(l.x + o.hp * u.x) < kLegRefuse && fabsf(l.y + o.hp * u.y) < kLegRefuse &&
-                              fabsf(l.z + o.hp * u.z) < kLegRefuse)) {
-            atomicOr(err, NEFE_ERR_NAN);
-            p = make_float3(-o.hp * u.x, -o.hp * u.y, -o.hp * u.z);
+        float l[3] = {u.x, u.y, u.z}, p[3];      // p: what the leg atom gets
+        bool same = true;
+        if (b.leg_refuse) {
+            const LegOut o = leg_of_edge(P, u, sh.r[e], sh.mom[0][t], sh.mom[1][t], sh.mom[2][t], Gt);
+            l[0] = o.x; l[1] = o.y; l[2] = o.z;
+            same = fabsf(o.x + o.hp * u.x) < kLegRefuse && fabsf(o.y + o.hp * u.y) < kLegRefuse &&
+                   fabsf(o.z + o.hp * u.z) < kLegRefuse;
+            p[0] = -o.hp * u.x; p[1] = -o.hp * u.y; p[2] = -o.hp * u.z;
+            if (!same) atomicOr(err, NEFE_ERR_NAN);
         }
-        const float unit = P.leg_scale / kLegScale;
-        p = split_leg(b, S, j, 1, err, p.x * unit, p.y * unit, p.z * unit);
-        l = split_leg(b, S, i, -1, err, l.x * unit, l.y * unit, l.z * unit);
-        red_force(b.lacc + 4 * (size_t)j, __float2int_rn(p.x * kLegScale), __float2int_rn(p.y * kLegScale),
-                  __float2int_rn(p.z * kLegScale));
-        atomicAdd(&sh.own[0][t], __float2int_rn(l.x * kLegScale));
-        atomicAdd(&sh.own[1][t], __float2int_rn(l.y * kLegScale));
-        atomicAdd(&sh.own[2][t], __float2int_rn(l.z * kLegScale));
+        int ql[3], qp[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            long long nl, np;
+            ql[k] = qp[k] = __float2int_rn(split_term(l[k] * unit, nl) * kLegScale);
+            np = nl;
+            if (!same) qp[k] = __float2int_rn(split_term(p[k] * unit, np) * kLegScale);
+            if (nl == kLegNan || np == kLegNan) {
+                atomicOr(err, NEFE_ERR_NAN);
+                if (b.leg_refuse) {              // (a refused term is left out)
+                    nl = nl == kLegNan ? 0 : nl;
+                    np = np == kLegNan ? 0 : np;
+                }
+            }
+            if (np) add_count(b, S, j, k, np);
+            if (nl) add_count(b, S, i, k, -nl);
+            atomicAdd(&sh.own[k][t], ql[k]);
+        }
+        red_force(b.lacc + 4 * (size_t)j, qp[0], qp[1], qp[2]);
     }
     __syncwarp();
 }
@@ -2695,11 +2709,12 @@ __device__ __noinline__ void refuse_own(const Bufs& b, const DevSys& S, const SW
     }
     if (lane < G && !(fabsf(ox) < kLegRefuse && fabsf(oy) < kLegRefuse && fabsf(oz) < kLegRefuse)) {
         atomicOr(err, NEFE_ERR_NAN);
-        const float unit = P.leg_scale / kLegScale;
-        const float3 o = split_leg(b, S, i, -1, err, ox * unit, oy * unit, oz * unit);
-        sh.own[0][t] += __float2int_rn(o.x * kLegScale);
-        sh.own[1][t] += __float2int_rn(o.y * kLegScale);
-        sh.own[2][t] += __float2int_rn(o.z * kLegScale);
+        const float unit = P.leg_scale / kLegScale, o[3] = {ox * unit, oy * unit, oz * unit};
+        for (int k = 0; k < 3; ++k) {
+            long long n;
+            sh.own[k][t] += __float2int_rn(split_term(o[k], n) * kLegScale);
+            if (n && n != kLegNan) add_count(b, S, i, k, -n);
+        }
     }
     __syncwarp();
 }
@@ -2917,6 +2932,7 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
             }
             if (!(fabsf(o.x) < fine && fabsf(o.y) < fine && fabsf(o.z) < fine && fabsf(o.hp) < pair_odd)) {
                 odd |= 1u << (e0 >> 5);
+                if (!b.leg_refuse) sh.u[e] = make_float4(o.x, o.y, o.z, 0.0f);
                 continue;
             }
             const int qx = __float2int_rn(o.x * P.leg_scale), qy = __float2int_rn(o.y * P.leg_scale),
