@@ -219,14 +219,14 @@ static void want_forces(Scratch1& S, int n, int precision) {
 // Both force passes of a stateless call.  FP64 pass B: one lane per atom from kGatherOne atoms on (its
 // epilogue runs on one lane per atom, so more lanes cost FP64 issue; fewer atoms want shorter chains).
 constexpr int kGatherOne = 20000;
-static int run_forces(const Scratch1& S, Bufs& b, int n, const nefe_sw_params* prm, int precision) {
+static int run_forces(const Scratch1& S, Bufs& b, int n, const double box[3], const nefe_sw_params* prm, int precision) {
     const int ntiles = (n + kTile - 1) / kTile;
     b.xc = S.xc; b.lscale = S.lscale;
     b.row4 = (b.cap & 3) == 0 && (reinterpret_cast<uintptr_t>(b.nbr) & 15) == 0;
     set_edge_items(b, precision, atoms_per_warp_log2(precision, n), ntiles);
     b.common = 1;
     if (precision == NEFE_FP32) {
-        b.xf = S.xf; b.lacc = S.lacc; b.lacc_hi = S.lacc_hi; b.hi_flag = S.hi_flag;
+        b.xf = S.xf; b.want_xf = 1 + frac_fine(box); b.lacc = S.lacc; b.lacc_hi = S.lacc_hi; b.hi_flag = S.hi_flag;
         b.swc_common = make_swc<float>(*prm);
         NEFE_CU(cudaMemsetAsync(S.lacc, 0, (size_t)(reinterpret_cast<char*>(S.hi_flag + ntiles) - reinterpret_cast<char*>(S.lacc)),
                                 S.s));
@@ -339,7 +339,7 @@ int nefe_sw_forces(const double* x, int n, const double box[3], double rcs, cons
         Bufs b = bufs_of(S, x, n);
         b.nbr = const_cast<int*>(nbr); b.cnt = const_cast<int*>(cnt); b.cap = cap;
         b.f_out = f; b.e_atom = e_atom;
-        if ((rc = run_forces(S, b, n, prm, precision))) return rc;
+        if ((rc = run_forces(S, b, n, box, prm, precision))) return rc;
     }
     if (energy_virial) launch_decode_ev(S.acc, energy_virial, &S.st->err, S.s);
     NEFE_CU(cudaGetLastError());
@@ -376,7 +376,7 @@ int nefe_sw_energy_grad(const double* x, int n, const double box[3], double rcs,
         Bufs b = bufs_of(S, x, n);
         b.nbr = const_cast<int*>(nbr); b.cnt = const_cast<int*>(cnt); b.cap = cap;
         b.f_out = fo; b.e_atom = nullptr; b.want_grad = 1;
-        if ((rc = run_forces(S, b, n, prm, precision))) return rc;
+        if ((rc = run_forces(S, b, n, box, prm, precision))) return rc;
     }
     launch_decode_grad(S.acc, energy_grad, S.s);
     NEFE_CU(cudaGetLastError());
@@ -425,7 +425,7 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
         Bufs b = bufs_of(S, x, n);
         b.uf_nbr = uf_nbr; b.uf_cnt = uf_cnt; b.uf_tiles = nullptr;
         b.xf = b.xfb = S.xf; b.xc = S.xc; b.lscale = S.lscale;
-        b.want_xf = precision == NEFE_FP32 ? 1 : 0;
+        b.want_xf = precision == NEFE_FP32 ? 1 + frac_fine(box) : 0;
         b.f_out = f; b.e_atom = e_atom;
         const int ntiles = (n + kTile - 1) / kTile;
         launch_cells(b, precision, ntiles, 1, 1, S.s, nullptr);

@@ -46,6 +46,10 @@ enum Baro { BARO_NONE = 0, BARO_ISO = 1, BARO_ANISO = 2 };
 constexpr float kLegScale = 4194304.0f;   // accumulator units per eV/A: 2^22
 constexpr float kLegFine = 8.0f;          // terms from here on are split (eV/A)
 
+// FP32: longest box whose fractional positions do with 32 bits an axis (A).  At 1024 A half a unit is
+// 1.2e-7 A, what an FP32 coordinate within a cell of 2 to 4 A is rounded by.
+constexpr double kFracCoarse = 1024.0;
+
 // Potential constants in the precision of the force kernel.
 template <typename T>
 struct SWc {

@@ -164,12 +164,20 @@ int not_ready(nefe_ctx* c, const char* what) {
 
 double rc_of(const HostSys& h) { return h.prm.a * h.prm.sigma; }
 
+// Bufs::want_xf where fractional positions are wanted.
+int frac_form(const nefe_ctx* c) {
+    int fine = 0;
+    if (c->prec == NEFE_FP32)
+        for (const HostSys& h : c->sys) fine |= frac_fine(h.box);
+    return 1 + fine;
+}
+
 // Pass A's form, and the positions that the kernels of that form read.
 void set_form(nefe_ctx* c, int lanes) {
     c->lanes = lanes;
     const bool scatter = c->prec == NEFE_FP32 && lanes == 0;
     // (the Uhlenbeck-Ford kernel reads fractions in FP32)
-    const int xf = scatter || c->prec == NEFE_FP64 || c->n_uf_tiles > 0 ? 1 : 0, xs = !scatter ? 1 : 0;
+    const int xf = scatter || c->prec == NEFE_FP64 || c->n_uf_tiles > 0 ? frac_form(c) : 0, xs = !scatter ? 1 : 0;
     // FP64: 8, 16, 32 lanes per atom set by hand stand for 16, 8, 4 atoms per warp
     set_edge_items(c->b, c->prec, c->prec == NEFE_FP64 && c->chosen ? (lanes <= 8 ? 4 : lanes == 16 ? 3 : 2) : atoms_per_warp_log2(c->prec, c->ntot),
                    c->ntiles);
@@ -1130,7 +1138,8 @@ int nefe_autotune(nefe_ctx* c) {
     c->b.leg_refuse = 1;
     Bufs b = c->b;
     if (c->prec == NEFE_FP32) {                  // every form is timed: both kinds of positions
-        b.want_xf = b.want_xs = 1;
+        b.want_xf = frac_form(c);
+        b.want_xs = 1;
         launch_positions(b, c->prec, c->ntiles, c->stream, &c->launches);
     }
     b.acc = c->d_acc_tmp;

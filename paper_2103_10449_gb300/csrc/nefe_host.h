@@ -63,6 +63,8 @@ inline void set_grid(DevState& st, const double box[3], const int n3[3]) {
     st.nbuild = 1;
 }
 
+inline int frac_fine(const double box[3]) { return std::fmax(box[0], std::fmax(box[1], box[2])) > kFracCoarse ? 1 : 0; }
+
 // Power of two by which the scatter form's force unit is finer than silicon's (eps/sigma = 1.035, in
 // the middle of an octave, so that fitted parameters keep the unit).
 inline int leg_power(const nefe_sw_params& p) {

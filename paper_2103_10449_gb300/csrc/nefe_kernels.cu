@@ -400,9 +400,39 @@ __device__ __forceinline__ uint2 pack_frac(const int4& f) {
     return make_uint2(y << 22 | z << 1, x << 11 | y >> 10);     // (lo, hi)
 }
 
-// Fractional position of x in the box of the last list build (frac32).
-__device__ __forceinline__ int4 frac_position(const double (&x)[3], const DevState& st) {
+// Fractional position of x in the box of the last list build (frac32).  A resolution of L 2^-32 is
+// finer than an FP32 coordinate within a cell up to some 1000 A; in longer boxes (fine) the next ten
+// bits of each axis are kept in .w, ten apiece.
+__device__ __forceinline__ int4 frac_position(const double (&x)[3], const DevState& st, int fine) {
+    if (fine) {
+        const long long a = frac42(x[0], st.ibox[0]), b = frac42(x[1], st.ibox[1]), c = frac42(x[2], st.ibox[2]);
+        constexpr int mask = (1 << kFracLow) - 1;
+        return make_int4((int)(unsigned)(a >> kFracLow), (int)(unsigned)(b >> kFracLow), (int)(unsigned)(c >> kFracLow),
+                         ((int)a & mask) | ((int)b & mask) << kFracLow | ((int)c & mask) << 2 * kFracLow);
+    }
     return make_int4(frac32(x[0], st.ibox[0]), frac32(x[1], st.ibox[1]), frac32(x[2], st.ibox[2]), 0);
+}
+// fb moved by (tx, ty, tz) units of 2^-32.
+__device__ __forceinline__ int4 frac_moved(const int4& fb, float tx, float ty, float tz, int fine) {
+    int4 f = make_int4(fb.x + __float2int_rn(tx), fb.y + __float2int_rn(ty), fb.z + __float2int_rn(tz), 0);
+    if (fine) {
+        constexpr int mask = (1 << kFracLow) - 1;
+        const auto low = [&](float t, int axis, int& hi) {
+            const int v = ((fb.w >> axis * kFracLow) & mask) + __float2int_rn((t - rintf(t)) * (float)(mask + 1));
+            hi += v >> kFracLow;
+            f.w |= (v & mask) << axis * kFracLow;
+        };
+        low(tx, 0, f.x); low(ty, 1, f.y); low(tz, 2, f.z);
+    }
+    return f;
+}
+// What the low bits (of fine positions) add to the difference j - i, in units of 2^-32.
+__device__ __forceinline__ float3 frac_low_diff(int wj, int wi) {
+    constexpr int mask = (1 << kFracLow) - 1;
+    constexpr float unit = 1.0f / (mask + 1);
+    return make_float3(unit * (float)((wj & mask) - (wi & mask)),
+                       unit * (float)((wj >> kFracLow & mask) - (wi >> kFracLow & mask)),
+                       unit * (float)((wj >> 2 * kFracLow & mask) - (wi >> 2 * kFracLow & mask)));
 }
 
 // The four rows of system s in lscale: L 2^-32 as FP32 value and remainder (what the fractional positions
@@ -465,7 +495,7 @@ __device__ void cells_count_tile(const Bufs& b, int tile, int th) {
     if (b.xfb && b.want_xf) {
         if (i == S.off) scale_of_box(b, ta.sys, st);
         const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
-        const int4 f = frac_position(x3, st);
+        const int4 f = frac_position(x3, st, b.want_xf > 1);
         if (b.xf) b.xf[i] = f;
         b.xfb[i] = f;
         b.xc[i] = pack_frac(f);
@@ -1688,7 +1718,7 @@ __device__ __forceinline__ void uf_pair(double xx, double pk, double c0, double&
 template <typename T> constexpr int kUfLanes = sizeof(T) == 8 ? 4 : 8;
 template <typename T> constexpr int kUfThreads = sizeof(T) == 8 ? 4 * kTile : kTile;
 template <typename T> constexpr int kUfBlocks = kTile * kUfLanes<T> / kUfThreads<T>;   // per tile
-template <typename T, int MODE>
+template <typename T, int MODE, bool FINE>
 __global__ void __launch_bounds__(kUfThreads<T>, sizeof(T) == 4 ? 5 : 1) k_uf(Bufs b) {
     dep_wait();
     using T4 = typename V4<T>::t;
@@ -1756,7 +1786,11 @@ __global__ void __launch_bounds__(kUfThreads<T>, sizeof(T) == 4 ? 5 : 1) k_uf(Bu
             if (!NEFE_IN_RANGE(e & kUfMask, b.ntot, &st.err)) continue;
             T dx, dy, dz;
             if constexpr (kFrac) {
-                const float gx = (float)(xj.x - fi.x), gy = (float)(xj.y - fi.y), gz = (float)(xj.z - fi.z);
+                float gx = (float)(xj.x - fi.x), gy = (float)(xj.y - fi.y), gz = (float)(xj.z - fi.z);
+                if constexpr (FINE) {
+                    const float3 g = frac_low_diff(xj.w, fi.w);
+                    gx += g.x; gy += g.y; gz += g.z;
+                }
                 dx = gx * Lh.x + gx * Ll.x; dy = gy * Lh.y + gy * Ll.y; dz = gz * Lh.z + gz * Ll.z;
             } else {
                 const T4 oh = soff[e >> kUfShift];
@@ -1847,7 +1881,7 @@ __global__ void __launch_bounds__(kTile) k_mirror(Bufs b) {
     if (b.xc) {
         const size_t N = b.ntot;
         const double x3[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
-        b.xc[i] = pack_frac(frac_position(x3, st));
+        b.xc[i] = pack_frac(frac_position(x3, st, 0));
         if (i == 0) scale_of_box(b, 0, st);
     }
 }
@@ -1915,8 +1949,7 @@ __device__ __forceinline__ T place_atom(const Bufs& b, const DevState& st, const
                 mv[k] = (float)d[k];
                 if (hmoved) mv[k] = fmaf(fmaf((float)qa[k], st.hb_f[k], (float)xav[k]), bm.omr[k], mv[k]);
             }
-            b.xc[i] = pack_frac(make_int4(fb.x + __float2int_rn(mv[0] * bm.to_frac[0]), fb.y + __float2int_rn(mv[1] * bm.to_frac[1]),
-                                          fb.z + __float2int_rn(mv[2] * bm.to_frac[2]), 0));
+            b.xc[i] = pack_frac(frac_moved(fb, mv[0] * bm.to_frac[0], mv[1] * bm.to_frac[1], mv[2] * bm.to_frac[2], 0));
         }
     } else {
         T mv[3];
@@ -1927,9 +1960,8 @@ __device__ __forceinline__ T place_atom(const Bufs& b, const DevState& st, const
             dd2 += mv[k] * mv[k];
         }
         if (b.want_xf) {
-            const int4 f = make_int4(fb.x + __float2int_rn(mul_rn(mv[0], bm.to_frac[0])),
-                                     fb.y + __float2int_rn(mul_rn(mv[1], bm.to_frac[1])),
-                                     fb.z + __float2int_rn(mul_rn(mv[2], bm.to_frac[2])), 0);
+            const int4 f = frac_moved(fb, mul_rn(mv[0], bm.to_frac[0]), mul_rn(mv[1], bm.to_frac[1]),
+                                      mul_rn(mv[2], bm.to_frac[2]), b.want_xf > 1);
             b.xf[i] = f;
             b.xc[i] = pack_frac(f);
         }
@@ -2018,7 +2050,7 @@ __global__ void __launch_bounds__(kTile) k_positions(Bufs b) {
     int4 fb = make_int4(0, 0, 0, 0);
     if (b.want_xf) {
         const double x[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
-        b.xfb[i] = fb = frac_position(x, st);
+        b.xfb[i] = fb = frac_position(x, st, b.want_xf > 1);
     }
     T d[3];
     for (int k = 0; k < 3; ++k) {
@@ -2773,7 +2805,8 @@ __device__ __forceinline__ void mark_row(const Bufs& b, int i, int part, int lpa
 
 // COMMON: every system has the same potential constants, which are then kernel arguments (operands of
 // the constant bank, no loads: 171 -> 155 us on the crystal); otherwise they are read from the table.
-template <bool EATOM, bool GRAD, bool COMMON, int BLOCKS>
+// FINE: positions carry ten more bits an axis (a test in the loop cost 8000 atoms 1.4 %).
+template <bool EATOM, bool GRAD, bool COMMON, int BLOCKS, bool FINE>
 __global__ void __launch_bounds__(kScatterThreads, BLOCKS)
 k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc) {
     dep_wait();
@@ -2854,7 +2887,11 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
             for (int u = 0; u < 2; ++u) {
                 const int e = e0 + 32 * u;
                 if (e >= E) break;
-                const float fx = (float)(xj[u].x - xi[u].x), fy = (float)(xj[u].y - xi[u].y), fz = (float)(xj[u].z - xi[u].z);
+                float fx = (float)(xj[u].x - xi[u].x), fy = (float)(xj[u].y - xi[u].y), fz = (float)(xj[u].z - xi[u].z);
+                if constexpr (FINE) {
+                    const float3 g = frac_low_diff(xj[u].w, xi[u].w);
+                    fx += g.x; fy += g.y; fz += g.z;
+                }
                 const float dx = fx * Lh.x + fx * Ll.x, dy = fy * Lh.y + fy * Ll.y, dz = fz * Lh.z + fz * Ll.z;
                 const float r2 = dx * dx + dy * dy + dz * dz;
                 // one Newton step: the hardware value's bias of a fraction of 1e-7 would scale every
@@ -4101,11 +4138,12 @@ void launch_uf_list(const Bufs& b0, int precision, int ntiles, int nsys, int for
 void launch_uf(const Bufs& b, int precision, int ntiles, int mode, cudaStream_t s, long* launches) {
     if (ntiles <= 0 || !b.uf_nbr) return;
     if (precision == NEFE_FP64) {
-        if (mode == FM_FORCES) launch_next(k_uf<double, FM_FORCES>, ntiles * kUfBlocks<double>, kUfThreads<double>, s, b);
-        else launch_next(k_uf<double, FM_STEP>, ntiles * kUfBlocks<double>, kUfThreads<double>, s, b);
+        if (mode == FM_FORCES) launch_next(k_uf<double, FM_FORCES, false>, ntiles * kUfBlocks<double>, kUfThreads<double>, s, b);
+        else launch_next(k_uf<double, FM_STEP, false>, ntiles * kUfBlocks<double>, kUfThreads<double>, s, b);
     } else {
-        if (mode == FM_FORCES) launch_next(k_uf<float, FM_FORCES>, ntiles * kUfBlocks<float>, kUfThreads<float>, s, b);
-        else launch_next(k_uf<float, FM_STEP>, ntiles * kUfBlocks<float>, kUfThreads<float>, s, b);
+        const auto go = [&](auto kernel) { launch_next(kernel, ntiles * kUfBlocks<float>, kUfThreads<float>, s, b); };
+        if (mode == FM_FORCES) b.want_xf > 1 ? go(k_uf<float, FM_FORCES, true>) : go(k_uf<float, FM_FORCES, false>);
+        else b.want_xf > 1 ? go(k_uf<float, FM_STEP, true>) : go(k_uf<float, FM_STEP, false>);
     }
     if (launches) *launches += 1;
 }
@@ -4132,7 +4170,7 @@ __global__ void __launch_bounds__(kTile) k_frac_positions(Bufs b) {
     if (i >= b.ntot) return;
     const size_t N = b.ntot;
     const double x[3] = {b.x[i], b.x[N + i], b.x[2 * N + i]};
-    const int4 f = frac_position(x, b.st[0]);
+    const int4 f = frac_position(x, b.st[0], b.want_xf > 1);
     b.xf[i] = f;
     b.xc[i] = pack_frac(f);
     if (i == 0) scale_of_box(b, 0, b.st[0]);
@@ -4180,11 +4218,16 @@ static void edges_fp32(const Bufs& b, int lanes, int ntiles, cudaStream_t s) {
             const int items = edge_items(b, ntiles);
             const auto go = [&](auto kernel) { launch_next_if(!b.uf_nbr || items <= kEarlyBlocks, kernel, items, kScatterThreads, s, b, b.swc_common); };
             const bool full = items >= 152 * kScatterBlocks;
-            if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks>);          // (stateless: one system)
-            else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks>);
-            else if (!b.common) go(k_edges_s<false, false, false, kScatterBlocks>);
-            else if (full) go(k_edges_s<false, false, true, kScatterBlocks>);
-            else go(k_edges_s<false, false, true, kScatterBlocksFew>);
+            if (b.want_xf > 1) {
+                if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks, true>);
+                else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks, true>);
+                else if (!b.common) go(k_edges_s<false, false, false, kScatterBlocks, true>);
+                else go(k_edges_s<false, false, true, kScatterBlocks, true>);
+            } else if (b.want_grad) go(k_edges_s<false, true, true, kScatterBlocks, false>);   // (stateless: one system)
+            else if (b.e_atom) go(k_edges_s<true, false, true, kScatterBlocks, false>);
+            else if (!b.common) go(k_edges_s<false, false, false, kScatterBlocks, false>);
+            else if (full) go(k_edges_s<false, false, true, kScatterBlocks, false>);
+            else go(k_edges_s<false, false, true, kScatterBlocksFew, false>);
             break;
         }
         case 1: launch_next(k_edges1<float>, ntiles * (kTile / kEdges1Threads), kEdges1Threads, s, b); break;

@@ -82,7 +82,8 @@ struct Bufs {
     int4* xf;                // FP32: fractional positions (x/L as 32-bit fixed point)
     int4* xfb;               // their values at the last list build
     uint2* xc;               // their top 21 bits per axis (pass A's row filter)
-    int want_xf, want_xs;    // per-step positions: fractional (scatter form; FP64: xc only), FP32 mirror (the others)
+    int want_xf, want_xs;    // per-step positions: fractional (scatter form; FP64: xc only; 2: with ten more
+                             // bits an axis in .w, see kFracCoarse), FP32 mirror (the others)
     int row4;                // row-major rows can be read 16 bytes at a time
     int* any_rebuild;        // engine: [0] some system's rebuild flag is set this step, [1] some
                              // rebuild_next is set (fused epilogue); NULL in the stateless calls

@@ -235,5 +235,16 @@ __device__ __forceinline__ int frac32(double x, double inv_L) {
     }
     return (int)(unsigned)(unsigned long long)__double_as_longlong(s);
 }
+// The same with kFracLow more bits (the fraction times 2^42, by the unit of 1.5 2^10), modulo 2^42.
+constexpr int kFracLow = 10;
+__device__ __forceinline__ long long frac42(double x, double inv_L) {
+    const double magic = 1536.0;                 // 1.5 2^10
+    double s = __fma_rn(x, inv_L, magic);
+    if ((__double_as_longlong(s) >> 52) != (__double_as_longlong(magic) >> 52)) {
+        const double t = __dmul_rn(x, inv_L);
+        s = __dadd_rn(t - floor(t), magic);
+    }
+    return __double_as_longlong(s) & ((1LL << (32 + kFracLow)) - 1);
+}
 
 }  // namespace nefe

@@ -583,3 +583,39 @@ def test_scatter_forces_of_weak_and_strong_potentials(N, scale):
         ctx.close()
     for a, b in zip(*v):
         assert np.abs(a - b).max() <= 1e-5 * np.abs(b).max()
+
+
+# ------------------------------------------------------------------ long boxes
+@pytest.mark.parametrize("L", [1000.0, 2000.0, 2.0e4, 2.0e5])
+def test_fp32_forces_in_long_boxes(N, L):
+    """A slab in a box of up to 2e5 A: the FP32 tolerance of a short box, stateless and in a context (velocity after
+    one step from rest), and for the Uhlenbeck-Ford term."""
+    x, box = I.diamond(3, 2, 2)
+    x = I.rattle(x, 0.1, 11) + np.array([0.61803 * L, 0.0, 0.0])
+    box = np.array([L, box[1], box[2]])
+    _close32(x, box, _forces32(N, x, box, 0.5, 48))
+    v = []
+    for precision in (N.NEFE_FP32, N.NEFE_FP64):
+        ctx = N.Context(precision=precision, skin=0.5, nbr_cap=48)
+        s = ctx.add_system(x, box, v=np.zeros_like(x))
+        ctx.run(1)
+        assert ctx.results(s)["error"] == 0
+        v.append(ctx.get_state(s)[1])
+        ctx.close()
+    assert np.abs(v[0] - v[1]).max() <= 1e-5 * np.abs(v[1]).max()
+
+
+@pytest.mark.parametrize("L", [1000.0, 2.0e4, 2.0e5])
+def test_fp32_uf_forces_in_long_boxes(N, L):
+    """1e-6 of the largest force: ten times the rounding of an FP32 distance."""
+    uf, skin = (25.0, 2.0, 2200.0, 8.0), 0.5
+    x, box = I.diamond(2, 4, 4)
+    x = I.rattle(x, 0.1, 12) + np.array([0.61803 * L, 0.0, 0.0])
+    box = np.array([L, 22.0, 22.0])
+    n = len(x)
+    e_o, f_o, vir_o, ea_o = O.uf_energy(x, box, uf)
+    f = torch.zeros(3 * n, dtype=torch.float64, device="cuda")
+    ea = torch.zeros(n, dtype=torch.float64, device="cuda")
+    N.nefe_uf_forces(soa(x), n, box, RC + skin, skin, N.uf_params(*uf), N.NEFE_FP32, f, ea, None)
+    f = f.cpu().numpy().reshape(3, n).T
+    assert np.abs(f - f_o).max() <= 1e-6 * np.abs(f_o).max()
