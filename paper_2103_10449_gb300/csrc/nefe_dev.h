@@ -31,7 +31,8 @@ enum Acc {
     ACC_VIR,            // 6: SW virial xx yy zz xy xz yz (unscaled)
     ACC_KT = ACC_VIR + 6,   // 6: sum m v_a v_b (eV)
     ACC_XI = ACC_KT + 6,    // 3: sum of thermostat normals of the current step
-    ACC_DTH = ACC_XI + 3,   // 7: dE/d(A, B, p, q, a, lambda3, gamma) (stateless gradient call)
+    ACC_DTH = ACC_XI + 3,   // 7: dE/d(A, B, p, q, a, lambda3, gamma) (stateless gradient call); FP64
+                            //    engine: remainders of U_int and the virial in 2^-40 units
     ACC_XIN = ACC_DTH + 7,  // 3: sum of the next step's thermostat normals, drawn by an epilogue
                             //    that already moved the atoms (becomes ACC_XI at the next step)
     ACC_N = ACC_XIN + 3

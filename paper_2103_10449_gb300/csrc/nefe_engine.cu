@@ -574,6 +574,7 @@ int setup(nefe_ctx* c) {
     // 149 us with 4, 56 us with 1); below 20,000 atoms the shorter chain of 4 lanes wins
     if (c->prec == NEFE_FP64 && !c->gchosen) c->glanes = c->ntot >= 20000 ? 1 : 4;
     b.xf = c->d_xf; b.xfb = c->d_xfb; b.lscale = c->d_lscale; b.xc = c->d_xc;
+    if (c->prec == NEFE_FP64) b.acc_lo = c->d_acc;
     b.swc_common = swc_common; b.swp_common = swp_common; b.common = common ? 1 : 0;
     set_form(c, c->lanes);
 
@@ -1143,6 +1144,7 @@ int nefe_autotune(nefe_ctx* c) {
         launch_positions(b, c->prec, c->ntiles, c->stream, &c->launches);
     }
     b.acc = c->d_acc_tmp;
+    if (b.acc_lo) b.acc_lo = b.acc;
     b.f_out = c->d_ftmp;
     b.e_atom = nullptr;
     cudaEvent_t e0, e1;

@@ -171,13 +171,19 @@ template <> struct Noise<float> {
 // In FP64 the threads' values are converted first (2^-40 units) and summed as integers: FP64 adds
 // run at 2 lanes a cycle, and five of them per value and warp were a third of the epilogue.  The
 // integer sum of a block (at most 128 threads) stays below 2^62 when every value is below 2^15; a
-// block that holds a larger value (or one that is not finite) takes the FP64 sums.  The remainders of the conversion to 2^-32 are
-// kept in their own slots where the caller has some (acc_lo: stateless calls, whose small blocks
-// would round several times as often as a 128-atom block does).
+// block that holds a larger value (or one that is not finite) takes the FP64 sums.  The remainders of
+// the conversion to 2^-32 are kept in slots of their own (acc_lo) where blocks are small: 8 atoms to a
+// block round four times as often as 32.
 // ------------------------------------------------------------------------------------
+// Rows of the remainders of pass A's sums (U_int, virial).  The engine keeps them in the rows of
+// dE/dtheta, which it has no other use for (and which its saved states hold); the stateless calls have
+// a second array of the sums' layout.
+__device__ __forceinline__ int engine_lo_row(int a) { return ACC_DTH + max(a - 1, 0); }
+
 template <typename T, int K>
 __device__ __forceinline__ void block_sum_to_acc(T (&v)[K], long long* acc_sys, int first,
-                                                 unsigned* err, long long* acc_lo = nullptr) {
+                                                 unsigned* err, long long* acc_lo = nullptr,
+                                                 bool engine = false) {
     if constexpr (sizeof(T) == 8) {
         __shared__ long long ired[kTile / 32][K];
         constexpr double most = 4194304.0 / kTile;
@@ -197,12 +203,14 @@ __device__ __forceinline__ void block_sum_to_acc(T (&v)[K], long long* acc_sys, 
             if (threadIdx.x < K) {
                 long long s = 0;
                 for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += ired[i][threadIdx.x];
-                const size_t slot = (size_t)(first + threadIdx.x) * kSlots + (blockIdx.x % kSlots);
+                const int a = first + (int)threadIdx.x, slot = (int)(blockIdx.x % kSlots);
                 const long long units = s;
                 s = (s + 128) >> 8;
-                if (s != 0) atomicAdd(reinterpret_cast<unsigned long long*>(&acc_sys[slot]), (unsigned long long)s);
+                if (s != 0)
+                    atomicAdd(reinterpret_cast<unsigned long long*>(&acc_sys[a * kSlots + slot]), (unsigned long long)s);
                 if (acc_lo && units != s * 256)
-                    atomicAdd(reinterpret_cast<unsigned long long*>(&acc_lo[slot]), (unsigned long long)(units - s * 256));
+                    atomicAdd(reinterpret_cast<unsigned long long*>(&acc_lo[(engine ? engine_lo_row(a) : a) * kSlots + slot]),
+                              (unsigned long long)(units - s * 256));
             }
             return;
         }
@@ -3221,7 +3229,8 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
         reinterpret_cast<double4*>(b.P)[i] = mk4(fx, fy, fz, en);
     }
     long long* acc = b.acc + (size_t)ta.sys * ACC_N * kSlots;
-    block_sum_to_acc<double, 8>(red8, acc, ACC_UINT, &st.err, b.acc_lo);
+    const bool engine = b.acc_lo == b.acc;
+    block_sum_to_acc<double, 8>(red8, acc, ACC_UINT, &st.err, engine ? acc : b.acc_lo, engine);
     if constexpr (GRAD) block_sum_to_acc<double, 7>(gth, acc, ACC_DTH, &st.err, b.acc_lo);
 }
 
@@ -3789,10 +3798,14 @@ __global__ void __launch_bounds__(kTile) k_group(Bufs b, const DevGroup* groups,
     __shared__ __align__(16) GroupShared sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mine = warp == 1 ? gr.b : gr.a;    // the member of warps 0 and 1
-    // slot sums (fixed order: deterministic), in flight together with the descriptors
+    // slot sums (fixed order: deterministic), in flight together with the descriptors; lane 16 + a takes the
+    // remainders of sum a where pass A keeps them (FP64)
     double sum = 0.0;
-    if (mode != 0 && warp < nm && lane < ACC_XI)
-        sum = (double)slot_sum(b.acc + (size_t)mine * ACC_N * kSlots + (size_t)lane * kSlots) * (1.0 / kFix);
+    const int a_lo = lane - 16;
+    const bool rest = b.acc_lo && a_lo >= 0 && a_lo < ACC_KT && a_lo != ACC_UREF;
+    if (mode != 0 && warp < nm && (lane < ACC_XI || rest))
+        sum = (double)slot_sum(b.acc + ((size_t)mine * ACC_N + (rest ? engine_lo_row(a_lo) : lane)) * kSlots) *
+              (rest ? 0x1p-40 : 1.0 / kFix);
     for (int mi = 0; mi < nm; ++mi) {
         StagedSys& m = sh.m[mi];
         stage_sys(b, mi == 0 ? gr.a : gr.b, m);
@@ -3805,6 +3818,7 @@ __global__ void __launch_bounds__(kTile) k_group(Bufs b, const DevGroup* groups,
     __syncthreads();
     if (warp < nm && mode != 0) {
         DevState& st = sh.m[warp].st;
+        sum += __shfl_down_sync(0xffffffffu, sum, 16);
         if (lane == ACC_UINT) st.u_int = sum;
         else if (lane == ACC_UREF) st.u_ref = sum;
         else if (lane < ACC_KT) st.vir[lane - ACC_VIR] = sum;

@@ -14,7 +14,8 @@ struct Bufs {
     const DevSys* sys;
     DevState* st;
     long long* acc;          // [nsys][ACC_N][kSlots]
-    long long* acc_lo;       // stateless: remainders of the sums in 2^-40 units, the same layout, or NULL
+    long long* acc_lo;       // remainders of the sums in 2^-40 units: stateless, an array of the same layout;
+                             // FP64 engine, acc itself (engine_lo_row); or NULL
     const int4* tiles;       // 128-atom tiles: system, first atom, atom count
     double* x;               // FP64 anchor positions (positions at the last list build), SoA
     void* dhi;               // displacement since the last build, kernel precision, SoA (may be NULL)

@@ -619,3 +619,21 @@ def test_fp32_uf_forces_in_long_boxes(N, L):
     N.nefe_uf_forces(soa(x), n, box, RC + skin, skin, N.uf_params(*uf), N.NEFE_FP32, f, ea, None)
     f = f.cpu().numpy().reshape(3, n).T
     assert np.abs(f - f_o).max() <= 1e-6 * np.abs(f_o).max()
+
+
+# ------------------------------------------------------------------ sums of the FP64 engine
+@pytest.mark.parametrize("seed", [1, 2, 3, 4])
+def test_fp64_engine_sums_keep_their_remainders(N, seed):
+    """Energy and pressure of 64 atoms in blocks of 8, as test_fp64_sums_keep_their_remainders: 1e-13 of the
+    energy (at rest the pressure is the virial's alone)."""
+    x, box = I.diamond(2, 2, 2)
+    x = I.rattle(x, 0.1, seed)
+    ctx = N.Context(precision=N.NEFE_FP64, skin=0.5, nbr_cap=48)
+    s = ctx.add_system(x, box, v=np.zeros_like(x))
+    ctx.setup()
+    r = ctx.results(s)
+    ctx.close()
+    e_o, _, vir_o, _ = O.sw_energy(x, box)
+    V = float(np.prod(box))
+    assert abs(r["U"] - e_o) <= 1e-13 * abs(e_o)
+    assert np.abs(r["P"] * V / O.EV_A3_TO_GPA - vir_o).max() <= 2e-13 * abs(e_o)
