@@ -1350,7 +1350,7 @@ int nefe_get_shell_stats(nefe_ctx* c, double* mean_count, int* max_count) {
     for (int s = 0; s < c->nsys; ++s) {
         if (S[s].pot != POT_SW) continue;
         for (int i = 0; i < S[s].n; ++i) {
-            const int v = shn[S[s].off + i];
+            const int e = shn[S[s].off + i], v = (e & 0xffff) - (e >> 16);
             sum += v;
             mx = std::max(mx, v);
         }

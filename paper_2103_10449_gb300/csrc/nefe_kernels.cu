@@ -3033,6 +3033,28 @@ struct __align__(16) EdgesDShared {
     unsigned short slot[kListEdgesD];   // cell-offset code << 8 | shell slot
     double mom[10][32];
 };
+// Takes the marked entries at or beyond the cutoff (in the filter's margin) out of (lo, hi).  Only where
+// an atom has more marked entries than its shell holds: a shell's slots are for edges.
+__device__ __noinline__ void drop_margin(const Bufs& b, const DevState& st, double rc2, int i, int part, int lpa, unsigned& lo,
+                                         unsigned& hi) {
+    const double4* X = reinterpret_cast<const double4*>(b.xs);
+    const double4 xi = X[i];
+    unsigned w[2] = {lo, hi};
+    for (int q = 0; q < 2; ++q)
+        for (unsigned left = w[q]; left; left &= left - 1u) {
+            const int bit = __ffs(left) - 1, k = bit + 32 * q;
+            const unsigned e = (unsigned)b.nbr[nbr_at(b, i, 8 * (((k >> 3) << lpa) + part) + (k & 7))];
+            int j = (int)(e & kIndexMask);
+            if (j >= b.ntot) j = i;
+            const int code = (int)(e >> kCodeShift);
+            const double4 xj = X[j];
+            const double dx = (xj.x - xi.x) + (code % 3 - 1) * st.h[0], dy = (xj.y - xi.y) + ((code / 3) % 3 - 1) * st.h[1],
+                         dz = (xj.z - xi.z) + (code / 9 - 1) * st.h[2];
+            if (dx * dx + dy * dy + dz * dz >= rc2) w[q] &= ~(1u << bit);
+        }
+    lo = w[0];
+    hi = w[1];
+}
 // The next step's thermostat noise of 32 atoms (a quarter of a tile, one warp per Box-Muller pair) into
 // xi_next, by blocks of pass A beyond the edges' own.  It depends on the step and the atom only, and in
 // a small context it is the longest part of k_kick_drift (a chain of FP64 logarithm, root and sine, on as
@@ -3078,9 +3100,14 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
     const double4* X = reinterpret_cast<const double4*>(b.xs);
     unsigned lo = 0u, hi = 0u;
     if (valid) mark_row(b, i, lane >> lg, lpa, b.lscale[4 * ta.sys], (float)P.rc2, &st.err, lo, hi);
-    const int ml = __popc(lo) + __popc(hi);      // edges of this lane, then of its atom
+    int ml = __popc(lo) + __popc(hi);            // edges of this lane, then of its atom
     int m = ml, before = 0;                      // before: of the atom's lanes before this one
     for (int o = 16; o >= G; o >>= 1) m += __shfl_xor_sync(kAll, m, o);
+    if (__any_sync(kAll, m > kShell)) {          // rare
+        if (m > kShell) drop_margin(b, st, P.rc2, i, lane >> lg, lpa, lo, hi);
+        m = ml = __popc(lo) + __popc(hi);
+        for (int o = 16; o >= G; o >>= 1) m += __shfl_xor_sync(kAll, m, o);
+    }
     {
         int inc = ml;                            // inclusive scan over the atom's lanes (stride G)
         for (int o = G; o < 32; o <<= 1) {
@@ -3095,7 +3122,7 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
         if (t >= o) incl += y;
     }
     const int total = __shfl_sync(kAll, incl, G - 1);
-    int mtrue = 0;
+    int outside = 0;                             // of the lane's entries, those of the filter's margin
     double red8[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // energy, -, virial
     double gth[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     double fx = 0.0, fy = 0.0, fz = 0.0, en = 0.0;
@@ -3154,9 +3181,10 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
             const unsigned bal = __ballot_sync(kAll, on);
             if (on) {
                 const int e = base + __popc(bal & below);
-                const double g = sh.v[5][e];
-                mtrue += g > 0.0 ? 1 : 0;
-                mom_add(M, sh.v[0][e], sh.v[1][e], sh.v[2][e], g);
+                const double ux = sh.v[0][e], uy = sh.v[1][e], uz = sh.v[2][e];
+                // (beyond the cutoff the unit vector is 0: high words, no FP64 comparison)
+                outside += ((__double2hiint(ux) | __double2hiint(uy) | __double2hiint(uz)) << 1) == 0 ? 1 : 0;
+                mom_add(M, ux, uy, uz, sh.v[5][e]);
             }
             base += __popc(bal);
         }
@@ -3215,7 +3243,7 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
     }
     red8[5] *= 0.5; red8[6] *= 0.5; red8[7] *= 0.5;
     for (int o = 16; o >= G; o >>= 1) {
-        mtrue += __shfl_xor_sync(kAll, mtrue, o);
+        outside += __shfl_xor_sync(kAll, outside, o);
         fx += __shfl_xor_sync(kAll, fx, o);
         fy += __shfl_xor_sync(kAll, fy, o);
         fz += __shfl_xor_sync(kAll, fz, o);
@@ -3224,7 +3252,7 @@ k_edges_d(const __grid_constant__ Bufs b, const __grid_constant__ SWp<double> Pc
     if (lane < G && valid) {
         if (m > kShell) atomicOr(&st.err, NEFE_ERR_SHELL_OVERFLOW);
         const int ms = min(m, kShell);
-        b.shn[i] = ms;
+        b.shn[i] = ms | outside << 16;
         if (ms < kShell) b.shj[(size_t)i * kShell + ms] = -1;
         reinterpret_cast<double4*>(b.P)[i] = mk4(fx, fy, fz, en);
     }
@@ -3305,7 +3333,7 @@ __global__ void __launch_bounds__(kTile) k_gather(Bufs b) {
         }
         if (S.pot == POT_SW) {
             const T4* Fl = reinterpret_cast<const T4*>(b.shd);
-            const int m = b.shn[i];
+            const int m = b.shn[i] & 0xffff;     // (FP64: with the margin's entries, see k_edges_d)
             // NB shell entries per lane in flight: neighbour index, the first 8 entries of the
             // neighbour's index list (one 32-byte sector), then the leg force
             constexpr int NB = L >= 2 ? 1 : 2;

@@ -637,3 +637,40 @@ def test_fp64_engine_sums_keep_their_remainders(N, seed):
     V = float(np.prod(box))
     assert abs(r["U"] - e_o) <= 1e-13 * abs(e_o)
     assert np.abs(r["P"] * V / O.EV_A3_TO_GPA - vir_o).max() <= 2e-13 * abs(e_o)
+
+
+# ------------------------------------------------------------------ shells of 32
+def _ball(r_out):
+    """An atom, 32 neighbours spread over a sphere inside the cutoff, one more at r_out."""
+    k = np.arange(33) + 0.5
+    z, t = 1.0 - 2.0 * k / 33, math.pi * (1.0 + 5.0 ** 0.5) * k
+    u = np.stack([np.sqrt(1.0 - z * z) * np.cos(t), np.sqrt(1.0 - z * z) * np.sin(t), z], 1)
+    r = np.full((33, 1), 3.55)
+    r[16] = r_out
+    return np.concatenate([[[0.0, 0.0, 0.0]], u * r])
+
+
+def test_fp64_shell_of_32_with_one_more_just_outside(N):
+    """The row filter's margin (1.4e-3 A in a box of 500 A) is not the cutoff: 32 neighbours and one 1e-4 A outside are
+    a shell of 32, in the sums, the forces and the shell statistics."""
+    box = np.array([500.0, 500.0, 500.0])
+    x = _ball(RC + 1e-4) + 250.0
+    f, ev = _sw(N, x, box, _silicon(N), N.NEFE_FP64, cap=64)
+    e_o, f_o, vir_o, _ = O.sw_energy(x, box)
+    assert np.abs(f - f_o).max() <= 1e-10 * np.abs(f_o).max()
+    assert abs(ev[0] - e_o) <= 1e-10 * abs(e_o)
+    ctx = N.Context(precision=N.NEFE_FP64, skin=0.5, nbr_cap=64)
+    s = ctx.add_system(x, box, v=np.zeros_like(x))
+    ctx.setup()
+    r, st = ctx.results(s), ctx.shell_stats()
+    ctx.close()
+    assert r["error"] == 0 and r["U"] == pytest.approx(e_o, rel=1e-10)
+    d = x[:, None] - x[None]
+    m = ((d * d).sum(2) < RC * RC).sum(1) - 1
+    assert m.max() == 32 and st == (m.mean(), 32)
+
+
+def test_fp64_shell_of_33_is_refused(N):
+    box = np.array([500.0, 500.0, 500.0])
+    with pytest.raises(N.NefeError):
+        _sw(N, _ball(RC - 1e-4) + 250.0, box, _silicon(N), N.NEFE_FP64, cap=64)
