@@ -76,6 +76,7 @@ struct nefe_ctx {
     uint2* d_xc = nullptr;
     int4 *d_xf = nullptr, *d_xfb = nullptr;                               // fractional positions (FP32)
     bool chosen = false;     // pass A's form was set by nefe_set_tuning or the autotuner
+    bool refuse = false;     // the scatter form was set by nefe_set_tuning, which refuses terms of 48 eV/A
     bool gchosen = false;    // pass B's lanes likewise
     bool stale_pos = false;  // the positions' forms have to be made anew before the next step
     void* d_uf_F = nullptr;
@@ -184,7 +185,7 @@ void set_form(nefe_ctx* c, int lanes) {
     if (c->b.want_xf != xf || c->b.want_xs != xs) c->stale_pos = true;
     c->b.want_xf = xf;
     c->b.want_xs = xs;
-    c->b.leg_refuse = c->chosen ? 1 : 0;
+    c->b.leg_refuse = c->refuse ? 1 : 0;
 }
 
 // Both force passes, chunk by chunk; with slot >= 0 (profiling capture) events bracket
@@ -1134,10 +1135,31 @@ int nefe_autotune(nefe_ctx* c) {
     int rc = setup(c);
     if (rc) return rc;
     if ((rc = set_device(c))) return rc;
-    if (!c->chosen) drop_graph(c);               // what the forms refuse is captured in the step graph
+    if (c->refuse) drop_graph(c);                // what the form refuses is captured in the step graph
     c->chosen = c->gchosen = true;
-    c->b.leg_refuse = 1;
+    c->refuse = false;
+    c->b.leg_refuse = 0;
     Bufs b = c->b;
+    // The trial launches work on the live positions and descriptors.  What they leave in the states (error
+    // bits: a variant's shells may be too small) is taken back after each, and one that adds an error is
+    // not a candidate.
+    std::vector<DevState> st0(c->nsys), st1(c->nsys);
+    NEFE_CU(cudaMemcpyAsync(st0.data(), c->d_st, sizeof(DevState) * c->nsys, cudaMemcpyDeviceToHost, c->stream));
+    NEFE_CU(cudaStreamSynchronize(c->stream));
+    auto took_back = [&] {                       // true where an error was added
+        bool bad = false;
+        if (cudaMemcpyAsync(st1.data(), c->d_st, sizeof(DevState) * c->nsys, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+            cudaStreamSynchronize(c->stream) != cudaSuccess)
+            return false;                        // (reported by the checks below)
+        for (int s = 0; s < c->nsys; ++s) bad = bad || (st1[s].err & ~st0[s].err) != 0;
+        cudaMemcpyAsync(c->d_st, st0.data(), sizeof(DevState) * c->nsys, cudaMemcpyHostToDevice, c->stream);
+        cudaStreamSynchronize(c->stream);
+        return bad;
+    };
+    if (c->prec == NEFE_FP64 && c->stale_pos) {
+        launch_positions(b, c->prec, c->ntiles, c->stream, &c->launches);
+        c->stale_pos = false;
+    }
     if (c->prec == NEFE_FP32) {                  // every form is timed: both kinds of positions
         b.want_xf = frac_form(c);
         b.want_xs = 1;
@@ -1194,6 +1216,7 @@ int nefe_autotune(nefe_ctx* c) {
             set_edge_items(b, c->prec, lg_of(l), c->ntiles);
             us = time_us([&] { launch_edges(b, c->prec, l, c->ntiles, FM_FORCES, c->stream, &c->launches); });
         }
+        if (took_back()) continue;
         ranked_a.push_back({us, l});
         if (us < best) { best = us; best_l = l; }
     }
@@ -1201,11 +1224,17 @@ int nefe_autotune(nefe_ctx* c) {
     cudaFree(tv0);
     cudaFree(tf0);
     std::sort(ranked_a.begin(), ranked_a.end());
+    // the gather form whose pass B is timed: the best one, beside the scatter form one thread per atom
+    int la = best_l;
+    if (best_l == 0)
+        for (const auto& r : ranked_a)
+            if (r.second == 1 || (r.second != 0 && la == 0)) la = r.second;
     set_edge_items(b, c->prec, lg_of(best_l), c->ntiles);
-    launch_edges(b, c->prec, best_l == 0 ? 1 : best_l, c->ntiles, FM_FORCES, c->stream, &c->launches);
-    double best_g = 1e30;
+    double best_g = 0.0;
     int best_gl = c->glanes;
-    {
+    if (la != 0) {
+        launch_edges(b, c->prec, la, c->ntiles, FM_FORCES, c->stream, &c->launches);
+        best_g = 1e30;
         // pass B is timed in its step form (springs, Langevin, kick) on scratch copies of the
         // velocities and the force, so the state is left as it was
         const size_t el = c->prec == NEFE_FP64 ? sizeof(double) : sizeof(float);
@@ -1219,7 +1248,6 @@ int nefe_autotune(nefe_ctx* c) {
         bs.F = tf;
         // each variant right after pass A, as in a step (pass B reads what pass A just wrote);
         // the scatter form was timed with its own pass B above
-        const int la = best_l == 0 ? 1 : best_l;
         double base_a = best;
         for (const auto& r : ranked_a)
             if (r.second == la) base_a = r.first;
@@ -1230,6 +1258,7 @@ int nefe_autotune(nefe_ctx* c) {
             });
             if (us < best_g) { best_g = us; best_gl = l; }
         }
+        took_back();
         best_g -= base_a;
         // a gather-form pair faster than the scatter form (pass A + its pass B) replaces it
         if (best_l == 0 && base_a + best_g < scatter_us) best_l = la;
@@ -1272,8 +1301,9 @@ int nefe_set_tuning(nefe_ctx* c, int lanes) {
     if (!c) return fail(NEFE_EINVAL, "context is NULL");
     if (!lanes_supported(lanes) || (c->prec == NEFE_FP64 && (lanes == 0 || lanes == 1 || lanes == 4)))
         return fail(NEFE_EINVAL, "unsupported lanes per atom %d", lanes);
-    if (lanes != c->lanes || !c->chosen) drop_graph(c);
+    if (lanes != c->lanes || !c->chosen || c->refuse != (lanes == 0)) drop_graph(c);
     c->chosen = true;
+    c->refuse = lanes == 0;
     set_form(c, lanes);
     return NEFE_OK;
 }

@@ -674,3 +674,32 @@ def test_fp64_shell_of_33_is_refused(N):
     box = np.array([500.0, 500.0, 500.0])
     with pytest.raises(N.NefeError):
         _sw(N, _ball(RC - 1e-4) + 250.0, box, _silicon(N), N.NEFE_FP64, cap=64)
+
+
+# ------------------------------------------------------------------ autotuner
+def test_autotune_does_not_narrow_what_a_context_takes(N):
+    """A pair at 1.3 A (terms above 48 eV/A) in an autotuned context, as in one left alone: no error, neither from the
+    trial launches nor from the steps."""
+    x, box = I.diamond(3, 3, 3)
+    d = x[4] - x[0]
+    x[4] = x[0] + d * (1.3 / np.linalg.norm(d))
+    ctx = N.Context(precision=N.NEFE_FP32, skin=0.5, nbr_cap=48)
+    s = ctx.add_system(x, box, v=np.zeros_like(x))
+    ctx.autotune()
+    assert ctx.results(s)["error"] == 0
+    ctx.run(1)
+    assert ctx.results(s)["error"] == 0
+    ctx.close()
+
+
+def test_autotune_of_shells_above_the_thread_form(N):
+    """28 neighbours inside the cutoff: more than the one-thread form's 20, which flags its trial; the context takes
+    another form and stays without error."""
+    x, box = I.diamond(4, 4, 4, a=4.4)
+    x = I.rattle(x, 0.02, 9)
+    ctx = N.Context(precision=N.NEFE_FP32, skin=0.3, nbr_cap=64)
+    s = ctx.add_system(x, box, v=np.zeros_like(x))
+    lanes, _ = ctx.autotune()
+    ctx.run(1)
+    assert lanes != 1 and ctx.results(s)["error"] == 0
+    ctx.close()
