@@ -417,7 +417,10 @@ NEFE_API int nefe_load(nefe_ctx* ctx, const char* path);
  * continues bit for bit as without the call; the snapshot needs about as much free device
  * memory as the state, and without it the kernel-level choice stands).  nefe_get_tuning
  * reports pass A's lanes and the time per MD step of the chosen pair (kernel-level: the two
- * passes' summed time); nefe_set_tuning fixes pass A's lanes.  Blocking. */
+ * passes' summed time); nefe_set_tuning fixes pass A's lanes.  Blocking.
+ * FP32, scatter form (0): set by nefe_set_tuning, or chosen by nefe_autotune for systems of at most 14
+ * neighbours inside the cutoff on average, it flags (NEFE_ERR_NAN) and leaves out force terms of 48 eV/A
+ * and more.  As the default it takes any term, as the other forms do. */
 NEFE_API int nefe_autotune(nefe_ctx* ctx);
 NEFE_API int nefe_get_tuning(nefe_ctx* ctx, int* lanes_per_atom, double* best_us);
 NEFE_API int nefe_set_tuning(nefe_ctx* ctx, int lanes_per_atom);

@@ -76,7 +76,8 @@ struct nefe_ctx {
     uint2* d_xc = nullptr;
     int4 *d_xf = nullptr, *d_xfb = nullptr;                               // fractional positions (FP32)
     bool chosen = false;     // pass A's form was set by nefe_set_tuning or the autotuner
-    bool refuse = false;     // the scatter form was set by nefe_set_tuning, which refuses terms of 48 eV/A
+    bool refuse = false;     // terms of 48 eV/A are refused: the scatter form was set by nefe_set_tuning, or by
+                             // the autotuner for shells of up to kRefuseShell
     bool gchosen = false;    // pass B's lanes likewise
     bool stale_pos = false;  // the positions' forms have to be made anew before the next step
     void* d_uf_F = nullptr;
@@ -1129,6 +1130,12 @@ static int refine_in_steps(nefe_ctx* c, const std::vector<std::pair<double, int>
     return NEFE_OK;
 }
 
+// An autotuned context in the scatter form has always flagged terms of 48 eV/A and more, and runs of crystals
+// that meet one (a random start) stay flagged.  The form once lost to the gather form, which takes any term, where
+// shells are larger (beta-tin, 18 neighbours; diamond, the liquid and pairs of phases have 4 to 13): there, where
+// it wins now, nothing is refused either.
+static constexpr double kRefuseShell = 14.0;
+
 int nefe_autotune(nefe_ctx* c) {
     NvtxRange nvtx_("nefe_autotune");
     if (!c) return fail(NEFE_EINVAL, "context is NULL");
@@ -1279,7 +1286,14 @@ int nefe_autotune(nefe_ctx* c) {
     c->llanes = best_ll;
     c->b.list_lanes = best_ll;
     c->tune_us = best + best_g;
-    return refine_in_steps(c, ranked_a);
+    if ((rc = refine_in_steps(c, ranked_a))) return rc;
+    if (c->lanes == 0) {
+        double mean = 0.0;
+        if ((rc = nefe_get_shell_stats(c, &mean, nullptr))) return rc;
+        c->refuse = mean <= kRefuseShell;
+        c->b.leg_refuse = c->refuse ? 1 : 0;
+    }
+    return NEFE_OK;
 }
 
 int nefe_get_lanes(nefe_ctx* c, int lanes[3]) {

@@ -703,3 +703,26 @@ def test_autotune_of_shells_above_the_thread_form(N):
     ctx.run(1)
     assert lanes != 1 and ctx.results(s)["error"] == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("kind,error", [("beta_tin", 0), ("diamond", 4)])
+def test_autotuned_scatter_form_refuses_where_it_always_did(N, kind, error):
+    """256,000 atoms, one of 32 systems with a pair at 1.3 A, in contexts whose fastest form is the scatter form: beta-tin
+    (18 neighbours, once faster in the gather form, which takes any term) is not refused, diamond is, as before."""
+    x, box = I.beta_tin(10, 10, 20) if kind == "beta_tin" else I.diamond(10, 10, 10)
+    x = I.rattle(x, 0.02, 4)
+    ctx = N.Context(precision=N.NEFE_FP32, skin=0.5, nbr_cap=48)
+    for r in range(32):
+        y = x.copy()
+        if r == 3:
+            d = y[1:] - y[0]
+            d -= box * np.rint(d / box)
+            k = np.argmin((d * d).sum(1))
+            y[k + 1] = y[0] + d[k] * (1.3 / np.linalg.norm(d[k]))
+        ctx.add_system(y, box, v=np.zeros_like(y))
+    lanes, _ = ctx.autotune()
+    assert all(r["error"] == 0 for r in ctx.results_all())
+    ctx.run(1)
+    assert lanes == 0
+    assert [r["error"] for r in ctx.results_all()] == [error if r == 3 else 0 for r in range(32)]
+    ctx.close()
