@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(32) k_sw_edges(const __grid_constant__ AdArgs<
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     if (b0 + u >= ci) continue;
-                    const float dx = (float)(xj[u].x - xi.x) * A.Lf[0], dy = (float)(xj[u].y - xi.y) * A.Lf[1],
-                                dz = (float)(xj[u].z - xi.z) * A.Lf[2];
+                    const float dx = (float)wrap_sub(xj[u].x, xi.x) * A.Lf[0], dy = (float)wrap_sub(xj[u].y, xi.y) * A.Lf[1],
+                                dz = (float)wrap_sub(xj[u].z, xi.z) * A.Lf[2];
                     if (dx * dx + dy * dy + dz * dz < A.rcf2) {
                         if (m < kAdCand) sj[m] = j[u];
                         ++m;
@@ -301,7 +301,8 @@ __device__ __forceinline__ void frac_atom(const FracArgs& F, int i, const double
     xf[i] = f;
     if (!ref) return;
     const int4 r = ref[i];
-    const float dx = (float)(f.x - r.x) * F.Lf[0], dy = (float)(f.y - r.y) * F.Lf[1], dz = (float)(f.z - r.z) * F.Lf[2];
+    const float dx = (float)wrap_sub(f.x, r.x) * F.Lf[0], dy = (float)wrap_sub(f.y, r.y) * F.Lf[1],
+                dz = (float)wrap_sub(f.z, r.z) * F.Lf[2];
     if (F.force || !(dx * dx + dy * dy + dz * dz < F.thr2)) *rebuild = 1;
 }
 __global__ void __launch_bounds__(kAdThreads) k_frac(int n, FracArgs F, const double* x, int4* xf, const int4* ref,

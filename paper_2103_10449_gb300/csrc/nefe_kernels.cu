@@ -422,12 +422,12 @@ __device__ __forceinline__ int4 frac_position(const double (&x)[3], const DevSta
 }
 // fb moved by (tx, ty, tz) units of 2^-32.
 __device__ __forceinline__ int4 frac_moved(const int4& fb, float tx, float ty, float tz, int fine) {
-    int4 f = make_int4(fb.x + __float2int_rn(tx), fb.y + __float2int_rn(ty), fb.z + __float2int_rn(tz), 0);
+    int4 f = make_int4(wrap_add(fb.x, __float2int_rn(tx)), wrap_add(fb.y, __float2int_rn(ty)), wrap_add(fb.z, __float2int_rn(tz)), 0);
     if (fine) {
         constexpr int mask = (1 << kFracLow) - 1;
         const auto low = [&](float t, int axis, int& hi) {
             const int v = ((fb.w >> axis * kFracLow) & mask) + __float2int_rn((t - rintf(t)) * (float)(mask + 1));
-            hi += v >> kFracLow;
+            hi = wrap_add(hi, v >> kFracLow);
             f.w |= (v & mask) << axis * kFracLow;
         };
         low(tx, 0, f.x); low(ty, 1, f.y); low(tz, 2, f.z);
@@ -1794,7 +1794,7 @@ __global__ void __launch_bounds__(kUfThreads<T>, sizeof(T) == 4 ? 5 : 1) k_uf(Bu
             if (!NEFE_IN_RANGE(e & kUfMask, b.ntot, &st.err)) continue;
             T dx, dy, dz;
             if constexpr (kFrac) {
-                float gx = (float)(xj.x - fi.x), gy = (float)(xj.y - fi.y), gz = (float)(xj.z - fi.z);
+                float gx = (float)wrap_sub(xj.x, fi.x), gy = (float)wrap_sub(xj.y, fi.y), gz = (float)wrap_sub(xj.z, fi.z);
                 if constexpr (FINE) {
                     const float3 g = frac_low_diff(xj.w, fi.w);
                     gx += g.x; gy += g.y; gz += g.z;
@@ -2800,9 +2800,9 @@ __device__ __forceinline__ void mark_row(const Bufs& b, int i, int part, int lpa
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const float dx = (float)((int)pj[u].y - xi) * L.x,
-                        dy = (float)((int)__funnelshift_l(pj[u].x, pj[u].y, 21) - yi) * L.y,
-                        dz = (float)((int)(pj[u].x << 10) - zi) * L.z;
+            const float dx = (float)wrap_sub((int)pj[u].y, xi) * L.x,
+                        dy = (float)wrap_sub((int)__funnelshift_l(pj[u].x, pj[u].y, 21), yi) * L.y,
+                        dz = (float)wrap_sub((int)(pj[u].x << 10), zi) * L.z;
             if (dx * dx + dy * dy + dz * dz < act2) oct |= 1u << u;
         }
         // entries past the length are the atom itself
@@ -2895,7 +2895,8 @@ k_edges_s(const __grid_constant__ Bufs b, const __grid_constant__ SWc<float> Pc)
             for (int u = 0; u < 2; ++u) {
                 const int e = e0 + 32 * u;
                 if (e >= E) break;
-                float fx = (float)(xj[u].x - xi[u].x), fy = (float)(xj[u].y - xi[u].y), fz = (float)(xj[u].z - xi[u].z);
+                float fx = (float)wrap_sub(xj[u].x, xi[u].x), fy = (float)wrap_sub(xj[u].y, xi[u].y),
+                      fz = (float)wrap_sub(xj[u].z, xi[u].z);
                 if constexpr (FINE) {
                     const float3 g = frac_low_diff(xj[u].w, xi[u].w);
                     fx += g.x; fy += g.y; fz += g.z;

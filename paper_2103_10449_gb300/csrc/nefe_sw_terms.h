@@ -226,6 +226,8 @@ inline SWp<Dd> sw_params_dual(const nefe_sw_params& p, const double* d) {
 // last place is 2^-32: the sum's low word is the fraction.  Beyond 2^19 boxes (or not finite) the
 // remainder is taken first.
 // ------------------------------------------------------------------------------------
+__device__ __forceinline__ int wrap_sub(int a, int b) { return (int)((unsigned)a - (unsigned)b); }
+__device__ __forceinline__ int wrap_add(int a, int b) { return (int)((unsigned)a + (unsigned)b); }
 __device__ __forceinline__ int frac32(double x, double inv_L) {
     const double magic = 1572864.0;              // 1.5 2^20
     double s = __fma_rn(x, inv_L, magic);
