@@ -439,6 +439,11 @@ NEFE_API int nefe_set_list_tuning(nefe_ctx* ctx, int lanes_per_atom);
  * warp per cell and no system has a Uhlenbeck-Ford term.  NEFE_EINVAL for other values. */
 NEFE_API int nefe_set_cooperative_rebuild(nefe_ctx* ctx, int on);
 
+/* Gives back the device memory that the library's stateless calls keep between calls (at most 256 MB a
+ * device).  Any thread, any time: scratch in use stays valid until its call has ended, and the next call
+ * starts anew.  A host program that resets a device (cudaDeviceReset) calls it before. */
+NEFE_API int nefe_release_scratch(void);
+
 /* Failure detection of the time-bounded grid barrier (the one device-side wait of the library,
  * in the engine's single-launch list rebuild; the paper has no counterpart).  Launches a small
  * grid whose barrier can never complete (it expects one block more than it has), with a limit of

@@ -611,7 +611,7 @@ struct nefe_adj {
     template <typename P>
     cudaError_t alloc(P** p, size_t bytes) {
         void* q = nullptr;
-        cudaError_t e = cudaMalloc(&q, bytes < 16 ? 16 : bytes);
+        cudaError_t e = device_alloc(&q, bytes < 16 ? 16 : bytes);
         if (e == cudaSuccess) owned.push_back(q);
         *p = static_cast<P*>(q);
         return e;

@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <shared_mutex>
 #include <vector>
 
 #include "nefe.h"
@@ -53,41 +54,69 @@ int check_box(const double box[3], double rcs) {
 // The library's scratch pool of a device.  The default pool hands its memory back to the driver
 // at every synchronisation, so each call mapped its scratch anew (457 -> 207 us for a waited-for
 // list and force call of 1723 atoms); this one keeps up to kScratchKeep bytes mapped between calls
-// (anything above goes back at the next synchronisation).  Allocation and release are stream
-// ordered, so calls on several streams and threads share it safely.
+// (anything above goes back at the next synchronisation) until nefe_release_scratch, or until an
+// allocation of the library finds the device full.  Allocation and release are stream ordered, so
+// calls on several streams and threads share it safely; the lock keeps a pool from being destroyed
+// between its look-up and its use (what is allocated from it then stays valid until it is freed).
 constexpr uint64_t kScratchKeep = 256ull << 20;
 constexpr int kPoolDevices = 64;
 
-static std::mutex g_pool_mu;
+static std::shared_mutex g_pool_mu;
 static cudaMemPool_t g_pool[kPoolDevices] = {};
+
+static cudaError_t make_pool(int dev) {
+    std::unique_lock<std::shared_mutex> lock(g_pool_mu);
+    if (g_pool[dev]) return cudaSuccess;
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = cudaMemPoolCreate(&pool, &props);
+    if (e != cudaSuccess) return e;
+    uint64_t keep = kScratchKeep;
+    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e == cudaSuccess) g_pool[dev] = pool;
+    else cudaMemPoolDestroy(pool);
+    return e;
+}
+
+cudaError_t scratch_release() {
+    std::unique_lock<std::shared_mutex> lock(g_pool_mu);
+    cudaError_t first = cudaSuccess;
+    for (cudaMemPool_t& pool : g_pool) {
+        if (!pool) continue;
+        const cudaError_t e = cudaMemPoolDestroy(pool);
+        if (e != cudaSuccess && first == cudaSuccess) first = e;
+        pool = nullptr;
+    }
+    return first;
+}
 
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
     *p = nullptr;
+    if (bytes < 16) bytes = 16;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= kPoolDevices) return cudaMallocAsync(p, bytes < 16 ? 16 : bytes, s);
-    cudaMemPool_t pool;
-    {
-        std::lock_guard<std::mutex> lock(g_pool_mu);
-        if (!g_pool[dev]) {
-            cudaMemPoolProps props;
-            std::memset(&props, 0, sizeof(props));
-            props.allocType = cudaMemAllocationTypePinned;
-            props.handleTypes = cudaMemHandleTypeNone;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = dev;
-            if ((e = cudaMemPoolCreate(&g_pool[dev], &props)) != cudaSuccess) {
-                g_pool[dev] = nullptr;
-                return e;
-            }
-            uint64_t keep = kScratchKeep;
-            e = cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
-            if (e != cudaSuccess) return e;
+    if (dev >= kPoolDevices) return cudaMallocAsync(p, bytes, s);
+    for (;;) {
+        {
+            std::shared_lock<std::shared_mutex> lock(g_pool_mu);
+            if (g_pool[dev]) return cudaMallocFromPoolAsync(p, bytes, g_pool[dev], s);
         }
-        pool = g_pool[dev];
+        if ((e = make_pool(dev)) != cudaSuccess) return e;
     }
-    return cudaMallocFromPoolAsync(p, bytes < 16 ? 16 : bytes, pool, s);
+}
+
+cudaError_t device_alloc(void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    scratch_release();                           // what the pool kept may be what is missing
+    return cudaMalloc(p, bytes);
 }
 
 namespace {
@@ -439,6 +468,12 @@ int nefe_uf_forces(const double* x, int n, const double box[3], double rcs, doub
     if ((rc = read_error(S, &err))) return rc;
     if (err & NEFE_ERR_NBR_OVERFLOW) return fail(NEFE_EOVERFLOW, "nefe_uf_forces: a row exceeded %d", kUfCap);
     if (err & (NEFE_ERR_BOX | NEFE_ERR_CELL)) return fail(NEFE_EINVAL, "nefe_uf_forces: cell grid error");
+    return NEFE_OK;
+}
+
+int nefe_release_scratch(void) {
+    NvtxRange nvtx_("nefe_release_scratch");
+    NEFE_CU(scratch_release());
     return NEFE_OK;
 }
 

@@ -146,7 +146,7 @@ int set_device(nefe_ctx* c) {
 template <typename P>
 int dalloc(nefe_ctx* c, P** p, size_t bytes) {
     void* q = nullptr;
-    cudaError_t e = cudaMalloc(&q, bytes < 16 ? 16 : bytes);
+    cudaError_t e = device_alloc(&q, bytes < 16 ? 16 : bytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     c->allocs.push_back(q);
     *p = static_cast<P*>(q);
@@ -1050,7 +1050,7 @@ static int refine_in_steps(nefe_ctx* c, const std::vector<std::pair<double, int>
     size_t total = 0;
     for (const Blob& x : bl) total += (x.bytes + 255) / 256 * 256;
     char* snap = nullptr;
-    if (cudaMalloc(&snap, total) != cudaSuccess) {
+    if (device_alloc(reinterpret_cast<void**>(&snap), total) != cudaSuccess) {
         cudaGetLastError();
         return NEFE_OK;
     }
@@ -1203,8 +1203,8 @@ int nefe_autotune(nefe_ctx* c) {
     // accumulators); the gather form's pass B is timed below
     const size_t el_ = c->prec == NEFE_FP64 ? sizeof(double) : sizeof(float);
     void *tv0 = nullptr, *tf0 = nullptr;
-    NEFE_CU(cudaMalloc(&tv0, el_ * 3 * c->ntot));
-    NEFE_CU(cudaMalloc(&tf0, 4 * el_ * c->ntot));
+    NEFE_CU(device_alloc(&tv0, el_ * 3 * c->ntot));
+    NEFE_CU(device_alloc(&tf0, 4 * el_ * c->ntot));
     NEFE_CU(cudaMemcpyAsync(tv0, c->d_v, el_ * 3 * c->ntot, cudaMemcpyDeviceToDevice, c->stream));
     Bufs b0 = b;
     b0.v = tv0;
@@ -1247,8 +1247,8 @@ int nefe_autotune(nefe_ctx* c) {
         const size_t el = c->prec == NEFE_FP64 ? sizeof(double) : sizeof(float);
         const size_t v4 = 4 * el;
         void *tv = nullptr, *tf = nullptr;
-        NEFE_CU(cudaMalloc(&tv, el * 3 * c->ntot));
-        NEFE_CU(cudaMalloc(&tf, v4 * c->ntot));
+        NEFE_CU(device_alloc(&tv, el * 3 * c->ntot));
+        NEFE_CU(device_alloc(&tf, v4 * c->ntot));
         NEFE_CU(cudaMemcpyAsync(tv, c->d_v, el * 3 * c->ntot, cudaMemcpyDeviceToDevice, c->stream));
         Bufs bs = b;
         bs.v = tv;

@@ -132,6 +132,10 @@ inline bool valid_uf(const nefe_uf_params* u) {
 
 // Stream-ordered device scratch from the library's own memory pool of the current device.
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+// Gives the pools of all devices back (what is still allocated from them, once it is freed).
+cudaError_t scratch_release();
+// cudaMalloc, which takes back what the pools keep where the device is full.
+cudaError_t device_alloc(void** p, size_t bytes);
 
 // Single-system descriptors and scratch for the stateless calls and the adjoint context: the
 // arrays are collected with want() and carved out of one stream-ordered allocation by commit(),

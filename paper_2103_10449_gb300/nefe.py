@@ -144,6 +144,7 @@ SIGNATURES = {
     "nefe_set_list_tuning": [_vp, ctypes.c_int],
     "nefe_set_rebuild_policy": [_vp, ctypes.c_int],
     "nefe_check_barrier_timeout": [ctypes.c_int, ctypes.c_double],
+    "nefe_release_scratch": [],
     "nefe_set_cooperative_rebuild": [_vp, ctypes.c_int],
     "nefe_get_rebuild_policy": [_vp, _c_int_p],
     "nefe_launch_count": [_vp, ctypes.POINTER(ctypes.c_long)],
@@ -284,6 +285,11 @@ def nefe_sw_dual(x, w, n, box, rcs, nbr, cnt, cap, prm, dtheta, f, fd, out16, st
 def nefe_langevin_noise(seed, sys_id, step, n, precision, xi, stream=None):
     _check(load().nefe_langevin_noise(int(seed), int(sys_id), int(step), int(n), int(precision), _ptr(xi),
                                       _stream(stream)))
+
+
+def nefe_release_scratch():
+    """Gives the device memory that the stateless calls keep between calls back to the driver."""
+    _check(load().nefe_release_scratch())
 
 
 def nefe_check_barrier_timeout(device=0, limit_ms=50.0):

@@ -726,3 +726,20 @@ def test_autotuned_scatter_form_refuses_where_it_always_did(N, kind, error):
     assert lanes == 0
     assert [r["error"] for r in ctx.results_all()] == [error if r == 3 else 0 for r in range(32)]
     ctx.close()
+
+
+# ------------------------------------------------------------------ scratch kept between calls
+def test_scratch_is_given_back(N):
+    """The stateless calls keep up to 256 MB mapped; nefe_release_scratch returns them (a call of 110,592 atoms in FP64
+    wants some 150 MB, of which the list's and the force call's share is kept), twice in a row as well, and the
+    next call finds its scratch again."""
+    x, box = I.diamond(24, 24, 24)
+    x = I.rattle(x, 0.05, 2)
+    first = _sw(N, x, box, _silicon(N), N.NEFE_FP64)
+    torch.cuda.empty_cache()
+    kept = torch.cuda.mem_get_info()[0]
+    N.nefe_release_scratch()
+    assert torch.cuda.mem_get_info()[0] - kept >= 64 << 20
+    N.nefe_release_scratch()
+    again = _sw(N, x, box, _silicon(N), N.NEFE_FP64)
+    assert np.array_equal(first[0], again[0]) and np.array_equal(first[1], again[1])
