@@ -152,7 +152,7 @@ void want1(Scratch1& S, int n, const int n3[3], int prec, bool cells) {
     S.want(&S.acc, sizeof(long long) * 2 * ACC_N * kSlots);     // sums, then their remainders
     S.want(&S.swc, sizeof(SwcBytes));
     const size_t v4 = prec == NEFE_FP64 ? sizeof(double4) : sizeof(float4);
-    S.want(&S.xs, v4 * N);
+    if (cells || prec == NEFE_FP64) S.want(&S.xs, v4 * N);      // (the FP32 force passes read fractions)
     if (cells) {
         const size_t C = (size_t)S.ncells;
         S.want(&S.xa, v4 * N);
@@ -241,7 +241,7 @@ static void want_forces(Scratch1& S, int n, int precision) {
     } else {
         S.want(&S.shd, sizeof(double4) * N * kShell);
         S.want(&S.shj, sizeof(int) * N * kShell);
-        S.want(&S.P, 3 * sizeof(double4) * N);
+        S.want(&S.P, sizeof(double4) * N);
     }
 }
 

@@ -463,7 +463,7 @@ int setup(nefe_ctx* c) {
     if (c->prec == NEFE_FP32 && (rc = dalloc(c, &c->d_spill, (v4 + sizeof(float)) * N * kSpill1))) return rc;
     if ((rc = dalloc(c, &c->d_shj, sizeof(int) * N * (size_t)kShell))) return rc;
     if ((rc = dalloc(c, &c->d_shn, sizeof(int) * N))) return rc;
-    if ((rc = dalloc(c, &c->d_P, 3 * v4 * N))) return rc;
+    if ((rc = dalloc(c, &c->d_P, (c->prec == NEFE_FP64 ? 1 : 3) * v4 * N))) return rc;   // (FP64 sums its virial in pass A)
     if (c->prec == NEFE_FP32) {
         if ((rc = dalloc(c, &c->d_lacc, 4 * sizeof(int) * N))) return rc;
         if ((rc = dalloc(c, &c->d_lacc_hi, 3 * sizeof(long long) * N))) return rc;

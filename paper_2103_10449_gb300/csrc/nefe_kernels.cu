@@ -3276,8 +3276,6 @@ __device__ __forceinline__ void finish_atom(const Bufs& b, const DevSys& S, cons
                                             const T (&pv)[3], const T (&pz)[3], const T* s_xm, T (&red)[14],
                                             bool keep, T (&vo)[3], T (&Fo)[3]);
 template <typename T>
-__device__ __forceinline__ void noise_mean(const Bufs& b, const DevSys& S, int sys, T* s_xm);
-template <typename T>
 __device__ __forceinline__ void noise_mean_staged(const DevSys& S, const long long (*xi)[kSlots], T* s_xm);
 
 template <typename T, int MODE, int L>
@@ -3482,29 +3480,14 @@ __device__ __forceinline__ void finish_atom(const Bufs& b, const DevSys& S, cons
 }
 
 // Per-system mean of this step's thermostat noise (the "zero yes" removal), from the
-// fixed-point sums of k_kick_drift, into s_xm[3].  Threads 0..2 write; the caller syncs.
-// The same mean from the noise sums' slots already copied to shared memory (3 x kSlots).
+// fixed-point sums of k_kick_drift, into s_xm[3]: xi holds their slots, already copied to shared memory
+// (3 x kSlots).  Threads 0..2 write; the caller syncs.
 template <typename T>
 __device__ __forceinline__ void noise_mean_staged(const DevSys& S, const long long (*xi)[kSlots], T* s_xm) {
     if (threadIdx.x < 3) {
         long long sum = 0;
         for (int sl = 0; sl < kSlots; ++sl) sum += xi[threadIdx.x][sl];
         if constexpr (sizeof(T) == 4) {
-            const float hi = (float)(int)(sum >> 32);
-            const float lo = (float)(unsigned)(sum & 0xffffffffLL) * 0x1p-32f;
-            s_xm[threadIdx.x] = (hi + lo) * S.inv_n_f;
-        } else {
-            s_xm[threadIdx.x] = (T)((double)sum / kFix / (double)S.n);
-        }
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void noise_mean(const Bufs& b, const DevSys& S, int sys, T* s_xm) {
-    if (threadIdx.x < 3) {
-        const long long* acc = b.acc + (size_t)sys * ACC_N * kSlots + (size_t)(ACC_XI + threadIdx.x) * kSlots;
-        const long long sum = slot_sum(acc);
-        if constexpr (sizeof(T) == 4) {   // sum 2^-32 / n from its 32-bit halves, FP32 only
             const float hi = (float)(int)(sum >> 32);
             const float lo = (float)(unsigned)(sum & 0xffffffffLL) * 0x1p-32f;
             s_xm[threadIdx.x] = (hi + lo) * S.inv_n_f;

@@ -32,7 +32,7 @@ struct Bufs {
     int* shj;                // [ntot][kShell] shell neighbour indices
     int* shn;                // shell size (FP64: entries, and << 16 those of them outside the cutoff)
     void* spill;             // thread-per-atom pass A: shell entries beyond its shared table, or NULL
-    void* P;                 // [ntot] pass-A force (.w = atom energy), then [ntot][2] its virial (T4)
+    void* P;                 // [ntot] pass-A force (.w = atom energy), then in FP32 [ntot][2] its virial (T4)
     int4* q;                 // unwrapped cell index per axis, from the last build
     int* cell_of;
     int* perm;
