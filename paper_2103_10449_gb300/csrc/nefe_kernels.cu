@@ -3509,8 +3509,10 @@ __device__ __forceinline__ void noise_mean_staged(const DevSys& S, const long lo
 // sums go to ACC_XIN and the rebuild flag to rebuild_next, which the next k_group moves into
 // place.  The last step of every launch sequence runs unfused, so the state between calls is
 // the usual one (positions and velocities at a full step).
+// FP32: nine blocks an SM (56 registers, one spilled on the rare path of the large terms); left to itself the
+// kernel takes 61 and holds eight: 128 x 8000 atoms 82.75 -> 82.15 ms a pass, 64 pairs 64.4 -> 63.95.
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kTile) k_finish(Bufs b, int fuse) {
+__global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 9 : 1) k_finish(Bufs b, int fuse) {
     dep_wait();
     using T4 = typename V4<T>::t;
     const int tile = blockIdx.x + b.tile_base;
