@@ -91,9 +91,9 @@ struct nefe_ctx {
     double* d_trace = nullptr;
     std::vector<void*> allocs;
     int lanes = 8;           // pass A lanes per atom (1 = one thread per atom, 4, 8, 16, 32; 0 = the
-                             // scatter form, whose pass B is k_finish: the FP32 default, faster than
-                             // the gather form at every size (8000 atoms: 36 -> 30 us a step; 256,000
-                             // atoms: 190 -> 110 us)
+                             // scatter form, whose pass B is k_finish: the FP32 default, faster in the
+                             // step than every gather form at every size measured (512 atoms 21.6 -> 19.3 us a
+                             // step against the best of them, 8000 26.0 -> 22.8, 256,000 141 -> 92)
     int glanes = 4;          // pass B lanes per atom (1, 2, 4, 8)
     int llanes = 0;          // list build: 0 one warp per cell; 8, 16, 32 lanes per atom
     int rebuild_all = 0;     // rebuild policy (nefe_set_rebuild_policy)
@@ -1142,7 +1142,7 @@ int nefe_autotune(nefe_ctx* c) {
     int rc = setup(c);
     if (rc) return rc;
     if ((rc = set_device(c))) return rc;
-    if (c->refuse) drop_graph(c);                // what the form refuses is captured in the step graph
+    if (!c->chosen || c->refuse) drop_graph(c);  // the form and what it refuses are captured in the step graph
     c->chosen = c->gchosen = true;
     c->refuse = false;
     c->b.leg_refuse = 0;
@@ -1292,6 +1292,7 @@ int nefe_autotune(nefe_ctx* c) {
         if ((rc = nefe_get_shell_stats(c, &mean, nullptr))) return rc;
         c->refuse = mean <= kRefuseShell;
         c->b.leg_refuse = c->refuse ? 1 : 0;
+        if (c->refuse) drop_graph(c);
     }
     return NEFE_OK;
 }
