@@ -185,7 +185,9 @@ NEFE_API int nefe_neighbor_build(const double* x, int n, const double box[3], do
  *               three-body term to its centre atom).
  *   energy_virial device out [7] or NULL: total energy then the virial W_ab =
  *               sum over terms of sum_legs (x_leg - x_centre)_a f_leg_b as
- *               xx, yy, zz, xy, xz, yz (eV), each summed in FP64.
+ *               xx, yy, zz, xy, xz, yz (eV), summed in fixed point (order independent): FP64 in units
+ *               of 2^-40 eV (2^-32 a block where a thread's share reaches 2^15 eV), FP32 the
+ *               blocks' sums in units of 2^-16 eV.
  *   shell_overflow host out or NULL: 1 if some atom had more than 32 neighbours inside
  *               a*sigma (their forces are then incomplete).  Reading it synchronises.
  * Returns NEFE_EINVAL, NEFE_ENOMEM, NEFE_ECUDA or NEFE_EOVERFLOW (shell overflow).

@@ -2585,9 +2585,11 @@ __device__ __forceinline__ int3 force_of_acc(int4 q) {
 // G: 32 where that gives every SM kScatterFull warps; smaller systems take 16 or 8 atoms to a warp,
 // whose chain of row groups and edge iterations is shorter by as much (8000 atoms: 8.9 -> 6.8 us).
 // A list holds kListEdges edges; atoms whose edges do not fit wait for the next batch.
-// Against the form before: 1,024,000-atom crystal at skin 1.6 A (28 row entries, 5.5 edges an atom)
-// 168 -> 155 us; 1,008,516 atoms of diamond / beta-tin pairs (12.8 edges) 345 -> 253 us; against the
-// gather form's two passes, 96,000 atoms under barostats 73 -> 42 us, 8000 atoms 13.5 -> 11.5 us.
+// Against the forms before, live in the step: 1,024,000-atom crystal at skin 1.6 A (28 row entries, 5.8
+// edges an atom) 171.5 -> 151 us, or 167 with leg_refuse (its screen has the own sums of a warp computed
+// again wherever half a pair force reaches 6 eV/A); 1,008,516 atoms of diamond / beta-tin pairs (12.8
+// edges), with leg_refuse, 308-357 -> 232-255 us; against the gather form's two passes, 96,000 atoms under
+// barostats 85 -> 50 us, 8000 atoms 22.9 -> 19.4.
 constexpr int kListEdges = 224;         // 32 atoms of a crystal hold 186 +- 5; smaller lists leave more L1 and warps
 constexpr int kEdgesDBlocks = 7;         // blocks of k_edges_d an SM holds (shared memory)
 // The atoms of a block of the edge-list kernels: of tile `tile`, from atom `first` on, 2^lg to a warp.
@@ -4224,10 +4226,13 @@ int atoms_per_warp_log2(int precision, int ntot) {
 }
 
 // The last quarter of what the chip holds at once is cut into blocks of half the size, where there is
-// more than that to do: the launch ends on the SMs that drew the last blocks.  192,000 atoms 44.1 ->
-// 41.8 us, 512,000 304.8 -> 297.0, 1,024,000 192.6 -> 190.8, 128,000 in FP64 448 -> 440; a larger share or
-// quarter-size blocks give less, their lists being shorter, and just above one filling (136,000 atoms)
-// it costs 5 %.
+// more than that to do: the launch ends on the SMs that drew the last blocks.  Pass A without and with
+// it: liquid, 192,000 atoms 77.4 -> 74.6 us, 256,000 88.5 -> 86.6, 1,024,000 313.5 -> 309.9; beta-tin 176,000
+// 79.4 -> 76.6, 512,000 179.5 -> 175.3; crystal (skin 1.6 A) 192,000 36.9 -> 36.1, 1,024,000 152.2 -> 151.3; FP64
+// crystal 48,000 158.8 -> 154.6, 128,000 355.6 -> 352.1.  It costs crystals whose last filling is between three
+// quarters and full anyway: 256,000 atoms 38.9 -> 41.1 us, 384,000 55.8 -> 58.2 (liquids and beta-tin gain 2 %
+// there).  A larger share or quarter-size blocks give less, their lists being shorter, and just above one
+// filling (136,000 atoms) it costs 5 %.
 void set_edge_items(Bufs& b, int precision, int lg, int ntiles) {
     const int resident = 152 * (precision == NEFE_FP64 ? kEdgesDBlocks : kScatterBlocks);
     const bool cut = (long long)ntiles << (6 - lg) > resident + resident / 4;
